@@ -92,7 +92,9 @@ typedef struct {
                                   kernel per iteration, one block per system with whole xy planes in
                                   a shared-memory ring (grids whose nx*ny plane fits, about 1800
                                   points); where a plane does not fit, its cluster form (below); where
-                                  neither fits, as 1.  5 = the fused kernel warp-specialised: producer
+                                  neither fits, as 1; before either of them, grids that fit on chip
+                                  run the Lanczos kernel (a thread-block cluster keeps a system's
+                                  real Lanczos vector in shared memory; the same iterates).  5 = the fused kernel warp-specialised: producer
                                   threads form the next plane while consumer threads apply the
                                   stencil (planes of up to ~416 blocks of 2 x 2 points; else as 4).
                                   6 = the fused kernel's cluster form: the 2..8 blocks of a thread-
@@ -100,7 +102,8 @@ typedef struct {
                                   the rows past their band from each other's shared memory, here
                                   with rings small enough for two blocks per SM (else as 4).
                                   0 = automatic: as 4.  rpa_autotune sets it.  The plain FP64 form
-                                  always uses 1; periodic grids run 4 (even nx) or 1. */
+                                  runs the Lanczos kernel (0 and 4, grids that fit) or 1; on periodic
+                                  grids the fused kernel needs even nx (else the Lanczos kernel or 1). */
     int independent_frequencies; /* != 0: every frequency starts from V0 instead of the subspace of
                                   the next higher frequency (no warm start, Algorithm 1 carries it);
                                   with fixed_subspace_iters = 1 E_c is then the Rayleigh-Ritz energy
@@ -163,7 +166,8 @@ typedef struct {
 
 typedef struct {
     long long sternheimer_solves;   /* systems solved */
-    long long cocg_iterations;      /* COCG iterations summed over systems (inner ones for mixed) */
+    long long cocg_iterations;      /* COCG iterations summed over systems (inner ones for mixed;
+                                       Lanczos kernel: steps on real vectors) */
     long long refinement_steps;     /* FP64 residual evaluations summed over systems (mixed) */
     long long stencil_points;       /* grid points x stencil applications in COCG (work measure) */
     int subspace_iterations[64];    /* per frequency, ascending omega */
@@ -327,9 +331,9 @@ rpa_status rpa_coulomb_apply_noalloc(rpa_ctx *ctx, double power, const double *i
  * setting its stencil_shape and z_chunks options.  Candidates 0..5: the two-kernel variants
  * stencil_shape = 1, 2, 3 (columns per thread and threads per block, i.e. the xy tile shape)
  * crossed with one or two z chunks per column, index 2 (stencil_shape - 1) + (z_chunks - 1);
- * candidate 6: the fused single-pass kernel (stencil_shape 4); candidate 7: its warp-specialised
+ * candidate 6: the Lanczos kernel or the fused single-pass kernel (stencil_shape 4); candidate 7: its warp-specialised
  * form (stencil_shape 5); candidate 8: its cluster form with two blocks per SM (stencil_shape 6).
- * The plain FP64 form has one configuration (candidate 0).  times_ms_host (may be NULL) receives RPA_AUTOTUNE_CANDIDATES
+ * The plain FP64 form has candidate 0 and, where the grid fits on chip, 6.  times_ms_host (may be NULL) receives RPA_AUTOTUNE_CANDIDATES
  * timings, -1 for a candidate that does not apply; *chosen_host (may be NULL) the index of the
  * chosen one.  The context's results do not depend on the choice beyond rounding. */
 rpa_status rpa_autotune(rpa_ctx *ctx, double omega, const double *V_dev, int n_r, int *chosen_host,

@@ -12,7 +12,7 @@
 #include <thread>
 #include <vector>
 
-#include "internal.cuh"
+#include "lanczos.cuh"
 
 namespace rpa {
 
@@ -85,7 +85,7 @@ Ctx::~Ctx() {
         cudaFree(muf[a]);
     }
     for (DevBuf *b : {&cocg_state, &cocg_partials, &sys_state, &rhs, &pc_coef, &coul_tmp, &blockA, &blockB,
-                      &blockC, &blockD, &small, &slot_idx, &dense_scratch, &proj_buf, &coef_buf, &blockE})
+                      &blockC, &blockD, &small, &slot_idx, &dense_scratch, &proj_buf, &coef_buf, &blockE, &lanczos_ws})
         b->release();
     if (h_state) cudaFreeHost(h_state);
     if (h_count) cudaFreeHost(h_count);
@@ -130,13 +130,19 @@ int add_queue_stats(Ctx &c, const QueueStats &h) {
     return worst;
 }
 
+// Message of the device's timed-out wait flag (Ctx::d_tc_err).
+static const char *timed_out(int flag) {
+    return flag == 2 ? "a block of the Lanczos kernel timed out waiting for its neighbours"
+                     : "a tensor-core contraction timed out waiting for its MMAs";
+}
+
 void check_tensor_core_status(Ctx &c, cudaStream_t s) {
     int h = 0;
     RPA_CUDA(cudaMemcpyAsync(&h, c.d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, s));
     RPA_CUDA(cudaStreamSynchronize(s));
     if (h) {
         RPA_CUDA(cudaMemsetAsync(c.d_tc_err, 0, sizeof(int), s));
-        fail(RPA_ERR_CUDA, "a tensor-core contraction timed out waiting for its MMAs");
+        fail(RPA_ERR_CUDA, "%s", timed_out(h));
     }
 }
 
@@ -297,7 +303,7 @@ int finish_call(Ctx &c, cudaStream_t s) {
     std::memcpy(&tcerr, c.h_rb + kRbTc, sizeof(int));
     if (tcerr) {
         RPA_CUDA(cudaMemsetAsync(c.d_tc_err, 0, sizeof(int), s));
-        fail(RPA_ERR_CUDA, "a tensor-core contraction timed out waiting for its MMAs");
+        fail(RPA_ERR_CUDA, "%s", timed_out(tcerr));
     }
     QueueStats q;
     std::memcpy(&q, c.h_rb + kRbStats, sizeof q);
@@ -494,11 +500,13 @@ rpa_status rpa_autotune(rpa_ctx *ctx, double omega, const double *V_dev, int n_r
         double *t2 = (double *)c.blockB.ensure(blk);
         double *R = (double *)c.blockC.ensure(blk);
         // candidates 0..5: split kernel variant v (stencil_shape v + 1) with z chunks z + 1, index
-        // 2 v + z; candidate 6: the fused single-pass kernel (stencil_shape 4), candidate 7 its
+        // 2 v + z; candidate 6: the on-chip Lanczos kernel or the fused single-pass kernel
+        // (stencil_shape 4; the plain form: the Lanczos kernel where it applies), candidate 7 its
         // warp-specialised form (stencil_shape 5), where a plane fits; candidate 8 its cluster form
         // with two blocks per SM (stencil_shape 6), where the plane's bands fit
         const bool mixed = c.opt.prec == RPA_MIXED;
-        const bool fused_ok = mixed && fused_kernel_applies(c);
+        LanczosPlan lz{};
+        const bool fused_ok = lanczos_plan(c, n_r * c.ns, lz) || (mixed && fused_kernel_applies(c));
         const bool ws_ok = mixed && fused_kernel_applies(c, true);
         const bool cl_ok = mixed && fused_kernel_applies(c, false, true);
         double best = 1e300;
@@ -762,14 +770,17 @@ rpa_status rpa_ec_gradient(rpa_ctx *ctx, int n_r, const double *V0_dev, double *
             fail(RPA_ERR_INVALID, "rpa_ec_gradient differentiates the Rayleigh-Ritz energy: set sq_order = 0");
         const int saved = c.opt.project_solution;
         c.opt.project_solution = 1;
+        c.keep_cocg = V_out_dev != nullptr;
         try {
             worst = ec_impl(c, n_r, V0_dev, lambdas_host, ec_host, ec_per_omega_host, stats, as_stream(stream),
                             grad_dev, V_out_dev);
         } catch (...) {
             c.opt.project_solution = saved;
+            c.keep_cocg = false;
             throw;
         }
         c.opt.project_solution = saved;
+        c.keep_cocg = false;
     });
     if (st != RPA_OK) return st;
     if (worst != RPA_OK) g_last_error = "a Sternheimer system did not converge";

@@ -30,6 +30,7 @@
 #include <cooperative_groups.h>
 
 #include "internal.cuh"
+#include "lanczos.cuh"
 
 namespace rpa {
 
@@ -48,24 +49,6 @@ constexpr int kWarpsPerBlock = kThreads / 32;
 // ~N_d^-1/2 >= 1e-3, so this is rare in a healthy solve.
 constexpr double kNearBreak = 1e-5;
 
-enum Phase : int { kEmpty = 0, kInner = 1, kInnerDone = 2, kFinished = 3, kLoading = 4 };
-
-struct Slot {
-    double rho_re[2], rho_im[2];    // r^T r of the last two iterations (by parity of the iteration)
-    double alpha_re, alpha_im, beta_re, beta_im;
-    double shift_re, shift_im;
-    double bnorm, ref_norm, rnorm;  // ||b||; inner solve: norms of the scaled FP32 residual
-    double scale;                   // mixed: the FP32 inner solve works on scale * (b - A x64)
-    int phase, sys, n, j;
-    int iters, total_iters, refines, status;
-    int discard;                    // mixed: the inner solve went non-finite; its correction is dropped
-    int nearbreak;                  // mixed: inner solves ended at a near-breakdown
-};
-
-template <typename T> struct Cx;
-template <> struct Cx<float> { using t = float2; };
-template <> struct Cx<double> { using t = double2; };
-
 struct Grid3 {
     int nx, ny, nz;
     long long nd;
@@ -76,16 +59,6 @@ struct Grid3 {
 __device__ __forceinline__ int wrap_index(int a, int n) {
     a %= n;
     return a < 0 ? a + n : a;
-}
-
-template <typename T> struct Coef {
-    T a[kRadius + 1];
-};
-
-template <typename T> Coef<T> cast_coef(const StencilCoef &c) {
-    Coef<T> r;
-    for (int k = 0; k <= kRadius; ++k) r.a[k] = (T)c.a[k];
-    return r;
 }
 
 // Everything the kernels need, passed by value.
@@ -2854,7 +2827,14 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
                        (!ring1 && cluster_plan(c.nx, c.ny, smem_optin, false, ncl, band_pairs)));
     const RingFn ring_fn = ws ? (even_nx ? k_cocg_ring_ws<true> : k_cocg_ring_ws<false>)
                               : clus ? (even_nx ? k_cocg_ring_cl<true> : k_cocg_ring_cl<false>) : ring1_fn;
-    const bool use_ring = mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
+    // systems that fit on chip: the Lanczos kernel
+    if (c.lz_key[0] != S || c.lz_key[1] != c.opt.prec) {
+        c.lz_ok = lanczos_plan(c, S, c.lz_plan);
+        c.lz_key[0] = S;
+        c.lz_key[1] = c.opt.prec;
+    }
+    const bool use_lz = c.lz_ok && !precond && !c.keep_cocg && (want == 0 || want == 4);
+    const bool use_ring = !use_lz && mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
     const int variant = (want >= 1 && want <= 3 && !(per && want == 3)) ? want - 1 : 0;
     const PaShape shape = mixed ? kPaShapes32[variant] : kPaShape64;
     Tiles tl = pick_tiles(c.nx, c.ny, shape.max_threads, shape.pairs != 0);
@@ -3031,6 +3011,26 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         }
     }
 
+    LanczosArgs<float> lz32{};
+    LanczosArgs<double> lz64{};
+    if (use_lz) {
+        c.lz_plan.ws = c.lanczos_ws.ensure(c.lz_plan.ws_bytes);
+        auto fill = [&](auto &a) {
+            a.slots = slots;
+            a.list = list;                 // built by k_ring_list, which also clears the counter
+            a.cnt = cnt;
+            a.grab = cnt + 1;
+        };
+        fill(lz32);
+        fill(lz64);
+        lz32.r = (const float2 *)r;
+        lz32.x = (float2 *)xin;
+        lz32.vloc = c.vloc32;
+        lz64.r = (const double2 *)r;
+        lz64.x = x64;
+        lz64.vloc = c.vloc64;
+    }
+
     // the Laplacian preconditioner: z = M r in three passes (see k_pc_xy, k_pc_z)
     PcArgs<float> pc32{};
     PcArgs<double> pc64{};
@@ -3100,7 +3100,10 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     const char *tn = mixed ? "c64" : "c128";
     char names[3][32];
     std::snprintf(names[0], 32, "-");
-    if (use_ring) {
+    if (use_lz) {
+        std::snprintf(names[1], 32, "k_lanczos<%s>", mixed ? "f32" : "f64");
+        std::snprintf(names[2], 32, "-");
+    } else if (use_ring) {
         std::snprintf(names[1], 32, ws ? "k_cocg_ring_ws<%s>" : clus ? "k_cocg_ring_cl<%s>" : "k_cocg_ring<%s>", tn);
         std::snprintf(names[2], 32, "-");
     } else {
@@ -3112,12 +3115,14 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     // and writes x, r; the fused kernel reads and writes x, r, p, q, except in the first sweep of an
     // inner solve, which reads r and writes p, q (V is read once per plane and block, not per system,
     // and is not counted)
-    const double bytes_per_point[3] = {0.0, use_ring ? 8 * csz : 4 * csz + rsz, use_ring ? 0.0 : 6 * csz};
+    // the Lanczos kernel writes and reads every vector once
+    const double bytes_per_point[3] = {0.0, use_lz ? 2 * rsz : use_ring ? 8 * csz : 4 * csz + rsz,
+                                       use_lz || use_ring ? 0.0 : 6 * csz};
     if (prof) {
         RPA_CUDA(cudaMemsetAsync(c.d_prof_points, 0, sizeof(unsigned long long) * 3, st));
         P.prof = c.d_prof_points;
         for (int par = 0; par < 2; ++par) ia_pa[par].prof = ia_b[par].prof = c.d_prof_points;
-        ra.prof = c.d_prof_points;
+        ra.prof = lz32.prof = lz64.prof = c.d_prof_points;
     }
     // Two graph instances of one epoch (alternating, so that the events of one can be read while
     // the other runs); without graphs the same launches go straight to the stream.
@@ -3179,6 +3184,16 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
             if (capturing) RPA_CUDA(cudaEventRecordWithFlags(e, ss, cudaEventRecordExternal));
             else RPA_CUDA(cudaEventRecord(e, ss));
         };
+        if (use_lz) {
+            k_ring_list<<<1, 1024, 0, ss>>>(P);
+            rec(0);
+            if (mixed) lanczos_launch(c, c.lz_plan, lz32, ss);
+            else lanczos_launch(c, c.lz_plan, lz64, ss);
+            rec(1);
+            RPA_LAUNCH("inner solves (Lanczos)");
+            maintenance(ss);
+            return;
+        }
         if (use_ring) {
             k_ring_list<<<1, 1024, 0, ss>>>(P);
             rec(0);
@@ -3238,7 +3253,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         maintenance(ss);
     };
     const int per_maint = (mixed ? 8 : 5) + (P.project ? 2 : 0) + (P.cproject ? 5 : 0);
-    const int per_epoch = (use_ring ? 2 : (precond ? 7 : 4) * kEpoch) + per_maint;
+    const int per_epoch = (use_lz || use_ring ? 2 : (precond ? 7 : 4) * kEpoch) + per_maint;
 
     // device-driven queue: CUDA graphs, no profiling, no per-system outputs wanted
     const bool device_loop = use_graph && !prof && !iters_out && !status_out;
@@ -3262,7 +3277,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     auto collect_epoch = [&](long long k) {
         if (!prof) return;
         const int set = (int)(k & 1);
-        for (int t = 0; t < (use_ring ? 1 : kTimed); ++t) {   // the fused kernel: one timed launch
+        for (int t = 0; t < (use_lz || use_ring ? 1 : kTimed); ++t) {   // the fused kernels: one timed launch
             float ms = 0.f;
             RPA_CUDA(cudaEventElapsedTime(&ms, evs[((size_t)set * kTimed + t) * 2], evs[((size_t)set * kTimed + t) * 2 + 1]));
             prof_ms[1 + t % 2] += ms;
@@ -3340,6 +3355,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         ++checked;
     }
     sync_stream(c, st);
+    if (use_lz) check_tensor_core_status(c, st);
     while (checked < issued) collect_epoch(checked++);
     for (auto &e : ev) cudaEventDestroy(e);
     for (int g = 0; g < 2; ++g)
@@ -3349,7 +3365,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     if (prof) {
         unsigned long long pts[3];
         RPA_CUDA(cudaMemcpy(pts, c.d_prof_points, sizeof pts, cudaMemcpyDeviceToHost));
-        for (int k = 1; k < (use_ring ? 2 : 3); ++k) {
+        for (int k = 1; k < (use_lz || use_ring ? 2 : 3); ++k) {
             const int sl = prof_slot(c, names[k]);
             c.stats.prof_ms[sl] += prof_ms[k];
             c.stats.prof_launches[sl] += prof_n[k];

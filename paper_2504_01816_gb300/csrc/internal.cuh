@@ -83,6 +83,17 @@ struct QueueStats {
     int unfinished;     // a queue stopped at its epoch bound with systems left
 };
 
+// How a queue's systems are spread over the SMs by the Lanczos kernel (lanczos.cu): a cluster of
+// ncl blocks per system, `clusters` of them resident, each thread with W x 2 x zc points (W = 16 bytes).
+struct LanczosPlan {
+    int variant, mixed, zc, ncl, clusters, threads;
+    int hw, hh, nch;               // units per row, row pairs, z chunks of a block
+    int pitch, plane, lead;        // elements of a slab row and plane, and before the first plane
+    int reach, hist;
+    size_t smem, ws_stride, ws_bytes;
+    void *ws;                      // ws_bytes of workspace, set by the caller
+};
+
 struct BatchCoord;   // rendezvous of rpa_ec_batch's threads (api.cu)
 
 // ------------------------------------------------------------------------------------------
@@ -130,10 +141,19 @@ struct Ctx {
     DevBuf coef_buf;              // per-column coefficients of the gradient pass
     DevBuf blockE;                // subspace of the previous iteration (gradient)
     DevBuf dense_scratch;         // split-K partial sums
+    DevBuf lanczos_ws;            // Lanczos vectors of the systems in flight
+    LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, prec}
+    int lz_key[2] = {-1, -1};
+    bool lz_ok = false;
+    // rpa_ec_gradient with the final subspace as an output runs the COCG kernels: a subspace is R L^-T
+    // with the conditioning of R, and after the exact integer pieces of the tensor-core contractions
+    // (whose last digits turn on 1e-12 of their operands) the Lanczos kernel's rounding moves it by
+    // 2e-9 relative, more than a change of kernels may; the energies and the gradient move by 1e-10.
+    bool keep_cocg = false;
     SysState *h_state = nullptr;  // pinned host mirror of the slot states
     size_t h_state_cap = 0;
     int *h_count = nullptr;       // pinned host counter
-    int *d_tc_err = nullptr;      // set by a tensor-core contraction that gave up waiting on its MMAs
+    int *d_tc_err = nullptr;      // set by a kernel that gave up waiting: 1 a tensor-core contraction, 2 Lanczos
     QueueStats *d_qstats = nullptr;   // device accumulator of queue statistics
     int *d_loop = nullptr;            // epoch counter of a device-driven queue
     char *h_rb = nullptr;             // pinned read-back block (Ritz values, scalars, statistics)
@@ -171,7 +191,7 @@ inline bool use_tensor_cores(const Ctx &c) {
 inline bool use_tensor_cores_kronecker(const Ctx &c) {
     return c.opt.contractions == 2 || (c.opt.contractions == 0 && c.opt.prec == RPA_MIXED);
 }
-// Fails with RPA_ERR_CUDA if a tensor-core contraction reported a timed-out wait (synchronises s).
+// Fails with RPA_ERR_CUDA if a kernel reported a timed-out wait (synchronises s).
 void check_tensor_core_status(Ctx &c, cudaStream_t s);
 void coulomb_setup(Ctx &c);
 // Same operator with its scratch in the library's fixed device array (no allocation).

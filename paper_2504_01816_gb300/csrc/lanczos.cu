@@ -1,0 +1,1188 @@
+// Sternheimer inner solves by real Lanczos recurrences, a whole system on chip (arXiv 2504.01816:
+// Sternheimer equation, Eq. 9; COCG, Section "Implementation").
+//
+// COCG for (B + i w) x = b with B = H - eps_n real symmetric and a real b builds its iterates in the
+// real Krylov space of B and b: its residuals are complex multiples of the real Lanczos vectors v_k
+// of B.  This kernel runs the Lanczos recurrence itself,
+//     u = B v_k - c_k v_{k-1},  a_k = u.v_k / v_k.v_k,  v_{k+1} = (u - a_k v_k) / g_{k+1},  c_k = g_k,
+// and takes the COCG iterate from the LU factors of the tridiagonal T + i w (d_k = a_k + i w -
+// g_k c_k / d_{k-1}, z_k = -g_k z_{k-1} / d_{k-1}, ||r_k|| = g_{k+1} |z_k / d_k|): the same iterates as
+// COCG for half the stencil arithmetic and half the state.  |d_k| >= |w|, so for w != 0 the factors
+// cannot break down.  A complex right-hand side r (the residual of a refinement) is turned to
+// e^{-i phi} r = r_a + i r_b with r_a.r_b = 0 and ||r_a|| largest, and its two real parts are solved one
+// after the other; after a first inner solve r_b is the rounding noise of that solve (1e-3..1e-2 of
+// r_a) and takes a third of r_a's steps.
+//
+// A thread-block cluster of C blocks owns one system at a time.  Block c keeps the planes
+// [c nz / C, (c + 1) nz / C) of v_k with six halo planes on either side in shared memory; v_{k-1}, u and
+// v_{k+1} share one register array (each thread owns W x 2 x ZC points: W = 16 bytes of x, two rows, ZC
+// planes), so an iteration reads nothing from memory but V_loc (from L2) and writes only v_k, by a bulk
+// copy from shared memory, kept for the solution x = sum_k y_k v_k.  That sum is formed at the end, with
+// the vectors streamed back through the slab (or, when the history is full, by plain loads, and then with
+// the COCG direction p handed over).  Between blocks an iteration has two dependences and no cluster
+// barrier: the halo planes arrive by bulk copies through distributed shared memory that count on the
+// receiver's mbarrier, and overlap the x and y neighbours' part of the stencil; the three dot products are
+// sent to every block with st.async, which also tells a block that its neighbours' halos may be
+// overwritten.  Every block of a cluster computes the same scalars from the same sums in the same order,
+// so all take the same decisions.  The factors, the stopping test and the slot's state belong to an extra
+// warp that works while the others compute the next stencil; a solve therefore ends one stencil late.
+//
+// What bounds it: shared-memory loads.  A unit of W x 2 points and ZC planes takes 2 (ZC + 12) 16-byte
+// loads for the z neighbours of all its planes (held against the ZC accumulators in turn), and per
+// plane 12 for the y and 2 XL for the x neighbours: 58 bytes a point for ZC = 5 in FP32 against 240 for
+// a plane-by-plane march on complex values; the FP64 form is bound by the FP64 pipe (46 operations a
+// point).  Measured (GB300, tol 1e-11, whole chi0 application, against the fused and split COCG kernels):
+// 40^3, 1024 systems 212 -> 125 ms; 24^3, 4 systems 9.8 -> 2.1 ms; 37 x 43 x 29, 77 systems 25 -> 8.5 ms;
+// FP64 15^3, 32 systems 15.9 -> 3.2 ms, 32^3, 128 systems 197 -> 92 ms.  At 40^3 (four blocks a system) an
+// iteration takes 22.6 thousand cycles: x and y neighbours 9.2 (5.7 of shared-memory loads and 2.5 of
+// copies), z neighbours 3.0, halo 1.1, sums 2.1, update 2.7, and per iteration of a solve 3.8 for the
+// solution and 1.2 for the start.  One form with 64-bit index arithmetic per halo store took 230 ms, one
+// with cluster barriers 138 ms, one with the solution's code inlined (spills) 158 ms.
+#include <algorithm>
+#include <cmath>
+
+#include "lanczos.cuh"
+
+namespace rpa {
+
+namespace {
+
+constexpr int kHistMax = 128;            // Lanczos vectors kept between two updates of x
+
+constexpr int kStages = 4;               // vectors of the history in flight at the end of a solve
+
+// W values of one row: 16 bytes.
+template <typename T> struct Pk;
+template <> struct Pk<float> {
+    static constexpr int W = 4;
+    float2 p[2];
+    __device__ __forceinline__ float get(int i) const { return i & 1 ? p[i >> 1].y : p[i >> 1].x; }
+    __device__ __forceinline__ void set(int i, float v) { (i & 1 ? p[i >> 1].y : p[i >> 1].x) = v; }
+    __device__ __forceinline__ void fma(float c, const Pk &v) {
+        const float2 cc = make_float2(c, c);
+        p[0] = __ffma2_rn(cc, v.p[0], p[0]);
+        p[1] = __ffma2_rn(cc, v.p[1], p[1]);
+    }
+    __device__ __forceinline__ void fma(const Pk &c, const Pk &v) {
+        p[0] = __ffma2_rn(c.p[0], v.p[0], p[0]);
+        p[1] = __ffma2_rn(c.p[1], v.p[1], p[1]);
+    }
+    __device__ __forceinline__ void mul(float c) {
+        const float2 cc = make_float2(c, c);
+        p[0] = __fmul2_rn(cc, p[0]);
+        p[1] = __fmul2_rn(cc, p[1]);
+    }
+    __device__ __forceinline__ void mul(const Pk &c) {
+        p[0] = __fmul2_rn(c.p[0], p[0]);
+        p[1] = __fmul2_rn(c.p[1], p[1]);
+    }
+    __device__ __forceinline__ float sum() const { return (p[0].x + p[0].y) + (p[1].x + p[1].y); }
+    __device__ __forceinline__ void zero() { p[0] = p[1] = make_float2(0.f, 0.f); }
+};
+template <> struct Pk<double> {
+    static constexpr int W = 2;
+    double2 p;
+    __device__ __forceinline__ double get(int i) const { return i ? p.y : p.x; }
+    __device__ __forceinline__ void set(int i, double v) { (i ? p.y : p.x) = v; }
+    __device__ __forceinline__ void fma(double c, const Pk &v) {
+        p.x = ::fma(c, v.p.x, p.x);
+        p.y = ::fma(c, v.p.y, p.y);
+    }
+    __device__ __forceinline__ void fma(const Pk &c, const Pk &v) {
+        p.x = ::fma(c.p.x, v.p.x, p.x);
+        p.y = ::fma(c.p.y, v.p.y, p.y);
+    }
+    __device__ __forceinline__ void mul(double c) {
+        p.x *= c;
+        p.y *= c;
+    }
+    __device__ __forceinline__ void mul(const Pk &c) {
+        p.x *= c.p.x;
+        p.y *= c.p.y;
+    }
+    __device__ __forceinline__ double sum() const { return p.x + p.y; }
+    __device__ __forceinline__ void zero() { p = make_double2(0.0, 0.0); }
+};
+__device__ __forceinline__ Pk<float> pk_load(const float *a) {
+    const float4 t = *reinterpret_cast<const float4 *>(a);
+    Pk<float> r;
+    r.p[0] = make_float2(t.x, t.y);
+    r.p[1] = make_float2(t.z, t.w);
+    return r;
+}
+__device__ __forceinline__ Pk<double> pk_load(const double *a) {
+    Pk<double> r;
+    r.p = *reinterpret_cast<const double2 *>(a);
+    return r;
+}
+// The same from the history, past L1: the bulk stores that write it do not update L1's lines.
+__device__ __forceinline__ Pk<float> pk_load_l2(const float *a) {
+    const float4 t = __ldcg(reinterpret_cast<const float4 *>(a));
+    Pk<float> r;
+    r.p[0] = make_float2(t.x, t.y);
+    r.p[1] = make_float2(t.z, t.w);
+    return r;
+}
+__device__ __forceinline__ Pk<double> pk_load_l2(const double *a) {
+    Pk<double> r;
+    r.p = __ldcg(reinterpret_cast<const double2 *>(a));
+    return r;
+}
+__device__ __forceinline__ void pk_store(float *a, const Pk<float> &v) {
+    *reinterpret_cast<float4 *>(a) = make_float4(v.p[0].x, v.p[0].y, v.p[1].x, v.p[1].y);
+}
+__device__ __forceinline__ void pk_store(double *a, const Pk<double> &v) { *reinterpret_cast<double2 *>(a) = v.p; }
+__device__ __forceinline__ unsigned map_rank(unsigned addr, int rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    __syncwarp();                        // the aligned forms need the warp together
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void mbar_init(unsigned long long *b) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(b)) : "memory");
+}
+// Wait for a phase of an mbarrier; false after ~1 s of cycles.
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+    const long long t0 = clock64();
+    for (;;) {
+        unsigned done;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+        if (clock64() - t0 > 2000000000LL) return false;
+    }
+}
+
+// acc += sum_d cf[d] (x - d and x + d neighbours) for W values; X holds the row from x - PAD on.
+__device__ __forceinline__ void x_part(Pk<float> &acc, const Pk<float> (&X)[5], const Coef<float> &cf) {
+    auto at = [&](int o) -> float { return X[(8 + o) >> 2].get((8 + o) & 3); };
+    auto pr = [&](int o) -> float2 { return X[(8 + o) >> 2].p[((8 + o) & 3) >> 1]; };   // o even
+#pragma unroll
+    for (int d = 1; d <= kRadius; ++d) {
+        if (d & 1) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc.set(i, fmaf(cf.a[d], at(i - d) + at(i + d), acc.get(i)));
+        } else {
+            const float2 c = make_float2(cf.a[d], cf.a[d]);
+#pragma unroll
+            for (int i = 0; i < 2; ++i) acc.p[i] = __ffma2_rn(c, __fadd2_rn(pr(2 * i - d), pr(2 * i + d)), acc.p[i]);
+        }
+    }
+}
+__device__ __forceinline__ void x_part(Pk<double> &acc, const Pk<double> (&X)[7], const Coef<double> &cf) {
+    auto at = [&](int o) -> double { return X[(6 + o) >> 1].get((6 + o) & 1); };
+#pragma unroll
+    for (int d = 1; d <= kRadius; ++d)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) acc.set(i, ::fma(cf.a[d], at(i - d) + at(i + d), acc.get(i)));
+}
+
+// Three sums into a block of the cluster, counted on its barrier.
+__device__ __forceinline__ void send_sums(unsigned to, unsigned bar, float a, float b, float c) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(to),
+                 "f"(a), "f"(b), "f"(c), "f"(0.f), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void send_sums(unsigned to, unsigned bar, double a, double b, double c) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(to), "d"(a),
+                 "d"(b), "r"(bar)
+                 : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f64 [%0], {%1, %2}, [%3];" ::"r"(to + 16),
+                 "d"(c), "d"(0.0), "r"(bar)
+                 : "memory");
+}
+
+template <typename T> struct Vec4;
+template <> struct Vec4<float> { using t = float4; };
+template <> struct Vec4<double> { using t = double4_16a; };
+
+// The scalar lane's state of a solve (in shared memory: the other threads' registers hold points).
+struct ScalarState {
+    double dr, di;                       // 1 / d_{k-1}
+    double zr, zi;                       // z_{k-1}
+    double gam;                          // g_k
+    double ak, ck, ig;                   // the step whose factors are pending: a_k, c_k, 1 / g_{k+1}
+    double thr, d0, w, rn2;              // threshold, diagonal of B but V_loc, omega, sum of ||r||^2
+    int sweeps, fail;                    // fail: 1 limit, 2 breakdown, 3 non-finite
+};
+
+// Shared memory of a block, before its slab of planes.
+template <typename T> struct Shared {
+    using V4 = typename Vec4<T>::t;
+    V4 coef[kHistMax];                   // y_j (re, im), direction coefficient (re, im)
+    V4 prev;                             // the same for the direction handed over
+    T part[2][16][4];                    // the blocks' sums of a reduction (alternating)
+    T red[3][32];
+    T vec[4];                            // a', 1/g, g (FP64)
+    double dr[kHistMax], di[kHistMax], zr[kHistMax], zi[kHistMax], g[kHistMax];   // factors by history place
+    double start[4];                     // cos phi, sin phi, ||r_a||, ||r_b||
+    ScalarState F;
+    unsigned long long bar, pbar[2], fbar[kStages];   // arrival of the halo, of the sums, of a vector
+    unsigned fphase;                     // phase of each fbar
+    int item, flag;
+    int nto, to[4 * 12];                 // the copies that fill the neighbours' halos
+    unsigned expect;                     // bytes that arrive in this block's halo
+    LanczosArgs<T> A;                    // for the functions off the hot path
+};
+template <typename T> constexpr int shared_bytes() { return (int)((sizeof(Shared<T>) + 127) / 128 * 128); }
+
+extern __shared__ __align__(128) unsigned char lz_smem[];
+template <typename T> __device__ __forceinline__ Shared<T> &sh() { return *reinterpret_cast<Shared<T> *>(lz_smem); }
+
+// A thread's points: W values of x from gx, rows gy and gy + 1, local planes lz0 .. lz0 + ZC - 1.
+template <typename T, int ZC> struct Geo {
+    static constexpr int W = Pk<T>::W, PAD = W == 4 ? 8 : 6;   // PAD: elements before a row, at least the radius
+    int rank, z0, nzl;                   // the block's planes
+    bool unit, row1;                     // has points; row gy + 1 lies inside the box
+    int gx, gy, lz0, nvx, nvz;           // nvx, nvz: points of a row, planes inside the box
+    int c0, c1;                          // its rows' first points in the slab (plane lz0)
+    int nthr;                            // threads that may hold points
+    __device__ __forceinline__ Geo(const LanczosArgs<T> &A) {
+        const int tid = threadIdx.x, per_chunk = A.hw * A.hh;
+        rank = (int)(blockIdx.x % (unsigned)A.ncl);
+        z0 = rank * A.nz / A.ncl;
+        nzl = (rank + 1) * A.nz / A.ncl - z0;
+        unit = tid < per_chunk * A.nch;
+        const int ch = unit ? tid / per_chunk : 0;
+        const int by = unit ? (tid - ch * per_chunk) / A.hw : 0;
+        gx = unit ? W * (tid - ch * per_chunk - by * A.hw) : 0;
+        gy = 2 * by;
+        lz0 = ch * ZC;
+        nvx = min(W, A.nx - gx);
+        row1 = gy + 1 < A.ny;
+        nvz = unit ? max(0, min(ZC, nzl - lz0)) : 0;
+        c0 = (lz0 + kRadius) * A.plane + gy * A.pitch + PAD + gx;
+        c1 = row1 ? c0 + A.pitch : c0;
+        nthr = (int)blockDim.x - 32;
+    }
+    // private 16-byte place of (z, r) in a vector of the workspace, in elements
+    __device__ __forceinline__ size_t priv(int z, int r) const { return ((size_t)(2 * z + r) * nthr + threadIdx.x) * W; }
+    // index of the row's first point on the grid
+    __device__ __forceinline__ long long grid(const LanczosArgs<T> &A, int z, int r) const {
+        return ((long long)(z0 + lz0 + z) * A.ny + gy + r) * A.nx + gx;
+    }
+};
+// The block's arrays in the workspace: V_loc, the direction (re, im), the history (laid out as in the slab).
+template <typename T, int ZC> struct Work {
+    T *V, *Pd, *H;
+    size_t vec, hvec;
+    __device__ __forceinline__ Work(const LanczosArgs<T> &A) {
+        vec = (size_t)2 * ZC * (blockDim.x - 32) * Pk<T>::W;
+        hvec = (size_t)A.nch * ZC * A.plane;
+        V = A.ws + (size_t)blockIdx.x * A.ws_stride;
+        Pd = V + vec;
+        H = Pd + 2 * vec;
+    }
+};
+template <typename T> __device__ __forceinline__ T *slab_of(const LanczosArgs<T> &A) {
+    return reinterpret_cast<T *>(lz_smem + shared_bytes<T>()) + A.lead;   // after the zero word or the first rows of zeros
+}
+
+// W values of a row into the slab (periodic: and the images past the row's ends).
+template <typename T, int MODE>
+__device__ __forceinline__ void put(T *own, int gx, int nvx, int nx, const Pk<T> &v) {
+    constexpr int W = Pk<T>::W, PAD = W == 4 ? 8 : 6;
+    if (nvx == W) {
+        pk_store(own, v);
+    } else {
+        for (int i = 0; i < nvx; ++i) own[i] = v.get(i);
+    }
+    if (MODE == 1) {
+        if (nx % W == 0) {
+            if (gx < PAD) pk_store(own + nx, v);
+            if (gx >= nx - PAD) pk_store(own - nx, v);
+        } else {
+            for (int i = 0; i < nvx; ++i) {
+                const int x = gx + i;
+                if (x < kRadius) own[i + nx] = v.get(i);
+                if (x >= nx - kRadius) own[i - nx] = v.get(i);
+            }
+        }
+    }
+}
+
+// The block's own planes are stored: before the bulk copies read them.
+__device__ __forceinline__ void planes_stored() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+}
+// The planes to the halos of the blocks that need them (one bulk copy a block and side), by the scalar
+// lane once they are stored and no block reads its last halo any more; the phase of sh().bar is complete
+// when this block's own halo has arrived.
+template <typename T> __device__ __forceinline__ void send_halos(T *slab) {
+    Shared<T> &S = sh<T>();
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(&S.bar), base = (unsigned)__cvta_generic_to_shared(slab);
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(S.expect) : "memory");
+    for (int e = 0; e < S.nto; ++e) {
+        const int t = S.to[4 * e];
+        asm volatile(
+            "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                map_rank(base, t) + (unsigned)S.to[4 * e + 1]),
+            "r"(base + (unsigned)S.to[4 * e + 2]), "r"(S.to[4 * e + 3]), "r"(map_rank(bar, t))
+            : "memory");
+    }
+}
+// The block's planes to place h of the history, by the scalar lane once they are stored; they may change
+// again after keep_wait.
+template <typename T> __device__ __forceinline__ void keep(const T *slab, T *H, size_t hvec, int h, int nzl, int plane) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                     __cvta_generic_to_global(H + (size_t)h * hvec)),
+                 "r"((unsigned)__cvta_generic_to_shared(slab + kRadius * plane)), "r"(nzl * plane * (int)sizeof(T))
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void keep_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
+// Block sums of three values per thread, all-gathered over the cluster into part[ng & 1]: every block
+// sends its sums to all (st.async, which counts on the receiver's barrier) and waits for all.  A block
+// sends only after all its threads are done with the stencil, so the wait also says that no block reads
+// its halo any more.  The sums alternate between two buffers and barriers: a block may be one
+// reduction ahead of another, never two.
+template <typename T> __device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int *err) {
+    Shared<T> &S = sh<T>();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (int)(blockDim.x >> 5);
+    T v[3] = {a, b, c};
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) S.red[q][warp] = v[q];
+    __syncthreads();
+    const unsigned pb = (unsigned)__cvta_generic_to_shared(&S.pbar[ng & 1]);
+    if (warp == 0) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) v[q] = lane < nwarp ? S.red[q][lane] : (T)0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+        if (lane == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(pb),
+                         "r"((unsigned)(ncl * 4 * (int)sizeof(T)))
+                         : "memory");
+        if (lane < ncl)
+            send_sums(map_rank((unsigned)__cvta_generic_to_shared(&S.part[ng & 1][rank][0]), lane), map_rank(pb, lane),
+                      v[0], v[1], v[2]);
+        __syncwarp();
+    }
+    if (!mbar_wait(pb, (ng >> 1) & 1)) atomicExch(err, 2);
+    ++ng;
+}
+template <typename T> __device__ __forceinline__ void sum_parts(unsigned ng, int ncl, T &a, T &b, T &c) {   // after gather3
+    const T(&pp)[16][4] = sh<T>().part[(ng & 1) ^ 1];
+    a = b = c = (T)0;
+    for (int t = 0; t < ncl; ++t) {
+        a += pp[t][0];
+        b += pp[t][1];
+        c += pp[t][2];
+    }
+}
+
+// The pending step's factors, by the scalar lane while the others compute the next stencil: d_k and z_k of
+// the LU of T + i w, the residual and the stopping test (flag: 0 go on, 1 converged, 2 limit, 3 breakdown,
+// 4 non-finite); j its place in the history, steps the steps so far.
+template <typename T> __device__ __forceinline__ void factor(int j, int steps, int maxit) {
+    Shared<T> &S = sh<T>();
+    ScalarState &F = S.F;
+    const double ig = F.ig, g1 = ig > 0.0 ? 1.0 / ig : 0.0;
+    const double lr = F.gam * F.dr, li = F.gam * F.di;               // l_k = g_k / d_{k-1}
+    const double er = F.ak - lr * F.ck, ei = F.w - li * F.ck;
+    const double q = er * er + ei * ei, iq = 1.0 / q;
+    const double zr = steps > 1 ? -(lr * F.zr - li * F.zi) : F.zr;
+    const double zi = steps > 1 ? -(lr * F.zi + li * F.zr) : 0.0;
+    const double dr = er * iq, di = -ei * iq;
+    const double yr = zr * dr - zi * di, yi = zr * di + zi * dr;
+    const double rn = g1 * sqrt(yr * yr + yi * yi);
+    S.dr[j] = F.dr = dr;
+    S.di[j] = F.di = di;
+    S.zr[j] = F.zr = zr;
+    S.zi[j] = F.zi = zi;
+    S.g[j] = F.gam;
+    F.gam = g1;
+    F.sweeps += 1;
+    int flag = 0;
+    if (!isfinite(rn) || !(ig == ig)) flag = 4;
+    else if (!(q > 0.0)) flag = 3;
+    else if (rn <= F.thr) flag = 1;
+    else if (steps >= maxit) flag = 2;
+    if (flag) F.rn2 += flag < 3 ? rn * rn : (double)INFINITY;
+    if (flag > 1) F.fail = max(F.fail, flag - 1);
+    S.flag = flag;
+}
+
+// Off the hot path, in functions of their own so that the iteration keeps its registers.
+
+// The thread's sums of Re(r)^2, Im(r)^2 and Re(r) Im(r) over its points of slot s.
+template <typename T, int ZC> __device__ __noinline__ void start_sums(int s, T &rr, T &ii, T &ri) {
+    using C = typename Cx<T>::t;
+    const LanczosArgs<T> &A = sh<T>().A;
+    const Geo<T, ZC> G(A);
+    const C *const rg = A.r + (long long)s * A.nd;
+    T a = 0, b = 0, c = 0;
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+        if (r == 0 || G.row1) {
+            C v[ZC][G.W];
+#pragma unroll
+            for (int z = 0; z < ZC; ++z) {
+                const C *src = rg + G.grid(A, z, r);
+#pragma unroll
+                for (int i = 0; i < G.W; ++i) v[z][i] = z < G.nvz && i < G.nvx ? src[i] : C{0, 0};
+            }
+#pragma unroll
+            for (int z = 0; z < ZC; ++z)
+#pragma unroll
+                for (int i = 0; i < G.W; ++i) {
+                    a += v[z][i].x * v[z][i].x;
+                    b += v[z][i].y * v[z][i].y;
+                    c += v[z][i].x * v[z][i].y;
+                }
+        }
+    rr = a;
+    ii = b;
+    ri = c;
+}
+
+// v_0 = f_re Re(r) + f_im Im(r) of slot s into the slab.
+template <typename T, int ZC, int MODE> __device__ __noinline__ void start_vector(int s, T f_re, T f_im) {
+    using C = typename Cx<T>::t;
+    const LanczosArgs<T> &A = sh<T>().A;
+    const Geo<T, ZC> G(A);
+    const C *const rg = A.r + (long long)s * A.nd;
+    T *const slab = slab_of(A);
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+        if (r == 0 || G.row1) {
+            C v[ZC][G.W];
+#pragma unroll
+            for (int z = 0; z < ZC; ++z) {
+                const C *src = rg + G.grid(A, z, r);
+#pragma unroll
+                for (int i = 0; i < G.W; ++i) v[z][i] = z < G.nvz && i < G.nvx ? src[i] : C{0, 0};
+            }
+#pragma unroll
+            for (int z = 0; z < ZC; ++z)
+                if (z < G.nvz) {
+                    Pk<T> w;
+#pragma unroll
+                    for (int i = 0; i < G.W; ++i) w.set(i, f_re * v[z][i].x + f_im * v[z][i].y);
+                    put<T, MODE>(slab + (r ? G.c1 : G.c0) + z * A.plane, G.gx, G.nvx, A.nx, w);
+                }
+        }
+}
+
+// x += sum_j y_j v_j over the n vectors of the history (and the direction handed over by the last time,
+// have_p); with go_on also the COCG direction p of the last of them.  (er, ei): the part's phase.
+template <typename T, int ZC, int MODE>
+__device__ __noinline__ void flush(int s, int n, bool go_on, bool have_p, double er, double ei) {
+    using P = Pk<T>;
+    using C = typename Cx<T>::t;
+    using V4 = typename Vec4<T>::t;
+    constexpr int W = P::W;
+    Shared<T> &S = sh<T>();
+    const LanczosArgs<T> &A = S.A;
+    const Geo<T, ZC> G(A);
+    const Work<T, ZC> K(A);
+    T *const slab = slab_of(A);
+    C *const xg = A.x + (long long)s * A.nd;
+    const bool scalar = (int)threadIdx.x == G.nthr;
+    const int planeE = A.plane;
+    if (scalar) {
+        // U y = z backwards; p = sum_j q_j v_j + q_prev p_prev likewise
+        double yr = 0, yi = 0, qr = 0, qi = 0;
+        for (int j = n - 1; j >= 0; --j) {
+            const double cn = j + 1 < n ? (double)(T)S.g[j + 1] : 0.0;
+            const double dr = S.dr[j], di = S.di[j];
+            const double tr = S.zr[j] - cn * yr, ti = S.zi[j] - cn * yi;
+            yr = tr * dr - ti * di;
+            yi = tr * di + ti * dr;
+            V4 c;
+            c.x = (T)(er * yr - ei * yi);
+            c.y = (T)(er * yi + ei * yr);
+            if (go_on) {
+                const double ur = j == n - 1 ? 1.0 : -cn * qr, ui = j == n - 1 ? 0.0 : -cn * qi;
+                qr = ur * dr - ui * di;
+                qi = ur * di + ui * dr;
+            }
+            c.z = (T)qr;
+            c.w = (T)qi;
+            S.coef[j] = c;
+        }
+        const double c0d = (double)(T)S.g[0];
+        V4 c;
+        c.x = (T)(-c0d * (er * yr - ei * yi));
+        c.y = (T)(-c0d * (er * yi + ei * yr));
+        c.z = (T)(-c0d * qr);
+        c.w = (T)(-c0d * qi);
+        S.prev = c;
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the history is written
+    }
+    planes_stored();
+    auto add_x = [&](int z, int r, const P &xr, const P &xi) {
+        C *dst = xg + G.grid(A, z, r);
+        C q[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) q[i] = i < G.nvx ? dst[i] : C{0, 0};
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (i < G.nvx) {
+                q[i].x += xr.get(i);
+                q[i].y += xi.get(i);
+                dst[i] = q[i];
+            }
+    };
+    auto add_prev = [&](const V4 &c, bool dir, size_t o, P &xr, P &xi) {
+        const T cr = dir ? c.z : c.x, ci = dir ? c.w : c.y;
+        const P qr = pk_load(K.Pd + o), qi = pk_load(K.Pd + K.vec + o);
+        xr.fma(cr, qr);
+        xr.fma(-ci, qi);
+        xi.fma(cr, qi);
+        xi.fma(ci, qr);
+    };
+    if (!go_on && A.stages > 1) {
+        // the vectors through the slab (which is free now), A.stages bulk copies ahead
+        const int sp = A.nzl_max * planeE;               // elements of a stage
+        const unsigned bytes = (unsigned)(G.nzl * planeE * (int)sizeof(T));
+        auto fetch = [&](int j, int q) {
+            const unsigned fb = (unsigned)__cvta_generic_to_shared(&S.fbar[q]);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(slab + q * sp)),
+                         "l"(__cvta_generic_to_global(K.H + (size_t)j * K.hvec)), "r"(bytes), "r"(fb)
+                         : "memory");
+        };
+        if (scalar)
+            for (int j = 0; j < min(n, A.stages); ++j) fetch(j, j);
+        P xr[ZC][2], xi[ZC][2];
+#pragma unroll
+        for (int z = 0; z < ZC; ++z)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                xr[z][r].zero();
+                xi[z][r].zero();
+            }
+        unsigned ph = S.fphase;
+        const T *const st0 = slab + G.c0 - kRadius * planeE;
+        const int d1 = G.c1 - G.c0;
+        for (int j = 0, q = 0; j < n; ++j, q = q + 1 == A.stages ? 0 : q + 1) {
+            if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.fbar[q]), (ph >> q) & 1)) atomicExch(A.err, 2);
+            ph ^= 1u << q;
+            const V4 c = S.coef[j];
+            const T *const st = st0 + q * sp;
+#pragma unroll
+            for (int z = 0; z < ZC; ++z)
+                if (z < G.nvz)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        const P v = pk_load(st + (r ? d1 : 0) + z * planeE);
+                        xr[z][r].fma(c.x, v);
+                        xi[z][r].fma(c.y, v);
+                    }
+            __syncthreads();
+            if (scalar && j + A.stages < n) fetch(j + A.stages, q);
+        }
+        if (scalar) S.fphase = ph;
+#pragma unroll
+        for (int z = 0; z < ZC; ++z)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (z < G.nvz && (r == 0 || G.row1)) {
+                    if (have_p) add_prev(S.prev, false, G.priv(z, r), xr[z][r], xi[z][r]);
+                    add_x(z, r, xr[z][r], xi[z][r]);
+                }
+        // halo planes outside the box are zero again
+        if (MODE != 1) {
+            P zero;
+            zero.zero();
+            for (int e = W * (int)threadIdx.x; e < max(0, kRadius - G.z0) * planeE; e += W * (int)blockDim.x)
+                pk_store(slab + e, zero);
+            for (int e = (A.nz - G.z0 + kRadius) * planeE + W * (int)threadIdx.x; e < (G.nzl + 2 * kRadius) * planeE;
+                 e += W * (int)blockDim.x)
+                pk_store(slab + e, zero);
+        }
+    } else if (G.nvz > 0) {
+        for (int pass = 0; pass < (go_on ? 2 : 1); ++pass)           // x, then p
+            for (int r = 0; r < (G.row1 ? 2 : 1); ++r) {
+                const T *const hr = K.H + (r ? G.c1 : G.c0) - kRadius * planeE;
+                P xr[ZC], xi[ZC];
+#pragma unroll
+                for (int z = 0; z < ZC; ++z) {
+                    xr[z].zero();
+                    xi[z].zero();
+                }
+#pragma unroll 2
+                for (int j = 0; j < n; ++j) {
+                    const V4 c = S.coef[j];
+                    const T cr = pass ? c.z : c.x, ci = pass ? c.w : c.y;
+#pragma unroll
+                    for (int z = 0; z < ZC; ++z) {
+                        const P v = pk_load_l2(hr + (size_t)j * K.hvec + z * planeE);
+                        xr[z].fma(cr, v);
+                        xi[z].fma(ci, v);
+                    }
+                }
+#pragma unroll
+                for (int z = 0; z < ZC; ++z) {
+                    const size_t o = G.priv(z, r);
+                    if (have_p) add_prev(S.prev, pass != 0, o, xr[z], xi[z]);
+                    if (pass) {
+                        pk_store(K.Pd + o, xr[z]);
+                        pk_store(K.Pd + K.vec + o, xi[z]);
+                    } else if (z < G.nvz) {
+                        add_x(z, r, xr[z], xi[z]);
+                    }
+                }
+            }
+    }
+    __syncthreads();                                     // the coefficients are read before they change
+}
+
+// Once a block: its slab cleared, barriers, the halo copies, V_loc by threads.
+template <typename T, int ZC> __device__ __noinline__ void block_setup(const LanczosArgs<T> *args, bool per) {
+    Shared<T> &S = sh<T>();
+    const LanczosArgs<T> &A = *args;
+    const Geo<T, ZC> G(A);
+    const Work<T, ZC> K(A);
+    for (int e = threadIdx.x; e < A.smem_words; e += blockDim.x)
+        reinterpret_cast<int4 *>(lz_smem + shared_bytes<T>())[e] = make_int4(0, 0, 0, 0);
+    if ((int)threadIdx.x < G.nthr)
+        for (int z = 0; z < ZC; ++z)
+            for (int r = 0; r < 2; ++r) {
+                Pk<T> v;
+#pragma unroll
+                for (int i = 0; i < G.W; ++i)
+                    v.set(i, z < G.nvz && (r == 0 || G.row1) && i < G.nvx ? A.vloc[G.grid(A, z, r) + i] : (T)0);
+                pk_store(K.V + G.priv(z, r), v);
+            }
+    if ((int)threadIdx.x == G.nthr) {
+        mbar_init(&S.bar);
+        for (int q = 0; q < 2; ++q) mbar_init(&S.pbar[q]);
+        for (int q = 0; q < kStages; ++q) mbar_init(&S.fbar[q]);
+        S.fphase = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // the copies: this block's planes [g0, g1) that lie in the halo of rank t (periodic: of its image)
+        const int ncl = A.ncl, nz = A.nz, z0 = G.z0, z1 = G.z0 + G.nzl, pb = A.plane * (int)sizeof(T);
+        int n = 0, bytes = 0;
+        for (int dt = -A.reach; dt <= A.reach; ++dt) {
+            int t = G.rank + dt, base = 0;
+            if (dt == 0) continue;
+            if (t < 0 || t >= ncl) {
+                if (!per) continue;
+                const int w = t < 0 ? -((ncl - 1 - t) / ncl) : t / ncl;
+                t -= w * ncl;
+                base = w * nz;
+            }
+            const int t0 = base + t * nz / ncl, t1 = base + (t + 1) * nz / ncl;   // rank t's planes
+            const int g0 = max(z0, t0 - kRadius), g1 = min(z1, t1 + kRadius);
+            if (g0 < g1) {
+                S.to[4 * n] = t;
+                S.to[4 * n + 1] = (g0 - t0 + kRadius) * pb;
+                S.to[4 * n + 2] = (g0 - z0 + kRadius) * pb;
+                S.to[4 * n + 3] = (g1 - g0) * pb;
+                ++n;
+            }
+            // and rank t's planes in this block's halo
+            bytes += max(0, min(t1, z1 + kRadius) - max(t0, z0 - kRadius)) * pb;
+        }
+        S.nto = n;
+        S.expect = (unsigned)bytes;
+    }
+}
+
+// MODE: 0 zero values outside the box, kept as rows of zeros between the planes; 1 periodic; 2 zero
+// values outside the box, read from a zero word (less shared memory, a select per row)
+template <typename T, int ZC, int MAXT, int MODE>
+__global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ LanczosArgs<T> A, const __grid_constant__ Coef<T> cf) {
+    using P = Pk<T>;
+    constexpr bool PER = MODE == 1;
+    constexpr int W = P::W;
+    constexpr int PAD = Geo<T, ZC>::PAD;
+    constexpr int XL = (2 * PAD + W) / W;               // 16-byte loads of a row's x neighbours
+    Shared<T> &S = sh<T>();
+    const int tid = threadIdx.x, ncl = A.ncl;
+    if (tid == 0) S.A = A;
+    __syncthreads();
+    block_setup<T, ZC>(&S.A, PER);
+    const Geo<T, ZC> G(A);
+    const bool scalar = tid == G.nthr;
+    T *const slab = slab_of(A);
+    const int n_items = *A.cnt;
+    unsigned phase = 0, ng = 0;                         // halo phase, reductions so far
+    cluster_barrier();                                  // every block runs, has cleared its slab and set its barriers
+    for (;;) {
+        // the next system, from the end of the list (the highest orbitals, the longest solves, first)
+        if (G.rank == 0 && tid < ncl) {
+            int it = 0;
+            if (tid == 0) it = atomicAdd(A.grab, 1);
+            it = __shfl_sync((1u << ncl) - 1u, it, 0);
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                             map_rank((unsigned)__cvta_generic_to_shared(&S.item), tid)),
+                         "r"(it)
+                         : "memory");
+        }
+        cluster_barrier();
+        if (S.item >= n_items) break;
+        const int s = A.list[n_items - 1 - S.item];
+        // the right-hand side's phase and the norms of its two parts
+        {
+            T rr, ii, ri;
+            start_sums<T, ZC>(s, rr, ii, ri);
+            gather3(rr, ii, ri, ng, ncl, G.rank, A.err);
+            if (scalar) {
+                T a, b, c;
+                sum_parts(ng, ncl, a, b, c);
+                // phi = arg(r^T r) / 2; r_a^2 = sum + |r^T r| / 2, r_b^2 = sum - |r^T r| / 2
+                const double sum = 0.5 * ((double)a + (double)b), D = 0.5 * ((double)a - (double)b), O = (double)c;
+                const double m = sqrt(D * D + O * O);
+                double cs = 1.0, sn = 0.0;
+                if (m > 0.0 && (double)b > 0.0) {
+                    cs = sqrt(fmax(0.0, 0.5 * (1.0 + D / m)));
+                    sn = copysign(sqrt(fmax(0.0, 0.5 * (1.0 - D / m))), O);
+                }
+                S.start[0] = cs;
+                S.start[1] = sn;
+                S.start[2] = sqrt(sum + m);
+                S.start[3] = (double)b > 0.0 ? sqrt(fmax(0.0, sum - m)) : 0.0;
+                S.F.sweeps = S.F.fail = 0;
+                S.F.rn2 = 0.0;
+                S.F.d0 = A.d0 + A.slots[s].shift_re;     // the shift of H: -eps_n, omega
+                S.F.w = A.slots[s].shift_im;
+            }
+            __syncthreads();
+        }
+        for (int pt = 0; pt < 2; ++pt) {
+            T f_re, f_im;
+            {
+                const Slot &sl = A.slots[s];
+                const double thr_all = A.mixed ? fmax(A.inner_tol * sl.ref_norm, 0.3 * A.tol * sl.bnorm * sl.scale)
+                                               : A.tol * sl.bnorm;
+                const double na = S.start[2], nb = S.start[3], beta = pt ? nb : na;
+                // The parts' residuals add as orthogonal vectors nearly do.  A small r_b (rounding noise of the
+                // last inner solve) gets a small share of the threshold, comparable parts equal shares.
+                const double thr = thr_all * (nb == 0.0 ? 1.0 : nb > 0.1 * na ? 0.7 : pt ? 0.3 : 0.95);
+                if (!(beta > thr)) {                     // nothing to solve for (uniform over the cluster)
+                    if (scalar) {
+                        S.F.rn2 += beta * beta;
+                        if (!(beta <= thr)) S.F.fail = 3;   // not a number
+                    }
+                    continue;
+                }
+                if (scalar) {
+                    S.F.dr = S.F.di = S.F.zi = S.F.gam = 0.0;
+                    S.F.zr = beta;
+                    S.F.thr = thr;
+                    S.flag = 0;
+                }
+                // v_0 = part / ||part||
+                const double ib = 1.0 / beta;
+                f_re = (T)((pt ? -S.start[1] : S.start[0]) * ib);
+                f_im = (T)((pt ? S.start[0] : S.start[1]) * ib);
+            }
+            start_vector<T, ZC, MODE>(s, f_re, f_im);
+            planes_stored();
+            if (scalar) {
+                const Work<T, ZC> K(A);
+                send_halos(slab);
+                keep(slab, K.H, K.hvec, 0, G.nzl, A.plane);
+            }
+            P acc[ZC][2];
+#pragma unroll
+            for (int z = 0; z < ZC; ++z) {
+                acc[z][0].zero();
+                acc[z][1].zero();
+            }
+            T dg = (T)S.F.d0, cc = 0;                    // diagonal used (shifted by the last a_k), c_k
+            int k = 0, kb = 0, n = 0;                    // step, first vector of the history, vectors to flush
+            bool have_p = false;
+            for (;;) {
+                // the unit's first point, its second row, the row and plane strides: made opaque so that the
+                // hundreds of addresses formed from them are not kept (and spilled) across iterations
+                int c0 = G.c0, d1 = G.c1 - G.c0, pitch = A.pitch, planeE = A.plane;
+                asm volatile("" : "+r"(c0), "+r"(d1), "+r"(pitch), "+r"(planeE));
+                const T *const b0 = slab + c0;
+                if (scalar) {
+                    if (k > kb) factor<T>(k - 1 - kb, k, A.maxit);
+                    keep_wait();
+                }
+                // ---- u = B v_k - c_k v_{k-1} (shifted), sums v.v, u.v, u.u.  The x and y neighbours and the
+                // diagonal lie in the block's own planes: first, while the halo is on its way.
+                T svv = 0, suv = 0, suu = 0;
+                P mask;                                  // 1 for points inside the box
+#pragma unroll
+                for (int i = 0; i < W; ++i) mask.set(i, i < G.nvx ? (T)1 : (T)0);
+                if (G.unit) {
+                    // the row r rows from the unit's first (pl)
+                    auto yrow = [&](const T *pl, int r) -> const T * {
+                        if (MODE == 0) return pl + r * pitch;
+                        int y = G.gy + r;
+                        if (MODE == 2)
+                            return y >= 0 && y < A.ny ? pl + r * pitch
+                                                      : reinterpret_cast<const T *>(lz_smem + shared_bytes<T>());
+                        y = y < 0 ? y + A.ny : y >= A.ny ? y - A.ny : y;
+                        return pl + (y - G.gy) * pitch;
+                    };
+                    const T *const wv = A.ws + (size_t)blockIdx.x * A.ws_stride + (size_t)tid * W;
+                    const int vs = G.nthr * W;
+                    P vn[2];
+                    vn[0] = pk_load(wv);
+                    vn[1] = pk_load(wv + vs);
+#pragma unroll
+                    for (int z = 0; z < ZC; ++z) {
+                        P &a0 = acc[z][0], &a1 = acc[z][1];
+                        a0.mul(-cc);
+                        a1.mul(-cc);
+                        if (z < G.nvz) {
+                            const T *const pl = b0 + z * planeE;
+                            const P pv0 = vn[0], pv1 = vn[1];
+                            if (z + 1 < ZC) {
+                                vn[0] = pk_load(wv + (2 * z + 2) * vs);
+                                vn[1] = pk_load(wv + (2 * z + 3) * vs);
+                            }
+                            P ctr0, ctr1, nb1;
+                            {
+                                P X[XL];
+#pragma unroll
+                                for (int m = 0; m < XL; ++m) X[m] = pk_load(pl - PAD + m * W);
+                                ctr0 = X[PAD / W];
+                                x_part(a0, X, cf);
+                            }
+                            {
+                                P X[XL];
+#pragma unroll
+                                for (int m = 0; m < XL; ++m) X[m] = pk_load(pl + d1 - PAD + m * W);
+                                ctr1 = X[PAD / W];
+                                x_part(a1, X, cf);
+                            }
+                            nb1 = G.row1 ? ctr1 : pk_load(yrow(pl, 1));
+                            a0.fma(cf.a[1], nb1);
+                            a1.fma(cf.a[1], ctr0);
+#pragma unroll
+                            for (int d = 1; d <= kRadius; ++d) {
+                                const P lo = pk_load(yrow(pl, -d)), hi = pk_load(yrow(pl, 1 + d));
+                                a0.fma(cf.a[d], lo);
+                                a1.fma(cf.a[d], hi);
+                                if (d < kRadius) {
+                                    a1.fma(cf.a[d + 1], lo);
+                                    a0.fma(cf.a[d + 1], hi);
+                                }
+                            }
+                            a0.fma(dg, ctr0);
+                            a1.fma(dg, ctr1);
+                            a0.fma(pv0, ctr0);
+                            a1.fma(pv1, ctr1);
+                            if (PER) {                   // a periodic row's images are no points
+                                ctr0.mul(mask);
+                                ctr1.mul(mask);
+                            }
+                            P t;
+                            t.zero();
+                            t.fma(ctr0, ctr0);
+                            if (G.row1) t.fma(ctr1, ctr1);
+                            svv += t.sum();
+                        }
+                    }
+                }
+                if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.bar), phase)) atomicExch(A.err, 2);
+                phase ^= 1u;
+                if (G.unit) {
+                    const T *const bz = b0 - kRadius * planeE;
+#pragma unroll
+                    for (int p = 0; p < ZC + 2 * kRadius; ++p) {
+                        const P v0 = pk_load(bz + p * planeE), v1 = pk_load(bz + d1 + p * planeE);
+#pragma unroll
+                        for (int z = 0; z < ZC; ++z) {
+                            const int d = p - z - kRadius < 0 ? z + kRadius - p : p - z - kRadius;
+                            if (d >= 1 && d <= kRadius) {
+                                acc[z][0].fma(cf.a[d], v0);
+                                acc[z][1].fma(cf.a[d], v1);
+                            }
+                        }
+                    }
+                    P t1, t2;
+                    t1.zero();
+                    t2.zero();
+#pragma unroll
+                    for (int z = 0; z < ZC; ++z)
+                        if (z < G.nvz) {
+                            P &a0 = acc[z][0], &a1 = acc[z][1];
+                            a0.mul(mask);                // u = 0 outside the box
+                            a1.mul(mask);
+                            const P v0 = pk_load(b0 + z * planeE), v1 = pk_load(b0 + d1 + z * planeE);
+                            t1.fma(a0, v0);
+                            t2.fma(a0, a0);
+                            if (G.row1) {
+                                t1.fma(a1, v1);
+                                t2.fma(a1, a1);
+                            }
+                        }
+                    suv = t1.sum();
+                    suu = t2.sum();
+                }
+                gather3(svv, suv, suu, ng, ncl, G.rank, A.err);
+                if (k > kb && S.flag) {                  // the last step ended the solve
+                    n = k - kb;
+                    break;
+                }
+                // ---- a' = u.v / v.v, 1/g with g = ||u - a' v||
+                T ap = 0, ig = 0;
+                if (sizeof(T) == 4 || scalar) {
+                    T a, b, c;
+                    sum_parts(ng, ncl, a, b, c);
+                    ap = b / a;
+                    const T b2 = c - ap * b;
+                    ig = b2 > (T)0 ? (T)1 / sqrt(b2) : (T)0;
+                    if (!isfinite(a) || !isfinite(c)) ig = (T)nan("");
+                }
+                if (sizeof(T) == 8) {
+                    if (scalar) {
+                        S.vec[0] = ap;
+                        S.vec[1] = ig;
+                        S.vec[2] = ig > (T)0 ? (T)1 / ig : (T)0;
+                    }
+                    __syncthreads();
+                    ap = S.vec[0];
+                    ig = S.vec[1];
+                }
+                if (scalar) {
+                    S.F.ak = S.F.d0 - (double)dg + (double)ap;   // a_k of B
+                    S.F.ck = (double)cc;
+                    S.F.ig = (double)ig;
+                    if (A.prof && G.rank == 0) atomicAdd(A.prof + 1, (unsigned long long)A.nd);
+                }
+                // ---- v_{k+1} into the slab; the registers keep v_k
+                const T m_ag = -ap * ig;
+#pragma unroll
+                for (int z = 0; z < ZC; ++z)
+                    if (z < G.nvz) {
+#pragma unroll
+                        for (int r = 0; r < 2; ++r)
+                            if (r == 0 || G.row1) {
+                                T *const own = slab + c0 + (r ? d1 : 0) + z * planeE;
+                                const P v = pk_load(own);
+                                P w = acc[z][r];
+                                w.mul(ig);
+                                w.fma(m_ag, v);
+                                put<T, MODE>(own, G.gx, G.nvx, A.nx, w);
+                                acc[z][r] = v;
+                            }
+                    }
+                // the next stencil: its diagonal shifted by a_k (u.v stays small against u.u)
+                cc = sizeof(T) == 8 ? S.vec[2] : ig > (T)0 ? (T)1 / ig : (T)0;
+                dg -= ap;
+                planes_stored();
+                ++k;
+                if (k - kb == A.hist) {                  // the history is full: into x and p
+                    if (scalar) factor<T>(k - 1 - kb, k, A.maxit);
+                    __syncthreads();
+                    n = k - kb;
+                    if (S.flag) break;
+                    flush<T, ZC, MODE>(s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+                    have_p = true;
+                    kb = k;
+                    const Work<T, ZC> K(A);
+                    const T *const hl = K.H + (size_t)(A.hist - 1) * K.hvec - kRadius * A.plane;   // v_{k-1} again
+#pragma unroll
+                    for (int z = 0; z < ZC; ++z) {
+                        acc[z][0] = pk_load_l2(hl + G.c0 + z * A.plane);
+                        acc[z][1] = pk_load_l2(hl + G.c1 + z * A.plane);
+                    }
+                }
+                if (scalar) {
+                    const Work<T, ZC> K(A);
+                    send_halos(slab);
+                    keep(slab, K.H, K.hvec, k - kb, G.nzl, planeE);
+                }
+            }
+            if (S.flag < 4)                              // nothing is kept of a solve that went non-finite
+                flush<T, ZC, MODE>(s, n, false, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+            // the flush uses the whole slab: no neighbour's next planes before every block is done with it
+            // (and no thread still reads the flag)
+            cluster_barrier();
+        }
+        // the slot's state
+        if (scalar && G.rank == 0) {
+            Slot &sl = A.slots[s];
+            const ScalarState &F = S.F;
+            sl.iters = F.sweeps;
+            sl.total_iters += F.sweeps;
+            sl.rnorm = sqrt(F.rn2);
+            if (A.mixed) {
+                if (F.fail == 3) sl.discard = 1;
+                if (F.fail >= 2) sl.status = RPA_ERR_BREAKDOWN;
+                sl.phase = kInnerDone;
+            } else {
+                sl.status = F.fail == 0 ? RPA_OK : F.fail == 1 ? RPA_ERR_NOT_CONVERGED : RPA_ERR_BREAKDOWN;
+                sl.phase = kFinished;
+            }
+        }
+    }
+    cluster_barrier();                                  // no block leaves while another may write its memory
+}
+
+struct Variant {
+    int zc, max_threads;
+};
+constexpr Variant kVar32[3] = {{3, 640}, {4, 640}, {5, 512}};
+constexpr Variant kVar64[2] = {{2, 640}, {4, 512}};
+
+using Fn32 = void (*)(LanczosArgs<float>, Coef<float>);
+using Fn64 = void (*)(LanczosArgs<double>, Coef<double>);
+// by variant and MODE (FP64 has no rows of zeros: its arithmetic, not its loads, is the limit)
+const Fn32 kFn32[3][2] = {{k_lanczos<float, 3, 640, 0>, k_lanczos<float, 3, 640, 1>},
+                          {k_lanczos<float, 4, 640, 0>, k_lanczos<float, 4, 640, 1>},
+                          {k_lanczos<float, 5, 512, 0>, k_lanczos<float, 5, 512, 1>}};
+const Fn64 kFn64[2][2] = {{k_lanczos<double, 2, 640, 2>, k_lanczos<double, 2, 640, 1>},
+                          {k_lanczos<double, 4, 512, 2>, k_lanczos<double, 4, 512, 1>}};
+
+const void *kernel_of(bool mixed, int v, bool per) {
+    return mixed ? (const void *)kFn32[v][per] : (const void *)kFn64[v][per];
+}
+
+void cluster_config(cudaLaunchConfig_t &lc, cudaLaunchAttribute &at, int ncl, int blocks, int threads, size_t smem,
+                    cudaStream_t s) {
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ncl;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    lc.gridDim = dim3((unsigned)blocks, 1, 1);
+    lc.blockDim = dim3((unsigned)threads, 1, 1);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+}
+
+}  // namespace
+
+bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
+    if (c.opt.precondition || c.nz < kRadius + 2 || c.ny < kRadius || c.nx < kRadius) return false;
+    const bool mixed = c.opt.prec == RPA_MIXED;
+    int sms = 0, optin = 0;
+    RPA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device));
+    RPA_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c.device));
+    const int W = mixed ? 4 : 2, pad = mixed ? 8 : 6;
+    const size_t tsz = mixed ? 4 : 8;
+    const int hw = (c.nx + W - 1) / W, hh = (c.ny + 1) / 2;
+    // row pitch in 16-byte words: the row and its padding (periodic: images on both sides), and two rows
+    // spanning hw words modulo 8 (odd hw: one more), so that 8 consecutive units hit different banks
+    int p16 = c.opt.periodic ? (2 * pad + c.nx + W - 1) / W : (pad + hw * W) / W;
+    if (mixed)
+        while ((2 * p16 - (hw + hw % 2)) % 8 != 0) ++p16;
+    // FP32, zero values outside the box: planes follow each other with kRadius rows of zeros in between
+    const int zrows = c.opt.periodic || !mixed ? 0 : kRadius;
+    const int pitch = p16 * W, plane = pitch * (c.ny + zrows), lead = std::max(W, pitch * zrows);
+    const int nvar = mixed ? 3 : 2;
+    double best_cost = 1e300;
+    bool found = false;
+    for (int v = 0; v < nvar; ++v) {
+        const Variant var = mixed ? kVar32[v] : kVar64[v];
+        const void *fn = kernel_of(mixed, v, c.opt.periodic != 0);
+        cudaFuncAttributes fa{};
+        RPA_CUDA(cudaFuncGetAttributes(&fa, fn));
+        for (int ncl = 1; ncl <= 16; ncl *= 2) {
+            if (ncl > c.nz) break;
+            const int nzl = (c.nz + ncl - 1) / ncl, nch = (nzl + var.zc - 1) / var.zc;
+            const long long units = (long long)hw * hh * nch;
+            const int threads = (int)std::min<long long>((units + 31) / 32 * 32 + 32, 1 << 20);
+            if (threads > var.max_threads) continue;
+            const size_t elems = (size_t)lead + (size_t)plane * (nch * var.zc + 2 * kRadius) + 2 * pad;
+            const size_t smem = (elems * tsz + 15) / 16 * 16 + (mixed ? shared_bytes<float>() : shared_bytes<double>());
+            if (smem + fa.sharedSizeBytes > (size_t)optin) continue;
+            RPA_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            allow_dynamic_smem(fn, smem);
+            cudaLaunchConfig_t lc{};
+            cudaLaunchAttribute at{};
+            cluster_config(lc, at, ncl, ncl * sms, threads, smem, nullptr);
+            int ncs = 0;
+            if (cudaOccupancyMaxActiveClusters(&ncs, fn, &lc) != cudaSuccess || ncs < 1) {
+                (void)cudaGetLastError();
+                continue;
+            }
+            // cycles per iteration of the blocks sharing an SM, and the rounds the systems take
+            const double pts = (double)(threads - 32) * 2 * W * var.zc;
+            const int used = std::min(ncs, nsys);
+            const double share = std::max(1.0, (double)used * ncl / sms);
+            const double sync = 3500.0 + 300.0 * std::log2((double)ncl);
+            const double cyc = std::max(share * pts * (mixed ? 0.6 : 24.0), pts * (mixed ? 0.6 : 24.0) + sync);
+            const double rounds = nsys <= ncs ? 1.0 : (double)nsys / ncs + 0.3;
+            const double cost = rounds * cyc;
+            if (cost < best_cost) {
+                best_cost = cost;
+                found = true;
+                best.variant = v;
+                best.mixed = mixed;
+                best.ncl = ncl;
+                best.clusters = used;
+                best.threads = threads;
+                best.smem = smem;
+                best.hw = hw;
+                best.hh = hh;
+                best.nch = nch;
+                best.pitch = pitch;
+                best.plane = plane;
+                best.lead = lead;
+                best.reach = (kRadius + c.nz / ncl - 1) / (c.nz / ncl);
+                best.zc = var.zc;
+            }
+        }
+    }
+    if (!found) return false;
+    const size_t vec = (size_t)2 * best.zc * (best.threads - 32) * W, hvec = (size_t)best.nch * best.zc * best.plane;
+    // history: as many vectors as 2 GB hold, 16 .. kHistMax
+    const size_t per_vec = hvec * tsz * best.clusters * best.ncl;
+    best.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, ((size_t)2 << 30) / per_vec));
+    best.ws_stride = 3 * vec + hvec * best.hist;
+    best.ws_bytes = best.ws_stride * tsz * best.clusters * best.ncl;
+    return true;
+}
+
+template <typename T> static void launch(const Ctx &c, const LanczosPlan &p, LanczosArgs<T> a, cudaStream_t s) {
+    a.ws = (T *)p.ws;
+    a.ws_stride = p.ws_stride;
+    a.nd = c.nd;
+    a.nx = c.nx;
+    a.ny = c.ny;
+    a.nz = c.nz;
+    a.tol = c.opt.tol;
+    a.inner_tol = c.opt.inner_tol;
+    a.maxit = c.opt.maxit;
+    a.mixed = p.mixed;
+    a.ncl = p.ncl;
+    a.hw = p.hw;
+    a.hh = p.hh;
+    a.nch = p.nch;
+    a.pitch = p.pitch;
+    a.plane = p.plane;
+    a.lead = p.lead;
+    a.nzl_max = (c.nz + p.ncl - 1) / p.ncl;
+    a.stages = std::min(kStages, (p.nch * p.zc + 2 * kRadius) / a.nzl_max);
+    a.err = c.d_tc_err;
+    a.reach = p.reach;
+    a.hist = p.hist;
+    a.smem_words = (int)((p.smem - shared_bytes<T>()) / 16);
+    a.d0 = 3.0 * c.coef.a[0];
+    const Coef<T> cf = cast_coef<T>(c.coef);
+    const void *fn = kernel_of(p.mixed, p.variant, c.opt.periodic != 0);
+    allow_dynamic_smem(fn, p.smem);
+    RPA_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t lc{};
+    cudaLaunchAttribute at{};
+    cluster_config(lc, at, p.ncl, p.ncl * p.clusters, p.threads, p.smem, s);
+    void *args[2] = {(void *)&a, (void *)&cf};
+    RPA_CUDA(cudaLaunchKernelExC(&lc, fn, args));
+}
+
+void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<float> &a, cudaStream_t s) { launch(c, p, a, s); }
+void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<double> &a, cudaStream_t s) { launch(c, p, a, s); }
+
+}  // namespace rpa
