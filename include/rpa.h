@@ -272,20 +272,21 @@ rpa_status rpa_ec_gradient(rpa_ctx *ctx, int n_r, const double *V0_dev, double *
  * rpa_apply_nuchi0_batch does for every context k what rpa_apply_nuchi0 does for one: R_dev[k] =
  * nu^1/2 chi0(i omega) nu^1/2 V_dev[k] (symmetric != 0) or nu chi0 V_dev[k], ncols[k] columns in
  * [0, 1024] (N_d x ncols[k], column-major, no aliasing).  The Sternheimer systems (Eq. 9) of all the
- * contexts run together in the block COCG kernels (block size max(1, block_cocg)): one launch per
- * kernel and iteration for the whole batch, every system with its own grid, operator, orbitals and
- * stopping rule.  The contexts must be distinct, on one device, with equal prec, tol, inner_tol,
+ * contexts are in flight together: with block_cocg = 0 each context's queue runs on a stream of its
+ * own, on the kernels it runs alone; with block_cocg > 0 they run in the block COCG kernels, one launch
+ * per kernel and iteration for the whole batch, every system with its own grid, operator, orbitals
+ * and stopping rule.  The contexts must be distinct, on one device, with equal prec, tol, inner_tol,
  * maxit, max_refine and block_cocg, and without precondition or project_solution (else
- * RPA_ERR_INVALID); the first context's batch_systems and profile apply.  Synchronises `stream`.
- * Returns the worst per-system status. */
+ * RPA_ERR_INVALID); with block_cocg > 0 the first context's batch_systems and profile apply.
+ * Synchronises `stream`.  Returns the worst per-system status. */
 rpa_status rpa_apply_nuchi0_batch(rpa_ctx *const *ctxs, int n, double omega, const double *const *V_dev,
                                   double *const *R_dev, const int *ncols, int symmetric, void *stream);
 
 /* rpa_ec for every context k of a batch: n_r[k] trial vectors V0_dev[k], each context with its own
- * frequencies, subspace iteration and stopping rule (Algorithm 1), and the chi0 applications of
- * the contexts still iterating run together as in rpa_apply_nuchi0_batch (one host thread per
- * context drives its subspace iteration; the last to reach its chi0 application runs the batch,
- * and a context that has finished drops out of later batches).  Outputs per context, each pointer
+ * frequencies, subspace iteration and stopping rule (Algorithm 1), one host thread and stream per
+ * context.  With block_cocg > 0 the chi0 applications of the contexts still iterating run together as
+ * in rpa_apply_nuchi0_batch (the last to reach its chi0 application runs the batch, and a context that
+ * has finished drops out of later batches).  Outputs per context, each pointer
  * may be NULL: lambdas_host[k] (n_omega x n_r[k] Ritz values), ec_host[2k] and ec_host[2k + 1]
  * (E_c and E_c per atom), ec_per_omega_host[k] (n_omega values), stats[k] (the launches and
  * synchronisations of a batch are counted in

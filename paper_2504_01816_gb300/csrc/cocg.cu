@@ -2828,10 +2828,11 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     const RingFn ring_fn = ws ? (even_nx ? k_cocg_ring_ws<true> : k_cocg_ring_ws<false>)
                               : clus ? (even_nx ? k_cocg_ring_cl<true> : k_cocg_ring_cl<false>) : ring1_fn;
     // systems that fit on chip: the Lanczos kernel
-    if (c.lz_key[0] != S || c.lz_key[1] != c.opt.prec) {
+    if (c.lz_key[0] != S || c.lz_key[1] != c.opt.prec || c.lz_key[2] != c.batch_load) {
         c.lz_ok = lanczos_plan(c, S, c.lz_plan);
         c.lz_key[0] = S;
         c.lz_key[1] = c.opt.prec;
+        c.lz_key[2] = c.batch_load;
     }
     const bool use_lz = c.lz_ok && !precond && !c.keep_cocg && (want == 0 || want == 4);
     const bool use_ring = !use_lz && mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
@@ -3494,7 +3495,7 @@ int response_square(Ctx &c, double omega, const double *dv, const double *coef, 
 }
 
 int chi0_apply(Ctx &c, double omega, const double *dv, double *drho, int ncols, cudaStream_t s) {
-    if (c.coord) return batch_chi0(c, omega, dv, drho, ncols, s);
+    if (c.coord && c.opt.block_cocg > 0) return batch_chi0(c, omega, dv, drho, ncols, s);
     if (c.opt.block_cocg > 0) return chi0_apply_block(c, omega, dv, drho, ncols, s);
     RPA_CUDA(cudaMemsetAsync(drho, 0, sizeof(double) * (size_t)ncols * c.nd, s));
     const int nsys = c.ns * ncols;

@@ -142,8 +142,8 @@ struct Ctx {
     DevBuf blockE;                // subspace of the previous iteration (gradient)
     DevBuf dense_scratch;         // split-K partial sums
     DevBuf lanczos_ws;            // Lanczos vectors of the systems in flight
-    LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, prec}
-    int lz_key[2] = {-1, -1};
+    LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, prec, batch_load}
+    int lz_key[3] = {-1, -1, -1};
     bool lz_ok = false;
     // rpa_ec_gradient with the final subspace as an output runs the COCG kernels: a subspace is R L^-T
     // with the conditioning of R, and after the exact integer pieces of the tensor-core contractions
@@ -170,6 +170,9 @@ struct Ctx {
     unsigned long long *d_prof_points = nullptr;   // RPA_PROF_SLOTS counters
     // rpa_ec_batch: the rendezvous this context's chi0 applications go to (nullptr otherwise)
     BatchCoord *coord = nullptr;
+    // a batch without block COCG: this context's stream, and the systems of the whole batch
+    cudaStream_t batch_stream = nullptr;
+    int batch_load = 0;
     // CUDA graphs: epochs of COCG iterations are captured on a private stream and replayed
     bool use_graphs = true;
     cudaStream_t cap_stream = nullptr;
@@ -250,8 +253,8 @@ struct Chi0Request {
 // max(1, block_cocg) and the iteration settings and workspaces of the first context.  The
 // statistics of each context get its own systems.
 int chi0_apply_batch(const std::vector<Chi0Request> &reqs, cudaStream_t s, std::vector<int> *status = nullptr);
-// While a context is attached to a BatchCoord, its chi0 applications are posted there and run
-// together with the other contexts' (batch_chi0).
+// While a context with block_cocg > 0 is attached to a BatchCoord, its chi0 applications are posted there
+// and run together with the other contexts' (batch_chi0).
 int batch_chi0(Ctx &c, double omega, const double *dv, double *drho, int ncols, cudaStream_t s);
 
 // Same as sternheimer_batch, with b replaced by P_c b first.

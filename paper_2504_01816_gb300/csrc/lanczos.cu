@@ -1110,11 +1110,12 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
             }
             // cycles per iteration of the blocks sharing an SM, and the rounds the systems take
             const double pts = (double)(threads - 32) * 2 * W * var.zc;
-            const int used = std::min(ncs, nsys);
-            const double share = std::max(1.0, (double)used * ncl / sms);
+            // (a batch's other contexts run beside this one)
+            const int used = std::min(ncs, nsys), all = std::max(nsys, c.batch_load), busy = std::min(ncs, all);
+            const double share = std::max(1.0, (double)busy * ncl / sms);
             const double sync = 3500.0 + 300.0 * std::log2((double)ncl);
             const double cyc = std::max(share * pts * (mixed ? 0.6 : 24.0), pts * (mixed ? 0.6 : 24.0) + sync);
-            const double rounds = nsys <= ncs ? 1.0 : (double)nsys / ncs + 0.3;
+            const double rounds = all <= ncs ? 1.0 : (double)all / ncs + 0.3;
             const double cost = rounds * cyc;
             if (cost < best_cost) {
                 best_cost = cost;
