@@ -3016,6 +3016,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     LanczosArgs<double> lz64{};
     if (use_lz) {
         c.lz_plan.ws = c.lanczos_ws.ensure(c.lz_plan.ws_bytes);
+        lanczos_prepare(c, c.lz_plan, st);
         auto fill = [&](auto &a) {
             a.slots = slots;
             a.list = list;                 // built by k_ring_list, which also clears the counter
@@ -3102,7 +3103,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     char names[3][32];
     std::snprintf(names[0], 32, "-");
     if (use_lz) {
-        std::snprintf(names[1], 32, "k_lanczos<%s>", mixed ? "f32" : "f64");
+        std::snprintf(names[1], 32, c.lz_plan.stream ? "k_lanczos_stream<%s>" : "k_lanczos<%s>", mixed ? "f32" : "f64");
         std::snprintf(names[2], 32, "-");
     } else if (use_ring) {
         std::snprintf(names[1], 32, ws ? "k_cocg_ring_ws<%s>" : clus ? "k_cocg_ring_cl<%s>" : "k_cocg_ring<%s>", tn);
@@ -3116,8 +3117,8 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     // and writes x, r; the fused kernel reads and writes x, r, p, q, except in the first sweep of an
     // inner solve, which reads r and writes p, q (V is read once per plane and block, not per system,
     // and is not counted)
-    // the Lanczos kernel writes and reads every vector once
-    const double bytes_per_point[3] = {0.0, use_lz ? 2 * rsz : use_ring ? 8 * csz : 4 * csz + rsz,
+    // the Lanczos kernel writes and reads every vector once; streaming, also u
+    const double bytes_per_point[3] = {0.0, use_lz ? (c.lz_plan.stream ? 5 : 2) * rsz : use_ring ? 8 * csz : 4 * csz + rsz,
                                        use_lz || use_ring ? 0.0 : 6 * csz};
     if (prof) {
         RPA_CUDA(cudaMemsetAsync(c.d_prof_points, 0, sizeof(unsigned long long) * 3, st));

@@ -422,6 +422,74 @@ template <typename T> __device__ __forceinline__ void factor(int j, int steps, i
 
 // Off the hot path, in functions of their own so that the iteration keeps its registers.
 
+// The scalar lane, from the right-hand side's sums (Re^2, Im^2, Re Im): its phase phi = arg(r^T r) / 2 and the
+// norms of its two parts, r_a^2 = sum + |r^T r| / 2, r_b^2 = sum - |r^T r| / 2.
+template <typename T> __device__ __noinline__ void start_state(T a, T b, T c, double d0, double w) {
+    Shared<T> &S = sh<T>();
+    const double sum = 0.5 * ((double)a + (double)b), D = 0.5 * ((double)a - (double)b), O = (double)c;
+    const double m = sqrt(D * D + O * O);
+    double cs = 1.0, sn = 0.0;
+    if (m > 0.0 && (double)b > 0.0) {
+        cs = sqrt(fmax(0.0, 0.5 * (1.0 + D / m)));
+        sn = copysign(sqrt(fmax(0.0, 0.5 * (1.0 - D / m))), O);
+    }
+    S.start[0] = cs;
+    S.start[1] = sn;
+    S.start[2] = sqrt(sum + m);
+    S.start[3] = (double)b > 0.0 ? sqrt(fmax(0.0, sum - m)) : 0.0;
+    S.F.sweeps = S.F.fail = 0;
+    S.F.rn2 = 0.0;
+    S.F.d0 = d0;                                         // 3 a_0 and the shift of H: -eps_n
+    S.F.w = w;
+}
+
+// Start of part pt of slot s's solve (every thread): false if there is nothing to solve for (uniform over
+// the cluster), else v_0 = f_re Re(r) + f_im Im(r).
+template <typename T> __device__ __noinline__ bool start_part(const LanczosArgs<T> &A, int s, int pt, bool scalar, T &f_re, T &f_im) {
+    Shared<T> &S = sh<T>();
+    const Slot &sl = A.slots[s];
+    const double thr_all = A.mixed ? fmax(A.inner_tol * sl.ref_norm, 0.3 * A.tol * sl.bnorm * sl.scale)
+                                   : A.tol * sl.bnorm;
+    const double na = S.start[2], nb = S.start[3], beta = pt ? nb : na;
+    // The parts' residuals add as orthogonal vectors nearly do.  A small r_b (rounding noise of the last inner
+    // solve) gets a small share of the threshold, comparable parts equal shares.
+    const double thr = thr_all * (nb == 0.0 ? 1.0 : nb > 0.1 * na ? 0.7 : pt ? 0.3 : 0.95);
+    if (!(beta > thr)) {
+        if (scalar) {
+            S.F.rn2 += beta * beta;
+            if (!(beta <= thr)) S.F.fail = 3;            // not a number
+        }
+        return false;
+    }
+    if (scalar) {
+        S.F.dr = S.F.di = S.F.zi = S.F.gam = 0.0;
+        S.F.zr = beta;
+        S.F.thr = thr;
+        S.flag = 0;
+    }
+    const double ib = 1.0 / beta;
+    f_re = (T)((pt ? -S.start[1] : S.start[0]) * ib);
+    f_im = (T)((pt ? S.start[0] : S.start[1]) * ib);
+    return true;
+}
+
+// The slot's state after its solve (the scalar lane of the cluster's first block).
+template <typename T> __device__ __noinline__ void end_state(const LanczosArgs<T> &A, int s) {
+    Slot &sl = A.slots[s];
+    const ScalarState &F = sh<T>().F;
+    sl.iters = F.sweeps;
+    sl.total_iters += F.sweeps;
+    sl.rnorm = sqrt(F.rn2);
+    if (A.mixed) {
+        if (F.fail == 3) sl.discard = 1;
+        if (F.fail >= 2) sl.status = RPA_ERR_BREAKDOWN;
+        sl.phase = kInnerDone;
+    } else {
+        sl.status = F.fail == 0 ? RPA_OK : F.fail == 1 ? RPA_ERR_NOT_CONVERGED : RPA_ERR_BREAKDOWN;
+        sl.phase = kFinished;
+    }
+}
+
 // The thread's sums of Re(r)^2, Im(r)^2 and Re(r) Im(r) over its points of slot s.
 template <typename T, int ZC> __device__ __noinline__ void start_sums(int s, T &rr, T &ii, T &ri) {
     using C = typename Cx<T>::t;
@@ -741,53 +809,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
             if (scalar) {
                 T a, b, c;
                 sum_parts(ng, ncl, a, b, c);
-                // phi = arg(r^T r) / 2; r_a^2 = sum + |r^T r| / 2, r_b^2 = sum - |r^T r| / 2
-                const double sum = 0.5 * ((double)a + (double)b), D = 0.5 * ((double)a - (double)b), O = (double)c;
-                const double m = sqrt(D * D + O * O);
-                double cs = 1.0, sn = 0.0;
-                if (m > 0.0 && (double)b > 0.0) {
-                    cs = sqrt(fmax(0.0, 0.5 * (1.0 + D / m)));
-                    sn = copysign(sqrt(fmax(0.0, 0.5 * (1.0 - D / m))), O);
-                }
-                S.start[0] = cs;
-                S.start[1] = sn;
-                S.start[2] = sqrt(sum + m);
-                S.start[3] = (double)b > 0.0 ? sqrt(fmax(0.0, sum - m)) : 0.0;
-                S.F.sweeps = S.F.fail = 0;
-                S.F.rn2 = 0.0;
-                S.F.d0 = A.d0 + A.slots[s].shift_re;     // the shift of H: -eps_n, omega
-                S.F.w = A.slots[s].shift_im;
+                start_state<T>(a, b, c, A.d0 + A.slots[s].shift_re, A.slots[s].shift_im);
             }
             __syncthreads();
         }
         for (int pt = 0; pt < 2; ++pt) {
             T f_re, f_im;
-            {
-                const Slot &sl = A.slots[s];
-                const double thr_all = A.mixed ? fmax(A.inner_tol * sl.ref_norm, 0.3 * A.tol * sl.bnorm * sl.scale)
-                                               : A.tol * sl.bnorm;
-                const double na = S.start[2], nb = S.start[3], beta = pt ? nb : na;
-                // The parts' residuals add as orthogonal vectors nearly do.  A small r_b (rounding noise of the
-                // last inner solve) gets a small share of the threshold, comparable parts equal shares.
-                const double thr = thr_all * (nb == 0.0 ? 1.0 : nb > 0.1 * na ? 0.7 : pt ? 0.3 : 0.95);
-                if (!(beta > thr)) {                     // nothing to solve for (uniform over the cluster)
-                    if (scalar) {
-                        S.F.rn2 += beta * beta;
-                        if (!(beta <= thr)) S.F.fail = 3;   // not a number
-                    }
-                    continue;
-                }
-                if (scalar) {
-                    S.F.dr = S.F.di = S.F.zi = S.F.gam = 0.0;
-                    S.F.zr = beta;
-                    S.F.thr = thr;
-                    S.flag = 0;
-                }
-                // v_0 = part / ||part||
-                const double ib = 1.0 / beta;
-                f_re = (T)((pt ? -S.start[1] : S.start[0]) * ib);
-                f_im = (T)((pt ? S.start[0] : S.start[1]) * ib);
-            }
+            if (!start_part<T>(A, s, pt, scalar, f_re, f_im)) continue;
             start_vector<T, ZC, MODE>(s, f_re, f_im);
             planes_stored();
             if (scalar) {
@@ -1009,24 +1037,397 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
             // (and no thread still reads the flag)
             cluster_barrier();
         }
-        // the slot's state
-        if (scalar && G.rank == 0) {
-            Slot &sl = A.slots[s];
-            const ScalarState &F = S.F;
-            sl.iters = F.sweeps;
-            sl.total_iters += F.sweeps;
-            sl.rnorm = sqrt(F.rn2);
-            if (A.mixed) {
-                if (F.fail == 3) sl.discard = 1;
-                if (F.fail >= 2) sl.status = RPA_ERR_BREAKDOWN;
-                sl.phase = kInnerDone;
-            } else {
-                sl.status = F.fail == 0 ? RPA_OK : F.fail == 1 ? RPA_ERR_NOT_CONVERGED : RPA_ERR_BREAKDOWN;
-                sl.phase = kFinished;
-            }
-        }
+        if (scalar && G.rank == 0) end_state(A, s);
     }
     cluster_barrier();                                  // no block leaves while another may write its memory
+}
+
+// ---------------------------------------------------------------------------------------------
+// The same solve for grids that do not fit on chip (mixed form, zero values outside the box): u and the
+// vectors stay in memory and a cluster of C blocks marches along z, block c over a band of rows, with 14
+// planes of its band and six rows on either side in a shared-memory ring.  One sweep is one Lanczos step:
+// at step f a thread forms v_k = (u - a' v_{k-1}) / g of plane f from the last sweep's u and v_{k-1} (its
+// band's halo rows too: they are formed by every block that reads them, so that bands exchange nothing
+// within a sweep), stores it in the ring and as vector k of the history, and after one barrier
+// applies the stencil to plane f - 6, writing u = B v_k - c v_{k-1} in place.  v_{k-1} is vector k - 1 of
+// the history, so the history costs no traffic of its own: a point takes 16 bytes an iteration (u and
+// v_{k-1} in, u and v_k out; v_{k-1}, read again six planes later, and V_loc come from L2) and 4 at the
+// end, against 64 of the fused COCG kernel on complex vectors.
+//
+// What bounds it: memory bandwidth, then shared memory (46 16-byte loads per unit of 4 x 2 points).
+// ---------------------------------------------------------------------------------------------
+constexpr int kRing = 14;                // planes f-13 .. f: the slot written at step f+1 was last read at f-1
+
+struct StreamArgs {
+    LanczosArgs<float> L;                // slots, queue, tolerances, workspace; pitch, plane: of the ring
+    const float *v;                      // V_loc, rows padded to px
+    int bh, hp;                          // rows of a band (even), halo row pairs on either side
+    int px;                              // padded row length in memory (a multiple of 4)
+    size_t nv;                           // elements of a vector in memory: nz ny px
+};
+
+// rows of nx values -> rows padded to px
+__global__ void k_pad_rows(const float *__restrict__ in, float *__restrict__ out, int nx, int px, long long rows) {
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < rows * px; e += (long long)gridDim.x * blockDim.x) {
+        const long long r = e / px;
+        const int i = (int)(e - r * px);
+        out[e] = i < nx ? in[r * nx + i] : 0.f;
+    }
+}
+
+struct StreamGeo {
+    int rank, gx, gy, nvx;
+    bool front, own, row1;               // forms points; of the block's band; row gy + 1 is one of them
+    int ring, mem;                       // the first point in a ring plane, and in a plane in memory
+    __device__ __forceinline__ StreamGeo(const StreamArgs &A) {
+        const int t = threadIdx.x, hw = A.L.hw;
+        rank = (int)(blockIdx.x % (unsigned)A.L.ncl);
+        const int y0 = rank * A.bh, y1 = min(A.L.ny, y0 + A.bh), pair = t / hw;
+        gx = 4 * (t - pair * hw);
+        gy = y0 + 2 * (pair - A.hp);
+        front = pair < A.bh / 2 + 2 * A.hp && gy >= 0 && gy < A.L.ny;
+        own = front && gy >= y0 && gy < y1;
+        row1 = gy + 1 < A.L.ny;
+        nvx = min(4, A.L.nx - gx);
+        ring = (gy - y0 + kRadius) * A.L.pitch + 8 + gx;
+        mem = front ? gy * A.px + gx : 0;
+    }
+};
+
+// x += sum_j y_j v_j (and the COCG direction) over the n vectors of the history, as flush() does.
+__device__ __noinline__ void stream_flush(const StreamArgs *args, int s, int n, bool go_on, bool have_p, double er, double ei) {
+    using P = Pk<float>;
+    Shared<float> &S = sh<float>();
+    const StreamArgs &A = *args;
+    const StreamGeo G(A);
+    const int ncl = A.L.ncl;
+    float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)ncl) * A.L.ws_stride;
+    float *const Pd = U + 2 * A.nv, *const H = Pd + 2 * A.nv;
+    if ((int)threadIdx.x == (int)blockDim.x - 32) {
+        double yr = 0, yi = 0, qr = 0, qi = 0;
+        for (int j = n - 1; j >= 0; --j) {
+            const double cn = j + 1 < n ? (double)(float)S.g[j + 1] : 0.0, dr = S.dr[j], di = S.di[j];
+            const double tr = S.zr[j] - cn * yr, ti = S.zi[j] - cn * yi;
+            yr = tr * dr - ti * di;
+            yi = tr * di + ti * dr;
+            const double ur = j == n - 1 ? 1.0 : -cn * qr, ui = j == n - 1 ? 0.0 : -cn * qi;
+            qr = ur * dr - ui * di;
+            qi = ur * di + ui * dr;
+            S.coef[j] = make_float4((float)(er * yr - ei * yi), (float)(er * yi + ei * yr), (float)qr, (float)qi);
+        }
+        const double c0 = (double)(float)S.g[0];
+        S.prev = make_float4((float)(-c0 * (er * yr - ei * yi)), (float)(-c0 * (er * yi + ei * yr)), (float)(-c0 * qr),
+                             (float)(-c0 * qi));
+    }
+    __syncthreads();
+    if (G.own) {
+        float2 *const xg = A.L.x + (long long)s * A.L.nd;
+        for (int z = 0; z < A.L.nz; ++z)
+            for (int r = 0; r < (G.row1 ? 2 : 1); ++r) {
+                const size_t o = (size_t)z * A.L.ny * A.px + G.mem + r * A.px;
+                P xr, xi, pr, pi;
+                xr.zero();
+                xi.zero();
+                pr.zero();
+                pi.zero();
+                if (have_p) {
+                    const float4 c = S.prev;
+                    const P qr = pk_load(Pd + o), qi = pk_load(Pd + A.nv + o);
+                    xr.fma(c.x, qr);
+                    xr.fma(-c.y, qi);
+                    xi.fma(c.x, qi);
+                    xi.fma(c.y, qr);
+                    pr.fma(c.z, qr);
+                    pr.fma(-c.w, qi);
+                    pi.fma(c.z, qi);
+                    pi.fma(c.w, qr);
+                }
+                if (go_on) {
+#pragma unroll 8
+                    for (int j = 0; j < n; ++j) {
+                        const float4 c = S.coef[j];
+                        const P v = pk_load(H + (size_t)j * A.nv + o);
+                        xr.fma(c.x, v);
+                        xi.fma(c.y, v);
+                        pr.fma(c.z, v);
+                        pi.fma(c.w, v);
+                    }
+                    pk_store(Pd + o, pr);
+                    pk_store(Pd + A.nv + o, pi);
+                } else {
+#pragma unroll 8
+                    for (int j = 0; j < n; ++j) {
+                        const float4 c = S.coef[j];
+                        const P v = pk_load(H + (size_t)j * A.nv + o);
+                        xr.fma(c.x, v);
+                        xi.fma(c.y, v);
+                    }
+                }
+                float2 *dst = xg + ((long long)z * A.L.ny + G.gy + r) * A.L.nx + G.gx;
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < G.nvx) {
+                        float2 q = dst[i];
+                        q.x += xr.get(i);
+                        q.y += xi.get(i);
+                        dst[i] = q;
+                    }
+            }
+    }
+    __syncthreads();
+}
+
+// Sums of the right-hand side (f_re = f_im = 0: into sums) or u = f_re Re(r) + f_im Im(r).
+__device__ __noinline__ void stream_start(const StreamArgs *args, int s, float f_re, float f_im, bool store, float &rr,
+                                          float &ii, float &ri) {
+    const StreamArgs &A = *args;
+    const StreamGeo G(A);
+    float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)A.L.ncl) * A.L.ws_stride;
+    const float2 *const rg = A.L.r + (long long)s * A.L.nd;
+    float a = 0.f, b = 0.f, c = 0.f;
+    if (G.own)
+#pragma unroll 4
+        for (int z = 0; z < A.L.nz; ++z)
+#pragma unroll
+            for (int r = 0; r < 2; ++r)
+                if (r == 0 || G.row1) {
+                    const float2 *src = rg + ((long long)z * A.L.ny + G.gy + r) * A.L.nx + G.gx;
+                    Pk<float> w;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 v = i < G.nvx ? src[i] : make_float2(0.f, 0.f);
+                        a += v.x * v.x;
+                        b += v.y * v.y;
+                        c += v.x * v.y;
+                        w.set(i, f_re * v.x + f_im * v.y);
+                    }
+                    if (store) pk_store(U + (size_t)z * A.L.ny * A.px + G.mem + r * A.px, w);
+                }
+    rr = a;
+    ii = b;
+    ri = c;
+}
+
+__global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant__ StreamArgs A, const __grid_constant__ Coef<float> cf) {
+    using P = Pk<float>;
+    Shared<float> &S = sh<float>();
+    const int tid = threadIdx.x, ncl = A.L.ncl, nz = A.L.nz;
+    const StreamGeo G(A);
+    const bool scalar = tid == (int)blockDim.x - 32;
+    float *const ring = slab_of(A.L);
+    for (int e = tid; e < A.L.smem_words; e += blockDim.x)
+        reinterpret_cast<int4 *>(lz_smem + shared_bytes<float>())[e] = make_int4(0, 0, 0, 0);
+    if (scalar) {
+        for (int q = 0; q < 2; ++q) mbar_init(&S.pbar[q]);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)ncl) * A.L.ws_stride;
+    float *const H = U + 4 * A.nv;                       // after u (two buffers) and the direction (re, im)
+    const size_t pl = (size_t)A.L.ny * A.px;             // a plane in memory
+    const int n_items = *A.L.cnt;
+    unsigned ng = 0;
+    cluster_barrier();
+    for (;;) {
+        if (G.rank == 0 && tid < ncl) {
+            int it = 0;
+            if (tid == 0) it = atomicAdd(A.L.grab, 1);
+            it = __shfl_sync((1u << ncl) - 1u, it, 0);
+            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
+                             map_rank((unsigned)__cvta_generic_to_shared(&S.item), tid)),
+                         "r"(it)
+                         : "memory");
+        }
+        cluster_barrier();
+        if (S.item >= n_items) break;
+        const int s = A.L.list[n_items - 1 - S.item];
+        {
+            float rr, ii, ri;
+            stream_start(&A, s, 0.f, 0.f, false, rr, ii, ri);
+            gather3(rr, ii, ri, ng, ncl, G.rank, A.L.err);
+            if (scalar) {
+                float a, b, c;
+                sum_parts(ng, ncl, a, b, c);
+                start_state(a, b, c, A.L.d0 + A.L.slots[s].shift_re, A.L.slots[s].shift_im);
+            }
+            __syncthreads();
+        }
+        for (int pt = 0; pt < 2; ++pt) {
+            float f_re, f_im;
+            if (!start_part<float>(A.L, s, pt, scalar, f_re, f_im)) continue;
+            {
+                float d0, d1, d2;
+                stream_start(&A, s, f_re, f_im, true, d0, d1, d2);
+            }
+            cluster_barrier();                           // u is stored in every band
+            float ap = 0.f, ig = 1.f, cc = 0.f, dg = (float)S.F.d0;   // the first sweep: v_0 = u
+            int k = 0, kb = 0, n = 0;
+            bool have_p = false;
+            for (;;) {
+                // u alternates between two buffers: a band may be planes ahead of one that reads its rows
+                const float *const ui = U + (size_t)(k & 1) * A.nv;
+                float *const uo = U + (size_t)((k & 1) ^ 1) * A.nv;
+                const float *const vp = k == 0 ? U : H + (size_t)(k == kb ? A.L.hist - 1 : k - 1 - kb) * A.nv;
+                float *const vk = H + (size_t)(k - kb) * A.nv;
+                const float m_ag = -ap * ig;
+                float svv = 0.f, suv = 0.f, suu = 0.f;
+                P zero;
+                zero.zero();
+                // ring planes -6 .. -1 (slots 8 .. 13) are zero
+                if (G.front)
+                    for (int m = kRing - kRadius; m < kRing; ++m) {
+                        pk_store(ring + m * A.L.plane + G.ring, zero);
+                        if (G.row1) pk_store(ring + m * A.L.plane + G.ring + A.L.pitch, zero);
+                    }
+                P fu[2], fv[2];                          // u and v_{k-1} of the next front plane
+                auto load_front = [&](int f) {
+                    const size_t o = f * pl + G.mem;
+                    fu[0] = pk_load_l2(ui + o);
+                    fv[0] = pk_load_l2(vp + o);
+                    if (G.row1) {
+                        fu[1] = pk_load_l2(ui + o + A.px);
+                        fv[1] = pk_load_l2(vp + o + A.px);
+                    }
+                };
+                fu[1].zero();
+                fv[1].zero();
+                if (G.front) load_front(0);
+                for (int f = 0, slot = 0; f < nz + kRadius; ++f, slot = slot + 1 == kRing ? 0 : slot + 1) {
+                    const int z = f - kRadius;
+                    P lv[2], vv[2];                      // v_{k-1} and V_loc of the stencil's plane
+                    if (G.own && z >= 0) {
+                        const size_t o = z * pl + G.mem;
+                        lv[0] = pk_load_l2(vp + o);
+                        vv[0] = pk_load(A.v + o);
+                        lv[1] = G.row1 ? pk_load_l2(vp + o + A.px) : zero;
+                        vv[1] = G.row1 ? pk_load(A.v + o + A.px) : zero;
+                    }
+                    if (G.front) {
+                        P w[2] = {zero, zero};
+                        if (f < nz) {
+                            const size_t o = f * pl + G.mem;
+#pragma unroll
+                            for (int r = 0; r < 2; ++r)
+                                if (r == 0 || G.row1) {
+                                    w[r] = fu[r];
+                                    w[r].mul(ig);
+                                    w[r].fma(m_ag, fv[r]);
+                                    if (G.own) pk_store(vk + o + r * A.px, w[r]);
+                                }
+                        }
+                        float *const dst = ring + slot * A.L.plane + G.ring;
+                        pk_store(dst, w[0]);
+                        if (G.row1) pk_store(dst + A.L.pitch, w[1]);
+                        if (f + 1 < nz) load_front(f + 1);
+                    }
+                    __syncthreads();
+                    if (G.own && z >= 0) {
+                        const int cz = slot >= kRadius ? slot - kRadius : slot + kRing - kRadius;
+                        const float *const c0 = ring + cz * A.L.plane + G.ring;
+                        const int pitch = A.L.pitch, d1 = G.row1 ? pitch : 0;
+                        P a0, a1, ctr0, ctr1;
+                        a0.zero();
+                        a1.zero();
+                        a0.fma(-cc, lv[0]);
+                        a1.fma(-cc, lv[1]);
+                        {
+                            P X[5];
+#pragma unroll
+                            for (int m = 0; m < 5; ++m) X[m] = pk_load(c0 - 8 + 4 * m);
+                            ctr0 = X[2];
+                            x_part(a0, X, cf);
+                        }
+                        {
+                            P X[5];
+#pragma unroll
+                            for (int m = 0; m < 5; ++m) X[m] = pk_load(c0 + d1 - 8 + 4 * m);
+                            ctr1 = X[2];
+                            x_part(a1, X, cf);
+                        }
+                        const P nb1 = G.row1 ? ctr1 : pk_load(c0 + pitch);   // a row of zeros
+                        a0.fma(cf.a[1], nb1);
+                        a1.fma(cf.a[1], ctr0);
+#pragma unroll
+                        for (int d = 1; d <= kRadius; ++d) {
+                            const P lo = pk_load(c0 - d * pitch), hi = pk_load(c0 + (1 + d) * pitch);
+                            a0.fma(cf.a[d], lo);
+                            a1.fma(cf.a[d], hi);
+                            if (d < kRadius) {
+                                a1.fma(cf.a[d + 1], lo);
+                                a0.fma(cf.a[d + 1], hi);
+                            }
+                            const int sm = cz >= d ? cz - d : cz + kRing - d, sp = cz + d < kRing ? cz + d : cz + d - kRing;
+                            const float *const pm = ring + sm * A.L.plane + G.ring, *const pp = ring + sp * A.L.plane + G.ring;
+                            a0.fma(cf.a[d], pk_load(pm));
+                            a0.fma(cf.a[d], pk_load(pp));
+                            a1.fma(cf.a[d], pk_load(pm + d1));
+                            a1.fma(cf.a[d], pk_load(pp + d1));
+                        }
+                        a0.fma(dg, ctr0);
+                        a1.fma(dg, ctr1);
+                        a0.fma(vv[0], ctr0);
+                        a1.fma(vv[1], ctr1);
+                        P t0, t1, t2;
+                        t0.zero();
+                        t1.zero();
+                        t2.zero();
+#pragma unroll
+                        for (int i = 1; i < 4; ++i)      // u = 0 outside the box
+                            if (i >= G.nvx) {
+                                a0.set(i, 0.f);
+                                a1.set(i, 0.f);
+                            }
+                        const size_t o = z * pl + G.mem;
+                        pk_store(uo + o, a0);
+                        t0.fma(ctr0, ctr0);
+                        t1.fma(a0, ctr0);
+                        t2.fma(a0, a0);
+                        if (G.row1) {
+                            pk_store(uo + o + A.px, a1);
+                            t0.fma(ctr1, ctr1);
+                            t1.fma(a1, ctr1);
+                            t2.fma(a1, a1);
+                        }
+                        svv += t0.sum();
+                        suv += t1.sum();
+                        suu += t2.sum();
+                    }
+                }
+                // (also: every ring reader of the sweep is done)
+                gather3(svv, suv, suu, ng, ncl, G.rank, A.L.err);
+                {
+                    float a, b, c;
+                    sum_parts(ng, ncl, a, b, c);
+                    ap = b / a;
+                    const float b2 = c - ap * b;
+                    ig = b2 > 0.f ? 1.f / sqrtf(b2) : 0.f;
+                    if (!isfinite(a) || !isfinite(c)) ig = nanf("");
+                }
+                ++k;
+                if (scalar) {
+                    S.F.ak = S.F.d0 - (double)dg + (double)ap;
+                    S.F.ck = (double)cc;
+                    S.F.ig = (double)ig;
+                    factor<float>(k - 1 - kb, k, A.L.maxit);
+                    if (A.L.prof && G.rank == 0) atomicAdd(A.L.prof + 1, (unsigned long long)A.L.nd);
+                }
+                cc = ig > 0.f ? 1.f / ig : 0.f;
+                dg -= ap;
+                cluster_barrier();                       // u and v_k of every band are written; the decision is taken
+                n = k - kb;
+                if (S.flag) break;
+                if (n == A.L.hist) {                     // the history is full: into x and p
+                    stream_flush(&A, s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+                    have_p = true;
+                    kb = k;
+                }
+            }
+            if (S.flag < 4)
+                stream_flush(&A, s, n, false, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+            cluster_barrier();                           // no thread still reads the flag or this part's vectors
+        }
+        if (scalar && G.rank == 0) end_state(A.L, s);
+    }
+    cluster_barrier();
 }
 
 struct Variant {
@@ -1063,6 +1464,53 @@ void cluster_config(cudaLaunchConfig_t &lc, cudaLaunchAttribute &at, int ncl, in
 }
 
 }  // namespace
+
+// Plan of the streaming kernel: the fewest bands (1, 2, 4, 8) whose ring fits a block.
+static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan &p) {
+    if (c.opt.prec != RPA_MIXED || c.opt.periodic) return false;
+    const void *fn = (const void *)k_lanczos_stream;
+    const int hw = (c.nx + 3) / 4;
+    int p16 = 2 + hw;
+    while ((2 * p16 - (hw + hw % 2)) % 8 != 0) ++p16;
+    for (int ncl = 1; ncl <= 8; ncl *= 2) {
+        const int bh = ((c.ny + ncl - 1) / ncl + 1) / 2 * 2, hp = ncl > 1 ? kRadius / 2 : 0;
+        if (bh < 2 || (long long)bh * (ncl - 1) >= c.ny) return false;
+        const long long units = (long long)hw * (bh / 2 + 2 * hp);
+        const int threads = (int)std::min<long long>((units + 31) / 32 * 32 + 32, 1 << 20);
+        const int pitch = 4 * p16, plane = pitch * (bh + 2 * kRadius);
+        const size_t smem = shared_bytes<float>() + sizeof(float) * ((size_t)kRing * plane + 16);
+        if (threads > 512 || smem > (size_t)optin) continue;
+        RPA_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        allow_dynamic_smem(fn, smem);
+        cudaLaunchConfig_t lc{};
+        cudaLaunchAttribute at{};
+        cluster_config(lc, at, ncl, ncl * sms, threads, smem, nullptr);
+        int ncs = 0;
+        if (cudaOccupancyMaxActiveClusters(&ncs, fn, &lc) != cudaSuccess || ncs < 1) {
+            (void)cudaGetLastError();
+            continue;
+        }
+        p = LanczosPlan{};
+        p.stream = 1;
+        p.mixed = 1;
+        p.ncl = ncl;
+        p.clusters = std::min(ncs, nsys);
+        p.threads = threads;
+        p.smem = smem;
+        p.hw = hw;
+        p.pitch = pitch;
+        p.plane = plane;
+        p.bh = bh;
+        p.hp = hp;
+        const size_t nv = (size_t)c.nz * c.ny * 4 * hw;
+        // history: as many vectors as 8 GB hold, 16 .. kHistMax
+        p.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, ((size_t)8 << 30) / (nv * 4 * p.clusters)));
+        p.ws_stride = nv * (4 + p.hist);
+        p.ws_bytes = sizeof(float) * (p.ws_stride * p.clusters + nv);     // and V_loc
+        return true;
+    }
+    return false;
+}
 
 bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
     if (c.opt.precondition || c.nz < kRadius + 2 || c.ny < kRadius || c.nx < kRadius) return false;
@@ -1137,7 +1585,8 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
             }
         }
     }
-    if (!found) return false;
+    if (!found) return stream_plan(c, nsys, sms, optin, best);
+    best.stream = 0;
     const size_t vec = (size_t)2 * best.zc * (best.threads - 32) * W, hvec = (size_t)best.nch * best.zc * best.plane;
     // history: as many vectors as 2 GB hold, 16 .. kHistMax
     const size_t per_vec = hvec * tsz * best.clusters * best.ncl;
@@ -1147,7 +1596,7 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
     return true;
 }
 
-template <typename T> static void launch(const Ctx &c, const LanczosPlan &p, LanczosArgs<T> a, cudaStream_t s) {
+template <typename T> static void fill_args(const Ctx &c, const LanczosPlan &p, LanczosArgs<T> &a) {
     a.ws = (T *)p.ws;
     a.ws_stride = p.ws_stride;
     a.nd = c.nd;
@@ -1166,12 +1615,16 @@ template <typename T> static void launch(const Ctx &c, const LanczosPlan &p, Lan
     a.plane = p.plane;
     a.lead = p.lead;
     a.nzl_max = (c.nz + p.ncl - 1) / p.ncl;
-    a.stages = std::min(kStages, (p.nch * p.zc + 2 * kRadius) / a.nzl_max);
+    a.stages = p.stream ? 0 : std::min(kStages, (p.nch * p.zc + 2 * kRadius) / a.nzl_max);
     a.err = c.d_tc_err;
     a.reach = p.reach;
     a.hist = p.hist;
     a.smem_words = (int)((p.smem - shared_bytes<T>()) / 16);
     a.d0 = 3.0 * c.coef.a[0];
+}
+
+template <typename T> static void launch(const Ctx &c, const LanczosPlan &p, LanczosArgs<T> a, cudaStream_t s) {
+    fill_args(c, p, a);
     const Coef<T> cf = cast_coef<T>(c.coef);
     const void *fn = kernel_of(p.mixed, p.variant, c.opt.periodic != 0);
     allow_dynamic_smem(fn, p.smem);
@@ -1183,7 +1636,37 @@ template <typename T> static void launch(const Ctx &c, const LanczosPlan &p, Lan
     RPA_CUDA(cudaLaunchKernelExC(&lc, fn, args));
 }
 
-void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<float> &a, cudaStream_t s) { launch(c, p, a, s); }
+void lanczos_prepare(const Ctx &c, const LanczosPlan &p, cudaStream_t s) {
+    if (!p.stream) return;
+    const size_t nv = (size_t)c.nz * c.ny * 4 * p.hw;
+    k_pad_rows<<<(unsigned)std::min<size_t>((nv + 255) / 256, 2048), 256, 0, s>>>(
+        c.vloc32, (float *)p.ws + p.ws_stride * p.clusters, c.nx, 4 * p.hw, (long long)c.nz * c.ny);
+    RPA_LAUNCH("V_loc rows");
+    count_launches(1);
+}
+
+void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<float> &args, cudaStream_t s) {
+    if (!p.stream) {
+        launch(c, p, args, s);
+        return;
+    }
+    StreamArgs a{};
+    a.L = args;
+    fill_args(c, p, a.L);
+    a.px = 4 * p.hw;
+    a.nv = (size_t)c.nz * c.ny * a.px;
+    a.v = (const float *)p.ws + p.ws_stride * p.clusters;
+    a.bh = p.bh;
+    a.hp = p.hp;
+    const Coef<float> cf = cast_coef<float>(c.coef);
+    const void *fn = (const void *)k_lanczos_stream;
+    allow_dynamic_smem(fn, p.smem);
+    cudaLaunchConfig_t lc{};
+    cudaLaunchAttribute at{};
+    cluster_config(lc, at, p.ncl, p.ncl * p.clusters, p.threads, p.smem, s);
+    void *kargs[2] = {(void *)&a, (void *)&cf};
+    RPA_CUDA(cudaLaunchKernelExC(&lc, fn, kargs));
+}
 void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<double> &a, cudaStream_t s) { launch(c, p, a, s); }
 
 }  // namespace rpa

@@ -28,6 +28,8 @@ template <typename T> struct LanczosArgs {
 // Plan for nsys systems of this context; false where the grid does not fit on chip (or its slabs
 // would be mostly halo) and the COCG kernels run instead.
 bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &p);
+// Once a queue, before its launches (p.ws set).
+void lanczos_prepare(const Ctx &c, const LanczosPlan &p, cudaStream_t s);
 void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<float> &a, cudaStream_t s);
 void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<double> &a, cudaStream_t s);
 
