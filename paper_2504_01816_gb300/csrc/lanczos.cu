@@ -115,6 +115,9 @@ __device__ __forceinline__ Pk<double> pk_load(const double *a) {
     r.p = *reinterpret_cast<const double2 *>(a);
     return r;
 }
+// The same from a byte offset in the block's shared memory (a thread's offset plus ones that are the same for
+// all threads, which stay in the uniform registers of the load's address).
+template <typename T> __device__ __forceinline__ Pk<T> lds(int off);
 // The same from the history, past L1: the bulk stores that write it do not update L1's lines.
 __device__ __forceinline__ Pk<float> pk_load_l2(const float *a) {
     const float4 t = __ldcg(reinterpret_cast<const float4 *>(a));
@@ -235,6 +238,9 @@ template <typename T> struct Shared {
 template <typename T> constexpr int shared_bytes() { return (int)((sizeof(Shared<T>) + 127) / 128 * 128); }
 
 extern __shared__ __align__(128) unsigned char lz_smem[];
+template <typename T> __device__ __forceinline__ Pk<T> lds(int off) {
+    return pk_load(reinterpret_cast<const T *>(lz_smem + off));
+}
 template <typename T> __device__ __forceinline__ Shared<T> &sh() { return *reinterpret_cast<Shared<T> *>(lz_smem); }
 
 // A thread's points: W values of x from gx, rows gy and gy + 1, local planes lz0 .. lz0 + ZC - 1.
@@ -784,6 +790,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
     const Geo<T, ZC> G(A);
     const bool scalar = tid == G.nthr;
     T *const slab = slab_of(A);
+    const int slab_off = shared_bytes<T>() + A.lead * (int)sizeof(T);
+    const int pb = A.plane * (int)sizeof(T), rb = A.pitch * (int)sizeof(T);   // bytes of a plane, a row
+    constexpr int QB = 16;                              // bytes of W values
     const int n_items = *A.cnt;
     unsigned phase = 0, ng = 0;                         // halo phase, reductions so far
     cluster_barrier();                                  // every block runs, has cleared its slab and set its barriers
@@ -833,11 +842,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
             int k = 0, kb = 0, n = 0;                    // step, first vector of the history, vectors to flush
             bool have_p = false;
             for (;;) {
-                // the unit's first point, its second row, the row and plane strides: made opaque so that the
-                // hundreds of addresses formed from them are not kept (and spilled) across iterations
-                int c0 = G.c0, d1 = G.c1 - G.c0, pitch = A.pitch, planeE = A.plane;
-                asm volatile("" : "+r"(c0), "+r"(d1), "+r"(pitch), "+r"(planeE));
-                const T *const b0 = slab + c0;
+                // byte offsets of the unit's rows: made opaque so that the hundreds of addresses formed from
+                // them are not kept (and spilled) across iterations
+                int o0 = slab_off + G.c0 * (int)sizeof(T), o1 = slab_off + G.c1 * (int)sizeof(T);
+                asm volatile("" : "+r"(o0), "+r"(o1));
                 if (scalar) {
                     if (k > kb) factor<T>(k - 1 - kb, k, A.maxit);
                     keep_wait();
@@ -849,15 +857,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
 #pragma unroll
                 for (int i = 0; i < W; ++i) mask.set(i, i < G.nvx ? (T)1 : (T)0);
                 if (G.unit) {
-                    // the row r rows from the unit's first (pl)
-                    auto yrow = [&](const T *pl, int r) -> const T * {
-                        if (MODE == 0) return pl + r * pitch;
+                    // the row r rows from the unit's first, at offset o
+                    auto yrow = [&](int o, int r) -> P {
+                        if (MODE == 0) return lds<T>(o + r * rb);
                         int y = G.gy + r;
-                        if (MODE == 2)
-                            return y >= 0 && y < A.ny ? pl + r * pitch
-                                                      : reinterpret_cast<const T *>(lz_smem + shared_bytes<T>());
+                        if (MODE == 2) return lds<T>(y >= 0 && y < A.ny ? o + r * rb : shared_bytes<T>());
                         y = y < 0 ? y + A.ny : y >= A.ny ? y - A.ny : y;
-                        return pl + (y - G.gy) * pitch;
+                        return lds<T>(o + (y - G.gy) * rb);
                     };
                     const T *const wv = A.ws + (size_t)blockIdx.x * A.ws_stride + (size_t)tid * W;
                     const int vs = G.nthr * W;
@@ -870,7 +876,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                         a0.mul(-cc);
                         a1.mul(-cc);
                         if (z < G.nvz) {
-                            const T *const pl = b0 + z * planeE;
+                            const int q0 = o0 + z * pb, q1 = o1 + z * pb;
                             const P pv0 = vn[0], pv1 = vn[1];
                             if (z + 1 < ZC) {
                                 vn[0] = pk_load(wv + (2 * z + 2) * vs);
@@ -880,23 +886,23 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                             {
                                 P X[XL];
 #pragma unroll
-                                for (int m = 0; m < XL; ++m) X[m] = pk_load(pl - PAD + m * W);
+                                for (int m = 0; m < XL; ++m) X[m] = lds<T>(q0 + (m - PAD / W) * QB);
                                 ctr0 = X[PAD / W];
                                 x_part(a0, X, cf);
                             }
                             {
                                 P X[XL];
 #pragma unroll
-                                for (int m = 0; m < XL; ++m) X[m] = pk_load(pl + d1 - PAD + m * W);
+                                for (int m = 0; m < XL; ++m) X[m] = lds<T>(q1 + (m - PAD / W) * QB);
                                 ctr1 = X[PAD / W];
                                 x_part(a1, X, cf);
                             }
-                            nb1 = G.row1 ? ctr1 : pk_load(yrow(pl, 1));
+                            nb1 = G.row1 ? ctr1 : yrow(q0, 1);
                             a0.fma(cf.a[1], nb1);
                             a1.fma(cf.a[1], ctr0);
 #pragma unroll
                             for (int d = 1; d <= kRadius; ++d) {
-                                const P lo = pk_load(yrow(pl, -d)), hi = pk_load(yrow(pl, 1 + d));
+                                const P lo = yrow(q0, -d), hi = yrow(q0, 1 + d);
                                 a0.fma(cf.a[d], lo);
                                 a1.fma(cf.a[d], hi);
                                 if (d < kRadius) {
@@ -923,10 +929,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                 if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.bar), phase)) atomicExch(A.err, 2);
                 phase ^= 1u;
                 if (G.unit) {
-                    const T *const bz = b0 - kRadius * planeE;
 #pragma unroll
                     for (int p = 0; p < ZC + 2 * kRadius; ++p) {
-                        const P v0 = pk_load(bz + p * planeE), v1 = pk_load(bz + d1 + p * planeE);
+                        const P v0 = lds<T>(o0 + (p - kRadius) * pb), v1 = lds<T>(o1 + (p - kRadius) * pb);
 #pragma unroll
                         for (int z = 0; z < ZC; ++z) {
                             const int d = p - z - kRadius < 0 ? z + kRadius - p : p - z - kRadius;
@@ -945,7 +950,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                             P &a0 = acc[z][0], &a1 = acc[z][1];
                             a0.mul(mask);                // u = 0 outside the box
                             a1.mul(mask);
-                            const P v0 = pk_load(b0 + z * planeE), v1 = pk_load(b0 + d1 + z * planeE);
+                            const P v0 = lds<T>(o0 + z * pb), v1 = lds<T>(o1 + z * pb);
                             t1.fma(a0, v0);
                             t2.fma(a0, a0);
                             if (G.row1) {
@@ -995,7 +1000,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
 #pragma unroll
                         for (int r = 0; r < 2; ++r)
                             if (r == 0 || G.row1) {
-                                T *const own = slab + c0 + (r ? d1 : 0) + z * planeE;
+                                T *const own = reinterpret_cast<T *>(lz_smem + (r ? o1 : o0) + z * pb);
                                 const P v = pk_load(own);
                                 P w = acc[z][r];
                                 w.mul(ig);
@@ -1028,7 +1033,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                 if (scalar) {
                     const Work<T, ZC> K(A);
                     send_halos(slab);
-                    keep(slab, K.H, K.hvec, k - kb, G.nzl, planeE);
+                    keep(slab, K.H, K.hvec, k - kb, G.nzl, A.plane);
                 }
             }
             if (S.flag < 4)                              // nothing is kept of a solve that went non-finite
@@ -1214,7 +1219,10 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
     const int tid = threadIdx.x, ncl = A.L.ncl, nz = A.L.nz;
     const StreamGeo G(A);
     const bool scalar = tid == (int)blockDim.x - 32;
-    float *const ring = slab_of(A.L);
+    // byte offsets in shared memory: the unit's rows in ring slot 0; bytes of a ring plane, of a row
+    const int o0 = shared_bytes<float>() + G.ring * 4, pb = A.L.plane * 4, rb = A.L.pitch * 4;
+    const int o1 = G.row1 ? o0 + rb : o0;
+    auto at = [&](int off) -> float * { return reinterpret_cast<float *>(lz_smem + off); };
     for (int e = tid; e < A.L.smem_words; e += blockDim.x)
         reinterpret_cast<int4 *>(lz_smem + shared_bytes<float>())[e] = make_int4(0, 0, 0, 0);
     if (scalar) {
@@ -1275,32 +1283,45 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
                 // ring planes -6 .. -1 (slots 8 .. 13) are zero
                 if (G.front)
                     for (int m = kRing - kRadius; m < kRing; ++m) {
-                        pk_store(ring + m * A.L.plane + G.ring, zero);
-                        if (G.row1) pk_store(ring + m * A.L.plane + G.ring + A.L.pitch, zero);
+                        pk_store(at(o0 + m * pb), zero);
+                        if (G.row1) pk_store(at(o1 + m * pb), zero);
                     }
-                P fu[2], fv[2];                          // u and v_{k-1} of the next front plane
-                auto load_front = [&](int f) {
-                    const size_t o = f * pl + G.mem;
-                    fu[0] = pk_load_l2(ui + o);
-                    fv[0] = pk_load_l2(vp + o);
+                // u and v_{k-1} of the next two front planes; v_{k-1} and V_loc of the next stencil plane
+                P fu[2][2], fv[2][2], nlv[2], nvv[2];
+                const float *pu = ui + G.mem, *pv = vp + G.mem;
+                auto load_front = [&](int f, P (&u)[2], P (&v)[2]) {
+                    const size_t o = f * pl;
+                    u[0] = pk_load_l2(pu + o);
+                    v[0] = pk_load_l2(pv + o);
                     if (G.row1) {
-                        fu[1] = pk_load_l2(ui + o + A.px);
-                        fv[1] = pk_load_l2(vp + o + A.px);
+                        u[1] = pk_load_l2(pu + o + A.px);
+                        v[1] = pk_load_l2(pv + o + A.px);
                     }
                 };
-                fu[1].zero();
-                fv[1].zero();
-                if (G.front) load_front(0);
-                for (int f = 0, slot = 0; f < nz + kRadius; ++f, slot = slot + 1 == kRing ? 0 : slot + 1) {
-                    const int z = f - kRadius;
-                    P lv[2], vv[2];                      // v_{k-1} and V_loc of the stencil's plane
-                    if (G.own && z >= 0) {
-                        const size_t o = z * pl + G.mem;
-                        lv[0] = pk_load_l2(vp + o);
-                        vv[0] = pk_load(A.v + o);
-                        lv[1] = G.row1 ? pk_load_l2(vp + o + A.px) : zero;
-                        vv[1] = G.row1 ? pk_load(A.v + o + A.px) : zero;
+                auto load_centre = [&](int z) {
+                    const size_t o = z * pl;
+                    nlv[0] = pk_load_l2(pv + o);
+                    nvv[0] = pk_load(A.v + G.mem + o);
+                    if (G.row1) {
+                        nlv[1] = pk_load_l2(pv + o + A.px);
+                        nvv[1] = pk_load(A.v + G.mem + o + A.px);
                     }
+                };
+#pragma unroll
+                for (int r = 0; r < 2; ++r) fu[r][1] = fv[r][1] = nlv[r] = nvv[r] = zero;
+                if (G.front) {
+                    load_front(0, fu[0], fv[0]);
+                    if (nz > 1) load_front(1, fu[1], fv[1]);
+                }
+                auto step = [&](int f, int slot, P (&cu)[2], P (&cv)[2]) {
+                    const int z = f - kRadius;
+                    P lv[2], vv[2];
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        lv[r] = nlv[r];
+                        vv[r] = nvv[r];
+                    }
+                    if (G.own && z + 1 >= 0 && z + 1 < nz) load_centre(z + 1);
                     if (G.front) {
                         P w[2] = {zero, zero};
                         if (f < nz) {
@@ -1308,22 +1329,20 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
 #pragma unroll
                             for (int r = 0; r < 2; ++r)
                                 if (r == 0 || G.row1) {
-                                    w[r] = fu[r];
+                                    w[r] = cu[r];
                                     w[r].mul(ig);
-                                    w[r].fma(m_ag, fv[r]);
+                                    w[r].fma(m_ag, cv[r]);
                                     if (G.own) pk_store(vk + o + r * A.px, w[r]);
                                 }
                         }
-                        float *const dst = ring + slot * A.L.plane + G.ring;
-                        pk_store(dst, w[0]);
-                        if (G.row1) pk_store(dst + A.L.pitch, w[1]);
-                        if (f + 1 < nz) load_front(f + 1);
+                        pk_store(at(o0 + slot * pb), w[0]);
+                        if (G.row1) pk_store(at(o1 + slot * pb), w[1]);
+                        if (f + 2 < nz) load_front(f + 2, cu, cv);
                     }
                     __syncthreads();
                     if (G.own && z >= 0) {
                         const int cz = slot >= kRadius ? slot - kRadius : slot + kRing - kRadius;
-                        const float *const c0 = ring + cz * A.L.plane + G.ring;
-                        const int pitch = A.L.pitch, d1 = G.row1 ? pitch : 0;
+                        const int q0 = o0 + cz * pb, q1 = o1 + cz * pb;
                         P a0, a1, ctr0, ctr1;
                         a0.zero();
                         a1.zero();
@@ -1332,35 +1351,35 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
                         {
                             P X[5];
 #pragma unroll
-                            for (int m = 0; m < 5; ++m) X[m] = pk_load(c0 - 8 + 4 * m);
+                            for (int m = 0; m < 5; ++m) X[m] = lds<float>(q0 + (m - 2) * 16);
                             ctr0 = X[2];
                             x_part(a0, X, cf);
                         }
                         {
                             P X[5];
 #pragma unroll
-                            for (int m = 0; m < 5; ++m) X[m] = pk_load(c0 + d1 - 8 + 4 * m);
+                            for (int m = 0; m < 5; ++m) X[m] = lds<float>(q1 + (m - 2) * 16);
                             ctr1 = X[2];
                             x_part(a1, X, cf);
                         }
-                        const P nb1 = G.row1 ? ctr1 : pk_load(c0 + pitch);   // a row of zeros
+                        const P nb1 = G.row1 ? ctr1 : lds<float>(q0 + rb);   // a row of zeros
                         a0.fma(cf.a[1], nb1);
                         a1.fma(cf.a[1], ctr0);
 #pragma unroll
                         for (int d = 1; d <= kRadius; ++d) {
-                            const P lo = pk_load(c0 - d * pitch), hi = pk_load(c0 + (1 + d) * pitch);
+                            const P lo = lds<float>(q0 - d * rb), hi = lds<float>(q0 + (1 + d) * rb);
                             a0.fma(cf.a[d], lo);
                             a1.fma(cf.a[d], hi);
                             if (d < kRadius) {
                                 a1.fma(cf.a[d + 1], lo);
                                 a0.fma(cf.a[d + 1], hi);
                             }
-                            const int sm = cz >= d ? cz - d : cz + kRing - d, sp = cz + d < kRing ? cz + d : cz + d - kRing;
-                            const float *const pm = ring + sm * A.L.plane + G.ring, *const pp = ring + sp * A.L.plane + G.ring;
-                            a0.fma(cf.a[d], pk_load(pm));
-                            a0.fma(cf.a[d], pk_load(pp));
-                            a1.fma(cf.a[d], pk_load(pm + d1));
-                            a1.fma(cf.a[d], pk_load(pp + d1));
+                            const int sm = (cz >= d ? cz - d : cz + kRing - d) * pb;
+                            const int sp = (cz + d < kRing ? cz + d : cz + d - kRing) * pb;
+                            a0.fma(cf.a[d], lds<float>(o0 + sm));
+                            a0.fma(cf.a[d], lds<float>(o0 + sp));
+                            a1.fma(cf.a[d], lds<float>(o1 + sm));
+                            a1.fma(cf.a[d], lds<float>(o1 + sp));
                         }
                         a0.fma(dg, ctr0);
                         a1.fma(dg, ctr1);
@@ -1391,6 +1410,10 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
                         suv += t1.sum();
                         suu += t2.sum();
                     }
+                };
+                for (int f = 0, slot = 0; f < nz + kRadius; f += 2, slot = slot + 2 == kRing ? 0 : slot + 2) {
+                    step(f, slot, fu[0], fv[0]);
+                    if (f + 1 < nz + kRadius) step(f + 1, slot + 1, fu[1], fv[1]);
                 }
                 // (also: every ring reader of the sweep is done)
                 gather3(svv, suv, suu, ng, ncl, G.rank, A.L.err);
