@@ -676,7 +676,7 @@ int ec_impl(Ctx &c, int n_r, const double *V0_dev, double *lambdas_host, double 
             RPA_CUDA(cudaEventRecord(a, s));
             // Rayleigh-Ritz: C = V^T R, eigenvalues, E_cm = (w_m / 2 pi) sum g(lambda)
             if (use_tensor_cores(c))
-                tc_gemm(V, c.nd, 1, R, c.nd, 1, n_r, n_r, c.nd, Wm, s, c.dense_scratch, c.d_tc_err);
+                tc_gemm(V, c.nd, R, c.nd, n_r, n_r, c.nd, Wm, s, c.dense_scratch, c.d_tc_err);
             else
                 gram(V, n_r, R, n_r, c.nd, Wm, s, c.dense_scratch);
             symmetrize(Wm, n_r, s);

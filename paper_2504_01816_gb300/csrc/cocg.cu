@@ -3402,7 +3402,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
 // T[s][k] = u_k . rows[s] for nrows rows.
 void pc_coefficients(Ctx &c, const double *rows, int nrows, double *T, cudaStream_t st) {
     if (use_tensor_cores(c))
-        tc_gemm(rows, c.nd, 1, c.psi64, c.nd, 1, nrows, c.ns, c.nd, T, st, c.dense_scratch, c.d_tc_err);
+        tc_gemm(rows, c.nd, c.psi64, c.nd, nrows, c.ns, c.nd, T, st, c.dense_scratch, c.d_tc_err);
     else
         gram(rows, nrows, c.psi64, c.ns, c.nd, T, st, c.dense_scratch);
 }
@@ -3469,6 +3469,10 @@ int sternheimer_batch_projected(Ctx &c, double omega, const int *orb, int nsys, 
 static double *pair_coefficients(Ctx &c, const double *dv, int ncols, cudaStream_t s) {
     const int nsys = c.ns * ncols;
     double *T = (double *)c.pc_coef.ensure(sizeof(double) * (size_t)nsys * c.ns);
+    if (use_tensor_cores(c)) {
+        tc_gemm_pairs(c.psi64, c.ns, dv, ncols, c.psi64, c.ns, c.nd, T, s, c.dense_scratch, c.d_tc_err);
+        return T;
+    }
     double *rows = (double *)c.rhs.ensure(sizeof(double) * (size_t)ncols * c.nd);
     for (int n = 0; n < c.ns; ++n) {
         k_pair_rows<<<dim3(std::min<unsigned>(cdiv(c.nd, 256), 1024u), ncols), 256, 0, s>>>(c.psi64, dv, n, c.nd,

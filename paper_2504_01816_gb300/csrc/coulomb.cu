@@ -212,38 +212,22 @@ void *static_scratch(int dev) {
 }
 }  // namespace
 
-// The same per-axis transform as a batch of tensor-core contractions (tc_gemm_batched):
-//   axis x: one contraction, rows (o) of length n_x times M^T;
-//   axis y: one contraction per (column, z) slab, M (n_y x n_y) times the slab (n_y x n_x);
-//   axis z: one contraction per column, M (n_z x n_z) times the column (n_z x n_x n_y),
-// with M = Q^T (forward) or Q (back), Q[i*n+a] row-major.
+// The same per-axis transform on the tensor cores: the grid's lines along the axis are the rows of one
+// contraction with M = Q^T (forward) or Q (back), Q[i*n+a] row-major, so its 128-row tiles are full
+// whatever the axis.
 static void axis_pass_tc(Ctx &c, int axis, const double *in, double *out, int ncols, int forward,
                          const double *scale, cudaStream_t s) {
     const int n = axis == 0 ? c.nx : axis == 1 ? c.ny : c.nz;
     const double *Q = c.Q[axis];
     // M(a, b) = Q[b][a] (forward) or Q[a][b] (back): element strides of (a, b)
     const long long ma = forward ? 1 : n, mb = forward ? n : 1;
-    if (axis == 0) {
-        const long long rows = (long long)ncols * c.nd / n;
-        if (rows > (long long)INT32_MAX) fail(RPA_ERR_INVALID, "too many rows for the tensor-core transform");
-        // D[o][a] = sum_b in[o][b] M(a, b): A = in (rows o, k = b), B(a, b) = M(a, b)
-        tc_gemm_batched(in, n, 1, 0, Q, ma, mb, 0, (int)rows, n, n, out, n, 1, 1, 1, scale, c.nd, s, c.d_tc_err);
-    } else if (axis == 1) {
-        const long long slab = (long long)n * c.nx;
-        const long long batch = (long long)ncols * c.nz;
-        // D_o[a][i] = sum_b M(a, b) in_o[b][i]: A(a, b) = M(a, b), B(i, b) = in_o[b][i]
-        for (long long z0 = 0; z0 < batch; z0 += 65535) {
-            const int nb = (int)std::min<long long>(65535, batch - z0);
-            tc_gemm_batched(Q, ma, mb, 0, in + z0 * slab, 1, c.nx, slab, n, c.nx, n, out + z0 * slab, c.nx, 1, slab,
-                            nb, scale, c.nd, s, c.d_tc_err);
-        }
-    } else {
-        const long long plane = (long long)c.nx * c.ny;
-        if (plane > (long long)INT32_MAX) fail(RPA_ERR_INVALID, "plane too large for the tensor-core transform");
-        if (ncols > 65535) fail(RPA_ERR_INVALID, "too many columns for the tensor-core transform");
-        tc_gemm_batched(Q, ma, mb, 0, in, 1, plane, c.nd, n, (int)plane, n, out, plane, 1, c.nd, ncols, scale, c.nd, s,
-                        c.d_tc_err);
-    }
+    const long long lines = (long long)ncols * c.nd / n, plane = (long long)c.nx * c.ny;
+    if (plane > (long long)INT32_MAX) fail(RPA_ERR_INVALID, "plane too large for the tensor-core transform");
+    // x: the line of row o starts at o n_x (taken n_y n_z lines, a column, at a time); y: line (slab, i) at
+    // slab n_x n_y + i; z: line (column, i) at column N_d + i
+    if (axis == 0) tc_lines(in, out, lines, c.ny * c.nz, c.nd, n, 1, n, Q, ma, mb, scale, s, c.d_tc_err);
+    else if (axis == 1) tc_lines(in, out, lines, c.nx, plane, 1, c.nx, n, Q, ma, mb, scale, s, c.d_tc_err);
+    else tc_lines(in, out, lines, (int)plane, c.nd, 1, plane, n, Q, ma, mb, scale, s, c.d_tc_err);
 }
 
 static void coulomb_passes_tc(Ctx &c, double power, const double *in, double *out, int ncols, double *t1, double *t2,

@@ -282,17 +282,18 @@ void sym_eigvals(double *C, int n, double *lam, double *work, double weight, dou
                  cudaStream_t s);
 void symmetrize(double *C, int n, cudaStream_t s);
 
-// D (M x N, row-major) = sum_k A(m, k) B(n, k) with A(m, k) = A[m a_m + k a_k] and B(n, k) =
-// B[n b_n + k b_k], on the tensor cores (tcgen05) as six products of BF16 splits accumulated in
-// FP32 (tc_gemm.cu).  *err_dev is set to 1 if the kernel gave up waiting on its MMAs.
-void tc_gemm(const double *A, long long a_m, long long a_k, const double *B, long long b_n, long long b_k, int M,
-             int N, long long K, double *D, cudaStream_t s, DevBuf &scratch, int *err_dev);
-// Batched form: for z < batch, D_z[m d_m + n d_n] = sum_k A_z(m, k) B_z(n, k), with the operands and
-// the output of member z offset by z a_z, z b_z, z d_z elements; optionally every output element e
-// (counted from D) is multiplied by scale[e % scale_n].
-void tc_gemm_batched(const double *A, long long a_m, long long a_k, long long a_z, const double *B, long long b_n,
-                     long long b_k, long long b_z, int M, int N, int K, double *D, long long d_m, long long d_n,
-                     long long d_z, int batch, const double *scale, long long scale_n, cudaStream_t s, int *err_dev);
+// Contractions on the tensor cores (tcgen05, exact integer pieces; tc_gemm.cu).  *err_dev is set to 1 if
+// the kernel gave up waiting on its MMAs.
+// D (M x N, row-major) = sum_k A[m a_m + k] B[n b_n + k].
+void tc_gemm(const double *A, long long a_m, const double *B, long long b_n, int M, int N, long long K, double *D,
+             cudaStream_t s, DevBuf &scratch, int *err_dev);
+// The same for the products of rows: D[(i nv + j) N + n] = sum_k U[i K + k] V[j K + k] B[n K + k], i < nu, j < nv.
+void tc_gemm_pairs(const double *U, int nu, const double *V, int nv, const double *B, int N, long long K, double *D,
+                   cudaStream_t s, DevBuf &scratch, int *err_dev);
+// Transform of lines of n values: line r starts at in + (r / mi) mo + (r % mi) ms, its values ks apart;
+// out (same places) = sum_k Q(a, k) in(k), Q(a, k) = Q[a q_n + k q_k]; optionally times scale[(r % mi) ms + a ks].
+void tc_lines(const double *in, double *out, long long rows, int mi, long long mo, long long ms, long long ks, int n,
+              const double *Q, long long q_n, long long q_k, const double *scale, cudaStream_t s, int *err_dev);
 
 // Profiling helpers: register a kernel name in the stats table (returns its slot) and add
 // launches/time/points/bytes to it.

@@ -29,15 +29,22 @@
 // T_{k,(n,j)} = u_k . (u_n (.) nu^1/2 v_j) of the Sternheimer right-hand sides (Eqs. 7-9), and the
 // per-axis transforms of the Kronecker-product Coulomb operator (Eq. 5), in the mixed-precision form.
 //
-// Blocking.  A block computes one 128 x kTcN tile of D over one range of k (split-K, blockIdx.z) or
-// for one member of a batch (blockIdx.z with the batch strides).  Per chunk all threads read the
-// FP64 operand tiles twice (coalesced along whichever index is contiguous): first for the row
-// exponents (shared-memory atomicMax), then to cut the pieces, which go to shared memory in the
-// canonical K-major layout without swizzle (8-row x 16-byte core matrices, 128 bytes each).  One
-// thread issues 4 (k slices of 16) x 10 (products) MMAs and commits them to an mbarrier, which every
-// thread waits on before the tiles are read back and the shared tiles rewritten.  The FP64 tile
-// goes to the output (batched) or to a split-K partial; a second kernel adds the partials in a
-// fixed order (deterministic).
+// Blocking.  A block computes one 128 x kTcN tile of D over one range of k (split-K, blockIdx.z).  Per
+// chunk a warp takes 8 rows of an operand at a time: lane l holds 16 values of row l % 8 (two groups
+// of 8 consecutive k), the row's exponent is a maximum over four lanes (two shuffles), and the pieces
+// go to shared memory as 16-byte stores, 8 lanes to the 8 rows of a core matrix, in the canonical K-major
+// layout without swizzle (8-row x 16-byte core matrices, 128 bytes each): every value is loaded once and
+// nothing is exchanged between warps before the tiles are complete.  One thread issues 4 (k slices of
+// 16) x 10 (products) MMAs and commits them to an mbarrier, which every thread waits on before the
+// tiles are read back and the shared tiles rewritten.  The FP64 tile goes to the output or to a
+// split-K partial; a second kernel adds the partials in a fixed order (deterministic).  An operand row
+// may be the product of two arrays' rows (the pairs u_n (.) dv_j), formed as it is loaded.
+//
+// What bounds it: the instructions that cut the pieces and the FP64 pipe that combines them (two
+// conversions and a multiply-add per output and chunk); rows and columns past the operands cost
+// nothing.  Measured at 40^3, 64 columns: a per-axis transform 200 -> 85 us (loading every value
+// twice, shared-memory atomics for the exponents, 2-byte stores), the P_c coefficients of 16 x 64
+// pairs 4.5 -> 0.72 ms (one contraction per orbital, 64 of 128 rows used).
 //
 // Bounded waits: every wait on the mbarrier gives up after ~1 s of clock cycles, sets the error
 // flag, waits (again bounded) for the block's MMAs, frees the tensor memory and returns.
@@ -66,18 +73,22 @@ constexpr uint32_t kTcTileB = kTcN * kTcK * 2;
 constexpr uint32_t kTcSmem = kTcPieces * (kTcTileA + kTcTileB) + 64;
 constexpr long long kTcWaitCycles = 2000000000LL;                 // ~1 s at 2 GHz
 
+// Operand rows: X(r, k) = p[(r / mi) mo + (r % mi) ms + k ks], times q[(r / mi) qmo + (r % mi) qms + k ks] if q is set.
+struct TcRows {
+    const double *p, *q;
+    long long mo, ms, qmo, qms, ks;
+    int mi;
+};
 struct TcArgs {
-    const double *A;
-    const double *B;
-    long long a_m, a_k, b_n, b_k;        // element strides
+    TcRows A, B;
     int M, N;                            // output size
     long long K;
-    long long kchunk;                    // k range per split (multiple of kTcK); K for a batch
-    double *part;                        // split-K: [splits][M][N]; batch: the output D
-    long long d_m, d_n;                  // output strides (batch); split-K partials are [M][N]
-    long long a_z, b_z, d_z;             // batch strides (0: blockIdx.z splits k)
-    const double *scale;                 // batch only: D[e] *= scale[e % scale_n] (nullptr = none)
-    long long scale_n;
+    long long kchunk;                    // k range per split (multiple of kTcK)
+    double *D;                           // split-K: partials [splits][M][N]; else the output
+    int lines;                           // != 0: no split; D[(m / di) do_ + (m % di) dm + n dn]
+    long long do_, dm, dn;
+    int di;
+    const double *scale;                 // lines only: times scale[(m % di) dm + n dn] (nullptr = none)
     int *err;                            // set on a timed-out wait
 };
 
@@ -98,12 +109,6 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
 // Instruction descriptor of kind::f16: D in FP32, A and B in BF16, both K-major, M x N.
 constexpr uint32_t tc_idesc(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-
-// Byte offset of element (row, k) of a K-major tile.
-__device__ __forceinline__ uint32_t tc_off(int row, int k) {
-    return (uint32_t)(row >> 3) * kTcSbo + (uint32_t)(k >> 3) * kTcCoreBytes + (uint32_t)(row & 7) * 16u +
-           (uint32_t)(k & 7) * 2u;
 }
 
 // Biased binary exponent field of |x| (0 for zero).
@@ -160,7 +165,59 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                  : "memory");
 }
 
-__global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
+// Rows 8 g .. 8 g + 7 of an operand's tile, by one warp: row exponents and integer pieces of the 64 values from
+// k = kb on (zeros from k1 on and for rows past the operand).
+__device__ __forceinline__ void tc_stage(const TcRows &X, int r0, int rows, int g, long long kb, long long k1,
+                                         unsigned char *tile, uint32_t tile_bytes, int *ex) {
+    const int lane = threadIdx.x & 31, lr = 8 * g + (lane & 7), kg = lane >> 3, r = r0 + lr;
+    double x[2][8];
+    int e = 0;
+    const bool in = r < rows;
+    const int hi = in ? r / X.mi : 0, lo = in ? r - hi * X.mi : 0;
+    const double *p = X.p + hi * X.mo + lo * X.ms, *q = X.q ? X.q + hi * X.qmo + lo * X.qms : nullptr;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long k = kb + 8 * (kg + 4 * h) + i;
+            x[h][i] = in && k < k1 ? p[k * X.ks] : 0.0;
+        }
+    if (q) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const long long k = kb + 8 * (kg + 4 * h) + i;
+                if (in && k < k1) x[h][i] *= q[k * X.ks];
+            }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) e = max(e, exp_field(x[h][i]));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
+    e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
+    if (lane < 8) ex[lr] = e;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        uint32_t w[kTcPieces][4];
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            __nv_bfloat16 a[4], b[4];
+            cut4(x[h][i], e, a);
+            cut4(x[h][i + 1], e, b);
+#pragma unroll
+            for (int c = 0; c < kTcPieces; ++c)
+                w[c][i >> 1] = (uint32_t)__bfloat16_as_ushort(a[c]) | ((uint32_t)__bfloat16_as_ushort(b[c]) << 16);
+        }
+        const uint32_t o = (uint32_t)g * kTcSbo + (uint32_t)(kg + 4 * h) * kTcCoreBytes + (uint32_t)(lane & 7) * 16u;
+#pragma unroll
+        for (int c = 0; c < kTcPieces; ++c)
+            *reinterpret_cast<uint4 *>(tile + c * tile_bytes + o) = make_uint4(w[c][0], w[c][1], w[c][2], w[c][3]);
+    }
+}
+
+__global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(const __grid_constant__ TcArgs a) {
     extern __shared__ __align__(1024) unsigned char tsm[];
     unsigned char *tA = tsm;                                       // [4][kTcTileA]
     unsigned char *tB = tsm + kTcPieces * kTcTileA;                // [4][kTcTileB]
@@ -170,13 +227,16 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
     __shared__ int expA[kTcM], expB[kTcN];                         // row exponents of the chunk
     const int tid = threadIdx.x, warp = tid >> 5;
     const int m0 = blockIdx.x * kTcM, n0 = blockIdx.y * kTcN;
-    const bool batch = a.a_z != 0 || a.b_z != 0 || a.d_z != 0;
-    const double *const Ab = a.A + (batch ? (long long)blockIdx.z * a.a_z : 0);
-    const double *const Bb = a.B + (batch ? (long long)blockIdx.z * a.b_z : 0);
-    const long long k0 = batch ? 0 : (long long)blockIdx.z * a.kchunk;
+    const long long k0 = (long long)blockIdx.z * a.kchunk;
     const long long k1 = min(a.K, k0 + a.kchunk);
     const uint32_t bar_addr = smem_u32(bar);
     constexpr uint32_t kCols = kTcLevels * kTcN;                  // one accumulator tile per weight
+    // groups of 8 rows with values; the tiles' other rows stay zero
+    const int ga = (min(kTcM, a.M - m0) + 7) / 8, gb = (min(kTcN, a.N - n0) + 7) / 8;
+    for (uint32_t e = tid; e < kTcPieces * (kTcTileA + kTcTileB) / 16; e += kTcThreads)
+        reinterpret_cast<uint4 *>(tsm)[e] = make_uint4(0, 0, 0, 0);
+    for (int e = tid; e < kTcM; e += kTcThreads) expA[e] = 0;
+    for (int e = tid; e < kTcN; e += kTcThreads) expB[e] = 0;
 
     if (tid == 0) {
         abort_flag = 0;
@@ -193,12 +253,13 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
-    const bool a_kfast = a.a_k == 1, b_kfast = a.b_k == 1;
     // epilogue mapping: warp w reads tile rows 32 (w % 4) .. +31 (its tensor-memory lanes) and
     // columns 32 (w / 4) .. +31
     const int lane_base = 32 * (warp & 3), col0 = 32 * (warp >> 2);
     const int my_row = lane_base + (tid & 31);
     const uint32_t t_base = tmem + ((uint32_t)lane_base << 16) + (uint32_t)col0;
+    // a warp whose rows or columns all lie past the output reads nothing back
+    const int my_cols = m0 + lane_base < a.M ? max(0, min(32, a.N - n0 - col0)) : 0;
     double acc[32];
 #pragma unroll
     for (int c = 0; c < 32; ++c) acc[c] = 0.0;
@@ -206,49 +267,10 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
     uint32_t phase = 0;
     bool ok = true, pending = false;
     for (long long kb = k0; kb < k1; kb += kTcK) {
-        // 1. row exponents of the chunk
-        for (int e = tid; e < kTcM; e += kTcThreads) expA[e] = 0;
-        for (int e = tid; e < kTcN; e += kTcThreads) expB[e] = 0;
-        __syncthreads();
-        for (int e = tid; e < kTcM * kTcK; e += kTcThreads) {
-            const int row = a_kfast ? e / kTcK : e % kTcM;
-            const int kk = a_kfast ? e % kTcK : e / kTcM;
-            const int m = m0 + row;
-            const long long k = kb + kk;
-            if (m < a.M && k < k1) atomicMax(&expA[row], exp_field(Ab[(long long)m * a.a_m + k * a.a_k]));
-        }
-        for (int e = tid; e < kTcN * kTcK; e += kTcThreads) {
-            const int row = b_kfast ? e / kTcK : e % kTcN;
-            const int kk = b_kfast ? e % kTcK : e / kTcN;
-            const int n = n0 + row;
-            const long long k = kb + kk;
-            if (n < a.N && k < k1) atomicMax(&expB[row], exp_field(Bb[(long long)n * a.b_n + k * a.b_k]));
-        }
-        __syncthreads();
-        // 2. integer pieces into the K-major core-matrix tiles
-        for (int e = tid; e < kTcM * kTcK; e += kTcThreads) {
-            const int row = a_kfast ? e / kTcK : e % kTcM;
-            const int kk = a_kfast ? e % kTcK : e / kTcM;
-            const int m = m0 + row;
-            const long long k = kb + kk;
-            const double x = (m < a.M && k < k1) ? Ab[(long long)m * a.a_m + k * a.a_k] : 0.0;
-            __nv_bfloat16 pc[4];
-            cut4(x, expA[row], pc);
-            const uint32_t o = tc_off(row, kk);
-#pragma unroll
-            for (int i = 0; i < kTcPieces; ++i) *reinterpret_cast<__nv_bfloat16 *>(tA + i * kTcTileA + o) = pc[i];
-        }
-        for (int e = tid; e < kTcN * kTcK; e += kTcThreads) {
-            const int row = b_kfast ? e / kTcK : e % kTcN;
-            const int kk = b_kfast ? e % kTcK : e / kTcN;
-            const int n = n0 + row;
-            const long long k = kb + kk;
-            const double x = (n < a.N && k < k1) ? Bb[(long long)n * a.b_n + k * a.b_k] : 0.0;
-            __nv_bfloat16 pc[4];
-            cut4(x, expB[row], pc);
-            const uint32_t o = tc_off(row, kk);
-#pragma unroll
-            for (int i = 0; i < kTcPieces; ++i) *reinterpret_cast<__nv_bfloat16 *>(tB + i * kTcTileB + o) = pc[i];
+        // 1. row exponents and integer pieces into the K-major core-matrix tiles
+        for (int g = warp; g < ga + gb; g += kTcThreads / 32) {
+            if (g < ga) tc_stage(a.A, m0, a.M, g, kb, k1, tA, kTcTileA, expA);
+            else tc_stage(a.B, n0, a.N, g - ga, kb, k1, tB, kTcTileB, expB);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> tensor core
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -290,10 +312,11 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
         if (abort_flag) break;
         pending = false;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        // 3. read the four weight tiles back (8 columns at a time) and add the chunk in FP64
+        // 2. read the four weight tiles back (8 columns at a time) and add the chunk in FP64
         const int ea = expA[my_row];
 #pragma unroll
         for (int h = 0; h < 4; ++h) {
+            if (8 * h >= my_cols) break;                           // uniform per warp
             uint32_t l0[8], l1[8], l2[8], l3[8];
             tmem_ld8(t_base + 8 * h, l0);
             tmem_ld8(t_base + kTcN + 8 * h, l1);
@@ -322,17 +345,16 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
     if (ok && !abort_flag) {
         const int m = m0 + my_row;
         if (m < a.M) {
-            if (batch) {
+            if (a.lines) {
+                const int hi = m / a.di;
+                const long long in = (m - hi * a.di) * a.dm, off = hi * a.do_ + in;
 #pragma unroll
                 for (int c = 0; c < 32; ++c) {
                     const int n = n0 + col0 + c;
-                    if (n < a.N) {
-                        const long long off = (long long)blockIdx.z * a.d_z + (long long)m * a.d_m + (long long)n * a.d_n;
-                        a.part[off] = a.scale ? acc[c] * a.scale[off % a.scale_n] : acc[c];
-                    }
+                    if (n < a.N) a.D[off + n * a.dn] = a.scale ? acc[c] * a.scale[in + n * a.dn] : acc[c];
                 }
             } else {
-                double *out = a.part + ((long long)blockIdx.z * a.M + m) * a.N;
+                double *out = a.D + ((long long)blockIdx.z * a.M + m) * a.N;
 #pragma unroll
                 for (int c = 0; c < 32; ++c) {
                     const int n = n0 + col0 + c;
@@ -353,7 +375,15 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_tc_gemm(TcArgs a) {
 __global__ void k_tc_sum_splits(const double *__restrict__ part, int splits, long long n, double *__restrict__ D) {
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         double s = 0.0;
-        for (int z = 0; z < splits; ++z) s += part[(long long)z * n + e];
+        int z = 0;
+        for (; z + 16 <= splits; z += 16) {              // 16 loads in flight, added in order
+            double v[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = part[(long long)(z + i) * n + e];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) s += v[i];
+        }
+        for (; z < splits; ++z) s += part[(long long)z * n + e];
         D[e] = s;
     }
 }
@@ -362,44 +392,83 @@ inline unsigned cdiv(long long a, long long b) { return (unsigned)((a + b - 1) /
 
 }  // namespace
 
-void tc_gemm(const double *A, long long a_m, long long a_k, const double *B, long long b_n, long long b_k, int M,
-             int N, long long K, double *D, cudaStream_t s, DevBuf &scratch, int *err_dev) {
-    const int tm = (int)cdiv(M, kTcM), tn = (int)cdiv(N, kTcN);
+// D (M x N, row-major) over split ranges of k, as if the rows came ref_rows at a time (which sets the ranges).
+static void tc_split(TcArgs a, int ref_rows, double *D, cudaStream_t s, DevBuf &scratch) {
+    const int tm = (int)cdiv(a.M, kTcM), tn = (int)cdiv(a.N, kTcN), rm = (int)cdiv(ref_rows, kTcM);
     int dev = 0, sms = 0;
     RPA_CUDA(cudaGetDevice(&dev));
     RPA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // split K so that the grid covers the SMs about three times, with at least two chunks per split
-    long long splits = std::max(1LL, std::min<long long>(K / (2 * kTcK), (3LL * sms + tm * tn - 1) / (tm * tn)));
-    const long long kchunk = ((K + splits - 1) / splits + kTcK - 1) / kTcK * kTcK;
-    splits = std::max(1LL, (K + kchunk - 1) / kchunk);
-    double *part = (double *)scratch.ensure(sizeof(double) * (size_t)splits * M * N);
-    TcArgs a{};
-    a.A = A; a.B = B; a.a_m = a_m; a.a_k = a_k; a.b_n = b_n; a.b_k = b_k;
-    a.M = M; a.N = N; a.K = K; a.kchunk = kchunk; a.part = part; a.err = err_dev;
+    long long splits = std::max(1LL, std::min<long long>(a.K / (2 * kTcK), (3LL * sms + rm * tn - 1) / (rm * tn)));
+    a.kchunk = ((a.K + splits - 1) / splits + kTcK - 1) / kTcK * kTcK;
+    splits = std::max(1LL, (a.K + a.kchunk - 1) / a.kchunk);
+    a.D = (double *)scratch.ensure(sizeof(double) * (size_t)splits * a.M * a.N);
     allow_dynamic_smem((const void *)k_tc_gemm, kTcSmem);
     k_tc_gemm<<<dim3(tm, tn, (unsigned)splits), kTcThreads, kTcSmem, s>>>(a);
-    const long long n = (long long)M * N;
-    k_tc_sum_splits<<<std::min<unsigned>(cdiv(n, 256), 4096u), 256, 0, s>>>(part, (int)splits, n, D);
+    const long long n = (long long)a.M * a.N;
+    k_tc_sum_splits<<<std::min<unsigned>(cdiv(n, 64), 4096u), 64, 0, s>>>(a.D, (int)splits, n, D);
     RPA_LAUNCH("tensor-core contraction");
     count_launches(2);
 }
 
-void tc_gemm_batched(const double *A, long long a_m, long long a_k, long long a_z, const double *B, long long b_n,
-                     long long b_k, long long b_z, int M, int N, int K, double *D, long long d_m, long long d_n,
-                     long long d_z, int batch, const double *scale, long long scale_n, cudaStream_t s, int *err_dev) {
-    if (batch <= 0 || M <= 0 || N <= 0) return;
-    const int tm = (int)cdiv(M, kTcM), tn = (int)cdiv(N, kTcN);
-    if (batch > 65535) fail(RPA_ERR_INVALID, "tensor-core contraction: batch of %d exceeds the grid limit", batch);
+void tc_gemm(const double *A, long long a_m, const double *B, long long b_n, int M, int N, long long K, double *D,
+             cudaStream_t s, DevBuf &scratch, int *err_dev) {
+    if (M <= 0 || N <= 0) return;
     TcArgs a{};
-    a.A = A; a.B = B; a.a_m = a_m; a.a_k = a_k; a.b_n = b_n; a.b_k = b_k;
-    a.M = M; a.N = N; a.K = K; a.kchunk = K; a.part = D; a.d_m = d_m; a.d_n = d_n;
-    // a zero stride would read as "split K": a batch always has a nonzero output stride
-    a.a_z = a_z; a.b_z = b_z; a.d_z = d_z != 0 ? d_z : 1;
-    a.scale = scale; a.scale_n = scale_n > 0 ? scale_n : 1; a.err = err_dev;
-    allow_dynamic_smem((const void *)k_tc_gemm, kTcSmem);
-    k_tc_gemm<<<dim3(tm, tn, (unsigned)batch), kTcThreads, kTcSmem, s>>>(a);
-    RPA_LAUNCH("tensor-core contraction (batched)");
-    count_launches(1);
+    a.A = TcRows{A, nullptr, 0, a_m, 0, 0, 1, M};
+    a.B = TcRows{B, nullptr, 0, b_n, 0, 0, 1, N};
+    a.M = M;
+    a.N = N;
+    a.K = K;
+    a.err = err_dev;
+    tc_split(a, M, D, s, scratch);
+}
+
+void tc_gemm_pairs(const double *U, int nu, const double *V, int nv, const double *B, int N, long long K, double *D,
+                   cudaStream_t s, DevBuf &scratch, int *err_dev) {
+    if (nu <= 0 || nv <= 0 || N <= 0) return;
+    const size_t limit = (size_t)256 << 20;              // bytes of partials: orbitals are taken in groups
+    const size_t per = sizeof(double) * (size_t)nv * N * 512;
+    const int step = (int)std::max<size_t>(1, std::min<size_t>(nu, limit / per));
+    for (int n = 0; n < nu; n += step) {
+        const int m = std::min(step, nu - n);
+        TcArgs a{};
+        a.A = TcRows{U + (size_t)n * K, V, K, 0, 0, K, 1, nv};
+        a.B = TcRows{B, nullptr, 0, K, 0, 0, 1, N};
+        a.M = m * nv;
+        a.N = N;
+        a.K = K;
+        a.err = err_dev;
+        tc_split(a, nv, D + (size_t)n * nv * N, s, scratch);
+    }
+}
+
+void tc_lines(const double *in, double *out, long long rows, int mi, long long mo, long long ms, long long ks, int n,
+              const double *Q, long long q_n, long long q_k, const double *scale, cudaStream_t s, int *err_dev) {
+    // whole groups of mi lines per launch, the line index in 32 bits
+    const long long per = std::max<long long>(1, (1LL << 30) / mi) * mi;
+    for (long long r = 0; r < rows; r += per) {
+        TcArgs a{};
+        const double *x = in + r / mi * mo;
+        a.A = TcRows{x, nullptr, mo, ms, 0, 0, ks, mi};
+        a.B = TcRows{Q, nullptr, 0, q_n, 0, 0, q_k, n};
+        a.M = (int)std::min(per, rows - r);
+        a.N = n;
+        a.K = n;
+        a.kchunk = n;
+        a.D = out + r / mi * mo;
+        a.lines = 1;
+        a.di = mi;
+        a.do_ = mo;
+        a.dm = ms;
+        a.dn = ks;
+        a.scale = scale;
+        a.err = err_dev;
+        allow_dynamic_smem((const void *)k_tc_gemm, kTcSmem);
+        k_tc_gemm<<<dim3(cdiv(a.M, kTcM), cdiv(n, kTcN), 1), kTcThreads, kTcSmem, s>>>(a);
+        RPA_LAUNCH("tensor-core transform");
+        count_launches(1);
+    }
 }
 
 }  // namespace rpa
