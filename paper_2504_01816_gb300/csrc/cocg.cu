@@ -89,6 +89,7 @@ struct Params {
     // mixed form with projected right-hand sides: P_c on every FP32 correction and residual
     int cproject;
     int proj_re_only;           // only Re(u_k . x) is needed (the solutions retire into drho)
+    int norm_only;              // only the norms among the residuals' partial sums are read (no split kernels)
     float *Tp32;                // [S][ns][2]       Tp in FP32 (for FP32 updates)
     const float *psi32;         // ns x nd orbitals in FP32
     // Laplacian-preconditioned COCG: rho = r^T z from the per-plane partial sums of z = M r
@@ -1962,56 +1963,101 @@ __device__ __forceinline__ double next_scale(const Slot &sl) {
 // P.cproject) goes into x64 += d' / scale and, for the residual update, into dq (the idle q
 // buffer); d is cleared for the next inner solve.  A correction that went non-finite is dropped:
 // only d is cleared.
+// One work item is one chunk of grid points of G consecutive slots: an orbital value loaded (from L2)
+// serves all of them, and the loop over the orbitals is the outer one, with the chunk's points of a
+// thread in registers (72^3, 256 slots, 64 orbitals: 6.7 -> 3.1 ms a pass with G = 4 against a slot at a
+// time; with 16 orbitals the state's own bytes bound it and G = 4 lacks warps: G = 2).  G = 1 where few
+// slots are in flight.
+template <int G>
 __global__ void __launch_bounds__(kThreads) k_refine_x(Params P, double2 *__restrict__ x64, float2 *__restrict__ d,
                                                        float2 *__restrict__ dq) {
-    const long long items = (long long)P.S * P.nblk;
+    const int ngroups = (P.S + G - 1) / G;
+    const long long items = (long long)ngroups * P.nblk;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
-        const int s = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
-        const Slot &sl = P.slots[s];
-        if (sl.phase != kInnerDone) continue;
-        const bool keep = !sl.discard;
-        const double inv = 1.0 / sl.scale;
-        const long long off = (long long)s * P.g.nd;
-        const float *tp = P.Tp32 + (long long)s * P.ns * 2;
-        for (int t = 0; t < kPPT; ++t) {
-            const long long idx = (long long)chunk * kChunk + t * kThreads + threadIdx.x;
-            if (idx < P.g.nd) {
-                if (keep) {
-                    double2 xv = x64[off + idx];
-                    float2 dv = d[off + idx];
-                    if (P.cproject)
-                        for (int k = 0; k < P.ns; ++k) {
-                            const float u = P.psi32[(long long)k * P.g.nd + idx];
-                            dv.x -= tp[2 * k] * u;
-                            dv.y -= tp[2 * k + 1] * u;
-                        }
-                    xv.x += (double)dv.x * inv;
-                    xv.y += (double)dv.y * inv;
-                    x64[off + idx] = xv;
-                    dq[off + idx] = dv;
-                }
-                d[off + idx] = make_float2(0.f, 0.f);
-            }
+        const int g = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
+        bool keep[G], done[G], any = false;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            const int s = g * G + q;
+            done[q] = s < P.S && P.slots[s].phase == kInnerDone;
+            keep[q] = done[q] && !P.slots[s].discard;
+            any = any || done[q];
         }
+        if (!any) continue;                              // uniform per block
+        const long long i0 = (long long)chunk * kChunk + threadIdx.x;
+        float2 dv[G][kPPT];
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+#pragma unroll
+            for (int t = 0; t < kPPT; ++t) {
+                const long long idx = i0 + t * kThreads;
+                dv[q][t] = keep[q] && idx < P.g.nd ? d[(long long)(g * G + q) * P.g.nd + idx] : make_float2(0.f, 0.f);
+            }
+        if (P.cproject)
+            for (int k = 0; k < P.ns; ++k) {
+                float u[kPPT];
+#pragma unroll
+                for (int t = 0; t < kPPT; ++t) {
+                    const long long idx = i0 + t * kThreads;
+                    u[t] = idx < P.g.nd ? P.psi32[(long long)k * P.g.nd + idx] : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < G; ++q)
+                    if (keep[q]) {
+                        const float2 tp = *reinterpret_cast<const float2 *>(P.Tp32 + ((long long)(g * G + q) * P.ns + k) * 2);
+#pragma unroll
+                        for (int t = 0; t < kPPT; ++t) {
+                            dv[q][t].x -= tp.x * u[t];
+                            dv[q][t].y -= tp.y * u[t];
+                        }
+                    }
+            }
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+            if (done[q]) {
+                const long long off = (long long)(g * G + q) * P.g.nd;
+                const double inv = 1.0 / P.slots[g * G + q].scale;
+#pragma unroll
+                for (int t = 0; t < kPPT; ++t) {
+                    const long long idx = i0 + t * kThreads;
+                    if (idx < P.g.nd) {
+                        if (keep[q]) {
+                            double2 xv = x64[off + idx];
+                            xv.x += (double)dv[q][t].x * inv;
+                            xv.y += (double)dv[q][t].y * inv;
+                            x64[off + idx] = xv;
+                            dq[off + idx] = dv[q][t];
+                        }
+                        d[off + idx] = make_float2(0.f, 0.f);
+                    }
+                }
+            }
     }
 }
 
 // Error-free transformations on FP32 (Knuth's TwoSum; the product error from one fma), the
 // building blocks of double-float ("float-float") arithmetic: a value is an unevaluated sum
 // hi + lo of two FP32 numbers, ~48 significant bits (Ogita, Rump and Oishi, "Accurate sum and dot
-// product", 2005, use the same transformations).
+// product", 2005, use the same transformations).  The real and imaginary parts go through the same
+// operations, two to a packed FP32x2 instruction (a - b as one fma with -1).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(make_float2(-1.f, -1.f), b, a); }
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
     const float bb = __fsub_rn(s, a);
     e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
-// (S, E) += (hi, lo) * x for an FP32 x: the product's rounding error is exact through fma.
-__device__ __forceinline__ void df_mad(float hi, float lo, float x, float &S, float &E) {
-    const float p = __fmul_rn(hi, x);
-    const float pe = __fmaf_rn(hi, x, -p);
-    float t;
-    two_sum(S, p, S, t);
-    E += t + pe + lo * x;
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2 &s, float2 &e) {
+    s = __fadd2_rn(a, b);
+    const float2 bb = sub2(s, a);
+    e = __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+// (S, E) += (hi, lo) * x, element-wise: the product's rounding error is exact through fma (nhi = -hi).
+__device__ __forceinline__ void df_mad2(float2 hi, float2 nhi, float2 lo, float2 x, float2 &S, float2 &E) {
+    const float2 p = __fmul2_rn(hi, x);
+    const float2 npe = __ffma2_rn(nhi, x, p);            // -(hi x - p)
+    float2 t;
+    two_sum2(S, p, S, t);
+    E = __fadd2_rn(E, __ffma2_rn(lo, x, sub2(t, npe)));
 }
 
 // (H + sigma) v at one point in double-float arithmetic for an FP32 complex v: the six
@@ -2019,48 +2065,41 @@ __device__ __forceinline__ void df_mad(float hi, float lo, float x, float &S, fl
 // (hi + lo) and accumulated with their rounding errors.  Zero outside the box.
 __device__ __forceinline__ void df_stencil(const float2 *__restrict__ v, long long idx, int i, int j, int k,
                                            const Grid3 &g, const Coef<float> &ch, const Coef<float> &cl, float dh,
-                                           float dl, float oh, float ol, float (&re)[2], float (&im)[2]) {
+                                           float dl, float oh, float ol, float2 &S, float2 &E) {
+    const float2 zero = make_float2(0.f, 0.f);
     const float2 c = v[idx];
-    float Sr = 0.f, Er = 0.f, Si = 0.f, Ei = 0.f;
-    df_mad(dh, dl, c.x, Sr, Er);          // (3 a0 + V + sigma_re) c
-    df_mad(dh, dl, c.y, Si, Ei);
-    df_mad(-oh, -ol, c.y, Sr, Er);        // i sigma_im c
-    df_mad(oh, ol, c.x, Si, Ei);
-    const long long sy = g.nx, sz = (long long)g.nx * g.ny;
+    S = E = zero;
+    df_mad2(make_float2(dh, dh), make_float2(-dh, -dh), make_float2(dl, dl), c, S, E);   // (3 a0 + V + sigma_re) c
+    df_mad2(make_float2(-oh, oh), make_float2(oh, -oh), make_float2(-ol, ol), make_float2(c.y, c.x), S, E);   // i sigma_im c
+    const float2 *const p = v + idx;
+    const int sy = g.nx, sz = g.nx * g.ny;
 #pragma unroll
     for (int s = 1; s <= kRadius; ++s) {
-        float ar = 0.f, er = 0.f, ai = 0.f, ei = 0.f, t;
-        auto add = [&](float2 u) {
-            two_sum(ar, u.x, ar, t);
-            er += t;
-            two_sum(ai, u.y, ai, t);
-            ei += t;
+        float2 a = zero, e = zero, t;
+        auto add = [&](bool in, int off) {
+            two_sum2(a, in ? p[off] : zero, a, t);
+            e = __fadd2_rn(e, t);
         };
         if (g.periodic) {
-            add(v[idx + (wrap_index(i - s, g.nx) - i)]);
-            add(v[idx + (wrap_index(i + s, g.nx) - i)]);
-            add(v[idx + (wrap_index(j - s, g.ny) - j) * sy]);
-            add(v[idx + (wrap_index(j + s, g.ny) - j) * sy]);
-            add(v[idx + (wrap_index(k - s, g.nz) - k) * sz]);
-            add(v[idx + (wrap_index(k + s, g.nz) - k) * sz]);
+            add(true, wrap_index(i - s, g.nx) - i);
+            add(true, wrap_index(i + s, g.nx) - i);
+            add(true, (wrap_index(j - s, g.ny) - j) * sy);
+            add(true, (wrap_index(j + s, g.ny) - j) * sy);
+            add(true, (wrap_index(k - s, g.nz) - k) * sz);
+            add(true, (wrap_index(k + s, g.nz) - k) * sz);
         } else {
-            if (i - s >= 0) add(v[idx - s]);
-            if (i + s < g.nx) add(v[idx + s]);
-            if (j - s >= 0) add(v[idx - s * sy]);
-            if (j + s < g.ny) add(v[idx + s * sy]);
-            if (k - s >= 0) add(v[idx - s * sz]);
-            if (k + s < g.nz) add(v[idx + s * sz]);
+            add(i - s >= 0, -s);
+            add(i + s < g.nx, s);
+            add(j - s >= 0, -s * sy);
+            add(j + s < g.ny, s * sy);
+            add(k - s >= 0, -s * sz);
+            add(k + s < g.nz, s * sz);
         }
-        // a_s (ar + er): the sum's low part times the coefficient's high part joins the error term
-        df_mad(ch.a[s], cl.a[s], ar, Sr, Er);
-        Er += ch.a[s] * er;
-        df_mad(ch.a[s], cl.a[s], ai, Si, Ei);
-        Ei += ch.a[s] * ei;
+        // a_s (a + e): the sum's low part times the coefficient's high part joins the error term
+        const float2 h = make_float2(ch.a[s], ch.a[s]);
+        df_mad2(h, make_float2(-ch.a[s], -ch.a[s]), make_float2(cl.a[s], cl.a[s]), a, S, E);
+        E = __ffma2_rn(h, e, E);
     }
-    re[0] = Sr;
-    re[1] = Er;
-    im[0] = Si;
-    im[1] = Ei;
 }
 
 // Mixed form: the FP64 residual of the slots whose inner solve ended, updated with their
@@ -2100,15 +2139,15 @@ __global__ void __launch_bounds__(kThreads) k_residual_df(Params P, double2 *__r
                     float dh, dl, e;                      // 3 a0 + V + sigma_re as a pair
                     two_sum(d0h, vhi[idx], dh, e);
                     dl = e + d0l + vlo[idx];
-                    float re[2], im[2];
-                    df_stencil(dq + off, idx, i, j, k, P.g, ch, cl, dh, dl, oh, ol, re, im);
-                    rv.x = fma(-((double)re[0] + (double)re[1]), inv, rv.x);
-                    rv.y = fma(-((double)im[0] + (double)im[1]), inv, rv.y);
+                    float2 hi, lo;
+                    df_stencil(dq + off, idx, i, j, k, P.g, ch, cl, dh, dl, oh, ol, hi, lo);
+                    rv.x = fma(-((double)hi.x + (double)lo.x), inv, rv.x);
+                    rv.y = fma(-((double)hi.y + (double)lo.y), inv, rv.y);
                     r64[off + idx] = rv;
                 }
                 const float2 rf = make_float2((float)(rv.x * sc), (float)(rv.y * sc));
                 r32[off + idx] = rf;
-                p32[off + idx] = make_float2(0.f, 0.f);         // direction buffer of iteration 0
+                if (p32) p32[off + idx] = make_float2(0.f, 0.f);   // direction buffer of iteration 0 (split kernels)
                 v0 += rf.x * rf.x - rf.y * rf.y;
                 v1 += 2.f * rf.x * rf.y;
                 v2 += rf.x * rf.x + rf.y * rf.y;
@@ -2239,36 +2278,81 @@ __global__ void __launch_bounds__(kThreads) k_cproj_dots(Params P, const float2 
 
 // P.cproject: r32 -= sum_k Tp[s][k] u_k for the slots whose inner solve ended; partials (into
 // partB): r32^T r32 and ||r32||^2 of the projected residual.
+// (the first two are read by the split kernels only: P.norm_only leaves them out).  Work items as k_refine_x.
+template <int G>
 __global__ void __launch_bounds__(kThreads) k_cproj_residual(Params P, float2 *__restrict__ r32) {
-    const long long items = (long long)P.S * P.nblk;
+    const int ngroups = (P.S + G - 1) / G;
+    const long long items = (long long)ngroups * P.nblk;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
-        const int s = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
-        if (P.slots[s].phase != kInnerDone) continue;
-        const long long off = (long long)s * P.g.nd;
-        const float *tp = P.Tp32 + (long long)s * P.ns * 2;
-        double v[3] = {0.0, 0.0, 0.0};
-        for (int t = 0; t < kPPT; ++t) {
-            const long long idx = (long long)chunk * kChunk + t * kThreads + threadIdx.x;
-            if (idx < P.g.nd) {
-                float2 rv = r32[off + idx];
-                for (int k = 0; k < P.ns; ++k) {
-                    const float u = P.psi32[(long long)k * P.g.nd + idx];
-                    rv.x -= tp[2 * k] * u;
-                    rv.y -= tp[2 * k + 1] * u;
+        const int g = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
+        bool act[G], any = false;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            const int s = g * G + q;
+            act[q] = s < P.S && P.slots[s].phase == kInnerDone;
+            any = any || act[q];
+        }
+        if (!any) continue;                              // uniform per block
+        const long long i0 = (long long)chunk * kChunk + threadIdx.x;
+        float2 rv[G][kPPT];
+#pragma unroll
+        for (int q = 0; q < G; ++q)
+#pragma unroll
+            for (int t = 0; t < kPPT; ++t) {
+                const long long idx = i0 + t * kThreads;
+                rv[q][t] = act[q] && idx < P.g.nd ? r32[(long long)(g * G + q) * P.g.nd + idx] : make_float2(0.f, 0.f);
+            }
+        for (int k = 0; k < P.ns; ++k) {
+            float u[kPPT];
+#pragma unroll
+            for (int t = 0; t < kPPT; ++t) {
+                const long long idx = i0 + t * kThreads;
+                u[t] = idx < P.g.nd ? P.psi32[(long long)k * P.g.nd + idx] : 0.f;
+            }
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+                if (act[q]) {
+                    const float2 tp = *reinterpret_cast<const float2 *>(P.Tp32 + ((long long)(g * G + q) * P.ns + k) * 2);
+#pragma unroll
+                    for (int t = 0; t < kPPT; ++t) {
+                        rv[q][t].x -= tp.x * u[t];
+                        rv[q][t].y -= tp.y * u[t];
+                    }
                 }
-                r32[off + idx] = rv;
-                v[0] += (double)rv.x * rv.x - (double)rv.y * rv.y;
-                v[1] += 2.0 * (double)rv.x * rv.y;
-                v[2] += (double)rv.x * rv.x + (double)rv.y * rv.y;
+        }
+        double v2[G];
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            v2[q] = 0.0;
+            double v[2] = {0.0, 0.0};
+            const long long off = (long long)(g * G + q) * P.g.nd;
+#pragma unroll
+            for (int t = 0; t < kPPT; ++t) {
+                const long long idx = i0 + t * kThreads;
+                if (act[q] && idx < P.g.nd) {
+                    const float2 r = rv[q][t];
+                    r32[off + idx] = r;
+                    if (!P.norm_only) {
+                        v[0] += (double)r.x * r.x - (double)r.y * r.y;
+                        v[1] += 2.0 * (double)r.x * r.y;
+                    }
+                    v2[q] += (double)r.x * r.x + (double)r.y * r.y;
+                }
+            }
+            if (!P.norm_only) {
+                block_sum<2>(v);
+                if (threadIdx.x == 0 && act[q]) {
+                    double *o = P.partB + ((long long)(g * G + q) * P.nblk + chunk) * 3;
+                    o[0] = v[0];
+                    o[1] = v[1];
+                }
             }
         }
-        block_sum<3>(v);
-        if (threadIdx.x == 0) {
-            double *o = P.partB + ((long long)s * P.nblk + chunk) * 3;
-            o[0] = v[0];
-            o[1] = v[1];
-            o[2] = v[2];
-        }
+        block_sum<G>(v2);
+        if (threadIdx.x == 0)
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+                if (act[q]) P.partB[((long long)(g * G + q) * P.nblk + chunk) * 3 + 2] = v2[q];
     }
 }
 
@@ -2319,46 +2403,79 @@ __global__ void k_state(Params P) {
     }
 }
 
-// Partial sums of u_k . x64 (complex) over each item of the finished slots, for k < ns.
-constexpr int kProjGroup = 8;   // orbitals reduced together (one block reduction per group)
+// Partial sums of u_k . x64 over each item of the finished slots, for k < ns: 32 sums at a time (NC = 1: the
+// real parts of 32 orbitals; NC = 2: both parts of 16), added over a warp's lanes by a transposing
+// butterfly (31 additions for all 32; the pairs of lanes are those of a shuffle-down tree, so the sums are
+// the same to the bit) and over the warps in the order of such a tree.  Bound by the FP64 pipe (one
+// multiply-add per point, orbital and part).  40^3, 1024 slots, 16 orbitals, real parts: 1.09 -> 0.55 ms
+// a pass against block reductions of 16 sums for 8 orbitals at a time.
+__device__ __forceinline__ double warp_transpose_sum(double (&a)[32]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 16; h >= 1; h >>= 1) {
+        const bool up = (lane & h) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double keep = up ? a[i + h] : a[i], send = up ? a[i] : a[i + h];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+        }
+    }
+    return a[0];
+}
+template <int NC>
 __global__ void __launch_bounds__(kThreads) k_proj_dots(Params P, const double2 *__restrict__ x64) {
+    constexpr int K = 32 / NC;                           // orbitals at a time
+    __shared__ double red[kWarpsPerBlock][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long items = (long long)P.S * P.nblk;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
         const int s = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
         if (P.slots[s].phase != kFinished) continue;
-        const long long off = (long long)s * P.g.nd;
-        double2 xv[kPPT];
+        const long long off = (long long)s * P.g.nd, i0 = (long long)chunk * kChunk + threadIdx.x;
+        double xv[kPPT][NC];
 #pragma unroll
         for (int t = 0; t < kPPT; ++t) {
-            const long long idx = (long long)chunk * kChunk + t * kThreads + threadIdx.x;
-            xv[t] = idx < P.g.nd ? x64[off + idx] : make_double2(0.0, 0.0);
+            const long long idx = i0 + t * kThreads;
+            const double2 v = idx < P.g.nd ? x64[off + idx] : make_double2(0.0, 0.0);
+            xv[t][0] = v.x;
+            if (NC == 2) xv[t][NC - 1] = v.y;
         }
-        for (int k0 = 0; k0 < P.ns; k0 += kProjGroup) {
-            double v[2 * kProjGroup];
+        for (int k0 = 0; k0 < P.ns; k0 += K) {
+            double a[32];
 #pragma unroll
-            for (int g = 0; g < kProjGroup; ++g) {
-                double a0 = 0.0, a1 = 0.0;
-                if (k0 + g < P.ns) {
+            for (int k = 0; k < K; ++k) {
+#pragma unroll
+                for (int c = 0; c < NC; ++c) a[k * NC + c] = 0.0;
+                if (k0 + k < P.ns) {
+                    const double *u = P.psi + (long long)(k0 + k) * P.g.nd;
 #pragma unroll
                     for (int t = 0; t < kPPT; ++t) {
-                        const long long idx = (long long)chunk * kChunk + t * kThreads + threadIdx.x;
+                        const long long idx = i0 + t * kThreads;
                         if (idx < P.g.nd) {
-                            const double u = P.psi[(long long)(k0 + g) * P.g.nd + idx];
-                            a0 += u * xv[t].x;
-                            if (!P.proj_re_only) a1 += u * xv[t].y;
+                            const double w = u[idx];
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) a[k * NC + c] += w * xv[t][c];
                         }
                     }
                 }
-                v[2 * g] = a0;
-                v[2 * g + 1] = a1;
             }
-            block_sum<2 * kProjGroup>(v);
-            if (threadIdx.x == 0)
-                for (int g = 0; g < kProjGroup && k0 + g < P.ns; ++g) {
-                    double *o = P.partP + (((long long)s * P.nblk + chunk) * P.ns + k0 + g) * 2;
-                    o[0] = v[2 * g];
-                    o[1] = v[2 * g + 1];
+            const double w = warp_transpose_sum(a);
+            __syncthreads();                             // the last sums are read
+            red[warp][lane] = w;
+            __syncthreads();
+            if (warp == 0) {
+                static_assert(kWarpsPerBlock == 8, "the warps' tree");
+                double v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = red[i][lane];
+                const double sum = ((v[0] + v[4]) + (v[2] + v[6])) + ((v[1] + v[5]) + (v[3] + v[7]));
+                const int k = k0 + lane / NC;
+                if (k < P.ns) {
+                    double *o = P.partP + (((long long)s * P.nblk + chunk) * P.ns + k) * 2;
+                    o[NC == 2 ? lane & 1 : 0] = sum;
+                    if (NC == 1) o[1] = 0.0;
                 }
+            }
         }
     }
 }
@@ -2460,15 +2577,18 @@ __global__ void k_retire_grad(Params P, const double2 *__restrict__ x64, const d
     }
 }
 
-// drho_j += (4/h^3) u_n (.) Re x64 for every finished slot, slots added in slot order.
+// drho_j += (4/h^3) u_n (.) Re x64 for every finished slot; the slots of a column are added in slot order.
+// blockIdx.y takes the columns j = blockIdx.y mod gridDim.y (columns do not share values of drho), so
+// that small grids fill the GPU.
 __global__ void k_retire_drho(Params P, const double2 *__restrict__ x64, const double *__restrict__ psi,
                               double *__restrict__ drho, double scale) {
+    const int nf = *P.fin_cnt;
     for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < P.g.nd;
          idx += (long long)gridDim.x * blockDim.x) {
-        const int nf = *P.fin_cnt;
         for (int i = 0; i < nf; ++i) {
             const int s = P.fin_list[i];
             const Slot &sl = P.slots[s];
+            if (sl.j % (int)gridDim.y != (int)blockIdx.y) continue;
             drho[(long long)sl.j * P.g.nd + idx] +=
                 scale * psi[(long long)sl.n * P.g.nd + idx] * solution_at(P, x64, s, idx).x;
         }
@@ -2569,52 +2689,90 @@ __global__ void __launch_bounds__(1024) k_refill(Params P, const int *__restrict
 //   b = sign * (base - sum_k T[sys][k] u_k),  base = u_n (.) vt_j (pair) or rhs[sys]
 // then x64 = 0, the FP64 residual r64 = b (mixed form), and the inner vectors start from r = b,
 // x = 0, p = 0.  Partials: r^T r, ||b||^2.
-template <typename T>
+// Work items as k_refine_x.  The direction buffers are cleared for the kernels that start from them only
+// (ndir of them: the split kernels take two, the fused COCG kernels write theirs before they read it).
+template <typename T, int G>
 __global__ void __launch_bounds__(kThreads) k_load(Params P, const double *__restrict__ psi, int ns,
                                                    const double *__restrict__ vt, const double *__restrict__ rhs,
                                                    const double *__restrict__ Tc, double sign, double2 *__restrict__ b,
                                                    double2 *__restrict__ x64, typename Cx<T>::t *__restrict__ xin,
                                                    typename Cx<T>::t *__restrict__ r, typename Cx<T>::t *__restrict__ p,
-                                                   long long pstride) {
+                                                   long long pstride, int ndir) {
     using C = typename Cx<T>::t;
-    const long long items = (long long)P.S * P.nblk;
+    const int ngroups = (P.S + G - 1) / G;
+    const long long items = (long long)ngroups * P.nblk;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
-        const int s = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
-        const Slot &sl = P.slots[s];
-        if (sl.phase != kLoading) continue;
-        const long long off = (long long)s * P.g.nd;
-        const double *tc = Tc ? Tc + (long long)sl.sys * ns : nullptr;
-        double v[3] = {0.0, 0.0, 0.0};
-        for (int t = 0; t < kPPT; ++t) {
-            const long long idx = (long long)chunk * kChunk + t * kThreads + threadIdx.x;
-            if (idx < P.g.nd) {
-                double base = vt ? psi[(long long)sl.n * P.g.nd + idx] * vt[(long long)sl.j * P.g.nd + idx]
-                                 : rhs[(long long)sl.sys * P.g.nd + idx];
-                if (tc)
-                    for (int k = 0; k < ns; ++k) base -= tc[k] * psi[(long long)k * P.g.nd + idx];
-                const double bv = sign * base;
-                b[off + idx] = make_double2(bv, 0.0);     // the FP64 residual of x64 = 0
-                x64[off + idx] = make_double2(0.0, 0.0);
-                C z;
-                z.x = (T)0;
-                z.y = (T)0;
-                C rv;
-                rv.x = (T)bv;
-                rv.y = (T)0;
-                if ((const void *)xin != (const void *)x64) xin[off + idx] = z;
-                r[off + idx] = rv;
-                p[off + idx] = z;
-                p[pstride + off + idx] = z;
-                v[0] += (double)rv.x * rv.x;
-                v[2] += bv * bv;
+        const int g = (int)(it / P.nblk), chunk = (int)(it % P.nblk);
+        bool act[G], any = false;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            const int s = g * G + q;
+            act[q] = s < P.S && P.slots[s].phase == kLoading;
+            any = any || act[q];
+        }
+        if (!any) continue;                              // uniform per block
+        const long long i0 = (long long)chunk * kChunk + threadIdx.x;
+        double bv[G][kPPT];
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            if (!act[q]) continue;
+            const Slot &sl = P.slots[g * G + q];
+#pragma unroll
+            for (int t = 0; t < kPPT; ++t) {
+                const long long idx = i0 + t * kThreads;
+                bv[q][t] = idx >= P.g.nd ? 0.0
+                           : vt          ? psi[(long long)sl.n * P.g.nd + idx] * vt[(long long)sl.j * P.g.nd + idx]
+                                         : rhs[(long long)sl.sys * P.g.nd + idx];
             }
         }
-        block_sum<3>(v);
-        if (threadIdx.x == 0) {
-            double *o = P.partB + ((long long)s * P.nblk + chunk) * 3;
-            o[0] = v[0];
-            o[1] = v[1];
-            o[2] = v[2];
+        if (Tc)
+            for (int k = 0; k < ns; ++k) {
+                double u[kPPT];
+#pragma unroll
+                for (int t = 0; t < kPPT; ++t) {
+                    const long long idx = i0 + t * kThreads;
+                    u[t] = idx < P.g.nd ? psi[(long long)k * P.g.nd + idx] : 0.0;
+                }
+#pragma unroll
+                for (int q = 0; q < G; ++q)
+                    if (act[q]) {
+                        const double c = Tc[(long long)P.slots[g * G + q].sys * ns + k];
+#pragma unroll
+                        for (int t = 0; t < kPPT; ++t) bv[q][t] -= c * u[t];
+                    }
+            }
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            double v[2] = {0.0, 0.0};                    // r^T r (real), ||b||^2
+            if (act[q]) {
+                const long long off = (long long)(g * G + q) * P.g.nd;
+#pragma unroll
+                for (int t = 0; t < kPPT; ++t) {
+                    const long long idx = i0 + t * kThreads;
+                    if (idx < P.g.nd) {
+                        const double bq = sign * bv[q][t];
+                        b[off + idx] = make_double2(bq, 0.0);     // the FP64 residual of x64 = 0
+                        x64[off + idx] = make_double2(0.0, 0.0);
+                        C z, rv;
+                        z.x = z.y = (T)0;
+                        rv.x = (T)bq;
+                        rv.y = (T)0;
+                        if ((const void *)xin != (const void *)x64) xin[off + idx] = z;
+                        r[off + idx] = rv;
+                        if (ndir > 0) p[off + idx] = z;
+                        if (ndir > 1) p[pstride + off + idx] = z;
+                        v[0] += (double)rv.x * rv.x;
+                        v[1] += bq * bq;
+                    }
+                }
+            }
+            block_sum<2>(v);
+            if (threadIdx.x == 0 && act[q]) {
+                double *o = P.partB + ((long long)(g * G + q) * P.nblk + chunk) * 3;
+                o[0] = v[0];
+                o[1] = 0.0;
+                o[2] = v[1];
+            }
         }
     }
 }
@@ -2899,6 +3057,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     P.cproject = mixed && sp.Tc != nullptr;
     P.project = c.opt.project_solution != 0 || sp.grad != nullptr || (P.cproject && c.opt.tol < 1e-9);
     P.proj_re_only = sp.drho != nullptr && sp.grad == nullptr;
+    P.norm_only = use_lz || use_ring;
     P.ns = c.ns;
     P.psi = c.psi64;
     P.psi32 = c.psi32;
@@ -2926,6 +3085,12 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     const long long items = (long long)S * nblk;
     const unsigned grid = (unsigned)std::max<long long>(1, std::min<long long>(items, (long long)dev_sms * 8));
     const unsigned wgrid = cdiv(S, kWarpsPerBlock);      // one warp per slot
+    // the kernels that go over the orbitals take four slots at a time where that leaves six blocks an SM
+    // (37 x 43 x 29, 77 slots, three: 127 -> 156 us for the loads; 40^3, 1024 slots: 622 -> 586)
+    const bool wide = (long long)cdiv(S, 4) * nblk >= 6LL * dev_sms;
+    const unsigned ggrid = (unsigned)std::max<long long>(
+        1, std::min<long long>(wide ? (long long)cdiv(S, 4) * nblk : items, (long long)dev_sms * 8));
+    const int ndir = use_lz || use_ring ? 0 : 2;         // direction buffers a queue's kernels start from
     const int per_row = shape.pairs ? tl.tx / 2 : tl.tx;
     const int pa_threads = (per_row * tl.ty + 31) / 32 * 32;
     // halo elements (pairs of elements for the two-column kernel) per plane
@@ -3147,34 +3312,36 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
                 k_cproj_dots<<<grid, kThreads, 0, ss>>>(P, (const float2 *)xin);
                 k_proj_sum<<<wgrid, kThreads, 0, ss>>>(P, kInnerDone);
             }
-            k_refine_x<<<grid, kThreads, 0, ss>>>(P, x64, (float2 *)xin, (float2 *)q);
-            k_residual_df<<<grid, kThreads, 0, ss>>>(P, b, (const float2 *)q, (float2 *)r, (float2 *)p, c.vloc32,
-                                                     c.vloc_lo, cf_hi, cf_lo, 3.0 * c.coef.a[0]);   // p = direction buffer 0
+            (!wide ? k_refine_x<1> : c.ns > 32 ? k_refine_x<4> : k_refine_x<2>)<<<c.ns > 32 ? ggrid : grid, kThreads, 0, ss>>>(P, x64, (float2 *)xin, (float2 *)q);
+            k_residual_df<<<grid, kThreads, 0, ss>>>(P, b, (const float2 *)q, (float2 *)r, ndir ? (float2 *)p : nullptr,
+                                                     c.vloc32, c.vloc_lo, cf_hi, cf_lo, 3.0 * c.coef.a[0]);
             if (P.cproject) {
                 k_cproj_dots<<<grid, kThreads, 0, ss>>>(P, (const float2 *)r);
                 k_proj_sum<<<wgrid, kThreads, 0, ss>>>(P, kInnerDone);
-                k_cproj_residual<<<grid, kThreads, 0, ss>>>(P, (float2 *)r);
+                (wide ? k_cproj_residual<4> : k_cproj_residual<1>)<<<ggrid, kThreads, 0, ss>>>(P, (float2 *)r);
             }
             k_state<<<wgrid, kThreads, 0, ss>>>(P);
         }
         k_finished_list<<<1, 1024, 0, ss>>>(P);
         if (P.project) {
-            k_proj_dots<<<grid, kThreads, 0, ss>>>(P, x64);
+            (P.proj_re_only ? k_proj_dots<1> : k_proj_dots<2>)<<<grid, kThreads, 0, ss>>>(P, x64);
             k_proj_sum<<<wgrid, kThreads, 0, ss>>>(P, kFinished);
         }
         if (sp.grad)
             k_retire_grad<<<std::min<unsigned>(cdiv(nd, 256), 2048u), 256, 0, ss>>>(P, x64, sp.coef, sp.grad, scale);
         else if (sp.drho)
-            k_retire_drho<<<std::min<unsigned>(cdiv(nd, 256), 2048u), 256, 0, ss>>>(P, x64, c.psi64, sp.drho, scale);
+            k_retire_drho<<<dim3(std::min<unsigned>(cdiv(nd, 256), 2048u), (unsigned)std::max(1, std::min(sp.pairs, 8))), 256,
+                            0, ss>>>(P, x64, c.psi64, sp.drho, scale);
         else
             k_retire_copy<<<grid, kThreads, 0, ss>>>(P, x64, sp.xout);
         k_refill<<<1, 1024, 0, ss>>>(P, sys_n, sys_j, c.eps_dev, sp.omega);
         if (mixed)
-            k_load<float><<<grid, kThreads, 0, ss>>>(P, c.psi64, c.ns, sp.vt, sp.rhs, sp.Tc, sp.sign, b, x64,
-                                                     (float2 *)xin, (float2 *)r, (float2 *)p, pstride);
+            (wide ? k_load<float, 4> : k_load<float, 1>)<<<ggrid, kThreads, 0, ss>>>(
+                P, c.psi64, c.ns, sp.vt, sp.rhs, sp.Tc, sp.sign, b, x64, (float2 *)xin, (float2 *)r, (float2 *)p, pstride, ndir);
         else
-            k_load<double><<<grid, kThreads, 0, ss>>>(P, c.psi64, c.ns, sp.vt, sp.rhs, sp.Tc, sp.sign, b, x64,
-                                                      (double2 *)xin, (double2 *)r, (double2 *)p, pstride);
+            (wide ? k_load<double, 4> : k_load<double, 1>)<<<ggrid, kThreads, 0, ss>>>(
+                P, c.psi64, c.ns, sp.vt, sp.rhs, sp.Tc, sp.sign, b, x64, (double2 *)xin, (double2 *)r, (double2 *)p, pstride,
+                ndir);
         k_state<<<wgrid, kThreads, 0, ss>>>(P);
         RPA_LAUNCH("cocg maintenance");
     };
