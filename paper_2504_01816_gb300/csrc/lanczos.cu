@@ -17,8 +17,9 @@
 // [c nz / C, (c + 1) nz / C) of v_k with six halo planes on either side in shared memory; v_{k-1}, u and
 // v_{k+1} share one register array (each thread owns W x 2 x ZC points: W = 16 bytes of x, two rows, ZC
 // planes), so an iteration reads nothing from memory but V_loc (from L2) and writes only v_k, by a bulk
-// copy from shared memory, kept for the solution x = sum_k y_k v_k.  That sum is formed at the end, with
-// the vectors streamed back through the slab (or, when the history is full, by plain loads, and then with
+// copy from shared memory, kept for the solution x = sum_k y_k v_k.  That sum is formed by two extra warps
+// while the others are at the next solve, from a history of two buffers; warps that come to the end of that
+// solve before take part in what is left of it (or, when the history is full, all form it at once, with
 // the COCG direction p handed over).  Between blocks an iteration has two dependences and no cluster
 // barrier: the halo planes arrive by bulk copies through distributed shared memory that count on the
 // receiver's mbarrier, and overlap the x and y neighbours' part of the stencil; the three dot products are
@@ -32,12 +33,14 @@
 // plane 12 for the y and 2 XL for the x neighbours: 58 bytes a point for ZC = 5 in FP32 against 240 for
 // a plane-by-plane march on complex values; the FP64 form is bound by the FP64 pipe (46 operations a
 // point).  Measured (GB300, tol 1e-11, whole chi0 application, against the fused and split COCG kernels):
-// 40^3, 1024 systems 212 -> 125 ms; 24^3, 4 systems 9.8 -> 2.1 ms; 37 x 43 x 29, 77 systems 25 -> 8.5 ms;
-// FP64 15^3, 32 systems 15.9 -> 3.2 ms, 32^3, 128 systems 197 -> 92 ms.  At 40^3 (four blocks a system) an
-// iteration takes 22.6 thousand cycles: x and y neighbours 9.2 (5.7 of shared-memory loads and 2.5 of
-// copies), z neighbours 3.0, halo 1.1, sums 2.1, update 2.7, and per iteration of a solve 3.8 for the
-// solution and 1.2 for the start.  One form with 64-bit index arithmetic per halo store took 230 ms, one
-// with cluster barriers 138 ms, one with the solution's code inlined (spills) 158 ms.
+// 40^3, 1024 systems 212 -> 98 ms; 24^3, 4 systems 9.9 -> 1.9 ms; 37 x 43 x 29, 77 systems 25 -> 6.8 ms;
+// FP64 15^3, 32 systems 15.9 -> 3.2 ms, 32^3, 128 systems 197 -> 79 ms.  At 40^3 (four blocks a system) an
+// iteration takes 20 thousand cycles: x and y neighbours 9.4 (5.7 of shared-memory loads and 2.5 of
+// copies), z neighbours 2.8, sums 2.3, update 2.2, halo 0.3, and per iteration of a solve 1.4 of waiting for
+// the solution before it and 2.0 for the start.  With the solution formed at the end of each solve, by all
+// warps: 22.4 thousand, 3.8 of them for it (and 9.6 of 26 where a system lies on two blocks).  One form with
+// 64-bit index arithmetic per halo store took 230 ms, one with cluster barriers 138 ms, one with the
+// solution's code inlined (spills) 158 ms, one that stored the history from registers 102 ms against 98.
 #include <algorithm>
 #include <cmath>
 
@@ -49,7 +52,8 @@ namespace {
 
 constexpr int kHistMax = 128;            // Lanczos vectors kept between two updates of x
 
-constexpr int kStages = 4;               // vectors of the history in flight at the end of a solve
+constexpr int kFlushThreads = 64;        // two warps that form the solutions
+constexpr int kExtra = 32 + kFlushThreads;   // threads without points: the scalar warp, the flush warps
 
 // W values of one row: 16 bytes.
 template <typename T> struct Pk;
@@ -149,8 +153,8 @@ __device__ __forceinline__ void cluster_barrier() {
 __device__ __forceinline__ void mbar_init(unsigned long long *b) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(b)) : "memory");
 }
-// Wait for a phase of an mbarrier; false after ~1 s of cycles.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+// Wait for a phase of an mbarrier; false after `limit` cycles (~1 s; the flush warps' wait for a whole solve longer).
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, long long limit = 2000000000LL) {
     const long long t0 = clock64();
     for (;;) {
         unsigned done;
@@ -160,7 +164,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
             : "r"(bar), "r"(parity)
             : "memory");
         if (done) return true;
-        if (clock64() - t0 > 2000000000LL) return false;
+        if (clock64() - t0 > limit) return false;
     }
 }
 
@@ -217,6 +221,12 @@ struct ScalarState {
     int sweeps, fail;                    // fail: 1 limit, 2 breakdown, 3 non-finite
 };
 
+// A solution to form, for the flush warps: slot s (-1: no more), n vectors of history buffer buf, the part's phase.
+struct Job {
+    int s, n, buf, have_p;
+    double er, ei;
+};
+
 // Shared memory of a block, before its slab of planes.
 template <typename T> struct Shared {
     using V4 = typename Vec4<T>::t;
@@ -225,12 +235,15 @@ template <typename T> struct Shared {
     T part[2][16][4];                    // the blocks' sums of a reduction (alternating)
     T red[3][32];
     T vec[4];                            // a', 1/g, g (FP64)
-    double dr[kHistMax], di[kHistMax], zr[kHistMax], zi[kHistMax], g[kHistMax];   // factors by history place
+    double dr[2][kHistMax], di[2][kHistMax], zr[2][kHistMax], zi[2][kHistMax], g[2][kHistMax];   // factors by history place
     double start[4];                     // cos phi, sin phi, ||r_a||, ||r_b||
     ScalarState F;
-    unsigned long long bar, pbar[2], fbar[kStages];   // arrival of the halo, of the sums, of a vector
-    unsigned fphase;                     // phase of each fbar
-    int item, flag;
+    unsigned long long bar, pbar[2], ibar[2];   // arrival of the halo, of the sums, of the next system
+    unsigned long long job_full, job_done;      // a job for the flush warps, and its end
+    Job job;
+    int next;                            // its first place that no warp has taken
+    unsigned opened;                     // jobs whose coefficients are there
+    int item[2], flag;
     int nto, to[4 * 12];                 // the copies that fill the neighbours' halos
     unsigned expect;                     // bytes that arrive in this block's halo
     LanczosArgs<T> A;                    // for the functions off the hot path
@@ -267,7 +280,7 @@ template <typename T, int ZC> struct Geo {
         nvz = unit ? max(0, min(ZC, nzl - lz0)) : 0;
         c0 = (lz0 + kRadius) * A.plane + gy * A.pitch + PAD + gx;
         c1 = row1 ? c0 + A.pitch : c0;
-        nthr = (int)blockDim.x - 32;
+        nthr = (int)blockDim.x - kExtra;
     }
     // private 16-byte place of (z, r) in a vector of the workspace, in elements
     __device__ __forceinline__ size_t priv(int z, int r) const { return ((size_t)(2 * z + r) * nthr + threadIdx.x) * W; }
@@ -276,16 +289,18 @@ template <typename T, int ZC> struct Geo {
         return ((long long)(z0 + lz0 + z) * A.ny + gy + r) * A.nx + gx;
     }
 };
-// The block's arrays in the workspace: V_loc, the direction (re, im), the history (laid out as in the slab).
+// The block's arrays in the workspace: V_loc by threads; the direction (re, im) and the history, laid out as in
+// the slab.
 template <typename T, int ZC> struct Work {
-    T *V, *Pd, *H;
-    size_t vec, hvec;
+    T *V, *Pd, *H;                       // H: two buffers, buf elements apart
+    size_t vec, hvec, buf;
     __device__ __forceinline__ Work(const LanczosArgs<T> &A) {
-        vec = (size_t)2 * ZC * (blockDim.x - 32) * Pk<T>::W;
+        vec = (size_t)2 * ZC * (blockDim.x - kExtra) * Pk<T>::W;
         hvec = (size_t)A.nch * ZC * A.plane;
         V = A.ws + (size_t)blockIdx.x * A.ws_stride;
         Pd = V + vec;
-        H = Pd + 2 * vec;
+        H = Pd + 2 * hvec;
+        buf = (size_t)A.hist * hvec;
     }
 };
 template <typename T> __device__ __forceinline__ T *slab_of(const LanczosArgs<T> &A) {
@@ -315,10 +330,12 @@ __device__ __forceinline__ void put(T *own, int gx, int nvx, int nx, const Pk<T>
     }
 }
 
+// Barrier of the threads that iterate (the flush warps run beside them).
+__device__ __forceinline__ void main_sync(int nmain) { asm volatile("bar.sync 1, %0;" ::"r"(nmain) : "memory"); }
 // The block's own planes are stored: before the bulk copies read them.
-__device__ __forceinline__ void planes_stored() {
+__device__ __forceinline__ void planes_stored(int nmain) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
+    main_sync(nmain);
 }
 // The planes to the halos of the blocks that need them (one bulk copy a block and side), by the scalar
 // lane once they are stored and no block reads its last halo any more; the phase of sh().bar is complete
@@ -352,9 +369,10 @@ __device__ __forceinline__ void keep_wait() { asm volatile("cp.async.bulk.wait_g
 // sends only after all its threads are done with the stencil, so the wait also says that no block reads
 // its halo any more.  The sums alternate between two buffers and barriers: a block may be one
 // reduction ahead of another, never two.
-template <typename T> __device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int *err) {
+template <typename T>
+__device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int nmain, int *err) {
     Shared<T> &S = sh<T>();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (int)(blockDim.x >> 5);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = nmain >> 5;
     T v[3] = {a, b, c};
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
@@ -363,7 +381,7 @@ template <typename T> __device__ __forceinline__ void gather3(T a, T b, T c, uns
     if (lane == 0)
 #pragma unroll
         for (int q = 0; q < 3; ++q) S.red[q][warp] = v[q];
-    __syncthreads();
+    main_sync(nmain);
     const unsigned pb = (unsigned)__cvta_generic_to_shared(&S.pbar[ng & 1]);
     if (warp == 0) {
 #pragma unroll
@@ -397,7 +415,7 @@ template <typename T> __device__ __forceinline__ void sum_parts(unsigned ng, int
 // The pending step's factors, by the scalar lane while the others compute the next stencil: d_k and z_k of
 // the LU of T + i w, the residual and the stopping test (flag: 0 go on, 1 converged, 2 limit, 3 breakdown,
 // 4 non-finite); j its place in the history, steps the steps so far.
-template <typename T> __device__ __forceinline__ void factor(int j, int steps, int maxit) {
+template <typename T> __device__ __forceinline__ void factor(int buf, int j, int steps, int maxit) {
     Shared<T> &S = sh<T>();
     ScalarState &F = S.F;
     const double ig = F.ig, g1 = ig > 0.0 ? 1.0 / ig : 0.0;
@@ -409,11 +427,11 @@ template <typename T> __device__ __forceinline__ void factor(int j, int steps, i
     const double dr = er * iq, di = -ei * iq;
     const double yr = zr * dr - zi * di, yi = zr * di + zi * dr;
     const double rn = g1 * sqrt(yr * yr + yi * yi);
-    S.dr[j] = F.dr = dr;
-    S.di[j] = F.di = di;
-    S.zr[j] = F.zr = zr;
-    S.zi[j] = F.zi = zi;
-    S.g[j] = F.gam;
+    S.dr[buf][j] = F.dr = dr;
+    S.di[buf][j] = F.di = di;
+    S.zr[buf][j] = F.zr = zr;
+    S.zi[buf][j] = F.zi = zi;
+    S.g[buf][j] = F.gam;
     F.gam = g1;
     F.sweeps += 1;
     int flag = 0;
@@ -555,170 +573,219 @@ template <typename T, int ZC, int MODE> __device__ __noinline__ void start_vecto
         }
 }
 
-// x += sum_j y_j v_j over the n vectors of the history (and the direction handed over by the last time,
-// have_p); with go_on also the COCG direction p of the last of them.  (er, ei): the part's phase.
-template <typename T, int ZC, int MODE>
-__device__ __noinline__ void flush(int s, int n, bool go_on, bool have_p, double er, double ei) {
+// The solution's coefficients, by one thread: x += sum_j y_j v_j over the n vectors of history buffer buf, y from
+// U y = z backwards (times the part's phase er + i ei), prev: of the direction handed over by the last time; the
+// COCG direction of the last vector, p = sum_j q_j v_j + q_prev p_prev, likewise.
+template <typename T> __device__ __noinline__ void coefficients(int buf, int n, double er, double ei) {
+    using V4 = typename Vec4<T>::t;
+    Shared<T> &S = sh<T>();
+    double yr = 0, yi = 0, qr = 0, qi = 0;
+    for (int j = n - 1; j >= 0; --j) {
+        const double cn = j + 1 < n ? (double)(T)S.g[buf][j + 1] : 0.0, dr = S.dr[buf][j], di = S.di[buf][j];
+        const double tr = S.zr[buf][j] - cn * yr, ti = S.zi[buf][j] - cn * yi;
+        yr = tr * dr - ti * di;
+        yi = tr * di + ti * dr;
+        const double ur = j == n - 1 ? 1.0 : -cn * qr, ui = j == n - 1 ? 0.0 : -cn * qi;
+        qr = ur * dr - ui * di;
+        qi = ur * di + ui * dr;
+        V4 c;
+        c.x = (T)(er * yr - ei * yi);
+        c.y = (T)(er * yi + ei * yr);
+        c.z = (T)qr;
+        c.w = (T)qi;
+        S.coef[j] = c;
+    }
+    const double c0 = (double)(T)S.g[buf][0];
+    V4 c;
+    c.x = (T)(-c0 * (er * yr - ei * yi));
+    c.y = (T)(-c0 * (er * yi + ei * yr));
+    c.z = (T)(-c0 * qr);
+    c.w = (T)(-c0 * qi);
+    S.prev = c;
+}
+
+// x of slot s += the history's sum at the 16-byte places e, e + nt .. of the block's planes (GO: and the
+// direction handed over formed anew), NP places a thread.  Two warps have to keep up with the others' iterations, and one warp
+// issues an instruction every four to five cycles: four 16-byte places at a time, so that a coefficient is
+// read once for four loads, whose addresses advance by additions (a first form with two places and products
+// in the addresses took 29 to 42 thousand cycles a vector of 16000 points, 9 with all 13 warps).
+template <typename T, int ZC, bool GO, int NP> __device__ __forceinline__ void add_history(const Job &J, int e, int nt) {
     using P = Pk<T>;
     using C = typename Cx<T>::t;
     using V4 = typename Vec4<T>::t;
-    constexpr int W = P::W;
+    constexpr int W = P::W, PAD = Geo<T, ZC>::PAD;
     Shared<T> &S = sh<T>();
     const LanczosArgs<T> &A = S.A;
-    const Geo<T, ZC> G(A);
     const Work<T, ZC> K(A);
-    T *const slab = slab_of(A);
-    C *const xg = A.x + (long long)s * A.nd;
-    const bool scalar = (int)threadIdx.x == G.nthr;
-    const int planeE = A.plane;
-    if (scalar) {
-        // U y = z backwards; p = sum_j q_j v_j + q_prev p_prev likewise
-        double yr = 0, yi = 0, qr = 0, qi = 0;
-        for (int j = n - 1; j >= 0; --j) {
-            const double cn = j + 1 < n ? (double)(T)S.g[j + 1] : 0.0;
-            const double dr = S.dr[j], di = S.di[j];
-            const double tr = S.zr[j] - cn * yr, ti = S.zi[j] - cn * yi;
-            yr = tr * dr - ti * di;
-            yi = tr * di + ti * dr;
-            V4 c;
-            c.x = (T)(er * yr - ei * yi);
-            c.y = (T)(er * yi + ei * yr);
-            if (go_on) {
-                const double ur = j == n - 1 ? 1.0 : -cn * qr, ui = j == n - 1 ? 0.0 : -cn * qi;
-                qr = ur * dr - ui * di;
-                qi = ur * di + ui * dr;
-            }
-            c.z = (T)qr;
-            c.w = (T)qi;
-            S.coef[j] = c;
-        }
-        const double c0d = (double)(T)S.g[0];
-        V4 c;
-        c.x = (T)(-c0d * (er * yr - ei * yi));
-        c.y = (T)(-c0d * (er * yi + ei * yr));
-        c.z = (T)(-c0d * qr);
-        c.w = (T)(-c0d * qi);
-        S.prev = c;
-        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the history is written
-    }
-    planes_stored();
-    auto add_x = [&](int z, int r, const P &xr, const P &xi) {
-        C *dst = xg + G.grid(A, z, r);
-        C q[W];
+    const int rank = (int)(blockIdx.x % (unsigned)A.ncl), z0 = rank * A.nz / A.ncl, nzl = (rank + 1) * A.nz / A.ncl - z0;
+    const int rows = nzl * A.ny, total = rows * A.hw, n = J.n;
+    const T *const H = K.H + J.buf * K.buf;
+    const size_t step = K.hvec;
+    const T *q[NP];
+    int o[NP];
 #pragma unroll
-        for (int i = 0; i < W; ++i) q[i] = i < G.nvx ? dst[i] : C{0, 0};
+    for (int h = 0; h < NP; ++h) {
+        const int m = min(e + h * nt, total - 1);    // past the end: the last place again, not stored
+        const int row = m / A.hw, z = row / A.ny;
+        o[h] = z * A.plane + (row - z * A.ny) * A.pitch + PAD + W * (m - row * A.hw);
+        q[h] = H + o[h];
+    }
+    P xr[NP], xi[NP], pr[NP], pi[NP];
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+        xr[h].zero();
+        xi[h].zero();
+        pr[h].zero();
+        pi[h].zero();
+    }
+    auto add = [&](int j, const P (&v)[NP]) {
+        const V4 c = S.coef[j];
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            xr[h].fma(c.x, v[h]);
+            xi[h].fma(c.y, v[h]);
+            if (GO) {
+                pr[h].fma(c.z, v[h]);
+                pi[h].fma(c.w, v[h]);
+            }
+        }
+    };
+    auto load = [&](P (&v)[NP]) {
+#pragma unroll
+        for (int h = 0; h < NP; ++h) {
+            v[h] = pk_load_l2(q[h]);
+            q[h] += step;
+        }
+    };
+    int j = 0;
+    for (; j + 4 <= n; j += 4) {
+        P v0[NP], v1[NP], v2[NP], v3[NP];
+        load(v0);
+        load(v1);
+        load(v2);
+        load(v3);
+        add(j, v0);
+        add(j + 1, v1);
+        add(j + 2, v2);
+        add(j + 3, v3);
+    }
+    for (; j < n; ++j) {
+        P v0[NP];
+        load(v0);
+        add(j, v0);
+    }
+    const V4 pv = S.prev;
+#pragma unroll
+    for (int h = 0; h < NP; ++h) {
+        if (e + h * nt >= total) continue;
+        if (J.have_p) {
+            const P qr = pk_load_l2(K.Pd + o[h]), qi = pk_load_l2(K.Pd + K.hvec + o[h]);
+            xr[h].fma(pv.x, qr);
+            xr[h].fma(-pv.y, qi);
+            xi[h].fma(pv.x, qi);
+            xi[h].fma(pv.y, qr);
+            if (GO) {
+                pr[h].fma(pv.z, qr);
+                pr[h].fma(-pv.w, qi);
+                pi[h].fma(pv.z, qi);
+                pi[h].fma(pv.w, qr);
+            }
+        }
+        if (GO) {
+            pk_store(K.Pd + o[h], pr[h]);
+            pk_store(K.Pd + K.hvec + o[h], pi[h]);
+        }
+        const int m = e + h * nt, row = m / A.hw, gx = W * (m - row * A.hw), nvx = min(W, A.nx - gx);
+        C *dst = A.x + (long long)J.s * A.nd + ((long long)z0 * A.ny + row) * A.nx + gx;
+        C c[W];
+#pragma unroll
+        for (int i = 0; i < W; ++i) c[i] = i < nvx ? __ldcg(dst + i) : C{0, 0};
 #pragma unroll
         for (int i = 0; i < W; ++i)
-            if (i < G.nvx) {
-                q[i].x += xr.get(i);
-                q[i].y += xi.get(i);
-                dst[i] = q[i];
-            }
-    };
-    auto add_prev = [&](const V4 &c, bool dir, size_t o, P &xr, P &xi) {
-        const T cr = dir ? c.z : c.x, ci = dir ? c.w : c.y;
-        const P qr = pk_load(K.Pd + o), qi = pk_load(K.Pd + K.vec + o);
-        xr.fma(cr, qr);
-        xr.fma(-ci, qi);
-        xi.fma(cr, qi);
-        xi.fma(ci, qr);
-    };
-    if (!go_on && A.stages > 1) {
-        // the vectors through the slab (which is free now), A.stages bulk copies ahead
-        const int sp = A.nzl_max * planeE;               // elements of a stage
-        const unsigned bytes = (unsigned)(G.nzl * planeE * (int)sizeof(T));
-        auto fetch = [&](int j, int q) {
-            const unsigned fb = (unsigned)__cvta_generic_to_shared(&S.fbar[q]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(bytes) : "memory");
-            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                             (unsigned)__cvta_generic_to_shared(slab + q * sp)),
-                         "l"(__cvta_generic_to_global(K.H + (size_t)j * K.hvec)), "r"(bytes), "r"(fb)
-                         : "memory");
-        };
-        if (scalar)
-            for (int j = 0; j < min(n, A.stages); ++j) fetch(j, j);
-        P xr[ZC][2], xi[ZC][2];
-#pragma unroll
-        for (int z = 0; z < ZC; ++z)
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                xr[z][r].zero();
-                xi[z][r].zero();
-            }
-        unsigned ph = S.fphase;
-        const T *const st0 = slab + G.c0 - kRadius * planeE;
-        const int d1 = G.c1 - G.c0;
-        for (int j = 0, q = 0; j < n; ++j, q = q + 1 == A.stages ? 0 : q + 1) {
-            if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.fbar[q]), (ph >> q) & 1)) atomicExch(A.err, 2);
-            ph ^= 1u << q;
-            const V4 c = S.coef[j];
-            const T *const st = st0 + q * sp;
-#pragma unroll
-            for (int z = 0; z < ZC; ++z)
-                if (z < G.nvz)
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        const P v = pk_load(st + (r ? d1 : 0) + z * planeE);
-                        xr[z][r].fma(c.x, v);
-                        xi[z][r].fma(c.y, v);
-                    }
-            __syncthreads();
-            if (scalar && j + A.stages < n) fetch(j + A.stages, q);
-        }
-        if (scalar) S.fphase = ph;
-#pragma unroll
-        for (int z = 0; z < ZC; ++z)
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-                if (z < G.nvz && (r == 0 || G.row1)) {
-                    if (have_p) add_prev(S.prev, false, G.priv(z, r), xr[z][r], xi[z][r]);
-                    add_x(z, r, xr[z][r], xi[z][r]);
-                }
-        // halo planes outside the box are zero again
-        if (MODE != 1) {
-            P zero;
-            zero.zero();
-            for (int e = W * (int)threadIdx.x; e < max(0, kRadius - G.z0) * planeE; e += W * (int)blockDim.x)
-                pk_store(slab + e, zero);
-            for (int e = (A.nz - G.z0 + kRadius) * planeE + W * (int)threadIdx.x; e < (G.nzl + 2 * kRadius) * planeE;
-                 e += W * (int)blockDim.x)
-                pk_store(slab + e, zero);
-        }
-    } else if (G.nvz > 0) {
-        for (int pass = 0; pass < (go_on ? 2 : 1); ++pass)           // x, then p
-            for (int r = 0; r < (G.row1 ? 2 : 1); ++r) {
-                const T *const hr = K.H + (r ? G.c1 : G.c0) - kRadius * planeE;
-                P xr[ZC], xi[ZC];
-#pragma unroll
-                for (int z = 0; z < ZC; ++z) {
-                    xr[z].zero();
-                    xi[z].zero();
-                }
-#pragma unroll 2
-                for (int j = 0; j < n; ++j) {
-                    const V4 c = S.coef[j];
-                    const T cr = pass ? c.z : c.x, ci = pass ? c.w : c.y;
-#pragma unroll
-                    for (int z = 0; z < ZC; ++z) {
-                        const P v = pk_load_l2(hr + (size_t)j * K.hvec + z * planeE);
-                        xr[z].fma(cr, v);
-                        xi[z].fma(ci, v);
-                    }
-                }
-#pragma unroll
-                for (int z = 0; z < ZC; ++z) {
-                    const size_t o = G.priv(z, r);
-                    if (have_p) add_prev(S.prev, pass != 0, o, xr[z], xi[z]);
-                    if (pass) {
-                        pk_store(K.Pd + o, xr[z]);
-                        pk_store(K.Pd + K.vec + o, xi[z]);
-                    } else if (z < G.nvz) {
-                        add_x(z, r, xr[z], xi[z]);
-                    }
-                }
+            if (i < nvx) {
+                c[i].x += xr[h].get(i);
+                c[i].y += xi[h].get(i);
+                dst[i] = c[i];
             }
     }
-    __syncthreads();                                     // the coefficients are read before they change
+}
+
+// The places of the job in hand that no warp has taken, NP rows of 32 at a time: by the flush warps, and by
+// the others once they are at the end of the next part (a place's sum is the same whoever forms it).
+template <typename T, int ZC, int NP> __device__ __noinline__ void take_places() {
+    Shared<T> &S = sh<T>();
+    const int rank = (int)(blockIdx.x % (unsigned)S.A.ncl), lane = (int)threadIdx.x & 31;
+    const int total = ((rank + 1) * S.A.nz / S.A.ncl - rank * S.A.nz / S.A.ncl) * S.A.ny * S.A.hw;
+    for (;;) {
+        int e = 0;
+        if (lane == 0) e = atomicAdd(&S.next, 32 * NP);
+        e = __shfl_sync(0xffffffffu, e, 0);
+        if (e >= total) break;
+        __threadfence_block();
+        add_history<T, ZC, false, NP>(S.job, e + lane, 32);
+    }
+    __threadfence();
+}
+
+// The flush warps: forms the solution of every finished part while the other warps go on with the next.
+template <typename T, int ZC> __device__ __noinline__ void flush_warps() {
+    Shared<T> &S = sh<T>();
+    const int t = (int)threadIdx.x - ((int)blockDim.x - kFlushThreads);
+    const unsigned full = (unsigned)__cvta_generic_to_shared(&S.job_full), done = (unsigned)__cvta_generic_to_shared(&S.job_done);
+    for (unsigned job = 1;; ++job) {
+        if (!mbar_wait(full, (job - 1) & 1, 200000000000LL)) {
+            atomicExch(S.A.err, 2);
+            return;
+        }
+        const Job J = S.job;
+        if (J.s < 0) return;
+        if (t == 0) {
+            coefficients<T>(J.buf, J.n, J.er, J.ei);
+            __threadfence_block();
+            atomicExch(&S.next, 0);
+            *(volatile unsigned *)&S.opened = job;
+        }
+        asm volatile("bar.sync 2, %0;" ::"r"(kFlushThreads) : "memory");
+        take_places<T, ZC, 4>();
+        asm volatile("bar.sync 2, %0;" ::"r"(kFlushThreads) : "memory");
+        if (t == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(done) : "memory");
+    }
+}
+
+// The threads that iterate, before the history's next use: the last job is done.
+template <typename T, int ZC> __device__ __forceinline__ void finish_job(int nmain) {
+    take_places<T, ZC, 2>();
+    main_sync(nmain);
+}
+// The scalar lane then: the flush warps are done with it too (njobs posted so far).
+template <typename T> __device__ __forceinline__ void jobs_done(unsigned njobs) {
+    Shared<T> &S = sh<T>();
+    if (njobs > 0 && !mbar_wait((unsigned)__cvta_generic_to_shared(&S.job_done), (njobs - 1) & 1)) atomicExch(S.A.err, 2);
+}
+// ... and the next.
+template <typename T> __device__ __forceinline__ void post_job(const Job &J, unsigned &njobs) {
+    Shared<T> &S = sh<T>();
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");    // the history is written
+    jobs_done<T>(njobs);
+    S.job = J;
+    ++njobs;
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(&S.job_full)) : "memory");
+}
+
+// The history is full: its sum into x, the direction handed over, by the threads that iterate.
+template <typename T, int ZC> __device__ __noinline__ void flush_full(const Job &J, unsigned njobs, int nmain) {
+    finish_job<T, ZC>(nmain);
+    if ((int)threadIdx.x == nmain - 32) {
+        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        jobs_done<T>(njobs);
+        coefficients<T>(J.buf, J.n, J.er, J.ei);
+    }
+    main_sync(nmain);
+    const int rank = (int)(blockIdx.x % (unsigned)sh<T>().A.ncl), nz = sh<T>().A.nz, ncl = sh<T>().A.ncl;
+    const int total = ((rank + 1) * nz / ncl - rank * nz / ncl) * sh<T>().A.ny * sh<T>().A.hw;
+    for (int e = threadIdx.x; e < total; e += 2 * nmain) add_history<T, ZC, true, 2>(J, e, nmain);
+    __threadfence();
+    main_sync(nmain);
 }
 
 // Once a block: its slab cleared, barriers, the halo copies, V_loc by threads.
@@ -741,8 +808,11 @@ template <typename T, int ZC> __device__ __noinline__ void block_setup(const Lan
     if ((int)threadIdx.x == G.nthr) {
         mbar_init(&S.bar);
         for (int q = 0; q < 2; ++q) mbar_init(&S.pbar[q]);
-        for (int q = 0; q < kStages; ++q) mbar_init(&S.fbar[q]);
-        S.fphase = 0;
+        for (int q = 0; q < 2; ++q) mbar_init(&S.ibar[q]);
+        mbar_init(&S.job_full);
+        mbar_init(&S.job_done);
+        S.next = 1 << 30;                                // no job
+        S.opened = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // the copies: this block's planes [g0, g1) that lie in the halo of rank t (periodic: of its image)
         const int ncl = A.ncl, nz = A.nz, z0 = G.z0, z1 = G.z0 + G.nzl, pb = A.plane * (int)sizeof(T);
@@ -788,49 +858,67 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
     __syncthreads();
     block_setup<T, ZC>(&S.A, PER);
     const Geo<T, ZC> G(A);
+    const int nmain = G.nthr + 32;                      // threads that iterate: points and the scalar warp
     const bool scalar = tid == G.nthr;
     T *const slab = slab_of(A);
     const int slab_off = shared_bytes<T>() + A.lead * (int)sizeof(T);
     const int pb = A.plane * (int)sizeof(T), rb = A.pitch * (int)sizeof(T);   // bytes of a plane, a row
     constexpr int QB = 16;                              // bytes of W values
     const int n_items = *A.cnt;
-    unsigned phase = 0, ng = 0;                         // halo phase, reductions so far
-    cluster_barrier();                                  // every block runs, has cleared its slab and set its barriers
-    for (;;) {
-        // the next system, from the end of the list (the highest orbitals, the longest solves, first)
-        if (G.rank == 0 && tid < ncl) {
-            int it = 0;
-            if (tid == 0) it = atomicAdd(A.grab, 1);
-            it = __shfl_sync((1u << ncl) - 1u, it, 0);
-            asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
-                             map_rank((unsigned)__cvta_generic_to_shared(&S.item), tid)),
-                         "r"(it)
-                         : "memory");
+    unsigned phase = 0, ng = 0, ns = 0, njobs = 0;      // halo phase; reductions, systems, jobs so far
+    int buf = 0;                                        // history buffer
+    // the next system, by the scalar lane of the first block, from the end of the list (the highest orbitals,
+    // the longest solves, first); every block receives its number in item[m & 1]
+    auto fetch = [&](unsigned m) {
+        if (G.rank == 0) {
+            const int it = atomicAdd(A.grab, 1);
+            for (int t = 0; t < ncl; ++t)
+                asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
+                                 map_rank((unsigned)__cvta_generic_to_shared(&S.item[m & 1]), t)),
+                             "r"(it), "r"(map_rank((unsigned)__cvta_generic_to_shared(&S.ibar[m & 1]), t))
+                             : "memory");
         }
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 4;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(&S.ibar[m & 1]))
+                     : "memory");
+    };
+    cluster_barrier();                                  // every block runs, has cleared its slab and set its barriers
+    if (tid >= nmain) {
+        flush_warps<T, ZC>();
         cluster_barrier();
-        if (S.item >= n_items) break;
-        const int s = A.list[n_items - 1 - S.item];
+        return;
+    }
+    if (scalar) fetch(0);
+    for (;; ++ns) {
+        if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.ibar[ns & 1]), (ns >> 1) & 1)) {
+            atomicExch(A.err, 2);
+            break;
+        }
+        const int it = S.item[ns & 1];
+        if (it >= n_items) break;
+        const int s = A.list[n_items - 1 - it];
         // the right-hand side's phase and the norms of its two parts
         {
             T rr, ii, ri;
             start_sums<T, ZC>(s, rr, ii, ri);
-            gather3(rr, ii, ri, ng, ncl, G.rank, A.err);
+            gather3(rr, ii, ri, ng, ncl, G.rank, nmain, A.err);
             if (scalar) {
+                fetch(ns + 1);                           // every block has read the number before this one
                 T a, b, c;
                 sum_parts(ng, ncl, a, b, c);
                 start_state<T>(a, b, c, A.d0 + A.slots[s].shift_re, A.slots[s].shift_im);
             }
-            __syncthreads();
+            main_sync(nmain);
         }
         for (int pt = 0; pt < 2; ++pt) {
             T f_re, f_im;
             if (!start_part<T>(A, s, pt, scalar, f_re, f_im)) continue;
             start_vector<T, ZC, MODE>(s, f_re, f_im);
-            planes_stored();
+            planes_stored(nmain);
             if (scalar) {
                 const Work<T, ZC> K(A);
                 send_halos(slab);
-                keep(slab, K.H, K.hvec, 0, G.nzl, A.plane);
+                keep(slab, K.H + buf * K.buf, K.hvec, 0, G.nzl, A.plane);
             }
             P acc[ZC][2];
 #pragma unroll
@@ -847,7 +935,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                 int o0 = slab_off + G.c0 * (int)sizeof(T), o1 = slab_off + G.c1 * (int)sizeof(T);
                 asm volatile("" : "+r"(o0), "+r"(o1));
                 if (scalar) {
-                    if (k > kb) factor<T>(k - 1 - kb, k, A.maxit);
+                    if (k > kb) factor<T>(buf, k - 1 - kb, k, A.maxit);
                     keep_wait();
                 }
                 // ---- u = B v_k - c_k v_{k-1} (shifted), sums v.v, u.v, u.u.  The x and y neighbours and the
@@ -961,7 +1049,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                     suv = t1.sum();
                     suu = t2.sum();
                 }
-                gather3(svv, suv, suu, ng, ncl, G.rank, A.err);
+                gather3(svv, suv, suu, ng, ncl, G.rank, nmain, A.err);
                 if (k > kb && S.flag) {                  // the last step ended the solve
                     n = k - kb;
                     break;
@@ -982,7 +1070,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                         S.vec[1] = ig;
                         S.vec[2] = ig > (T)0 ? (T)1 / ig : (T)0;
                     }
-                    __syncthreads();
+                    main_sync(nmain);
                     ap = S.vec[0];
                     ig = S.vec[1];
                 }
@@ -1012,18 +1100,19 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                 // the next stencil: its diagonal shifted by a_k (u.v stays small against u.u)
                 cc = sizeof(T) == 8 ? S.vec[2] : ig > (T)0 ? (T)1 / ig : (T)0;
                 dg -= ap;
-                planes_stored();
+                planes_stored(nmain);
                 ++k;
                 if (k - kb == A.hist) {                  // the history is full: into x and p
-                    if (scalar) factor<T>(k - 1 - kb, k, A.maxit);
-                    __syncthreads();
+                    if (scalar) factor<T>(buf, k - 1 - kb, k, A.maxit);
+                    main_sync(nmain);
                     n = k - kb;
                     if (S.flag) break;
-                    flush<T, ZC, MODE>(s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+                    flush_full<T, ZC>(Job{s, n, buf, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]},
+                                      njobs, nmain);
                     have_p = true;
                     kb = k;
                     const Work<T, ZC> K(A);
-                    const T *const hl = K.H + (size_t)(A.hist - 1) * K.hvec - kRadius * A.plane;   // v_{k-1} again
+                    const T *const hl = K.H + buf * K.buf + (size_t)(A.hist - 1) * K.hvec - kRadius * A.plane;   // v_{k-1} again
 #pragma unroll
                     for (int z = 0; z < ZC; ++z) {
                         acc[z][0] = pk_load_l2(hl + G.c0 + z * A.plane);
@@ -1033,17 +1122,25 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                 if (scalar) {
                     const Work<T, ZC> K(A);
                     send_halos(slab);
-                    keep(slab, K.H, K.hvec, k - kb, G.nzl, A.plane);
+                    keep(slab, K.H + buf * K.buf, K.hvec, k - kb, G.nzl, A.plane);
                 }
             }
-            if (S.flag < 4)                              // nothing is kept of a solve that went non-finite
-                flush<T, ZC, MODE>(s, n, false, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
-            // the flush uses the whole slab: no neighbour's next planes before every block is done with it
-            // (and no thread still reads the flag)
-            cluster_barrier();
+            finish_job<T, ZC>(nmain);
+            if (S.flag < 4) {                            // nothing is kept of a solve that went non-finite
+                if (scalar)
+                    post_job<T>(Job{s, n, buf, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]}, njobs);
+                buf ^= 1;                                // free again: its last job ended before this one was posted
+            }
+            main_sync(nmain);                            // no thread still reads the flag
         }
         if (scalar && G.rank == 0) end_state(A, s);
     }
+    // nothing is left to go on with: the last job by all warps, once its coefficients are there
+    if (scalar)
+        for (int i = 0; i < 1 << 20 && *(volatile unsigned *)&S.opened != njobs; ++i) {}
+    main_sync(nmain);
+    finish_job<T, ZC>(nmain);
+    if (scalar) post_job<T>(Job{-1, 0, 0, 0, 0.0, 0.0}, njobs);
     cluster_barrier();                                  // no block leaves while another may write its memory
 }
 
@@ -1109,20 +1206,7 @@ __device__ __noinline__ void stream_flush(const StreamArgs *args, int s, int n, 
     float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)ncl) * A.L.ws_stride;
     float *const Pd = U + 2 * A.nv, *const H = Pd + 2 * A.nv;
     if ((int)threadIdx.x == (int)blockDim.x - 32) {
-        double yr = 0, yi = 0, qr = 0, qi = 0;
-        for (int j = n - 1; j >= 0; --j) {
-            const double cn = j + 1 < n ? (double)(float)S.g[j + 1] : 0.0, dr = S.dr[j], di = S.di[j];
-            const double tr = S.zr[j] - cn * yr, ti = S.zi[j] - cn * yi;
-            yr = tr * dr - ti * di;
-            yi = tr * di + ti * dr;
-            const double ur = j == n - 1 ? 1.0 : -cn * qr, ui = j == n - 1 ? 0.0 : -cn * qi;
-            qr = ur * dr - ui * di;
-            qi = ur * di + ui * dr;
-            S.coef[j] = make_float4((float)(er * yr - ei * yi), (float)(er * yi + ei * yr), (float)qr, (float)qi);
-        }
-        const double c0 = (double)(float)S.g[0];
-        S.prev = make_float4((float)(-c0 * (er * yr - ei * yi)), (float)(-c0 * (er * yi + ei * yr)), (float)(-c0 * qr),
-                             (float)(-c0 * qi));
+        coefficients<float>(0, n, er, ei);
     }
     __syncthreads();
     if (G.own) {
@@ -1241,17 +1325,17 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
             if (tid == 0) it = atomicAdd(A.L.grab, 1);
             it = __shfl_sync((1u << ncl) - 1u, it, 0);
             asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
-                             map_rank((unsigned)__cvta_generic_to_shared(&S.item), tid)),
+                             map_rank((unsigned)__cvta_generic_to_shared(&S.item[0]), tid)),
                          "r"(it)
                          : "memory");
         }
         cluster_barrier();
-        if (S.item >= n_items) break;
-        const int s = A.L.list[n_items - 1 - S.item];
+        if (S.item[0] >= n_items) break;
+        const int s = A.L.list[n_items - 1 - S.item[0]];
         {
             float rr, ii, ri;
             stream_start(&A, s, 0.f, 0.f, false, rr, ii, ri);
-            gather3(rr, ii, ri, ng, ncl, G.rank, A.L.err);
+            gather3(rr, ii, ri, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
             if (scalar) {
                 float a, b, c;
                 sum_parts(ng, ncl, a, b, c);
@@ -1416,7 +1500,7 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
                     if (f + 1 < nz + kRadius) step(f + 1, slot + 1, fu[1], fv[1]);
                 }
                 // (also: every ring reader of the sweep is done)
-                gather3(svv, suv, suu, ng, ncl, G.rank, A.L.err);
+                gather3(svv, suv, suu, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
                 {
                     float a, b, c;
                     sum_parts(ng, ncl, a, b, c);
@@ -1430,7 +1514,7 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
                     S.F.ak = S.F.d0 - (double)dg + (double)ap;
                     S.F.ck = (double)cc;
                     S.F.ig = (double)ig;
-                    factor<float>(k - 1 - kb, k, A.L.maxit);
+                    factor<float>(0, k - 1 - kb, k, A.L.maxit);
                     if (A.L.prof && G.rank == 0) atomicAdd(A.L.prof + 1, (unsigned long long)A.L.nd);
                 }
                 cc = ig > 0.f ? 1.f / ig : 0.f;
@@ -1457,7 +1541,7 @@ struct Variant {
     int zc, max_threads;
 };
 constexpr Variant kVar32[3] = {{3, 640}, {4, 640}, {5, 512}};
-constexpr Variant kVar64[2] = {{2, 640}, {4, 512}};
+constexpr Variant kVar64[3] = {{2, 640}, {4, 640}, {8, 384}};
 
 using Fn32 = void (*)(LanczosArgs<float>, Coef<float>);
 using Fn64 = void (*)(LanczosArgs<double>, Coef<double>);
@@ -1465,8 +1549,9 @@ using Fn64 = void (*)(LanczosArgs<double>, Coef<double>);
 const Fn32 kFn32[3][2] = {{k_lanczos<float, 3, 640, 0>, k_lanczos<float, 3, 640, 1>},
                           {k_lanczos<float, 4, 640, 0>, k_lanczos<float, 4, 640, 1>},
                           {k_lanczos<float, 5, 512, 0>, k_lanczos<float, 5, 512, 1>}};
-const Fn64 kFn64[2][2] = {{k_lanczos<double, 2, 640, 2>, k_lanczos<double, 2, 640, 1>},
-                          {k_lanczos<double, 4, 512, 2>, k_lanczos<double, 4, 512, 1>}};
+const Fn64 kFn64[3][2] = {{k_lanczos<double, 2, 640, 2>, k_lanczos<double, 2, 640, 1>},
+                          {k_lanczos<double, 4, 640, 2>, k_lanczos<double, 4, 640, 1>},
+                          {k_lanczos<double, 8, 384, 2>, k_lanczos<double, 8, 384, 1>}};
 
 const void *kernel_of(bool mixed, int v, bool per) {
     return mixed ? (const void *)kFn32[v][per] : (const void *)kFn64[v][per];
@@ -1552,7 +1637,7 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
     // FP32, zero values outside the box: planes follow each other with kRadius rows of zeros in between
     const int zrows = c.opt.periodic || !mixed ? 0 : kRadius;
     const int pitch = p16 * W, plane = pitch * (c.ny + zrows), lead = std::max(W, pitch * zrows);
-    const int nvar = mixed ? 3 : 2;
+    const int nvar = 3;
     double best_cost = 1e300;
     bool found = false;
     for (int v = 0; v < nvar; ++v) {
@@ -1564,7 +1649,7 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
             if (ncl > c.nz) break;
             const int nzl = (c.nz + ncl - 1) / ncl, nch = (nzl + var.zc - 1) / var.zc;
             const long long units = (long long)hw * hh * nch;
-            const int threads = (int)std::min<long long>((units + 31) / 32 * 32 + 32, 1 << 20);
+            const int threads = (int)std::min<long long>((units + 31) / 32 * 32 + kExtra, 1 << 20);
             if (threads > var.max_threads) continue;
             const size_t elems = (size_t)lead + (size_t)plane * (nch * var.zc + 2 * kRadius) + 2 * pad;
             const size_t smem = (elems * tsz + 15) / 16 * 16 + (mixed ? shared_bytes<float>() : shared_bytes<double>());
@@ -1580,7 +1665,7 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
                 continue;
             }
             // cycles per iteration of the blocks sharing an SM, and the rounds the systems take
-            const double pts = (double)(threads - 32) * 2 * W * var.zc;
+            const double pts = (double)(threads - kExtra) * 2 * W * var.zc;
             // (a batch's other contexts run beside this one)
             const int used = std::min(ncs, nsys), all = std::max(nsys, c.batch_load), busy = std::min(ncs, all);
             const double share = std::max(1.0, (double)busy * ncl / sms);
@@ -1610,11 +1695,11 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
     }
     if (!found) return stream_plan(c, nsys, sms, optin, best);
     best.stream = 0;
-    const size_t vec = (size_t)2 * best.zc * (best.threads - 32) * W, hvec = (size_t)best.nch * best.zc * best.plane;
-    // history: as many vectors as 2 GB hold, 16 .. kHistMax
+    const size_t vec = (size_t)2 * best.zc * (best.threads - kExtra) * W, hvec = (size_t)best.nch * best.zc * best.plane;
+    // history: as many vectors as 2 GB hold in each of its two buffers, 16 .. kHistMax
     const size_t per_vec = hvec * tsz * best.clusters * best.ncl;
     best.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, ((size_t)2 << 30) / per_vec));
-    best.ws_stride = 3 * vec + hvec * best.hist;
+    best.ws_stride = vec + 2 * hvec + 2 * hvec * best.hist;
     best.ws_bytes = best.ws_stride * tsz * best.clusters * best.ncl;
     return true;
 }
@@ -1637,8 +1722,6 @@ template <typename T> static void fill_args(const Ctx &c, const LanczosPlan &p, 
     a.pitch = p.pitch;
     a.plane = p.plane;
     a.lead = p.lead;
-    a.nzl_max = (c.nz + p.ncl - 1) / p.ncl;
-    a.stages = p.stream ? 0 : std::min(kStages, (p.nch * p.zc + 2 * kRadius) / a.nzl_max);
     a.err = c.d_tc_err;
     a.reach = p.reach;
     a.hist = p.hist;

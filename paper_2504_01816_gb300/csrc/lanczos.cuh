@@ -20,7 +20,7 @@ template <typename T> struct LanczosArgs {
     int nx, ny, nz;
     double tol, inner_tol;
     int maxit, mixed;
-    int ncl, hw, hh, nch, pitch, plane, lead, reach, hist, nzl_max, stages, smem_words;
+    int ncl, hw, hh, nch, pitch, plane, lead, reach, hist, smem_words;
     int *err;                      // set on a timed-out wait
     double d0;                     // 3 a_0
 };

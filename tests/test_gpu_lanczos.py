@@ -81,6 +81,30 @@ def test_lanczos_past_its_history(rpa, project):
     assert np.all(np.abs(it - rit) <= np.maximum(3, 0.1 * rit)), (it, rit)
 
 
+@pytest.mark.parametrize("prec,grid,nsys", [
+    ("mixed", (20, 17, 16), 700),   # several solves a cluster, short: the solution warps keep up
+    ("mixed", (33, 31, 30), 160),   # large blocks: the other warps take part in what they leave
+    ("fp64", (17, 15, 16), 320),
+])
+def test_lanczos_solutions_formed_beside_the_next_solve(rpa, prec, grid, nsys):
+    """Every solution of a queue is its own system's, and the same whichever warps formed its points."""
+    s = synth.small_system(grid, h=0.5, n_s=2, n_wells=2, seed=29)
+    g = oracle.Grid(s.nx, s.ny, s.nz, s.h)
+    b = np.random.default_rng(9).standard_normal((nsys, s.n_d))
+    orbs = np.arange(nsys) % s.n_s
+    o = rpa.default_options()
+    o.tol, o.prec = 1e-10, rpa.RPA_MIXED if prec == "mixed" else rpa.RPA_FP64
+    with rpa.Context.from_system(s, o) as ctx:
+        bt = torch.as_tensor(b, device="cuda")
+        runs = [ctx.sternheimer_solve(0.4, orbs, bt, project=False) for _ in range(3)]
+        xs = [r[0].cpu().numpy() for r in runs]
+    assert all(r[3] == rpa.RPA_OK for r in runs)
+    assert np.array_equal(xs[0], xs[1]) and np.array_equal(xs[0], xs[2])
+    for i in range(nsys):
+        r = b[i] - oracle.apply_h(g, s.vloc, xs[0][i], -s.eps[orbs[i]] + 0.4j)
+        assert np.linalg.norm(r) <= 1.5 * 1e-10 * np.linalg.norm(b[i]), i
+
+
 @pytest.mark.parametrize("grid,nsys", [
     ((57, 61, 10), 3),              # rows of 14 units and one point, odd rows, bands of unequal height
     ((90, 90, 8), 2),               # wide planes: several bands, the fewest planes the kernel takes
