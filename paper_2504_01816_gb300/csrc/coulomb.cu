@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -115,6 +116,116 @@ __global__ void __launch_bounds__(256) k_axis(const double *__restrict__ in, dou
     }
 }
 
+// The same transform for eigenvectors that are symmetric or antisymmetric about the middle of the line, as
+// those of a symmetric Toeplitz matrix are: with s_i = x_i + x_{n-1-i} and d_i = x_i - x_{n-1-i} (i < h)
+// a symmetric component takes only the s_i and an antisymmetric one only the d_i, and back: half the
+// multiply-adds of the n x n product.  The FP64 pipe bounds it (two multiply-adds a clock and SM).  One
+// thread takes one symmetric and one antisymmetric sum of a line (two chains), a warp 32 lines, so that
+// the matrix is read by broadcast.  40^3, 64 columns, a pass: 341 -> 200 us (140 at the pipe's rate).
+__global__ void __launch_bounds__(256) k_axis_par(const double *__restrict__ in, double *__restrict__ out,
+                                                  const double *__restrict__ Qp, int n, long long inner,
+                                                  long long outer, int forward, const double *__restrict__ scale,
+                                                  long long nd) {
+    extern __shared__ double sh[];
+    const int h = (n + 1) / 2;
+    double *Ms = sh;                 // h x h, Ms[r * h + c]: result r from term c, symmetric; then antisymmetric
+    double *X = Ms + 2 * h * h;      // h x 33 of s (or symmetric components), then of d
+    double *Y = X + 2 * h * 33;      // inner == 1: results, n x 33
+    int *idx = reinterpret_cast<int *>(Y + (inner == 1 ? n * 33 : 0));   // eigenvectors: symmetric, antisymmetric
+    for (int e = threadIdx.x; e < 2 * h * h; e += blockDim.x) {
+        const int p = e / (h * h), r = (e - p * h * h) / h, c = e - p * h * h - r * h;
+        Ms[e] = Qp[(size_t)p * h * h + (forward ? r * h + c : c * h + r)];
+    }
+    for (int e = threadIdx.x; e < 2 * h; e += blockDim.x) idx[e] = reinterpret_cast<const int *>(Qp + 2 * h * h)[e];
+    long long o0, i0;
+    int wcount;
+    if (inner > 1) {
+        const long long tiles = (inner + 31) / 32;
+        o0 = blockIdx.x / tiles;
+        i0 = (blockIdx.x % tiles) * 32;
+        wcount = (int)min(32LL, inner - i0);
+    } else {
+        o0 = (long long)blockIdx.x * 32;
+        i0 = 0;
+        wcount = (int)min(32LL, outer - o0);
+    }
+    // element b of line w
+    auto addr = [&](int b, int w) { return inner > 1 ? (o0 * n + b) * inner + i0 + w : (o0 + w) * n + b; };
+    __syncthreads();                 // idx
+    for (int e = threadIdx.x; e < h * 32; e += blockDim.x) {
+        int i, w;
+        if (inner > 1) { i = e / 32; w = e % 32; }
+        else { w = e / h; i = e % h; }
+        double s = 0.0, d = 0.0;
+        if (w < wcount) {
+            const int b0 = forward ? i : idx[i], b1 = forward ? n - 1 - i : idx[h + i];   // -1: no such component
+            const double v0 = in[addr(b0, w)], v1 = b1 >= 0 ? in[addr(b1, w)] : 0.0;
+            s = !forward || b0 == b1 ? v0 : v0 + v1;
+            d = !forward ? v1 : b0 == b1 ? 0.0 : v0 - v1;
+        }
+        X[i * 33 + w] = s;
+        X[(h + i) * 33 + w] = d;
+    }
+    __syncthreads();
+    const int w = threadIdx.x & 31;
+    for (int r = threadIdx.x >> 5; r < h; r += (int)blockDim.x >> 5) {
+        const double *ms = Ms + r * h, *ma = ms + h * h, *xs = X + w, *xd = xs + h * 33;
+        double s = 0.0, d = 0.0;
+        for (int c = 0; c < h; ++c) {
+            s += ms[c] * xs[c * 33];
+            d += ma[c] * xd[c * 33];
+        }
+        if (w >= wcount) continue;
+        const int b0 = forward ? idx[r] : r, b1 = forward ? idx[h + r] : n - 1 - r;
+        const double v0 = forward ? s : s + d, v1 = forward ? d : s - d;
+        if (inner == 1) {
+            Y[b0 * 33 + w] = v0;
+            if (b1 >= 0 && b1 != b0) Y[b1 * 33 + w] = v1;
+            continue;
+        }
+        const long long a0 = addr(b0, w);
+        out[a0] = scale ? v0 * scale[a0 % nd] : v0;
+        if (b1 >= 0 && b1 != b0) {
+            const long long a1 = addr(b1, w);
+            out[a1] = scale ? v1 * scale[a1 % nd] : v1;
+        }
+    }
+    if (inner > 1) return;
+    __syncthreads();
+    for (int e = threadIdx.x; e < n * wcount; e += blockDim.x) {
+        const int l = e / n, b = e - l * n;
+        const long long a = addr(b, l);
+        out[a] = scale ? Y[b * 33 + l] * scale[a % nd] : Y[b * 33 + l];
+    }
+}
+
+// The eigenvectors by parity for k_axis_par (empty: one has no parity, as within the degenerate pairs of a
+// periodic axis).
+std::vector<double> by_parity(const std::vector<double> &Q, int n) {
+    const int h = (n + 1) / 2;
+    std::vector<double> F((size_t)2 * h * h + h, 0.0);
+    std::vector<int> idx(2 * (size_t)h, -1);
+    int cnt[2] = {0, 0};
+    for (int a = 0; a < n; ++a) {
+        double even = 0.0, odd = 0.0;
+        for (int i = 0; i < n; ++i) {
+            const double u = Q[(size_t)i * n + a], v = Q[(size_t)(n - 1 - i) * n + a];
+            even += 0.25 * (u + v) * (u + v);
+            odd += 0.25 * (u - v) * (u - v);
+        }
+        const int p = even < odd;
+        if (std::min(even, odd) > 1e-22 || cnt[p] >= (p ? n - h : h)) return {};
+        const int j = cnt[p]++;
+        idx[(size_t)p * h + j] = a;
+        for (int i = 0; i < h; ++i) {
+            const double u = Q[(size_t)i * n + a], v = Q[(size_t)(n - 1 - i) * n + a];
+            F[((size_t)p * h + j) * h + i] = 0.5 * (p ? u - v : u + v);
+        }
+    }
+    std::memcpy(F.data() + (size_t)2 * h * h, idx.data(), sizeof(int) * idx.size());
+    return F;
+}
+
 // Pointwise factor (4 pi / lam)^power of nu^power in the eigenbasis; lam = 0 only for the G = 0
 // mode of a periodic grid, which nu^power maps to zero.
 __global__ void k_scale_grid(const double *__restrict__ lam, double *__restrict__ sc, long long nd, double power) {
@@ -159,6 +270,11 @@ void coulomb_setup(Ctx &c) {
         }
         RPA_CUDA(cudaMalloc(&c.Q[a], sizeof(double) * n * n));
         RPA_CUDA(cudaMemcpy(c.Q[a], Q.data(), sizeof(double) * n * n, cudaMemcpyHostToDevice));
+        const std::vector<double> qp = by_parity(Q, n);
+        if (!qp.empty()) {
+            RPA_CUDA(cudaMalloc(&c.Qpar[a], sizeof(double) * qp.size()));
+            RPA_CUDA(cudaMemcpy(c.Qpar[a], qp.data(), sizeof(double) * qp.size(), cudaMemcpyHostToDevice));
+        }
         // the same factors for the Laplacian preconditioner of COCG, in FP64 and FP32
         std::vector<float> qf(Q.begin(), Q.end()), mf(mu[a].begin(), mu[a].end());
         RPA_CUDA(cudaMalloc(&c.mu[a], sizeof(double) * n));
@@ -185,6 +301,14 @@ static void axis_pass(Ctx &c, int axis, const double *in, double *out, int ncols
     const size_t sh = sizeof(double) * ((size_t)n * n + (size_t)n * 33);
     allow_dynamic_smem((const void *)k_axis, sh);   // rejects grid dimensions above ~150
     const long long blocks = inner > 1 ? outer * ((inner + 31) / 32) : (outer + 31) / 32;
+    if (c.Qpar[axis]) {
+        const int h = (n + 1) / 2;
+        const size_t shp = sizeof(double) * ((size_t)2 * h * h + (size_t)2 * h * 33 + (inner == 1 ? (size_t)n * 33 : 0) + h);
+        allow_dynamic_smem((const void *)k_axis_par, shp);
+        k_axis_par<<<(unsigned)blocks, 256, shp, s>>>(in, out, c.Qpar[axis], n, inner, outer, forward, scale, c.nd);
+        RPA_LAUNCH("coulomb axis transform by parity");
+        return;
+    }
     k_axis<<<(unsigned)blocks, 256, sh, s>>>(in, out, c.Q[axis], n, inner, outer, forward, scale, c.nd);
     RPA_LAUNCH("coulomb axis transform");
 }
