@@ -2786,15 +2786,6 @@ __global__ void k_init_slots(Slot *slots, int S) {
     slots[s] = z;
 }
 
-// rows[j] = u_n (.) dv_j for j < ncols (right-hand sides before projection, for one orbital).
-__global__ void k_pair_rows(const double *__restrict__ psi, const double *__restrict__ dv, int n, long long nd,
-                            double *__restrict__ rows) {
-    const int j = blockIdx.y;
-    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < nd;
-         idx += (long long)gridDim.x * blockDim.x)
-        rows[(long long)j * nd + idx] = psi[(long long)n * nd + idx] * dv[(long long)j * nd + idx];
-}
-
 // (n, j) of the pair systems q = n * ncols + j (chi0 and the adjoint's response).
 __global__ void k_pair_index(int *__restrict__ sys_n, int *__restrict__ sys_j, int nsys, int ncols) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -3640,14 +3631,7 @@ static double *pair_coefficients(Ctx &c, const double *dv, int ncols, cudaStream
         tc_gemm_pairs(c.psi64, c.ns, dv, ncols, c.psi64, c.ns, c.nd, T, s, c.dense_scratch, c.d_tc_err);
         return T;
     }
-    double *rows = (double *)c.rhs.ensure(sizeof(double) * (size_t)ncols * c.nd);
-    for (int n = 0; n < c.ns; ++n) {
-        k_pair_rows<<<dim3(std::min<unsigned>(cdiv(c.nd, 256), 1024u), ncols), 256, 0, s>>>(c.psi64, dv, n, c.nd,
-                                                                                             rows);
-        RPA_LAUNCH("pair rows");
-        count_launches(1);
-        pc_coefficients(c, rows, ncols, T + (size_t)n * ncols * c.ns, s);
-    }
+    gram_pairs(c.psi64, c.ns, dv, ncols, c.nd, T, s, c.dense_scratch);
     return T;
 }
 

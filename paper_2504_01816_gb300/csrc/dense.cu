@@ -65,6 +65,80 @@ __global__ void k_sum_splits(const double *__restrict__ part, int splits, long l
     }
 }
 
+// part[z][p][j] = sum_{r in chunk z} u_n[r] u_k[r] dv_j[r] for the orbital pairs p = (n, k), k <= n: one
+// contraction for all of them, the products of a pair formed as they are loaded.  Tiles and inner loop as
+// k_gram, the chunk as short as it takes to fill the GPU: with a contraction of at least 512 points for
+// each orbital, 15^3 with 4 orbitals ran 6 blocks at a time, 4 x 164 us; in one launch 9 us.
+__global__ void __launch_bounds__(256) k_gram_pairs(const double *__restrict__ psi, int npair,
+                                                    const double *__restrict__ dv, int ncols, long long len,
+                                                    long long chunk, double *__restrict__ part) {
+    __shared__ double sa[kKc][kTile + 1];
+    __shared__ double sb[kKc][kTile + 1];
+    __shared__ int pn[kTile], pk[kTile];
+    const int p0 = blockIdx.x * kTile, j0 = blockIdx.y * kTile;
+    const long long r0 = (long long)blockIdx.z * chunk;
+    const long long r1 = min(len, r0 + chunk);
+    if (threadIdx.x < kTile) {
+        const int p = min(p0 + (int)threadIdx.x, npair - 1);
+        int n = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);   // n (n + 1) / 2 <= p, to rounding
+        while (n * (n + 1) / 2 > p) --n;
+        while ((n + 1) * (n + 2) / 2 <= p) ++n;
+        pn[threadIdx.x] = n;
+        pk[threadIdx.x] = p - n * (n + 1) / 2;
+    }
+    __syncthreads();
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    double acc[2][2] = {{0, 0}, {0, 0}};
+    for (long long rb = r0; rb < r1; rb += kKc) {
+        for (int e = threadIdx.x; e < kTile * kKc; e += 256) {
+            const int row = e / kKc, kk = e % kKc;
+            const long long r = rb + kk;
+            sa[kk][row] = (p0 + row < npair && r < r1) ? psi[pn[row] * len + r] * psi[pk[row] * len + r] : 0.0;
+            sb[kk][row] = (j0 + row < ncols && r < r1) ? dv[(long long)(j0 + row) * len + r] : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int kk = 0; kk < kKc; ++kk) {
+            const double x0 = sa[kk][ty], x1 = sa[kk][ty + 16];
+            const double y0 = sb[kk][tx], y1 = sb[kk][tx + 16];
+            acc[0][0] += x0 * y0;
+            acc[0][1] += x0 * y1;
+            acc[1][0] += x1 * y0;
+            acc[1][1] += x1 * y1;
+        }
+        __syncthreads();
+    }
+    double *out = part + (long long)blockIdx.z * npair * ncols;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int p = p0 + ty + 16 * u, j = j0 + tx + 16 * v;
+            if (p < npair && j < ncols) out[(long long)p * ncols + j] = acc[u][v];
+        }
+}
+
+// T[(n, j)][k] = T[(k, j)][n] = sum of the chunks, one warp a value.
+__global__ void __launch_bounds__(256) k_sum_pairs(const double *__restrict__ part, int splits, int ns, int ncols,
+                                                   double *__restrict__ T) {
+    const int npair = ns * (ns + 1) / 2, lane = threadIdx.x & 31;
+    const long long total = (long long)npair * ncols;
+    for (long long e = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < total; e += ((long long)gridDim.x * blockDim.x) >> 5) {
+        double s = 0.0;
+        for (int z = lane; z < splits; z += 32) s += part[z * total + e];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane) continue;
+        const int p = (int)(e / ncols), j = (int)(e - (long long)p * ncols);
+        int n = (int)((sqrtf(8.f * (float)p + 1.f) - 1.f) * 0.5f);
+        while (n * (n + 1) / 2 > p) --n;
+        while ((n + 1) * (n + 2) / 2 <= p) ++n;
+        const int k = p - n * (n + 1) / 2;
+        T[((long long)n * ncols + j) * ns + k] = s;
+        T[((long long)k * ncols + j) * ns + n] = s;
+    }
+}
+
 // Y[c][r] = sum_k S[c][k] X[k][r]; blockIdx.y picks 16 output rows.
 __global__ void __launch_bounds__(256) k_combine(const double *__restrict__ S, int nc, int nk,
                                                  const double *__restrict__ X, long long len, double *__restrict__ Y) {
@@ -564,6 +638,20 @@ void gram(const double *A, int na, const double *B, int nb, long long len, doubl
     const long long n = (long long)na * nb;
     k_sum_splits<<<std::min<unsigned>(cdiv(n, 256), 4096u), 256, 0, s>>>(part, (int)splits, n, G);
     RPA_LAUNCH("gram");
+    count_launches(2);
+}
+
+void gram_pairs(const double *psi, int ns, const double *dv, int ncols, long long len, double *T, cudaStream_t s,
+                DevBuf &scratch) {
+    const int npair = ns * (ns + 1) / 2, tp = cdiv(npair, kTile), tj = cdiv(ncols, kTile);
+    long long splits = std::max(1LL, std::min<long long>(len / kKc, 1200 / std::max(1, tp * tj)));
+    const long long chunk = ((len + splits - 1) / splits + kKc - 1) / kKc * kKc;
+    splits = (len + chunk - 1) / chunk;
+    double *part = (double *)scratch.ensure(sizeof(double) * (size_t)splits * npair * ncols);
+    k_gram_pairs<<<dim3(tp, tj, (unsigned)splits), 256, 0, s>>>(psi, npair, dv, ncols, len, chunk, part);
+    RPA_LAUNCH("gram of the pairs");
+    k_sum_pairs<<<std::min<unsigned>(cdiv((long long)npair * ncols, 8), 4096u), 256, 0, s>>>(part, (int)splits, ns, ncols, T);
+    RPA_LAUNCH("gram of the pairs, sums");
     count_launches(2);
 }
 

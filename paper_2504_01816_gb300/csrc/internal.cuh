@@ -269,6 +269,9 @@ int sternheimer_batch_projected(Ctx &c, double omega, const int *orb, int nsys, 
 // G (na x nb, row-major) = A B^T with A: na rows of length len, B: nb rows of length len.
 void gram(const double *A, int na, const double *B, int nb, long long len, double *G, cudaStream_t s,
           DevBuf &scratch);
+// T[(n, j)][k] = sum_r u_k[r] u_n[r] dv_j[r], row n ncols + j of ns values.
+void gram_pairs(const double *psi, int ns, const double *dv, int ncols, long long len, double *T, cudaStream_t s,
+                DevBuf &scratch);
 // Y (nc rows) = S X, S: nc x nk row-major (device), X: nk rows of length len.
 void combine_rows(const double *S, int nc, int nk, const double *X, long long len, double *Y,
                   cudaStream_t s);
