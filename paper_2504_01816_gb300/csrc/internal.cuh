@@ -90,7 +90,7 @@ struct LanczosPlan {
     int hw, hh, nch;               // units per row, row pairs, z chunks of a block
     int pitch, plane, lead;        // elements of a slab row and plane, and before the first plane
     int reach, hist;
-    int stream, bh, hp;            // the streaming kernel: rows of a band, halo row pairs
+    int stream, bh, depth, unit_rows;   // the streaming kernel: rows of a band, planes in flight, rows a thread
     size_t smem, ws_stride, ws_bytes;
     void *ws;                      // ws_bytes of workspace, set by the caller
 };

@@ -238,8 +238,14 @@ template <typename T> struct Shared {
     double dr[2][kHistMax], di[2][kHistMax], zr[2][kHistMax], zi[2][kHistMax], g[2][kHistMax];   // factors by history place
     double start[4];                     // cos phi, sin phi, ||r_a||, ||r_b||
     ScalarState F;
-    unsigned long long bar, pbar[2], ibar[2];   // arrival of the halo, of the sums, of the next system
-    unsigned long long job_full, job_done;      // a job for the flush warps, and its end
+    unsigned long long bar, pbar[2];     // arrival of the halo, of the sums
+    union {
+        struct {
+            unsigned long long ibar[2];              // arrival of the next system
+            unsigned long long job_full, job_done;   // a job for the flush warps, and its end
+        };
+        unsigned long long full[4];      // streaming kernel: arrival of a stage's planes
+    };
     Job job;
     int next;                            // its first place that no warp has taken
     unsigned opened;                     // jobs whose coefficients are there
@@ -1146,25 +1152,33 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
 
 // ---------------------------------------------------------------------------------------------
 // The same solve for grids that do not fit on chip (mixed form, zero values outside the box): u and the
-// vectors stay in memory and a cluster of C blocks marches along z, block c over a band of rows, with 14
-// planes of its band and six rows on either side in a shared-memory ring.  One sweep is one Lanczos step:
-// at step f a thread forms v_k = (u - a' v_{k-1}) / g of plane f from the last sweep's u and v_{k-1} (its
-// band's halo rows too: they are formed by every block that reads them, so that bands exchange nothing
-// within a sweep), stores it in the ring and as vector k of the history, and after one barrier
-// applies the stencil to plane f - 6, writing u = B v_k - c v_{k-1} in place.  v_{k-1} is vector k - 1 of
-// the history, so the history costs no traffic of its own: a point takes 16 bytes an iteration (u and
-// v_{k-1} in, u and v_k out; v_{k-1}, read again six planes later, and V_loc come from L2) and 4 at the
-// end, against 64 of the fused COCG kernel on complex vectors.
+// vectors stay in memory and a cluster of C blocks marches along z, block c over a band of rows.  One
+// sweep is one Lanczos step: at step f a thread (4 x 1 or 4 x 2 points) forms v_k = (u - a' v_{k-1}) / g of plane f
+// from the last sweep's u and v_{k-1}, stores it in a plane in shared memory and as vector k of the history,
+// and after one barrier applies the x and y neighbours and the diagonal of the stencil.  Along z its values go
+// into sums for the planes f-6 .. f+6, which it holds in registers and shifts as it adds (a multiply-add
+// writes where the last one read), and plane f-6 of u = B v_k - c v_{k-1} is complete.  u.v is summed with
+// the sums that plane f has received so far, twice (B is symmetric).  The six halo rows on either side of
+// a band are formed by every block that reads them, so that bands exchange nothing within a sweep.  u and v_{k-1}
+// of the planes ahead, and V_loc, arrive by bulk copies, A.depth planes in flight.  v_{k-1} is vector
+// k - 1 of the history, so the history costs no traffic of its own: a point takes 16 bytes an iteration (u
+// and v_{k-1} in, u and v_k out) and 4 at the end, when the history comes back through the same stages,
+// against 64 of the fused COCG kernel on complex vectors.
 //
-// What bounds it: memory bandwidth, then shared memory (46 16-byte loads per unit of 4 x 2 points).
+// What bounds it: the latency of a plane's step (loads from a stage, one barrier, 16 to 20 loads of neighbours, a
+// hundred dependent multiply-adds) with the 7 to 14 warps that the sums' registers allow, and memory
+// bandwidth above 64^3.  A form that kept 14 planes in a shared-memory ring for the z neighbours took 46
+// shared-memory loads for 8 points against 20, and twice the bands.  Measured, whole chi0 application: 56^3,
+// 256 systems 239 ms with the COCG kernels, 111 with the ring, 83 in this form; 72^3, 256 systems 691, 352, 213.
 // ---------------------------------------------------------------------------------------------
-constexpr int kRing = 14;                // planes f-13 .. f: the slot written at step f+1 was last read at f-1
+constexpr int kStages = 4;               // planes in flight, at most
 
 struct StreamArgs {
-    LanczosArgs<float> L;                // slots, queue, tolerances, workspace; pitch, plane: of the ring
+    LanczosArgs<float> L;                // slots, queue, tolerances, workspace; pitch, plane: in shared memory
     const float *v;                      // V_loc, rows padded to px
-    int bh, hp;                          // rows of a band (even), halo row pairs on either side
+    int bh;                              // rows of a band (even)
     int px;                              // padded row length in memory (a multiple of 4)
+    int depth;                           // planes in flight
     size_t nv;                           // elements of a vector in memory: nz ny px
 };
 
@@ -1177,100 +1191,195 @@ __global__ void k_pad_rows(const float *__restrict__ in, float *__restrict__ out
     }
 }
 
-struct StreamGeo {
-    int rank, gx, gy, nvx;
-    bool front, own, row1;               // forms points; of the block's band; row gy + 1 is one of them
-    int ring, mem;                       // the first point in a ring plane, and in a plane in memory
+// A thread's points of a plane: 4 values of x from gx, R rows from gy.
+template <int R> struct StreamGeo {
+    int rank, y0, rows, gx, gy, nvx;     // the band's first row and rows inside the box; the unit's first point
+    bool own, row1;                      // has points; of R = 2 row gy + 1, too, lies inside the box
+    int mem;                             // the first point in a plane in memory
     __device__ __forceinline__ StreamGeo(const StreamArgs &A) {
-        const int t = threadIdx.x, hw = A.L.hw;
+        const int t = threadIdx.x, hw = A.L.hw, pair = t / hw;
         rank = (int)(blockIdx.x % (unsigned)A.L.ncl);
-        const int y0 = rank * A.bh, y1 = min(A.L.ny, y0 + A.bh), pair = t / hw;
+        y0 = rank * A.bh;
+        rows = min(A.bh, A.L.ny - y0);
         gx = 4 * (t - pair * hw);
-        gy = y0 + 2 * (pair - A.hp);
-        front = pair < A.bh / 2 + 2 * A.hp && gy >= 0 && gy < A.L.ny;
-        own = front && gy >= y0 && gy < y1;
-        row1 = gy + 1 < A.L.ny;
+        gy = y0 + R * pair;
+        own = R * pair < rows;
+        row1 = R == 2 && own && R * pair + 1 < rows;
         nvx = min(4, A.L.nx - gx);
-        ring = (gy - y0 + kRadius) * A.L.pitch + 8 + gx;
-        mem = front ? gy * A.px + gx : 0;
+        mem = own ? gy * A.px + gx : 0;
+    }
+};
+__device__ __forceinline__ void bulk_load(unsigned to, const float *from, int bytes, unsigned bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(to),
+                 "l"(__cvta_generic_to_global(from)), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void expect_bytes(unsigned bar, int bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Values written by the threads, before bulk copies (after a barrier) read them from memory.
+__device__ __forceinline__ void before_bulk() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// The stages: planes in flight, each with its barrier; every thread counts along.
+struct Stages {
+    int st;                              // next stage
+    unsigned ph;                         // bit s: parity of stage s's next arrival
+    bool ok;
+    __device__ __forceinline__ unsigned bar(int s) const {
+        return (unsigned)__cvta_generic_to_shared(&sh<float>().full[0]) + 8u * (unsigned)s;
+    }
+    __device__ __forceinline__ void wait(int *err) {
+        if (ok && !mbar_wait(bar(st), (ph >> st) & 1)) {
+            ok = false;
+            atomicExch(err, 2);
+        }
+    }
+    __device__ __forceinline__ void next(int depth) {
+        ph ^= 1u << st;
+        st = st + 1 == depth ? 0 : st + 1;
     }
 };
 
-// x += sum_j y_j v_j (and the COCG direction) over the n vectors of the history, as flush() does.
-__device__ __noinline__ void stream_flush(const StreamArgs *args, int s, int n, bool go_on, bool have_p, double er, double ei) {
+// x += sum_j y_j v_j over the n vectors of the history (go_on: by plain loads, and the COCG direction; else
+// three planes of the band of one vector a stage).
+template <int R>
+__device__ __noinline__ Stages stream_flush(const StreamArgs *args, int s, int n, bool go_on, bool have_p, double er,
+                                            double ei, Stages G4) {
     using P = Pk<float>;
+    constexpr int NP = 3;                // planes of the band that a stage holds
     Shared<float> &S = sh<float>();
     const StreamArgs &A = *args;
-    const StreamGeo G(A);
+    const StreamGeo<R> G(A);
     const int ncl = A.L.ncl;
+    const bool scalar = (int)threadIdx.x == (int)blockDim.x - 32;
     float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)ncl) * A.L.ws_stride;
     float *const Pd = U + 2 * A.nv, *const H = Pd + 2 * A.nv;
-    if ((int)threadIdx.x == (int)blockDim.x - 32) {
-        coefficients<float>(0, n, er, ei);
-    }
+    float2 *const xg = A.L.x + (long long)s * A.L.nd;
+    if (scalar) coefficients<float>(0, n, er, ei);
     __syncthreads();
-    if (G.own) {
-        float2 *const xg = A.L.x + (long long)s * A.L.nd;
-        for (int z = 0; z < A.L.nz; ++z)
-            for (int r = 0; r < (G.row1 ? 2 : 1); ++r) {
-                const size_t o = (size_t)z * A.L.ny * A.px + G.mem + r * A.px;
-                P xr, xi, pr, pi;
-                xr.zero();
-                xi.zero();
-                pr.zero();
-                pi.zero();
-                if (have_p) {
-                    const float4 c = S.prev;
-                    const P qr = pk_load(Pd + o), qi = pk_load(Pd + A.nv + o);
-                    xr.fma(c.x, qr);
-                    xr.fma(-c.y, qi);
-                    xi.fma(c.x, qi);
-                    xi.fma(c.y, qr);
-                    pr.fma(c.z, qr);
-                    pr.fma(-c.w, qi);
-                    pi.fma(c.z, qi);
-                    pi.fma(c.w, qr);
-                }
-                if (go_on) {
+    auto add_x = [&](int z, int r, P xr, P xi, P pr, P pi) {
+        const size_t o = ((size_t)z * A.L.ny + r) * A.px + G.mem;
+        if (have_p) {
+            const float4 c = S.prev;
+            const P qr = pk_load(Pd + o), qi = pk_load(Pd + A.nv + o);
+            xr.fma(c.x, qr);
+            xr.fma(-c.y, qi);
+            xi.fma(c.x, qi);
+            xi.fma(c.y, qr);
+            pr.fma(c.z, qr);
+            pr.fma(-c.w, qi);
+            pi.fma(c.z, qi);
+            pi.fma(c.w, qr);
+        }
+        if (go_on) {
+            pk_store(Pd + o, pr);
+            pk_store(Pd + A.nv + o, pi);
+        }
+        float2 *dst = xg + ((long long)z * A.L.ny + G.gy + r) * A.L.nx + G.gx;
+        float2 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = i < G.nvx ? dst[i] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < G.nvx) dst[i] = make_float2(q[i].x + xr.get(i), q[i].y + xi.get(i));
+    };
+    if (go_on) {
+        if (G.own)
+            for (int z = 0; z < A.L.nz; ++z)
+                for (int r = 0; r < (G.row1 ? 2 : 1); ++r) {
+                    const float *h = H + ((size_t)z * A.L.ny + r) * A.px + G.mem;
+                    P xr, xi, pr, pi;
+                    xr.zero();
+                    xi.zero();
+                    pr.zero();
+                    pi.zero();
 #pragma unroll 8
                     for (int j = 0; j < n; ++j) {
                         const float4 c = S.coef[j];
-                        const P v = pk_load(H + (size_t)j * A.nv + o);
+                        const P v = pk_load(h + (size_t)j * A.nv);
                         xr.fma(c.x, v);
                         xi.fma(c.y, v);
                         pr.fma(c.z, v);
                         pi.fma(c.w, v);
                     }
-                    pk_store(Pd + o, pr);
-                    pk_store(Pd + A.nv + o, pi);
-                } else {
-#pragma unroll 8
-                    for (int j = 0; j < n; ++j) {
-                        const float4 c = S.coef[j];
-                        const P v = pk_load(H + (size_t)j * A.nv + o);
-                        xr.fma(c.x, v);
-                        xi.fma(c.y, v);
-                    }
+                    add_x(z, r, xr, xi, pr, pi);
                 }
-                float2 *dst = xg + ((long long)z * A.L.ny + G.gy + r) * A.L.nx + G.gx;
+        __syncthreads();
+        return G4;
+    }
+    const size_t pl = (size_t)A.L.ny * A.px;
+    const int band = G.rows * A.px, su = (A.bh + 2 * kRadius) * A.px, stb = (2 * su + A.bh * A.px) * 4;
+    const int s0 = shared_bytes<float>() + (2 * A.L.plane + 16) * 4;
+    const int own_at = s0 + (G.own ? ((G.gy - G.y0) * A.px + G.gx) * 4 : 0), second = G.row1 ? A.px * 4 : 0;
+    const int npair = (A.L.nz + NP - 1) / NP, total = npair * n;
+    // planes NP zi .. of vector j into stage q
+    auto issue = [&](int zi, int j, int q) {
+        const int np = min(NP, A.L.nz - NP * zi);
+        expect_bytes(G4.bar(q), np * band * 4);
+        for (int m = 0; m < np; ++m)
+            bulk_load((unsigned)__cvta_generic_to_shared(lz_smem) + (unsigned)(s0 + q * stb + m * band * 4),
+                      H + (size_t)j * A.nv + (size_t)(NP * zi + m) * pl + (size_t)G.y0 * A.px, band * 4, G4.bar(q));
+    };
+    int iz = 0, ij = 0, iq = G4.st;      // the next to issue (the scalar lane's)
+    auto issue_next = [&]() {
+        if (iz >= npair) return;
+        issue(iz, ij, iq);
+        if (++ij == n) {
+            ij = 0;
+            ++iz;
+        }
+        iq = iq + 1 == A.depth ? 0 : iq + 1;
+    };
+    if (scalar) {
+        before_bulk();
+        for (int i = 0; i < min(total, A.depth); ++i) issue_next();
+    }
+    for (int zi = 0; zi < npair; ++zi) {
+        P xr[NP][R], xi[NP][R];
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (i < G.nvx) {
-                        float2 q = dst[i];
-                        q.x += xr.get(i);
-                        q.y += xi.get(i);
-                        dst[i] = q;
-                    }
+        for (int m = 0; m < NP; ++m)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                xr[m][r].zero();
+                xi[m][r].zero();
             }
+        for (int j = 0; j < n; ++j) {
+            G4.wait(A.L.err);
+            const int b = G4.st * stb;
+            P v[NP][R];
+#pragma unroll
+            for (int m = 0; m < NP; ++m)
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[m][r] = lds<float>(own_at + b + m * band * 4 + r * second);
+            const float4 c = S.coef[j];
+#pragma unroll
+            for (int m = 0; m < NP; ++m)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    xr[m][r].fma(c.x, v[m][r]);
+                    xi[m][r].fma(c.y, v[m][r]);
+                }
+            G4.next(A.depth);
+            __syncthreads();             // the stage is read
+            if (scalar) issue_next();
+        }
+        if (G.own)
+#pragma unroll
+            for (int m = 0; m < NP; ++m)
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (NP * zi + m < A.L.nz && (r == 0 || G.row1)) add_x(NP * zi + m, r, xr[m][r], xi[m][r], xr[m][r], xi[m][r]);
     }
     __syncthreads();
+    return G4;
 }
 
 // Sums of the right-hand side (f_re = f_im = 0: into sums) or u = f_re Re(r) + f_im Im(r).
+template <int R>
 __device__ __noinline__ void stream_start(const StreamArgs *args, int s, float f_re, float f_im, bool store, float &rr,
                                           float &ii, float &ri) {
     const StreamArgs &A = *args;
-    const StreamGeo G(A);
+    const StreamGeo<R> G(A);
     float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)A.L.ncl) * A.L.ws_stride;
     const float2 *const rg = A.L.r + (long long)s * A.L.nd;
     float a = 0.f, b = 0.f, c = 0.f;
@@ -1278,7 +1387,7 @@ __device__ __noinline__ void stream_start(const StreamArgs *args, int s, float f
 #pragma unroll 4
         for (int z = 0; z < A.L.nz; ++z)
 #pragma unroll
-            for (int r = 0; r < 2; ++r)
+            for (int r = 0; r < R; ++r)
                 if (r == 0 || G.row1) {
                     const float2 *src = rg + ((long long)z * A.L.ny + G.gy + r) * A.L.nx + G.gx;
                     Pk<float> w;
@@ -1297,27 +1406,52 @@ __device__ __noinline__ void stream_start(const StreamArgs *args, int s, float f
     ri = c;
 }
 
-__global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant__ StreamArgs A, const __grid_constant__ Coef<float> cf) {
+template <int R, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1)
+    k_lanczos_stream(const __grid_constant__ StreamArgs A, const __grid_constant__ Coef<float> cf) {
     using P = Pk<float>;
     Shared<float> &S = sh<float>();
-    const int tid = threadIdx.x, ncl = A.L.ncl, nz = A.L.nz;
-    const StreamGeo G(A);
+    const int tid = threadIdx.x, ncl = A.L.ncl, nz = A.L.nz, depth = A.depth;
+    const StreamGeo<R> G(A);
     const bool scalar = tid == (int)blockDim.x - 32;
-    // byte offsets in shared memory: the unit's rows in ring slot 0; bytes of a ring plane, of a row
-    const int o0 = shared_bytes<float>() + G.ring * 4, pb = A.L.plane * 4, rb = A.L.pitch * 4;
-    const int o1 = G.row1 ? o0 + rb : o0;
-    auto at = [&](int off) -> float * { return reinterpret_cast<float *>(lz_smem + off); };
+    // byte offsets in shared memory: the unit's rows in plane 0; bytes of a plane, of a row; the stages (u with
+    // its halo rows, v_{k-1} likewise, V_loc)
+    const int pb = A.L.plane * 4, rb = A.L.pitch * 4, mb = A.px * 4;
+    const int o0 = shared_bytes<float>() + ((G.gy - G.y0 + kRadius) * A.L.pitch + 8 + G.gx) * 4;
+    const int s0 = shared_bytes<float>() + 2 * pb + 64, su = (A.bh + 2 * kRadius) * mb, stb = 2 * su + A.bh * mb;
+    const int r0 = max(0, G.y0 - kRadius), nrow = min(A.L.ny, G.y0 + A.bh + kRadius) - r0;   // rows staged
+    // the unit's second row, if it lies outside the box: the first again, with factors 0
+    const int uo = G.own ? (G.gy - r0) * mb + G.gx * 4 : 0, vo = 2 * su + (G.own ? (G.gy - G.y0) * mb + G.gx * 4 : 0);
+    const int mb1 = G.row1 ? mb : 0;
+    const float in1 = G.row1 ? 1.f : 0.f;
+    // halo rows: units of one row by all threads that have points
+    const int nhalo = ncl > 1 ? 2 * kRadius * A.L.hw : 0, nthr = A.bh / R * A.L.hw;
+    // unit e: its place in a stage (-1: outside the box) and in plane 0
+    auto halo = [&](int e, int &from, int &to) {
+        const int hr = e / A.L.hw, lr = hr < kRadius ? hr - kRadius : A.bh + hr - kRadius, y = G.y0 + lr;
+        const int x = 4 * (e - hr * A.L.hw);
+        from = e < nhalo && y >= 0 && y < A.L.ny ? (y - r0) * mb + 4 * x : -1;
+        to = shared_bytes<float>() + ((lr + kRadius) * A.L.pitch + 8 + x) * 4;
+    };
+    int h_from = -1, h_to = 0;                           // the thread's first
+    if (tid < nthr) halo(tid, h_from, h_to);
     for (int e = tid; e < A.L.smem_words; e += blockDim.x)
         reinterpret_cast<int4 *>(lz_smem + shared_bytes<float>())[e] = make_int4(0, 0, 0, 0);
     if (scalar) {
         for (int q = 0; q < 2; ++q) mbar_init(&S.pbar[q]);
+        for (int q = 0; q < kStages; ++q) mbar_init(&S.full[q]);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    before_bulk();                                       // the zeros, before bulk copies into the same memory
     float *const U = A.L.ws + (size_t)(blockIdx.x / (unsigned)ncl) * A.L.ws_stride;
     float *const H = U + 4 * A.nv;                       // after u (two buffers) and the direction (re, im)
     const size_t pl = (size_t)A.L.ny * A.px;             // a plane in memory
     const int n_items = *A.L.cnt;
     unsigned ng = 0;
+    Stages G4{0, 0u, true};
+    P mask;                                              // 1 for points inside the box
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mask.set(i, i < G.nvx ? 1.f : 0.f);
     cluster_barrier();
     for (;;) {
         if (G.rank == 0 && tid < ncl) {
@@ -1334,7 +1468,7 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
         const int s = A.L.list[n_items - 1 - S.item[0]];
         {
             float rr, ii, ri;
-            stream_start(&A, s, 0.f, 0.f, false, rr, ii, ri);
+            stream_start<R>(&A, s, 0.f, 0.f, false, rr, ii, ri);
             gather3(rr, ii, ri, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
             if (scalar) {
                 float a, b, c;
@@ -1348,8 +1482,9 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
             if (!start_part<float>(A.L, s, pt, scalar, f_re, f_im)) continue;
             {
                 float d0, d1, d2;
-                stream_start(&A, s, f_re, f_im, true, d0, d1, d2);
+                stream_start<R>(&A, s, f_re, f_im, true, d0, d1, d2);
             }
+            before_bulk();
             cluster_barrier();                           // u is stored in every band
             float ap = 0.f, ig = 1.f, cc = 0.f, dg = (float)S.F.d0;   // the first sweep: v_0 = u
             int k = 0, kb = 0, n = 0;
@@ -1357,150 +1492,132 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
             for (;;) {
                 // u alternates between two buffers: a band may be planes ahead of one that reads its rows
                 const float *const ui = U + (size_t)(k & 1) * A.nv;
-                float *const uo = U + (size_t)((k & 1) ^ 1) * A.nv;
+                float *const uout = U + (size_t)((k & 1) ^ 1) * A.nv + G.mem;
                 const float *const vp = k == 0 ? U : H + (size_t)(k == kb ? A.L.hist - 1 : k - 1 - kb) * A.nv;
-                float *const vk = H + (size_t)(k - kb) * A.nv;
-                const float m_ag = -ap * ig;
-                float svv = 0.f, suv = 0.f, suu = 0.f;
-                P zero;
-                zero.zero();
-                // ring planes -6 .. -1 (slots 8 .. 13) are zero
-                if (G.front)
-                    for (int m = kRing - kRadius; m < kRing; ++m) {
-                        pk_store(at(o0 + m * pb), zero);
-                        if (G.row1) pk_store(at(o1 + m * pb), zero);
-                    }
-                // u and v_{k-1} of the next two front planes; v_{k-1} and V_loc of the next stencil plane
-                P fu[2][2], fv[2][2], nlv[2], nvv[2];
-                const float *pu = ui + G.mem, *pv = vp + G.mem;
-                auto load_front = [&](int f, P (&u)[2], P (&v)[2]) {
-                    const size_t o = f * pl;
-                    u[0] = pk_load_l2(pu + o);
-                    v[0] = pk_load_l2(pv + o);
-                    if (G.row1) {
-                        u[1] = pk_load_l2(pu + o + A.px);
-                        v[1] = pk_load_l2(pv + o + A.px);
-                    }
+                float *const vk = H + (size_t)(k - kb) * A.nv + G.mem;
+                auto issue = [&](int f, int q) {
+                    const unsigned to = (unsigned)__cvta_generic_to_shared(lz_smem) + (unsigned)(s0 + q * stb);
+                    const size_t o = f * pl + (size_t)r0 * A.px;
+                    expect_bytes(G4.bar(q), 2 * nrow * mb + G.rows * mb);
+                    bulk_load(to, ui + o, nrow * mb, G4.bar(q));
+                    bulk_load(to + su, vp + o, nrow * mb, G4.bar(q));
+                    bulk_load(to + 2 * su, A.v + f * pl + (size_t)G.y0 * A.px, G.rows * mb, G4.bar(q));
                 };
-                auto load_centre = [&](int z) {
-                    const size_t o = z * pl;
-                    nlv[0] = pk_load_l2(pv + o);
-                    nvv[0] = pk_load(A.v + G.mem + o);
-                    if (G.row1) {
-                        nlv[1] = pk_load_l2(pv + o + A.px);
-                        nvv[1] = pk_load(A.v + G.mem + o + A.px);
-                    }
-                };
-#pragma unroll
-                for (int r = 0; r < 2; ++r) fu[r][1] = fv[r][1] = nlv[r] = nvv[r] = zero;
-                if (G.front) {
-                    load_front(0, fu[0], fv[0]);
-                    if (nz > 1) load_front(1, fu[1], fv[1]);
+                if (scalar) {
+                    before_bulk();
+                    for (int f = 0, q = G4.st; f < min(depth, nz); ++f, q = q + 1 == depth ? 0 : q + 1) issue(f, q);
                 }
-                auto step = [&](int f, int slot, P (&cu)[2], P (&cv)[2]) {
-                    const int z = f - kRadius;
-                    P lv[2], vv[2];
+                const float m_ag = -ap * ig, ig1 = ig * in1, m_ag1 = m_ag * in1;
+                float *pu = uout, *pv = vk;              // planes f - 6 of u, f of v_k
+                float2 svv = make_float2(0.f, 0.f), suv = svv, suu = svv;
+                P acc[12][R];                            // sums of planes f-6 .. f+5
 #pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        lv[r] = nlv[r];
-                        vv[r] = nvv[r];
+                for (int j = 0; j < 12; ++j)
+#pragma unroll
+                    for (int r = 0; r < R; ++r) acc[j][r].zero();
+                // the next plane of u
+                auto put_u = [&](const P (&u)[R]) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        P t = u[r];
+                        t.mul(mask);
+                        if (r) t.mul(in1);
+                        if (r == 0 || G.row1) pk_store(pu + r * A.px, t);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) suu = __ffma2_rn(t.p[i], t.p[i], suu);
                     }
-                    if (G.own && z + 1 >= 0 && z + 1 < nz) load_centre(z + 1);
-                    if (G.front) {
-                        P w[2] = {zero, zero};
-                        if (f < nz) {
-                            const size_t o = f * pl + G.mem;
-#pragma unroll
-                            for (int r = 0; r < 2; ++r)
-                                if (r == 0 || G.row1) {
-                                    w[r] = cu[r];
-                                    w[r].mul(ig);
-                                    w[r].fma(m_ag, cv[r]);
-                                    if (G.own) pk_store(vk + o + r * A.px, w[r]);
-                                }
-                        }
-                        pk_store(at(o0 + slot * pb), w[0]);
-                        if (G.row1) pk_store(at(o1 + slot * pb), w[1]);
-                        if (f + 2 < nz) load_front(f + 2, cu, cv);
-                    }
-                    __syncthreads();
-                    if (G.own && z >= 0) {
-                        const int cz = slot >= kRadius ? slot - kRadius : slot + kRing - kRadius;
-                        const int q0 = o0 + cz * pb, q1 = o1 + cz * pb;
-                        P a0, a1, ctr0, ctr1;
-                        a0.zero();
-                        a1.zero();
-                        a0.fma(-cc, lv[0]);
-                        a1.fma(-cc, lv[1]);
-                        {
-                            P X[5];
-#pragma unroll
-                            for (int m = 0; m < 5; ++m) X[m] = lds<float>(q0 + (m - 2) * 16);
-                            ctr0 = X[2];
-                            x_part(a0, X, cf);
-                        }
-                        {
-                            P X[5];
-#pragma unroll
-                            for (int m = 0; m < 5; ++m) X[m] = lds<float>(q1 + (m - 2) * 16);
-                            ctr1 = X[2];
-                            x_part(a1, X, cf);
-                        }
-                        const P nb1 = G.row1 ? ctr1 : lds<float>(q0 + rb);   // a row of zeros
-                        a0.fma(cf.a[1], nb1);
-                        a1.fma(cf.a[1], ctr0);
-#pragma unroll
-                        for (int d = 1; d <= kRadius; ++d) {
-                            const P lo = lds<float>(q0 - d * rb), hi = lds<float>(q0 + (1 + d) * rb);
-                            a0.fma(cf.a[d], lo);
-                            a1.fma(cf.a[d], hi);
-                            if (d < kRadius) {
-                                a1.fma(cf.a[d + 1], lo);
-                                a0.fma(cf.a[d + 1], hi);
-                            }
-                            const int sm = (cz >= d ? cz - d : cz + kRing - d) * pb;
-                            const int sp = (cz + d < kRing ? cz + d : cz + d - kRing) * pb;
-                            a0.fma(cf.a[d], lds<float>(o0 + sm));
-                            a0.fma(cf.a[d], lds<float>(o0 + sp));
-                            a1.fma(cf.a[d], lds<float>(o1 + sm));
-                            a1.fma(cf.a[d], lds<float>(o1 + sp));
-                        }
-                        a0.fma(dg, ctr0);
-                        a1.fma(dg, ctr1);
-                        a0.fma(vv[0], ctr0);
-                        a1.fma(vv[1], ctr1);
-                        P t0, t1, t2;
-                        t0.zero();
-                        t1.zero();
-                        t2.zero();
-#pragma unroll
-                        for (int i = 1; i < 4; ++i)      // u = 0 outside the box
-                            if (i >= G.nvx) {
-                                a0.set(i, 0.f);
-                                a1.set(i, 0.f);
-                            }
-                        const size_t o = z * pl + G.mem;
-                        pk_store(uo + o, a0);
-                        t0.fma(ctr0, ctr0);
-                        t1.fma(a0, ctr0);
-                        t2.fma(a0, a0);
-                        if (G.row1) {
-                            pk_store(uo + o + A.px, a1);
-                            t0.fma(ctr1, ctr1);
-                            t1.fma(a1, ctr1);
-                            t2.fma(a1, a1);
-                        }
-                        svv += t0.sum();
-                        suv += t1.sum();
-                        suu += t2.sum();
-                    }
+                    pu += pl;
                 };
-                for (int f = 0, slot = 0; f < nz + kRadius; f += 2, slot = slot + 2 == kRing ? 0 : slot + 2) {
-                    step(f, slot, fu[0], fv[0]);
-                    if (f + 1 < nz + kRadius) step(f + 1, slot + 1, fu[1], fv[1]);
+                for (int f = 0; f < nz; ++f) {
+                    const int sb = s0 + G4.st * stb, po = (f & 1) * pb;
+                    int q0 = o0 + po;
+                    asm volatile("" : "+r"(q0));
+                    G4.wait(A.L.err);
+                    P w[R], a[R];
+                    if (G.own) {
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            a[r] = lds<float>(sb + su + uo + r * mb1);
+                            w[r] = lds<float>(sb + uo + r * mb1);
+                            w[r].mul(r ? ig1 : ig);
+                            w[r].fma(r ? m_ag1 : m_ag, a[r]);
+                            pk_store(reinterpret_cast<float *>(lz_smem + q0 + r * rb), w[r]);
+                            if (r == 0 || G.row1) pk_store(pv + r * A.px, w[r]);
+                            a[r].mul(-cc);
+                            a[r].fma(lds<float>(sb + vo + r * mb1), w[r]);
+                            a[r].fma(dg, w[r]);
+                        }
+                        pv += pl;
+                    }
+                    auto form_halo = [&](int from, int to) {
+                        if (from < 0) return;
+                        P h = lds<float>(sb + from);
+                        h.mul(ig);
+                        h.fma(m_ag, lds<float>(sb + su + from));
+                        pk_store(reinterpret_cast<float *>(lz_smem + po + to), h);
+                    };
+                    form_halo(h_from, h_to);
+                    if (tid < nthr)
+                        for (int e = tid + nthr; e < nhalo; e += nthr) {   // bands of fewer than 24 rows
+                            int from, to;
+                            halo(e, from, to);
+                            form_halo(from, to);
+                        }
+                    const int freed = G4.st;
+                    G4.next(depth);
+                    __syncthreads();                     // the plane is there, the stage is read
+                    if (scalar && f + depth < nz) issue(f + depth, freed);
+                    if (!G.own) continue;
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        P X[5];
+#pragma unroll
+                        for (int m = 0; m < 5; ++m) X[m] = m == 2 ? w[r] : lds<float>(q0 + r * rb + (m - 2) * 16);
+                        x_part(a[r], X, cf);
+                    }
+                    if (R == 2) {
+                        a[0].fma(cf.a[1], w[R - 1]);
+                        a[R - 1].fma(cf.a[1], w[0]);
+                    }
+#pragma unroll
+                    for (int d = 1; d <= kRadius; ++d) {
+                        const P lo = lds<float>(q0 - d * rb), hi = lds<float>(q0 + (R - 1 + d) * rb);
+                        a[0].fma(cf.a[d], lo);
+                        a[R - 1].fma(cf.a[d], hi);
+                        if (R == 2 && d < kRadius) {
+                            a[R - 1].fma(cf.a[d + 1], lo);
+                            a[0].fma(cf.a[d + 1], hi);
+                        }
+                    }
+                    P u[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        // acc[6]: plane f's neighbours below; the ones above give w.(B w) the same again
+                        P t = a[r];
+                        t.fma(2.f, acc[6][r]);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            svv = __ffma2_rn(w[r].p[i], w[r].p[i], svv);
+                            suv = __ffma2_rn(t.p[i], w[r].p[i], suv);
+                        }
+                        u[r] = acc[0][r];
+                        u[r].fma(cf.a[6], w[r]);
+#pragma unroll
+                        for (int j = 1; j < 12; ++j) {
+                            acc[j - 1][r] = acc[j][r];
+                            if (j == 6) acc[j - 1][r].fma(1.f, a[r]);   // plane f
+                            else acc[j - 1][r].fma(cf.a[j < 6 ? 6 - j : j - 6], w[r]);
+                        }
+                        acc[11][r] = w[r];
+                        acc[11][r].mul(cf.a[6]);
+                    }
+                    if (f >= kRadius) put_u(u);
                 }
-                // (also: every ring reader of the sweep is done)
-                gather3(svv, suv, suu, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
+                if (G.own)
+#pragma unroll
+                    for (int j = 0; j < kRadius; ++j) put_u(acc[j]);
+                before_bulk();                           // u and v_k, for the next sweep's copies
+                gather3(svv.x + svv.y, suv.x + suv.y, suu.x + suu.y, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
                 {
                     float a, b, c;
                     sum_parts(ng, ncl, a, b, c);
@@ -1523,13 +1640,13 @@ __global__ void __launch_bounds__(512, 1) k_lanczos_stream(const __grid_constant
                 n = k - kb;
                 if (S.flag) break;
                 if (n == A.L.hist) {                     // the history is full: into x and p
-                    stream_flush(&A, s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+                    G4 = stream_flush<R>(&A, s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1], G4);
                     have_p = true;
                     kb = k;
                 }
             }
             if (S.flag < 4)
-                stream_flush(&A, s, n, false, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]);
+                G4 = stream_flush<R>(&A, s, n, false, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1], G4);
             cluster_barrier();                           // no thread still reads the flag or this part's vectors
         }
         if (scalar && G.rank == 0) end_state(A.L, s);
@@ -1553,6 +1670,11 @@ const Fn64 kFn64[3][2] = {{k_lanczos<double, 2, 640, 2>, k_lanczos<double, 2, 64
                           {k_lanczos<double, 4, 640, 2>, k_lanczos<double, 4, 640, 1>},
                           {k_lanczos<double, 8, 384, 2>, k_lanczos<double, 8, 384, 1>}};
 
+const void *stream_kernel(int rows, int threads) {
+    return rows == 1 ? (const void *)k_lanczos_stream<1, 512>
+                     : threads <= 256 ? (const void *)k_lanczos_stream<2, 256> : (const void *)k_lanczos_stream<2, 384>;
+}
+
 const void *kernel_of(bool mixed, int v, bool per) {
     return mixed ? (const void *)kFn32[v][per] : (const void *)kFn64[v][per];
 }
@@ -1573,21 +1695,33 @@ void cluster_config(cudaLaunchConfig_t &lc, cudaLaunchAttribute &at, int ncl, in
 
 }  // namespace
 
-// Plan of the streaming kernel: the fewest bands (1, 2, 4, 8) whose ring fits a block.
-static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan &p) {
+// Plan of the streaming kernel: threads of one or two rows and 1 to 8 bands, of which a block's threads take every
+// point and whose planes fit, two in flight at least.  A plane of a band of bh rows takes time as bh + 10 (its
+// halo rows are only formed), three quarters of that for each of the blocks that share an SM (one waits
+// where another computes), and never less than one step's latency, which is longer for two rows a thread.
+// Measured, whole chi0 application in ms, with (rows, bands): 56^3, 256 systems (1, 2) 88, (1, 3) 108,
+// (1, 4) 82.5, (1, 5) 93, (1, 6) 118, (2, 2) 83, (2, 3) 123, (2, 4) 134; 72^3, 256 systems (1, 3) 246, (1, 4) 264,
+// (1, 6) 238, (2, 2) 213, (2, 3) 232, (2, 4) 289, (2, 6) 357.
+static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan &p, double &cycles) {
     if (c.opt.prec != RPA_MIXED || c.opt.periodic) return false;
-    const void *fn = (const void *)k_lanczos_stream;
-    const int hw = (c.nx + 3) / 4;
-    int p16 = 2 + hw;
-    while ((2 * p16 - (hw + hw % 2)) % 8 != 0) ++p16;
-    for (int ncl = 1; ncl <= 8; ncl *= 2) {
-        const int bh = ((c.ny + ncl - 1) / ncl + 1) / 2 * 2, hp = ncl > 1 ? kRadius / 2 : 0;
-        if (bh < 2 || (long long)bh * (ncl - 1) >= c.ny) return false;
-        const long long units = (long long)hw * (bh / 2 + 2 * hp);
+    const int hw = (c.nx + 3) / 4, px = 4 * hw;
+    double best = 1e300;
+    for (int q = 0; q < 16; ++q) {
+        const int rows = 1 + q / 8, ncl = 1 + q % 8;
+        const int bh = ((c.ny + ncl - 1) / ncl + 1) / 2 * 2;
+        if (bh < 2 || (long long)bh * (ncl - 1) >= c.ny) continue;
+        const long long units = (long long)hw * (bh / rows);
         const int threads = (int)std::min<long long>((units + 31) / 32 * 32 + 32, 1 << 20);
+        if (threads > (rows == 1 ? 512 : 384)) continue;
+        int p16 = 2 + hw;                // 16-byte words of a row: a unit's rows span hw of them modulo 8
+        while ((rows * p16 - (hw + (rows == 2 ? hw % 2 : 0))) % 8 != 0) ++p16;
         const int pitch = 4 * p16, plane = pitch * (bh + 2 * kRadius);
-        const size_t smem = shared_bytes<float>() + sizeof(float) * ((size_t)kRing * plane + 16);
-        if (threads > 512 || smem > (size_t)optin) continue;
+        const size_t stage = sizeof(float) * (size_t)px * (3 * bh + 4 * kRadius);
+        const size_t fixed = shared_bytes<float>() + sizeof(float) * (2 * (size_t)plane + 16);
+        if (fixed + 2 * stage > (size_t)optin) continue;
+        const int depth = (int)std::min<size_t>(kStages, ((size_t)optin - fixed) / stage);
+        const size_t smem = fixed + depth * stage;
+        const void *fn = stream_kernel(rows, threads);
         RPA_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         allow_dynamic_smem(fn, smem);
         cudaLaunchConfig_t lc{};
@@ -1598,6 +1732,13 @@ static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan 
             (void)cudaGetLastError();
             continue;
         }
+        const int all = std::max(nsys, c.batch_load);
+        const double share = (double)std::min(ncs, all) * ncl / sms, load = (rows == 1 ? 1.0 : 0.92) * hw * (bh + 10);
+        // cycles of a sweep (and what it costs at its end), times the rounds the systems take
+        const double cost = (all <= ncs ? 1.0 : (double)all / ncs + 0.3) *
+                            (20e3 + 5.4 * c.nz * std::max(rows == 1 ? 250.0 : 500.0, load * std::max(1.0, 0.75 * share)));
+        if (cost >= best) continue;
+        best = cost;
         p = LanczosPlan{};
         p.stream = 1;
         p.mixed = 1;
@@ -1609,15 +1750,17 @@ static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan 
         p.pitch = pitch;
         p.plane = plane;
         p.bh = bh;
-        p.hp = hp;
-        const size_t nv = (size_t)c.nz * c.ny * 4 * hw;
-        // history: as many vectors as 8 GB hold, 16 .. kHistMax
-        p.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, ((size_t)8 << 30) / (nv * 4 * p.clusters)));
-        p.ws_stride = nv * (4 + p.hist);
-        p.ws_bytes = sizeof(float) * (p.ws_stride * p.clusters + nv);     // and V_loc
-        return true;
+        p.depth = depth;
+        p.unit_rows = rows;
     }
-    return false;
+    if (best == 1e300) return false;
+    cycles = best;
+    const size_t nv = (size_t)c.nz * c.ny * px;
+    // history: as many vectors as 8 GB hold, 16 .. kHistMax
+    p.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, ((size_t)8 << 30) / (nv * 4 * p.clusters)));
+    p.ws_stride = nv * (4 + p.hist);
+    p.ws_bytes = sizeof(float) * (p.ws_stride * p.clusters + nv);         // and V_loc
+    return true;
 }
 
 bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
@@ -1693,7 +1836,17 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
             }
         }
     }
-    if (!found) return stream_plan(c, nsys, sms, optin, best);
+    // Clusters of 8 or 16 blocks leave SMs idle (15 and 7 are resident, of 19 and 9.5): with many systems the
+    // streaming kernel is faster then.  An iteration on chip takes 1.5 times the cycles above.  Measured, chi0 in
+    // ms, on chip and streaming: 44^3 32 systems 7.7, 15.4, 128 systems 23.7, 28.1, 256 systems 45.0, 40.7; 48^3
+    // 11.0, 19.0; 38.1, 30.4; 73.3, 46.4; with four blocks, 40^3, 4096 systems 357, 429; with two, 32^3 175, 212.
+    LanczosPlan sp;
+    double sc = 0.0;
+    if (stream_plan(c, nsys, sms, optin, sp, sc) && (!found || sc < 0.93 * 1.5 * best_cost)) {
+        best = sp;
+        return true;
+    }
+    if (!found) return false;
     best.stream = 0;
     const size_t vec = (size_t)2 * best.zc * (best.threads - kExtra) * W, hvec = (size_t)best.nch * best.zc * best.plane;
     // history: as many vectors as 2 GB hold in each of its two buffers, 16 .. kHistMax
@@ -1763,9 +1916,9 @@ void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<float>
     a.nv = (size_t)c.nz * c.ny * a.px;
     a.v = (const float *)p.ws + p.ws_stride * p.clusters;
     a.bh = p.bh;
-    a.hp = p.hp;
+    a.depth = p.depth;
     const Coef<float> cf = cast_coef<float>(c.coef);
-    const void *fn = (const void *)k_lanczos_stream;
+    const void *fn = stream_kernel(p.unit_rows, p.threads);
     allow_dynamic_smem(fn, p.smem);
     cudaLaunchConfig_t lc{};
     cudaLaunchAttribute at{};

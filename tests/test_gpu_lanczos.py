@@ -116,3 +116,19 @@ def test_streaming_lanczos_matches_oracle(rpa, grid, nsys, h, tol):
     if h < 0.2 and nsys > 3:
         pytest.skip("the oracle's time")
     solve_and_check(rpa, grid, "mixed", False, nsys, h=h, tol=tol, kernel="k_lanczos_stream")
+
+
+def test_on_chip_and_streaming_solutions_agree(rpa):
+    """Grids of more than four blocks a system: few systems are solved on chip, many by the streaming kernel."""
+    s = synth.small_system((46, 45, 44), h=0.5, n_s=1, n_wells=1, seed=5)
+    b = torch.as_tensor(np.random.default_rng(6).standard_normal((200, s.n_d)), device="cuda")
+    o = rpa.default_options()
+    o.tol, o.prec = 1e-10, rpa.RPA_MIXED
+    with rpa.Context.from_system(s, o) as ctx:
+        few = ctx.sternheimer_solve(0.4, np.zeros(3, int), b[:3], project=False)
+        many = ctx.sternheimer_solve(0.4, np.zeros(200, int), b, project=False)
+    assert few[3] == rpa.RPA_OK and many[3] == rpa.RPA_OK
+    x, y = few[0].cpu().numpy(), many[0][:3].cpu().numpy()
+    w = synth.fornberg_second_derivative(6)
+    top = 1.5 * (abs(w[0]) + 2.0 * np.abs(w[1:]).sum()) / 0.25 + float(np.abs(s.vloc).max()) + abs(-s.eps[0] + 0.4j)
+    assert np.linalg.norm(x - y) <= 2 * 1e-10 * top / 0.4 * np.linalg.norm(x)
