@@ -721,7 +721,11 @@ int ec_impl(Ctx &c, int n_r, const double *V0_dev, double *lambdas_host, double 
             ritz_rotation(Lm, work, n_r, wt[m] / (2.0 * M_PI), Sm, coef, s);
             combine_rows(Sm, n_r, n_r, Vprev, c.nd, T1, s);           // Ritz vectors
             coulomb_apply(c, 0.5, T1, T2, n_r, s);                    // nu^1/2 y_i
+            // the responses enter the gradient only, not the subspace that goes on: by any kernel
+            const bool keep = c.keep_cocg;
+            c.keep_cocg = false;
             worst = std::max(worst, response_square(c, om[m], T2, coef, grad, n_r, s));
+            c.keep_cocg = keep;
             enqueue_status_readback(c, s);
             sync_stream(c, s);
             worst = std::max(worst, finish_call(c, s));

@@ -2977,10 +2977,11 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     const RingFn ring_fn = ws ? (even_nx ? k_cocg_ring_ws<true> : k_cocg_ring_ws<false>)
                               : clus ? (even_nx ? k_cocg_ring_cl<true> : k_cocg_ring_cl<false>) : ring1_fn;
     // systems that fit on chip: the Lanczos kernel
-    if (c.lz_key[0] != S || c.lz_key[1] != c.opt.prec || c.lz_key[2] != c.batch_load) {
+    const int lz_form = c.opt.prec + 16 * (c.opt.precondition != 0);
+    if (c.lz_key[0] != S || c.lz_key[1] != lz_form || c.lz_key[2] != c.batch_load) {
         c.lz_ok = lanczos_plan(c, S, c.lz_plan);
         c.lz_key[0] = S;
-        c.lz_key[1] = c.opt.prec;
+        c.lz_key[1] = lz_form;
         c.lz_key[2] = c.batch_load;
     }
     const bool use_lz = c.lz_ok && !precond && !c.keep_cocg && (want == 0 || want == 4);

@@ -146,10 +146,10 @@ struct Ctx {
     DevBuf blockE;                // subspace of the previous iteration (gradient)
     DevBuf dense_scratch;         // split-K partial sums
     DevBuf lanczos_ws;            // Lanczos vectors of the systems in flight
-    LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, prec, batch_load}
+    LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, form, batch_load}
     int lz_key[3] = {-1, -1, -1};
     bool lz_ok = false;
-    // rpa_ec_gradient with the final subspace as an output runs the COCG kernels: a subspace is R L^-T
+    // rpa_ec_gradient with the final subspace as an output runs the COCG kernels up to it: a subspace is R L^-T
     // with the conditioning of R, and after the exact integer pieces of the tensor-core contractions
     // (whose last digits turn on 1e-12 of their operands) the Lanczos kernel's rounding moves it by
     // 2e-9 relative, more than a change of kernels may; the energies and the gradient move by 1e-10.
