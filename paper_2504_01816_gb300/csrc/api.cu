@@ -78,7 +78,6 @@ Ctx::~Ctx() {
     cudaFree(psi32);
     cudaFree(eps_dev);
     for (double *q : Q) cudaFree(q);
-    for (double *q : Qpar) cudaFree(q);
     cudaFree(lam);
     for (int a = 0; a < 3; ++a) {
         cudaFree(mu[a]);

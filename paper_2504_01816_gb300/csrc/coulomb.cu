@@ -268,13 +268,12 @@ void coulomb_setup(Ctx &c) {
             for (double m : mu[a])
                 if (!(m > 0.0)) fail(RPA_ERR_INVALID, "1D Laplacian not positive definite (n=%d)", n);
         }
-        RPA_CUDA(cudaMalloc(&c.Q[a], sizeof(double) * n * n));
-        RPA_CUDA(cudaMemcpy(c.Q[a], Q.data(), sizeof(double) * n * n, cudaMemcpyHostToDevice));
         const std::vector<double> qp = by_parity(Q, n);
-        if (!qp.empty()) {
-            RPA_CUDA(cudaMalloc(&c.Qpar[a], sizeof(double) * qp.size()));
-            RPA_CUDA(cudaMemcpy(c.Qpar[a], qp.data(), sizeof(double) * qp.size(), cudaMemcpyHostToDevice));
-        }
+        std::vector<double> both(Q);                     // one allocation and copy
+        both.insert(both.end(), qp.begin(), qp.end());
+        RPA_CUDA(cudaMalloc(&c.Q[a], sizeof(double) * both.size()));
+        RPA_CUDA(cudaMemcpy(c.Q[a], both.data(), sizeof(double) * both.size(), cudaMemcpyHostToDevice));
+        if (!qp.empty()) c.Qpar[a] = c.Q[a] + (size_t)n * n;
         // the same factors for the Laplacian preconditioner of COCG, in FP64 and FP32
         std::vector<float> qf(Q.begin(), Q.end()), mf(mu[a].begin(), mu[a].end());
         RPA_CUDA(cudaMalloc(&c.mu[a], sizeof(double) * n));

@@ -121,7 +121,7 @@ struct Ctx {
     // summed eigenvalue grid lam = mu_x + mu_y + mu_z (nd).
     double *Q[3] = {nullptr, nullptr, nullptr};
     double *lam = nullptr;
-    // The same eigenvectors by parity (null: not every one has a parity), h = ceil(n_a / 2): h x h components
+    // The same eigenvectors by parity, in the same allocation (null: not every one has a parity), h = ceil(n_a / 2): h x h components
     // i < h of the symmetric ones and of the antisymmetric ones, then their indices a (two lists of h ints).
     double *Qpar[3] = {nullptr, nullptr, nullptr};
     // Laplacian preconditioner of COCG: the 1D eigenvalues mu_a (FP64), FP32 copies of Q_a and mu_a,
