@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
 }
 
 // ---------------------------------------------------------------------------------------------
-// The same solve for grids that do not fit on chip (mixed form, zero values outside the box): u and the
+// The same solve for grids that do not fit on chip (mixed form): u and the
 // vectors stay in memory and a cluster of C blocks marches along z, block c over a band of rows.  One
 // sweep is one Lanczos step: at step f a thread (4 x 1 or 4 x 2 points) forms v_k = (u - a' v_{k-1}) / g of plane f
 // from the last sweep's u and v_{k-1}, stores it in a plane in shared memory and as vector k of the history,
@@ -1406,7 +1406,10 @@ __device__ __noinline__ void stream_start(const StreamArgs *args, int s, float f
     ri = c;
 }
 
-template <int R, int MAXT>
+// PER: periodic boundaries (R = 1): rows past the box are staged and formed at their images, a row's images beside
+// it in its padding, and the planes nz-6 .. nz-1 before and 0 .. 5 after the sweep, for their part along z alone
+// (the COCG kernels before: chi0 at 48^3, 128 systems 127 ms, now 55).
+template <int R, int MAXT, bool PER>
 __global__ void __launch_bounds__(MAXT, 1)
     k_lanczos_stream(const __grid_constant__ StreamArgs A, const __grid_constant__ Coef<float> cf) {
     using P = Pk<float>;
@@ -1419,18 +1422,20 @@ __global__ void __launch_bounds__(MAXT, 1)
     const int pb = A.L.plane * 4, rb = A.L.pitch * 4, mb = A.px * 4;
     const int o0 = shared_bytes<float>() + ((G.gy - G.y0 + kRadius) * A.L.pitch + 8 + G.gx) * 4;
     const int s0 = shared_bytes<float>() + 2 * pb + 64, su = (A.bh + 2 * kRadius) * mb, stb = 2 * su + A.bh * mb;
-    const int r0 = max(0, G.y0 - kRadius), nrow = min(A.L.ny, G.y0 + A.bh + kRadius) - r0;   // rows staged
+    // rows staged; planes before the first
+    const int r0 = PER ? G.y0 - kRadius : max(0, G.y0 - kRadius), nrow = PER ? G.rows + 2 * kRadius : min(A.L.ny, G.y0 + A.bh + kRadius) - r0;
+    constexpr int GH = PER ? kRadius : 0;
     // the unit's second row, if it lies outside the box: the first again, with factors 0
     const int uo = G.own ? (G.gy - r0) * mb + G.gx * 4 : 0, vo = 2 * su + (G.own ? (G.gy - G.y0) * mb + G.gx * 4 : 0);
     const int mb1 = G.row1 ? mb : 0;
     const float in1 = G.row1 ? 1.f : 0.f;
     // halo rows: units of one row by all threads that have points
-    const int nhalo = ncl > 1 ? 2 * kRadius * A.L.hw : 0, nthr = A.bh / R * A.L.hw;
+    const int nhalo = PER || ncl > 1 ? 2 * kRadius * A.L.hw : 0, nthr = A.bh / R * A.L.hw;
     // unit e: its place in a stage (-1: outside the box) and in plane 0
     auto halo = [&](int e, int &from, int &to) {
-        const int hr = e / A.L.hw, lr = hr < kRadius ? hr - kRadius : A.bh + hr - kRadius, y = G.y0 + lr;
+        const int hr = e / A.L.hw, lr = hr < kRadius ? hr - kRadius : G.rows + hr - kRadius, y = G.y0 + lr;
         const int x = 4 * (e - hr * A.L.hw);
-        from = e < nhalo && y >= 0 && y < A.L.ny ? (y - r0) * mb + 4 * x : -1;
+        from = e < nhalo && (PER || (y >= 0 && y < A.L.ny)) ? (y - r0) * mb + 4 * x : -1;
         to = shared_bytes<float>() + ((lr + kRadius) * A.L.pitch + 8 + x) * 4;
     };
     int h_from = -1, h_to = 0;                           // the thread's first
@@ -1497,15 +1502,22 @@ __global__ void __launch_bounds__(MAXT, 1)
                 float *const vk = H + (size_t)(k - kb) * A.nv + G.mem;
                 auto issue = [&](int f, int q) {
                     const unsigned to = (unsigned)__cvta_generic_to_shared(lz_smem) + (unsigned)(s0 + q * stb);
-                    const size_t o = f * pl + (size_t)r0 * A.px;
+                    if (PER) f = f < 0 ? f + nz : f >= nz ? f - nz : f;
                     expect_bytes(G4.bar(q), 2 * nrow * mb + G.rows * mb);
-                    bulk_load(to, ui + o, nrow * mb, G4.bar(q));
-                    bulk_load(to + su, vp + o, nrow * mb, G4.bar(q));
+                    for (int i = 0; i < nrow;) {         // once, but for a periodic band at the box's edge
+                        int y = r0 + i;
+                        if (PER) y = y < 0 ? y + A.L.ny : y % A.L.ny;
+                        const int m = PER ? min(nrow - i, A.L.ny - y) : nrow;
+                        const size_t o = f * pl + (size_t)y * A.px;
+                        bulk_load(to + i * mb, ui + o, m * mb, G4.bar(q));
+                        bulk_load(to + su + i * mb, vp + o, m * mb, G4.bar(q));
+                        i += m;
+                    }
                     bulk_load(to + 2 * su, A.v + f * pl + (size_t)G.y0 * A.px, G.rows * mb, G4.bar(q));
                 };
                 if (scalar) {
                     before_bulk();
-                    for (int f = 0, q = G4.st; f < min(depth, nz); ++f, q = q + 1 == depth ? 0 : q + 1) issue(f, q);
+                    for (int i = 0, q = G4.st; i < min(depth, nz + 2 * GH); ++i, q = q + 1 == depth ? 0 : q + 1) issue(i - GH, q);
                 }
                 const float m_ag = -ap * ig, ig1 = ig * in1, m_ag1 = m_ag * in1;
                 float *pu = uout, *pv = vk;              // planes f - 6 of u, f of v_k
@@ -1528,7 +1540,8 @@ __global__ void __launch_bounds__(MAXT, 1)
                     }
                     pu += pl;
                 };
-                for (int f = 0; f < nz; ++f) {
+                for (int f = -GH; f < nz + GH; ++f) {
+                    const bool real = !PER || (f >= 0 && f < nz);
                     const int sb = s0 + G4.st * stb, po = (f & 1) * pb;
                     int q0 = o0 + po;
                     asm volatile("" : "+r"(q0));
@@ -1541,23 +1554,31 @@ __global__ void __launch_bounds__(MAXT, 1)
                             w[r] = lds<float>(sb + uo + r * mb1);
                             w[r].mul(r ? ig1 : ig);
                             w[r].fma(r ? m_ag1 : m_ag, a[r]);
-                            pk_store(reinterpret_cast<float *>(lz_smem + q0 + r * rb), w[r]);
+                            if (PER) {
+                                if (!real) continue;
+                                put<float, 1>(reinterpret_cast<float *>(lz_smem + q0), G.gx, G.nvx, A.L.nx, w[r]);
+                            } else {
+                                pk_store(reinterpret_cast<float *>(lz_smem + q0 + r * rb), w[r]);
+                            }
                             if (r == 0 || G.row1) pk_store(pv + r * A.px, w[r]);
                             a[r].mul(-cc);
                             a[r].fma(lds<float>(sb + vo + r * mb1), w[r]);
                             a[r].fma(dg, w[r]);
                         }
-                        pv += pl;
+                        if (real) pv += pl;
                     }
                     auto form_halo = [&](int from, int to) {
                         if (from < 0) return;
                         P h = lds<float>(sb + from);
                         h.mul(ig);
                         h.fma(m_ag, lds<float>(sb + su + from));
-                        pk_store(reinterpret_cast<float *>(lz_smem + po + to), h);
+                        float *const at = reinterpret_cast<float *>(lz_smem + po + to);
+                        const int x = from % mb / 4;
+                        if (PER) put<float, 1>(at, x, min(4, A.L.nx - x), A.L.nx, h);
+                        else pk_store(at, h);
                     };
-                    form_halo(h_from, h_to);
-                    if (tid < nthr)
+                    if (real) form_halo(h_from, h_to);
+                    if (tid < nthr && real)
                         for (int e = tid + nthr; e < nhalo; e += nthr) {   // bands of fewer than 24 rows
                             int from, to;
                             halo(e, from, to);
@@ -1566,13 +1587,30 @@ __global__ void __launch_bounds__(MAXT, 1)
                     const int freed = G4.st;
                     G4.next(depth);
                     __syncthreads();                     // the plane is there, the stage is read
-                    if (scalar && f + depth < nz) issue(f + depth, freed);
+                    if (scalar && f + depth < nz + GH) issue(f + depth, freed);
                     if (!G.own) continue;
+                    if (!real) {                         // its part along z alone
+                        P u = acc[0][0];
+                        u.fma(cf.a[6], w[0]);
+#pragma unroll
+                        for (int j = 1; j < 12; ++j) {
+                            acc[j - 1][0] = acc[j][0];
+                            if (j != 6) acc[j - 1][0].fma(cf.a[j < 6 ? 6 - j : j - 6], w[0]);
+                        }
+                        acc[11][0] = w[0];
+                        acc[11][0].mul(cf.a[6]);
+                        if (f >= nz) {
+                            P t[R];
+                            t[0] = u;
+                            put_u(t);
+                        }
+                        continue;
+                    }
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
                         P X[5];
 #pragma unroll
-                        for (int m = 0; m < 5; ++m) X[m] = m == 2 ? w[r] : lds<float>(q0 + r * rb + (m - 2) * 16);
+                        for (int m = 0; m < 5; ++m) X[m] = m == 2 && !PER ? w[r] : lds<float>(q0 + r * rb + (m - 2) * 16);
                         x_part(a[r], X, cf);
                     }
                     if (R == 2) {
@@ -1613,7 +1651,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                     }
                     if (f >= kRadius) put_u(u);
                 }
-                if (G.own)
+                if (G.own && !PER)
 #pragma unroll
                     for (int j = 0; j < kRadius; ++j) put_u(acc[j]);
                 before_bulk();                           // u and v_k, for the next sweep's copies
@@ -1670,9 +1708,11 @@ const Fn64 kFn64[3][2] = {{k_lanczos<double, 2, 640, 2>, k_lanczos<double, 2, 64
                           {k_lanczos<double, 4, 640, 2>, k_lanczos<double, 4, 640, 1>},
                           {k_lanczos<double, 8, 384, 2>, k_lanczos<double, 8, 384, 1>}};
 
-const void *stream_kernel(int rows, int threads) {
-    return rows == 1 ? (const void *)k_lanczos_stream<1, 512>
-                     : threads <= 256 ? (const void *)k_lanczos_stream<2, 256> : (const void *)k_lanczos_stream<2, 384>;
+const void *stream_kernel(int rows, int threads, bool per) {
+    return per ? (const void *)k_lanczos_stream<1, 512, true>
+               : rows == 1 ? (const void *)k_lanczos_stream<1, 512, false>
+                           : threads <= 256 ? (const void *)k_lanczos_stream<2, 256, false>
+                                            : (const void *)k_lanczos_stream<2, 384, false>;
 }
 
 const void *kernel_of(bool mixed, int v, bool per) {
@@ -1703,17 +1743,18 @@ void cluster_config(cudaLaunchConfig_t &lc, cudaLaunchAttribute &at, int ncl, in
 // (1, 4) 82.5, (1, 5) 93, (1, 6) 118, (2, 2) 83, (2, 3) 123, (2, 4) 134; 72^3, 256 systems (1, 3) 246, (1, 4) 264,
 // (1, 6) 238, (2, 2) 213, (2, 3) 232, (2, 4) 289, (2, 6) 357.
 static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan &p, double &cycles) {
-    if (c.opt.prec != RPA_MIXED || c.opt.periodic) return false;
+    if (c.opt.prec != RPA_MIXED) return false;
+    const bool per = c.opt.periodic != 0;
     const int hw = (c.nx + 3) / 4, px = 4 * hw;
     double best = 1e300;
-    for (int q = 0; q < 16; ++q) {
+    for (int q = 0; q < (per ? 8 : 16); ++q) {
         const int rows = 1 + q / 8, ncl = 1 + q % 8;
         const int bh = ((c.ny + ncl - 1) / ncl + 1) / 2 * 2;
         if (bh < 2 || (long long)bh * (ncl - 1) >= c.ny) continue;
         const long long units = (long long)hw * (bh / rows);
         const int threads = (int)std::min<long long>((units + 31) / 32 * 32 + 32, 1 << 20);
         if (threads > (rows == 1 ? 512 : 384)) continue;
-        int p16 = 2 + hw;                // 16-byte words of a row: a unit's rows span hw of them modulo 8
+        int p16 = per ? (16 + c.nx + 3) / 4 : 2 + hw;   // 16-byte words of a row: a unit's rows span hw of them modulo 8
         while ((rows * p16 - (hw + (rows == 2 ? hw % 2 : 0))) % 8 != 0) ++p16;
         const int pitch = 4 * p16, plane = pitch * (bh + 2 * kRadius);
         const size_t stage = sizeof(float) * (size_t)px * (3 * bh + 4 * kRadius);
@@ -1721,7 +1762,7 @@ static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan 
         if (fixed + 2 * stage > (size_t)optin) continue;
         const int depth = (int)std::min<size_t>(kStages, ((size_t)optin - fixed) / stage);
         const size_t smem = fixed + depth * stage;
-        const void *fn = stream_kernel(rows, threads);
+        const void *fn = stream_kernel(rows, threads, per);
         RPA_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         allow_dynamic_smem(fn, smem);
         cudaLaunchConfig_t lc{};
@@ -1736,7 +1777,7 @@ static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan 
         const double share = (double)std::min(ncs, all) * ncl / sms, load = (rows == 1 ? 1.0 : 0.92) * hw * (bh + 10);
         // cycles of a sweep (and what it costs at its end), times the rounds the systems take
         const double cost = (all <= ncs ? 1.0 : (double)all / ncs + 0.3) *
-                            (20e3 + 5.4 * c.nz * std::max(rows == 1 ? 250.0 : 500.0, load * std::max(1.0, 0.75 * share)));
+                            (20e3 + 5.4 * (c.nz + (per ? 8 : 0)) * std::max(rows == 1 ? 250.0 : 500.0, load * std::max(1.0, 0.75 * share)));
         if (cost >= best) continue;
         best = cost;
         p = LanczosPlan{};
@@ -1918,7 +1959,7 @@ void lanczos_launch(const Ctx &c, const LanczosPlan &p, const LanczosArgs<float>
     a.bh = p.bh;
     a.depth = p.depth;
     const Coef<float> cf = cast_coef<float>(c.coef);
-    const void *fn = stream_kernel(p.unit_rows, p.threads);
+    const void *fn = stream_kernel(p.unit_rows, p.threads, c.opt.periodic != 0);
     allow_dynamic_smem(fn, p.smem);
     cudaLaunchConfig_t lc{};
     cudaLaunchAttribute at{};

@@ -132,3 +132,13 @@ def test_on_chip_and_streaming_solutions_agree(rpa):
     w = synth.fornberg_second_derivative(6)
     top = 1.5 * (abs(w[0]) + 2.0 * np.abs(w[1:]).sum()) / 0.25 + float(np.abs(s.vloc).max()) + abs(-s.eps[0] + 0.4j)
     assert np.linalg.norm(x - y) <= 2 * 1e-10 * top / 0.4 * np.linalg.norm(x)
+
+
+@pytest.mark.parametrize("grid,nsys", [
+    ((57, 61, 10), 2),              # rows of 14 units and one point, odd rows, bands of unequal height
+    ((64, 62, 9), 70),              # several solves a cluster
+    ((90, 70, 8), 1),               # images in whole units, the fewest planes
+])
+def test_periodic_streaming_lanczos_matches_oracle(rpa, grid, nsys):
+    """Periodic grids that do not fit on chip: images along every axis."""
+    solve_and_check(rpa, grid, "mixed", True, nsys, h=0.5, tol=1e-11, kernel="k_lanczos_stream")
