@@ -2984,7 +2984,8 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         c.lz_key[1] = lz_form;
         c.lz_key[2] = c.batch_load;
     }
-    const bool use_lz = c.lz_ok && !precond && !c.keep_cocg && (want == 0 || want == 4);
+    // (their vectors take up to 8 GB: where that is not to be had, the kernels that do without run)
+    const bool use_lz = c.lz_ok && !precond && !c.keep_cocg && (want == 0 || want == 4) && c.lanczos_ws.room(c.lz_plan.ws_bytes);
     const bool use_ring = !use_lz && mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
     const int variant = (want >= 1 && want <= 3 && !(per && want == 3)) ? want - 1 : 0;
     const PaShape shape = mixed ? kPaShapes32[variant] : kPaShape64;
@@ -3172,7 +3173,7 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     LanczosArgs<float> lz32{};
     LanczosArgs<double> lz64{};
     if (use_lz) {
-        c.lz_plan.ws = c.lanczos_ws.ensure(c.lz_plan.ws_bytes);
+        c.lz_plan.ws = c.lanczos_ws.ptr;
         lanczos_prepare(c, c.lz_plan, st);
         auto fill = [&](auto &a) {
             a.slots = slots;

@@ -47,6 +47,7 @@ struct DevBuf {
     void *ptr = nullptr;
     size_t bytes = 0;
     void *ensure(size_t need);
+    bool room(size_t need);       // the same, for a buffer that one can do without: false where memory is short
     void release();
     template <typename T> T *as() const { return static_cast<T *>(ptr); }
 };
