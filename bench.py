@@ -267,15 +267,20 @@ def roofline_of(agg, step_ms, peaks):
     bytes_per_launch = a["bytes"] / max(a["launches"], 1)
     achieved = bytes_per_launch / per_launch_s / 1e9
     pts_per_launch = a.get("points", 0.0) / max(a["launches"], 1)
-    return {"bound": "hbm", "kernel": name, "achieved": achieved, "peak": hbm, "unit": "GB/s",
+    # bytes a point and iteration: the complex kernels' x, r, p read and written once; the Lanczos
+    # kernels' kept vector written and read (on chip), and u in and out and v_{k-1} in (streaming)
+    floor = {"k_lanczos<f32>": 8, "k_lanczos<f64>": 16, "k_lanczos_stream<f32>": 20}.get(
+        name, 48 if "c64" in name else 96)
+    bound = {"k_lanczos<f32>": "shared memory", "k_lanczos<f64>": "fp64 pipe"}.get(name, "hbm")
+    return {"bound": bound, "kernel": name, "achieved": achieved, "peak": hbm, "unit": "GB/s",
             "frac": achieved / hbm, "traffic": kernel_traffic(name, bytes_per_launch),
             "algorithmic_bytes_per_launch": bytes_per_launch, "points_per_launch": pts_per_launch,
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (burst copy)" if peaks else "fallback 6.8 TB/s",
             "share_of_step": a["ms"] / step_ms, "avg_launch_us": 1e6 * per_launch_s,
-            "floor_bytes_per_point": 48 if "c64" in name else 96,
-            # the whole COCG iteration against the floor of x, r, p read and written once: all
-            # COCG kernels' time over the points of one of them (each processes every point once)
-            "iteration_frac_vs_floor": (48.0 if "c64" in name else 96.0) * a["points"]
+            "floor_bytes_per_point": floor,
+            # the whole iteration against that floor: all solver kernels' time over the points of
+            # one of them (each processes every point once)
+            "iteration_frac_vs_floor": floor * a["points"]
             / (sum(v["ms"] for v in agg.values()) / 1e3) / 1e9 / hbm}
 
 
