@@ -52,6 +52,12 @@ namespace {
 
 constexpr int kHistMax = 128;            // Lanczos vectors kept between two updates of x
 
+// FP64 form: where g^2 = u.u - (u.v)^2 / v.v comes out below this share of u.u (half its digits are gone: v is
+// nearly in an invariant subspace, as a right-hand side next to an eigenvector is), g is taken from the
+// sums of u - a' v itself.  Without it g is rounding noise and, where that is negative, the solve ends
+// with a residual of 1e-9 that it takes for 0.  The mixed form need not: its refinement forms the residual.
+constexpr double kNearSpace = 0x1p-26;
+
 constexpr int kFlushThreads = 64;        // two warps that form the solutions
 constexpr int kExtra = 32 + kFlushThreads;   // threads without points: the scalar warp, the flush warps
 
@@ -1069,15 +1075,51 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                     const T b2 = c - ap * b;
                     ig = b2 > (T)0 ? (T)1 / sqrt(b2) : (T)0;
                     if (!isfinite(a) || !isfinite(c)) ig = (T)nan("");
-                }
-                if (sizeof(T) == 8) {
-                    if (scalar) {
+                    if (sizeof(T) == 8) {
                         S.vec[0] = ap;
                         S.vec[1] = ig;
                         S.vec[2] = ig > (T)0 ? (T)1 / ig : (T)0;
+                        S.vec[3] = b2 < (T)kNearSpace * c ? a : (T)0;
                     }
+                }
+                if (sizeof(T) == 8) {
                     main_sync(nmain);
+                    const T vv = S.vec[3];
                     ap = S.vec[0];
+                    if (vv > (T)0) {                     // g by the sums of w = u - a' v itself, a' with w's rest along v
+                        P t1, t2;
+                        t1.zero();
+                        t2.zero();
+                        if (G.unit) {
+#pragma unroll
+                            for (int z = 0; z < ZC; ++z)
+                                if (z < G.nvz) {
+#pragma unroll
+                                    for (int r = 0; r < 2; ++r)
+                                        if (r == 0 || G.row1) {
+                                            const P v = lds<T>((r ? o1 : o0) + z * pb);
+                                            P w = acc[z][r];
+                                            w.fma(-ap, v);
+                                            w.mul(mask);
+                                            t1.fma(w, v);
+                                            t2.fma(w, w);
+                                        }
+                                }
+                        }
+                        gather3((T)0, t1.sum(), t2.sum(), ng, ncl, G.rank, nmain, A.err);
+                        if (scalar) {
+                            T a, b, c;
+                            sum_parts(ng, ncl, a, b, c);
+                            const T da = b / vv, b2 = c - da * b;
+                            ig = b2 > (T)0 ? (T)1 / sqrt(b2) : (T)0;
+                            if (!isfinite(c)) ig = (T)nan("");
+                            S.vec[0] = ap + da;
+                            S.vec[1] = ig;
+                            S.vec[2] = ig > (T)0 ? (T)1 / ig : (T)0;
+                        }
+                        main_sync(nmain);
+                        ap = S.vec[0];
+                    }
                     ig = S.vec[1];
                 }
                 if (scalar) {
