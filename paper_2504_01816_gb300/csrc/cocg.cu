@@ -3517,13 +3517,13 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         ++checked;
     }
     sync_stream(c, st);
-    if (use_lz) check_tensor_core_status(c, st);
     while (checked < issued) collect_epoch(checked++);
     for (auto &e : ev) cudaEventDestroy(e);
     for (int g = 0; g < 2; ++g)
         if (gexec[g] && (g == 0 || gexec[1] != gexec[0])) cudaGraphExecDestroy(gexec[g]);
     for (auto &e : evs) cudaEventDestroy(e);
     count_launches(launches + 1);
+    if (use_lz) check_tensor_core_status(c, st);
     if (prof) {
         unsigned long long pts[3];
         RPA_CUDA(cudaMemcpy(pts, c.d_prof_points, sizeof pts, cudaMemcpyDeviceToHost));

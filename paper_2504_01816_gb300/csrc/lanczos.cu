@@ -256,6 +256,8 @@ template <typename T> struct Shared {
     int next;                            // its first place that no warp has taken
     unsigned opened;                     // jobs whose coefficients are there
     int item[2], flag;
+    unsigned gone;                       // a wait ran out (wait_lost; 0: none did)
+    int taken;                           // on chip: the system taken last (first block)
     int nto, to[4 * 12];                 // the copies that fill the neighbours' halos
     unsigned expect;                     // bytes that arrive in this block's halo
     LanczosArgs<T> A;                    // for the functions off the hot path
@@ -342,8 +344,40 @@ __device__ __forceinline__ void put(T *own, int gx, int nvx, int nx, const Pk<T>
     }
 }
 
+// A wait ran out.  The threads of a block (on chip) or of a cluster (streaming: its blocks meet at cluster barriers) have
+// to go on alike: they end the solve when they next decide on it, behind a barrier (`left`), start no other
+// (start_part), and leave the launch before the next system.  The mark is the number of reductions (ng)
+// behind that barrier: a decision counts the marks up to its own number only, so that one made meanwhile by a
+// thread that is ahead does not divide those that still have to decide.
+template <typename T> __device__ __noinline__ void wait_lost(unsigned mark, int ncl) {
+    Shared<T> &S = sh<T>();
+    atomicExch(S.A.err, 2);
+    if (ncl == 0) atomicCAS(&S.gone, 0u, mark);          // this block; the first mark stands
+    for (int t = 0; t < ncl; ++t) {
+        unsigned old;
+        asm volatile("atom.relaxed.cluster.shared::cluster.cas.b32 %0, [%1], 0, %2;"
+                     : "=r"(old)
+                     : "r"(map_rank((unsigned)__cvta_generic_to_shared(&S.gone), t)), "r"(mark)
+                     : "memory");
+    }
+}
+template <typename T> __device__ __forceinline__ bool left(unsigned ng) {
+    const unsigned d = *(volatile unsigned *)&sh<T>().gone;
+    return d != 0 && d <= ng;
+}
+
 // Barrier of the threads that iterate (the flush warps run beside them).
 __device__ __forceinline__ void main_sync(int nmain) { asm volatile("bar.sync 1, %0;" ::"r"(nmain) : "memory"); }
+// The same, and whether any of them says so.
+__device__ __forceinline__ bool main_any(int nmain, bool say) {
+    int r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.s32 p, %2, 0;\n bar.red.or.pred q, 1, %1, p;\n selp.s32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(nmain), "r"((int)say)
+        : "memory");
+    return r != 0;
+}
 // The block's own planes are stored: before the bulk copies read them.
 __device__ __forceinline__ void planes_stored(int nmain) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -380,9 +414,9 @@ __device__ __forceinline__ void keep_wait() { asm volatile("cp.async.bulk.wait_g
 // sends its sums to all (st.async, which counts on the receiver's barrier) and waits for all.  A block
 // sends only after all its threads are done with the stencil, so the wait also says that no block reads
 // its halo any more.  The sums alternate between two buffers and barriers: a block may be one
-// reduction ahead of another, never two.
+// reduction ahead of another, never two.  tell: the blocks told of a lost wait (wait_lost).
 template <typename T>
-__device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int nmain, int *err) {
+__device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int nmain, int tell) {
     Shared<T> &S = sh<T>();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = nmain >> 5;
     T v[3] = {a, b, c};
@@ -411,7 +445,7 @@ __device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, in
                       v[0], v[1], v[2]);
         __syncwarp();
     }
-    if (!mbar_wait(pb, (ng >> 1) & 1)) atomicExch(err, 2);
+    if (!mbar_wait(pb, (ng >> 1) & 1)) wait_lost<T>(ng + 1, tell);
     ++ng;
 }
 template <typename T> __device__ __forceinline__ void sum_parts(unsigned ng, int ncl, T &a, T &b, T &c) {   // after gather3
@@ -481,8 +515,13 @@ template <typename T> __device__ __noinline__ void start_state(T a, T b, T c, do
 
 // Start of part pt of slot s's solve (every thread): false if there is nothing to solve for (uniform over
 // the cluster), else v_0 = f_re Re(r) + f_im Im(r).
-template <typename T> __device__ __noinline__ bool start_part(const LanczosArgs<T> &A, int s, int pt, bool scalar, T &f_re, T &f_im) {
+template <typename T> __device__ __noinline__ bool start_part(const LanczosArgs<T> &A, int s, int pt, bool scalar, unsigned ng, T &f_re,
+                                                                T &f_im) {
     Shared<T> &S = sh<T>();
+    if (left<T>(ng)) {                                   // no solve, and the system has failed
+        if (scalar) S.F.fail = 3;
+        return false;
+    }
     const Slot &sl = A.slots[s];
     const double thr_all = A.mixed ? fmax(A.inner_tol * sl.ref_norm, 0.3 * A.tol * sl.bnorm * sl.scale)
                                    : A.tol * sl.bnorm;
@@ -524,6 +563,16 @@ template <typename T> __device__ __noinline__ void end_state(const LanczosArgs<T
         sl.status = F.fail == 0 ? RPA_OK : F.fail == 1 ? RPA_ERR_NOT_CONVERGED : RPA_ERR_BREAKDOWN;
         sl.phase = kFinished;
     }
+}
+
+// A wait ran out, in this launch or before it: the call fails (err is set) and its systems end unsolved, so that the
+// queue does.  A slot that no cluster goes on with, and every system that none has taken yet.
+template <typename T> __device__ __noinline__ void fail_slot(const LanczosArgs<T> &A, int s) {
+    A.slots[s].status = RPA_ERR_CUDA;
+    A.slots[s].phase = kFinished;
+}
+template <typename T> __device__ __noinline__ void fail_rest(const LanczosArgs<T> &A, int n_items) {
+    for (int it; (it = atomicAdd(A.grab, 1)) < n_items;) fail_slot(A, A.list[n_items - 1 - it]);
 }
 
 // The thread's sums of Re(r)^2, Im(r)^2 and Re(r) Im(r) over its points of slot s.
@@ -769,28 +818,28 @@ template <typename T, int ZC> __device__ __forceinline__ void finish_job(int nma
     take_places<T, ZC, 2>();
     main_sync(nmain);
 }
-// The scalar lane then: the flush warps are done with it too (njobs posted so far).
-template <typename T> __device__ __forceinline__ void jobs_done(unsigned njobs) {
-    Shared<T> &S = sh<T>();
-    if (njobs > 0 && !mbar_wait((unsigned)__cvta_generic_to_shared(&S.job_done), (njobs - 1) & 1)) atomicExch(S.A.err, 2);
+// The scalar lane then: the flush warps are done with it too (njobs posted so far).  False where the wait ran out.
+template <typename T> __device__ __forceinline__ bool jobs_done(unsigned njobs, unsigned ng) {
+    const bool ok = njobs == 0 || mbar_wait((unsigned)__cvta_generic_to_shared(&sh<T>().job_done), (njobs - 1) & 1);
+    if (!ok) wait_lost<T>(ng + 1, 0);
+    return ok;
 }
-// ... and the next.
-template <typename T> __device__ __forceinline__ void post_job(const Job &J, unsigned &njobs) {
+// ... and the next (not posted where the wait ran out: the flush warps still read the last).
+template <typename T> __device__ __forceinline__ void post_job(const Job &J, unsigned &njobs, unsigned ng) {
     Shared<T> &S = sh<T>();
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");    // the history is written
-    jobs_done<T>(njobs);
+    if (!jobs_done<T>(njobs, ng)) return;
     S.job = J;
     ++njobs;
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"((unsigned)__cvta_generic_to_shared(&S.job_full)) : "memory");
 }
 
 // The history is full: its sum into x, the direction handed over, by the threads that iterate.
-template <typename T, int ZC> __device__ __noinline__ void flush_full(const Job &J, unsigned njobs, int nmain) {
+template <typename T, int ZC> __device__ __noinline__ void flush_full(const Job &J, unsigned njobs, unsigned ng, int nmain) {
     finish_job<T, ZC>(nmain);
     if ((int)threadIdx.x == nmain - 32) {
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-        jobs_done<T>(njobs);
-        coefficients<T>(J.buf, J.n, J.er, J.ei);
+        if (jobs_done<T>(njobs, ng)) coefficients<T>(J.buf, J.n, J.er, J.ei);
     }
     main_sync(nmain);
     const int rank = (int)(blockIdx.x % (unsigned)sh<T>().A.ncl), nz = sh<T>().A.nz, ncl = sh<T>().A.ncl;
@@ -798,6 +847,24 @@ template <typename T, int ZC> __device__ __noinline__ void flush_full(const Job 
     for (int e = threadIdx.x; e < total; e += 2 * nmain) add_history<T, ZC, true, 2>(J, e, nmain);
     __threadfence();
     main_sync(nmain);
+}
+
+// The end of a block that leaves after a wait has run out, by the scalar lane: the system taken last is given up,
+// the block's own copies are waited for, the flush warps sent home (they end by themselves where even their
+// last job's end does not come), and what is on its way to this block, sent before another one left, is given
+// half a millisecond to arrive.  The other blocks of the cluster leave likewise: they wait for this one's
+// sums, each wait for a second at most.
+template <typename T> __device__ __noinline__ void leave(int rank, int n_items, unsigned njobs, unsigned ng) {
+    Shared<T> &S = sh<T>();
+    const LanczosArgs<T> &A = S.A;
+    if (rank == 0) {
+        if (S.taken < n_items) fail_slot(A, A.list[n_items - 1 - S.taken]);
+        fail_rest(A, n_items);
+    }
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    post_job<T>(Job{-1, 0, 0, 0, 0.0, 0.0}, njobs, ng);
+    const long long t0 = clock64();
+    while (clock64() - t0 < 1000000LL) {}
 }
 
 // Once a block: its slab cleared, barriers, the halo copies, V_loc by threads.
@@ -824,6 +891,8 @@ template <typename T, int ZC> __device__ __noinline__ void block_setup(const Lan
         mbar_init(&S.job_full);
         mbar_init(&S.job_done);
         S.next = 1 << 30;                                // no job
+        S.gone = 0;
+        S.taken = 1 << 30;
         S.opened = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // the copies: this block's planes [g0, g1) that lie in the halo of rank t (periodic: of its image)
@@ -883,7 +952,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
     // the longest solves, first); every block receives its number in item[m & 1]
     auto fetch = [&](unsigned m) {
         if (G.rank == 0) {
-            const int it = atomicAdd(A.grab, 1);
+            const int err = *(volatile int *)A.err;
+            int it = atomicAdd(A.grab, 1);
+            if (err) {                                   // no more
+                if (it < n_items) fail_slot(A, A.list[n_items - 1 - it]);
+                fail_rest(A, n_items);
+                it = 1 << 30;
+            }
+            S.taken = it;
             for (int t = 0; t < ncl; ++t)
                 asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
                                  map_rank((unsigned)__cvta_generic_to_shared(&S.item[m & 1]), t)),
@@ -902,9 +978,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
     }
     if (scalar) fetch(0);
     for (;; ++ns) {
-        if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.ibar[ns & 1]), (ns >> 1) & 1)) {
-            atomicExch(A.err, 2);
-            break;
+        const bool here = mbar_wait((unsigned)__cvta_generic_to_shared(&S.ibar[ns & 1]), (ns >> 1) & 1);
+        if (!here) wait_lost<T>(ng + 1, 0);
+        if (main_any(nmain, !here || left<T>(ng))) {    // the item is not to be read, or a solve has ended so
+            if (scalar) leave<T>(G.rank, n_items, njobs, ng);
+            cluster_barrier();
+            return;
         }
         const int it = S.item[ns & 1];
         if (it >= n_items) break;
@@ -913,8 +992,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
         {
             T rr, ii, ri;
             start_sums<T, ZC>(s, rr, ii, ri);
-            gather3(rr, ii, ri, ng, ncl, G.rank, nmain, A.err);
-            if (scalar) {
+            gather3(rr, ii, ri, ng, ncl, G.rank, nmain, 0);
+            if (scalar && !left<T>(ng)) {
                 fetch(ns + 1);                           // every block has read the number before this one
                 T a, b, c;
                 sum_parts(ng, ncl, a, b, c);
@@ -924,7 +1003,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
         }
         for (int pt = 0; pt < 2; ++pt) {
             T f_re, f_im;
-            if (!start_part<T>(A, s, pt, scalar, f_re, f_im)) continue;
+            if (!start_part<T>(A, s, pt, scalar, ng, f_re, f_im)) continue;
             start_vector<T, ZC, MODE>(s, f_re, f_im);
             planes_stored(nmain);
             if (scalar) {
@@ -948,6 +1027,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                 asm volatile("" : "+r"(o0), "+r"(o1));
                 if (scalar) {
                     if (k > kb) factor<T>(buf, k - 1 - kb, k, A.maxit);
+                    if (left<T>(ng)) {
+                        S.F.fail = 3;
+                        S.flag = 4;
+                    }
                     keep_wait();
                 }
                 // ---- u = B v_k - c_k v_{k-1} (shifted), sums v.v, u.v, u.u.  The x and y neighbours and the
@@ -1026,7 +1109,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                         }
                     }
                 }
-                if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.bar), phase)) atomicExch(A.err, 2);
+                if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.bar), phase)) wait_lost<T>(ng + 1, 0);
                 phase ^= 1u;
                 if (G.unit) {
 #pragma unroll
@@ -1061,8 +1144,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                     suv = t1.sum();
                     suu = t2.sum();
                 }
-                gather3(svv, suv, suu, ng, ncl, G.rank, nmain, A.err);
-                if (k > kb && S.flag) {                  // the last step ended the solve
+                gather3(svv, suv, suu, ng, ncl, G.rank, nmain, 0);
+                if (S.flag) {                            // the last step ended the solve (k = kb: a lost wait)
                     n = k - kb;
                     break;
                 }
@@ -1106,7 +1189,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                                         }
                                 }
                         }
-                        gather3((T)0, t1.sum(), t2.sum(), ng, ncl, G.rank, nmain, A.err);
+                        gather3((T)0, t1.sum(), t2.sum(), ng, ncl, G.rank, nmain, 0);
                         if (scalar) {
                             T a, b, c;
                             sum_parts(ng, ncl, a, b, c);
@@ -1156,7 +1239,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                     n = k - kb;
                     if (S.flag) break;
                     flush_full<T, ZC>(Job{s, n, buf, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]},
-                                      njobs, nmain);
+                                      njobs, ng, nmain);
                     have_p = true;
                     kb = k;
                     const Work<T, ZC> K(A);
@@ -1167,7 +1250,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                         acc[z][1] = pk_load_l2(hl + G.c1 + z * A.plane);
                     }
                 }
-                if (scalar) {
+                if (scalar && !left<T>(ng)) {            // (a lost halo's barrier is not armed again)
                     const Work<T, ZC> K(A);
                     send_halos(slab);
                     keep(slab, K.H + buf * K.buf, K.hvec, k - kb, G.nzl, A.plane);
@@ -1176,8 +1259,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
             finish_job<T, ZC>(nmain);
             if (S.flag < 4) {                            // nothing is kept of a solve that went non-finite
                 if (scalar)
-                    post_job<T>(Job{s, n, buf, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]}, njobs);
+                    post_job<T>(Job{s, n, buf, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1]}, njobs, ng);
                 buf ^= 1;                                // free again: its last job ended before this one was posted
+            } else if (scalar) {
+                asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // its places are written anew
             }
             main_sync(nmain);                            // no thread still reads the flag
         }
@@ -1188,7 +1273,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
         for (int i = 0; i < 1 << 20 && *(volatile unsigned *)&S.opened != njobs; ++i) {}
     main_sync(nmain);
     finish_job<T, ZC>(nmain);
-    if (scalar) post_job<T>(Job{-1, 0, 0, 0, 0.0, 0.0}, njobs);
+    if (scalar) post_job<T>(Job{-1, 0, 0, 0, 0.0, 0.0}, njobs, ng);
     cluster_barrier();                                  // no block leaves while another may write its memory
 }
 
@@ -1270,7 +1355,7 @@ struct Stages {
     __device__ __forceinline__ unsigned bar(int s) const {
         return (unsigned)__cvta_generic_to_shared(&sh<float>().full[0]) + 8u * (unsigned)s;
     }
-    __device__ __forceinline__ void wait(int *err) {
+    __device__ __forceinline__ void wait(int *err) {   // !ok: no more copies; the scalar lane tells the cluster
         if (ok && !mbar_wait(bar(st), (ph >> st) & 1)) {
             ok = false;
             atomicExch(err, 2);
@@ -1364,7 +1449,7 @@ __device__ __noinline__ Stages stream_flush(const StreamArgs *args, int s, int n
     };
     int iz = 0, ij = 0, iq = G4.st;      // the next to issue (the scalar lane's)
     auto issue_next = [&]() {
-        if (iz >= npair) return;
+        if (iz >= npair || !G4.ok) return;
         issue(iz, ij, iq);
         if (++ij == n) {
             ij = 0;
@@ -1487,6 +1572,8 @@ __global__ void __launch_bounds__(MAXT, 1)
     if (scalar) {
         for (int q = 0; q < 2; ++q) mbar_init(&S.pbar[q]);
         for (int q = 0; q < kStages; ++q) mbar_init(&S.full[q]);
+        S.gone = 0;
+        S.A.err = A.L.err;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     before_bulk();                                       // the zeros, before bulk copies into the same memory
@@ -1503,7 +1590,10 @@ __global__ void __launch_bounds__(MAXT, 1)
     for (;;) {
         if (G.rank == 0 && tid < ncl) {
             int it = 0;
-            if (tid == 0) it = atomicAdd(A.L.grab, 1);
+            if (tid == 0) {
+                if (*(volatile int *)A.L.err) fail_rest(A.L, n_items);   // no more
+                it = atomicAdd(A.L.grab, 1);
+            }
             it = __shfl_sync((1u << ncl) - 1u, it, 0);
             asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(
                              map_rank((unsigned)__cvta_generic_to_shared(&S.item[0]), tid)),
@@ -1516,17 +1606,17 @@ __global__ void __launch_bounds__(MAXT, 1)
         {
             float rr, ii, ri;
             stream_start<R>(&A, s, 0.f, 0.f, false, rr, ii, ri);
-            gather3(rr, ii, ri, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
+            gather3(rr, ii, ri, ng, ncl, G.rank, (int)blockDim.x, ncl);
             if (scalar) {
                 float a, b, c;
                 sum_parts(ng, ncl, a, b, c);
                 start_state(a, b, c, A.L.d0 + A.L.slots[s].shift_re, A.L.slots[s].shift_im);
             }
-            __syncthreads();
+            cluster_barrier();                           // and every block knows of a lost wait (start_part)
         }
         for (int pt = 0; pt < 2; ++pt) {
             float f_re, f_im;
-            if (!start_part<float>(A.L, s, pt, scalar, f_re, f_im)) continue;
+            if (!start_part<float>(A.L, s, pt, scalar, ng, f_re, f_im)) continue;
             {
                 float d0, d1, d2;
                 stream_start<R>(&A, s, f_re, f_im, true, d0, d1, d2);
@@ -1557,7 +1647,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                     }
                     bulk_load(to + 2 * su, A.v + f * pl + (size_t)G.y0 * A.px, G.rows * mb, G4.bar(q));
                 };
-                if (scalar) {
+                if (scalar && G4.ok) {
                     before_bulk();
                     for (int i = 0, q = G4.st; i < min(depth, nz + 2 * GH); ++i, q = q + 1 == depth ? 0 : q + 1) issue(i - GH, q);
                 }
@@ -1629,7 +1719,7 @@ __global__ void __launch_bounds__(MAXT, 1)
                     const int freed = G4.st;
                     G4.next(depth);
                     __syncthreads();                     // the plane is there, the stage is read
-                    if (scalar && f + depth < nz + GH) issue(f + depth, freed);
+                    if (scalar && G4.ok && f + depth < nz + GH) issue(f + depth, freed);
                     if (!G.own) continue;
                     if (!real) {                         // its part along z alone
                         P u = acc[0][0];
@@ -1697,7 +1787,7 @@ __global__ void __launch_bounds__(MAXT, 1)
 #pragma unroll
                     for (int j = 0; j < kRadius; ++j) put_u(acc[j]);
                 before_bulk();                           // u and v_k, for the next sweep's copies
-                gather3(svv.x + svv.y, suv.x + suv.y, suu.x + suu.y, ng, ncl, G.rank, (int)blockDim.x, A.L.err);
+                gather3(svv.x + svv.y, suv.x + suv.y, suu.x + suu.y, ng, ncl, G.rank, (int)blockDim.x, ncl);
                 {
                     float a, b, c;
                     sum_parts(ng, ncl, a, b, c);
@@ -1712,13 +1802,15 @@ __global__ void __launch_bounds__(MAXT, 1)
                     S.F.ck = (double)cc;
                     S.F.ig = (double)ig;
                     factor<float>(0, k - 1 - kb, k, A.L.maxit);
+                    if (!G4.ok) wait_lost<float>(ng, ncl);
                     if (A.L.prof && G.rank == 0) atomicAdd(A.L.prof + 1, (unsigned long long)A.L.nd);
                 }
                 cc = ig > 0.f ? 1.f / ig : 0.f;
                 dg -= ap;
                 cluster_barrier();                       // u and v_k of every band are written; the decision is taken
                 n = k - kb;
-                if (S.flag) break;
+                // (a vote: as a plain condition it costs the plane loop 8 registers and 2.5% of the call)
+                if (__any_sync(0xffffffffu, S.flag != 0 || left<float>(ng))) break;
                 if (n == A.L.hist) {                     // the history is full: into x and p
                     G4 = stream_flush<R>(&A, s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1], G4);
                     have_p = true;
@@ -1730,6 +1822,10 @@ __global__ void __launch_bounds__(MAXT, 1)
             cluster_barrier();                           // no thread still reads the flag or this part's vectors
         }
         if (scalar && G.rank == 0) end_state(A.L, s);
+    }
+    if (!G4.ok) {                                        // planes that were asked for may still arrive: a second more
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000000LL) {}
     }
     cluster_barrier();
 }
