@@ -2985,7 +2985,14 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         c.lz_key[2] = c.batch_load;
     }
     // (their vectors take up to 8 GB: where that is not to be had, the kernels that do without run)
-    const bool use_lz = c.lz_ok && !precond && !c.keep_cocg && (want == 0 || want == 4) && c.lanczos_ws.room(c.lz_plan.ws_bytes);
+    // FP64 without P_c and with omega at rounding of the spectrum: the system is singular (its right-hand side has the
+    // orbital whose energy is the shift), the solution is that orbital over rounding, and the residual that the Lanczos
+    // factors imply says nothing of it (20 x 17 x 16, omega = 0, tol 1e-8: "converged" at 4e-2, where COCG's
+    // recursive residual does not get there).  The mixed form's refinement sees it.
+    double top = c.coef.a[0];
+    for (int k = 1; k <= kRadius; ++k) top += 2.0 * std::fabs(c.coef.a[k]);
+    const bool singular = !mixed && !sp.Tc && std::fabs(sp.omega) < 1e-15 * 3.0 * top;
+    const bool use_lz = c.lz_ok && !precond && !singular && !c.keep_cocg && (want == 0 || want == 4) && c.lanczos_ws.room(c.lz_plan.ws_bytes);
     const bool use_ring = !use_lz && mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
     const int variant = (want >= 1 && want <= 3 && !(per && want == 3)) ? want - 1 : 0;
     const PaShape shape = mixed ? kPaShapes32[variant] : kPaShape64;
