@@ -49,15 +49,63 @@ void allow_dynamic_smem(const void *kernel, size_t need) {
         RPA_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)avail));
 }
 
+namespace {
+
+std::mutex g_lanczos_mutex;              // guards the list and every context's lanczos_ws, lz_held
+std::vector<Ctx *> g_lanczos_owners;     // contexts that have asked for a Lanczos workspace
+
+// Frees the current device's Lanczos workspaces that no queue holds; whether there was one.
+bool give_back_workspaces() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lk(g_lanczos_mutex);
+    bool any = false;
+    for (Ctx *c : g_lanczos_owners) {
+        if (c->device != dev || c->lz_held || !c->lanczos_ws.ptr) continue;
+        if (c->lz_done && cudaEventSynchronize(c->lz_done) != cudaSuccess) return false;
+        c->lanczos_ws.release();
+        any = true;
+    }
+    return any;
+}
+
+}  // namespace
+
+cudaError_t device_malloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    (void)cudaGetLastError();
+    if (!give_back_workspaces()) return e;
+    e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+
+bool LanczosHold::take(size_t need) {
+    std::lock_guard<std::mutex> lk(g_lanczos_mutex);
+    if (!c.lz_done) RPA_CUDA(cudaEventCreateWithFlags(&c.lz_done, cudaEventDisableTiming));
+    if (!c.lanczos_ws.room(need)) return false;
+    if (std::find(g_lanczos_owners.begin(), g_lanczos_owners.end(), &c) == g_lanczos_owners.end())
+        g_lanczos_owners.push_back(&c);
+    held = c.lz_held = true;
+    return true;
+}
+
+LanczosHold::~LanczosHold() {
+    if (!held) return;
+    std::lock_guard<std::mutex> lk(g_lanczos_mutex);
+    if (cudaEventRecord(c.lz_done, s) != cudaSuccess) (void)cudaStreamSynchronize(s);
+    c.lz_held = false;
+}
+
 void *DevBuf::ensure(size_t need) {
     if (need <= bytes && ptr) return ptr;
     release();
     size_t want = std::max(need, (size_t)256);
-    cudaError_t e = cudaMalloc(&ptr, want);
+    cudaError_t e = device_malloc(&ptr, want);
     if (e != cudaSuccess) {
         ptr = nullptr;
         bytes = 0;
-        (void)cudaGetLastError();
         fail(RPA_ERR_OOM, "cudaMalloc of %zu bytes failed: %s", want, cudaGetErrorString(e));
     }
     bytes = want;
@@ -88,6 +136,11 @@ void DevBuf::release() {
 }
 
 Ctx::~Ctx() {
+    {
+        std::lock_guard<std::mutex> lk(g_lanczos_mutex);
+        g_lanczos_owners.erase(std::remove(g_lanczos_owners.begin(), g_lanczos_owners.end(), this), g_lanczos_owners.end());
+    }
+    if (lz_done) cudaEventDestroy(lz_done);
     cudaFree(vloc64);
     cudaFree(vloc32);
     cudaFree(vloc_lo);
@@ -404,12 +457,12 @@ rpa_status rpa_setup(rpa_ctx **out, int nx, int ny, int nz, double h, int fd_ord
             }
             c.coef.a[0] = -w0 / (2.0 * h * h);
             c.eps.assign(eps_host, eps_host + n_s);
-            RPA_CUDA(cudaMalloc(&c.vloc64, sizeof(double) * nd));
-            RPA_CUDA(cudaMalloc(&c.vloc32, sizeof(float) * nd));
-            RPA_CUDA(cudaMalloc(&c.vloc_lo, sizeof(float) * nd));
-            RPA_CUDA(cudaMalloc(&c.psi64, sizeof(double) * nd * n_s));
-            RPA_CUDA(cudaMalloc(&c.psi32, sizeof(float) * nd * n_s));
-            RPA_CUDA(cudaMalloc(&c.eps_dev, sizeof(double) * n_s));
+            RPA_CUDA(device_malloc(&c.vloc64, sizeof(double) * nd));
+            RPA_CUDA(device_malloc(&c.vloc32, sizeof(float) * nd));
+            RPA_CUDA(device_malloc(&c.vloc_lo, sizeof(float) * nd));
+            RPA_CUDA(device_malloc(&c.psi64, sizeof(double) * nd * n_s));
+            RPA_CUDA(device_malloc(&c.psi32, sizeof(float) * nd * n_s));
+            RPA_CUDA(device_malloc(&c.eps_dev, sizeof(double) * n_s));
             RPA_CUDA(cudaMemcpyAsync(c.vloc64, vloc_dev, sizeof(double) * nd, cudaMemcpyDeviceToDevice, s));
             RPA_CUDA(cudaMemcpyAsync(c.psi64, psi_dev, sizeof(double) * nd * n_s, cudaMemcpyDeviceToDevice, s));
             RPA_CUDA(cudaMemcpyAsync(c.eps_dev, eps_host, sizeof(double) * n_s, cudaMemcpyHostToDevice, s));
@@ -418,14 +471,14 @@ rpa_status rpa_setup(rpa_ctx **out, int nx, int ny, int nz, double h, int fd_ord
             k_to_float<<<(unsigned)((nd * n_s + 255) / 256), 256, 0, s>>>(c.psi64, c.psi32, nd * n_s);
             RPA_LAUNCH("setup");
             RPA_CUDA(cudaMallocHost((void **)&c.h_count, 8 * sizeof(int)));
-            RPA_CUDA(cudaMalloc(&c.d_tc_err, sizeof(int)));
+            RPA_CUDA(device_malloc(&c.d_tc_err, sizeof(int)));
             RPA_CUDA(cudaMemsetAsync(c.d_tc_err, 0, sizeof(int), s));
-            RPA_CUDA(cudaMalloc(&c.d_qstats, sizeof(QueueStats)));
+            RPA_CUDA(device_malloc(&c.d_qstats, sizeof(QueueStats)));
             RPA_CUDA(cudaMemsetAsync(c.d_qstats, 0, sizeof(QueueStats), s));
-            RPA_CUDA(cudaMalloc(&c.d_loop, sizeof(int)));
+            RPA_CUDA(device_malloc(&c.d_loop, sizeof(int)));
             RPA_CUDA(cudaMallocHost((void **)&c.h_rb, kReadBackBytes));
             for (auto &e : c.ev_apply) RPA_CUDA(cudaEventCreate(&e));
-            RPA_CUDA(cudaMalloc(&c.d_prof_points, sizeof(unsigned long long) * RPA_PROF_SLOTS));
+            RPA_CUDA(device_malloc(&c.d_prof_points, sizeof(unsigned long long) * RPA_PROF_SLOTS));
             RPA_CUDA(cudaStreamCreateWithFlags(&c.cap_stream, cudaStreamNonBlocking));
             {
                 const char *g = std::getenv("RPA_GRAPHS");

@@ -2895,10 +2895,11 @@ Tiles pick_tiles(int nx, int ny, int max_threads, bool pairs = false) {
 
 int choose_slots(const Ctx &c, int nsys) {
     if (c.opt.batch_systems > 0) return std::max(1, std::min(nsys, c.opt.batch_systems));
-    // All systems of a call in flight when they fit in 8 GB of slot storage; otherwise as many
-    // as fit (the queue refills the slots).
+    // All systems of a call in flight when they fit in 8 GB of slot storage (a batch's contexts together:
+    // each its share by systems); otherwise as many as fit (the queue refills the slots).
     const double slot_bytes = (double)c.nd * (c.opt.prec == RPA_MIXED ? 72.0 : 96.0);
-    long long S = std::max(1LL, (long long)(8.0e9 / slot_bytes));
+    const double share = c.batch_load > nsys ? (double)nsys / c.batch_load : 1.0;
+    long long S = std::max(1LL, (long long)(8.0e9 * share / slot_bytes));
     return (int)std::min<long long>(S, nsys);
 }
 
@@ -2976,24 +2977,6 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
                        (!ring1 && cluster_plan(c.nx, c.ny, smem_optin, false, ncl, band_pairs)));
     const RingFn ring_fn = ws ? (even_nx ? k_cocg_ring_ws<true> : k_cocg_ring_ws<false>)
                               : clus ? (even_nx ? k_cocg_ring_cl<true> : k_cocg_ring_cl<false>) : ring1_fn;
-    // systems that fit on chip: the Lanczos kernel
-    const int lz_form = c.opt.prec + 16 * (c.opt.precondition != 0);
-    if (c.lz_key[0] != S || c.lz_key[1] != lz_form || c.lz_key[2] != c.batch_load) {
-        c.lz_ok = lanczos_plan(c, S, c.lz_plan);
-        c.lz_key[0] = S;
-        c.lz_key[1] = lz_form;
-        c.lz_key[2] = c.batch_load;
-    }
-    // (their vectors take up to 8 GB: where that is not to be had, the kernels that do without run)
-    // FP64 without P_c and with omega at rounding of the spectrum: the system is singular (its right-hand side has the
-    // orbital whose energy is the shift), the solution is that orbital over rounding, and the residual that the Lanczos
-    // factors imply says nothing of it (20 x 17 x 16, omega = 0, tol 1e-8: "converged" at 4e-2, where COCG's
-    // recursive residual does not get there).  The mixed form's refinement sees it.
-    double top = c.coef.a[0];
-    for (int k = 1; k <= kRadius; ++k) top += 2.0 * std::fabs(c.coef.a[k]);
-    const bool singular = !mixed && !sp.Tc && std::fabs(sp.omega) < 1e-15 * 3.0 * top;
-    const bool use_lz = c.lz_ok && !precond && !singular && !c.keep_cocg && (want == 0 || want == 4) && c.lanczos_ws.room(c.lz_plan.ws_bytes);
-    const bool use_ring = !use_lz && mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
     const int variant = (want >= 1 && want <= 3 && !(per && want == 3)) ? want - 1 : 0;
     const PaShape shape = mixed ? kPaShapes32[variant] : kPaShape64;
     Tiles tl = pick_tiles(c.nx, c.ny, shape.max_threads, shape.pairs != 0);
@@ -3057,7 +3040,6 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     P.cproject = mixed && sp.Tc != nullptr;
     P.project = c.opt.project_solution != 0 || sp.grad != nullptr || (P.cproject && c.opt.tol < 1e-9);
     P.proj_re_only = sp.drho != nullptr && sp.grad == nullptr;
-    P.norm_only = use_lz || use_ring;
     P.ns = c.ns;
     P.psi = c.psi64;
     P.psi32 = c.psi32;
@@ -3068,6 +3050,27 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
         P.partP = pp + (size_t)S * c.ns * 2;
         P.Tp32 = (float *)(P.partP + (size_t)S * c.ns * 2 * nblk);
     }
+    // systems that fit on chip: the Lanczos kernel
+    const int lz_form = c.opt.prec + 16 * (c.opt.precondition != 0);
+    if (c.lz_key[0] != S || c.lz_key[1] != lz_form || c.lz_key[2] != c.batch_load) {
+        c.lz_ok = lanczos_plan(c, S, c.lz_plan);
+        c.lz_key[0] = S;
+        c.lz_key[1] = lz_form;
+        c.lz_key[2] = c.batch_load;
+    }
+    // (their vectors take up to 8 GB: where that is not to be had, the kernels that do without run; asked for
+    // last, when the queue has all that it cannot do without)
+    LanczosHold lz_hold(c, st);
+    // FP64 without P_c and with omega at rounding of the spectrum: the system is singular (its right-hand side has the
+    // orbital whose energy is the shift), the solution is that orbital over rounding, and the residual that the Lanczos
+    // factors imply says nothing of it (20 x 17 x 16, omega = 0, tol 1e-8: "converged" at 4e-2, where COCG's
+    // recursive residual does not get there).  The mixed form's refinement sees it.
+    double top = c.coef.a[0];
+    for (int k = 1; k <= kRadius; ++k) top += 2.0 * std::fabs(c.coef.a[k]);
+    const bool singular = !mixed && !sp.Tc && std::fabs(sp.omega) < 1e-15 * 3.0 * top;
+    const bool use_lz = c.lz_ok && !precond && !singular && !c.keep_cocg && (want == 0 || want == 4) && lz_hold.take(c.lz_plan.ws_bytes);
+    const bool use_ring = !use_lz && mixed && !precond && (want == 0 || want >= 4) && (ws || clus || ring1);
+    P.norm_only = use_lz || use_ring;
 
     // per parity: the stencil kernel's and the update kernel's views of P
     IterArgs ia_pa[2], ia_b[2];

@@ -271,16 +271,16 @@ void coulomb_setup(Ctx &c) {
         const std::vector<double> qp = by_parity(Q, n);
         std::vector<double> both(Q);                     // one allocation and copy
         both.insert(both.end(), qp.begin(), qp.end());
-        RPA_CUDA(cudaMalloc(&c.Q[a], sizeof(double) * both.size()));
+        RPA_CUDA(device_malloc(&c.Q[a], sizeof(double) * both.size()));
         RPA_CUDA(cudaMemcpy(c.Q[a], both.data(), sizeof(double) * both.size(), cudaMemcpyHostToDevice));
         if (!qp.empty()) c.Qpar[a] = c.Q[a] + (size_t)n * n;
         // the same factors for the Laplacian preconditioner of COCG, in FP64 and FP32
         std::vector<float> qf(Q.begin(), Q.end()), mf(mu[a].begin(), mu[a].end());
-        RPA_CUDA(cudaMalloc(&c.mu[a], sizeof(double) * n));
+        RPA_CUDA(device_malloc(&c.mu[a], sizeof(double) * n));
         RPA_CUDA(cudaMemcpy(c.mu[a], mu[a].data(), sizeof(double) * n, cudaMemcpyHostToDevice));
-        RPA_CUDA(cudaMalloc(&c.Qf[a], sizeof(float) * n * n));
+        RPA_CUDA(device_malloc(&c.Qf[a], sizeof(float) * n * n));
         RPA_CUDA(cudaMemcpy(c.Qf[a], qf.data(), sizeof(float) * n * n, cudaMemcpyHostToDevice));
-        RPA_CUDA(cudaMalloc(&c.muf[a], sizeof(float) * n));
+        RPA_CUDA(device_malloc(&c.muf[a], sizeof(float) * n));
         RPA_CUDA(cudaMemcpy(c.muf[a], mf.data(), sizeof(float) * n, cudaMemcpyHostToDevice));
     }
     std::vector<double> lam((size_t)c.nd);
@@ -288,7 +288,7 @@ void coulomb_setup(Ctx &c) {
         for (int j = 0; j < c.ny; ++j)
             for (int i = 0; i < c.nx; ++i)
                 lam[(size_t)i + (size_t)c.nx * (j + (size_t)c.ny * k)] = mu[0][i] + mu[1][j] + mu[2][k];
-    RPA_CUDA(cudaMalloc(&c.lam, sizeof(double) * c.nd));
+    RPA_CUDA(device_malloc(&c.lam, sizeof(double) * c.nd));
     RPA_CUDA(cudaMemcpy(c.lam, lam.data(), sizeof(double) * c.nd, cudaMemcpyHostToDevice));
 }
 

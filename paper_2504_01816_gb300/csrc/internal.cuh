@@ -40,6 +40,10 @@ void check_cuda(cudaError_t e, const char *what, const char *file, int line);
 #define RPA_CUDA(call) ::rpa::check_cuda((call), #call, __FILE__, __LINE__)
 #define RPA_LAUNCH(what) ::rpa::check_cuda(cudaGetLastError(), what, __FILE__, __LINE__)
 
+// cudaMalloc, again after the Lanczos workspaces that no running queue uses are given back (all contexts').
+cudaError_t device_malloc(void **p, size_t bytes);
+template <typename T> cudaError_t device_malloc(T **p, size_t bytes) { return device_malloc((void **)p, bytes); }
+
 // ------------------------------------------------------------------------------------------
 // Device buffer that only grows.
 // ------------------------------------------------------------------------------------------
@@ -146,7 +150,12 @@ struct Ctx {
     DevBuf coef_buf;              // per-column coefficients of the gradient pass
     DevBuf blockE;                // subspace of the previous iteration (gradient)
     DevBuf dense_scratch;         // split-K partial sums
-    DevBuf lanczos_ws;            // Lanczos vectors of the systems in flight
+    // Lanczos vectors of the systems in flight.  One can do without them (the COCG kernels run): any
+    // allocation of the library that fails takes them back from the contexts whose queue does not hold them
+    // (lz_held; lz_done: the last that did has run on the device), see LanczosHold.
+    DevBuf lanczos_ws;
+    bool lz_held = false;
+    cudaEvent_t lz_done = nullptr;
     LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, form, batch_load}
     int lz_key[3] = {-1, -1, -1};
     bool lz_ok = false;
@@ -196,6 +205,18 @@ void coulomb_apply(Ctx &c, double power, const double *in, double *out, int ncol
 inline bool use_tensor_cores(const Ctx &c) {
     return c.opt.contractions >= 2 || (c.opt.contractions == 0 && c.opt.prec == RPA_MIXED);
 }
+// A queue's hold on its context's Lanczos workspace, from its request (after every other buffer that the queue
+// needs) to the end of the work that the queue has put on its stream.
+struct LanczosHold {
+    Ctx &c;
+    cudaStream_t s;
+    bool held = false;
+    LanczosHold(Ctx &ctx, cudaStream_t st) : c(ctx), s(st) {}
+    LanczosHold(const LanczosHold &) = delete;
+    bool take(size_t bytes);      // false where memory is short
+    ~LanczosHold();
+};
+
 inline bool use_tensor_cores_kronecker(const Ctx &c) {
     return c.opt.contractions == 2 || (c.opt.contractions == 0 && c.opt.prec == RPA_MIXED);
 }
