@@ -673,7 +673,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
         const int zb = zc * tl.zlen, ze = min(nz, zb + tl.zlen);   // planes computed by this item
         const int gx = x0 + lx, gy = y0 + ly;
         const bool own = in_tile && gx < nx && gy < ny;
-        const int col = gy * nx + gx;
+        // the last tile along an axis may reach past it: zero there, on a periodic grid the images of the first
+        // columns, which its last columns' neighbours are
+        const bool have = own || (per && in_tile);
+        const int col = own ? gy * nx + gx : have ? wrap_index(gy, ny) * nx + wrap_index(gx, nx) : 0;
         auto pnew = [&](const C a, const C b) -> C {
             C o;
             o.x = a.x + br * b.x - bi * b.y;
@@ -730,10 +733,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
 #pragma unroll
         for (int m = 0; m < 2 * R + 1; ++m) {
             const int z = zplane(zb + m - R);
-            qv[m] = (own && z >= 0) ? pnew(rs[col + z * plane], po[col + z * plane]) : zero;
+            qv[m] = (have && z >= 0) ? pnew(rs[col + z * plane], po[col + z * plane]) : zero;
         }
         C f1r = zero, f1p = zero;          // raw front of plane z+R+1, consumed at the end of step z
-        if (own && zplane(zb + R + 1) >= 0) {
+        if (have && zplane(zb + R + 1) >= 0) {
             f1r = rs[col + zplane(zb + R + 1) * plane];
             f1p = po[col + zplane(zb + R + 1) * plane];
         }
@@ -766,7 +769,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
                         }
                 }
                 C f2r = zero, f2p = zero;
-                if (own && zplane(z + R + 2) >= 0) {
+                if (have && zplane(z + R + 2) >= 0) {
                     f2r = rs[col + zplane(z + R + 2) * plane];
                     f2p = po[col + zplane(z + R + 2) * plane];
                 }
@@ -797,7 +800,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
 
                 }
                 // the front loaded one plane ago takes the slot of plane z-6
-                qv[u] = (own && zplane(z + R + 1) >= 0) ? pnew(f1r, f1p) : zero;
+                qv[u] = (have && zplane(z + R + 1) >= 0) ? pnew(f1r, f1p) : zero;
                 f1r = f2r;
                 f1p = f2p;
             }
