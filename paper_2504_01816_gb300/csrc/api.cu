@@ -845,7 +845,7 @@ rpa_status rpa_ec_gradient(rpa_ctx *ctx, int n_r, const double *V0_dev, double *
             fail(RPA_ERR_INVALID, "rpa_ec_gradient differentiates the Rayleigh-Ritz energy: set sq_order = 0");
         const int saved = c.opt.project_solution;
         c.opt.project_solution = 1;
-        c.keep_cocg = V_out_dev != nullptr;
+        c.keep_cocg = true;
         try {
             worst = ec_impl(c, n_r, V0_dev, lambdas_host, ec_host, ec_per_omega_host, stats, as_stream(stream),
                             grad_dev, V_out_dev);
