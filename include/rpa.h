@@ -43,6 +43,17 @@
 extern "C" {
 #endif
 
+/* A context keeps the device memory of its largest calls until it is destroyed: up to 8 GB for the
+ * systems in flight (the contexts of a batch together) and up to 4 GB (grids solved on chip) or 8 GB
+ * (streamed) of Lanczos vectors (batches: about 16 GB together).  The Lanczos vectors are optional: a call that finds no
+ * room for them (512 MB stay free) runs the COCG kernels, and a device allocation of the library that
+ * fails takes back those that no running call uses, on all contexts of the device, before it reports
+ * RPA_ERR_OOM.
+ *
+ * How the Lanczos kernels spread a system over blocks, and whether it is solved on chip or streamed, is chosen
+ * by the number of systems in flight (in a batch: of all its contexts).  So a system's sums may be formed
+ * in another order, and its result differ within the tolerance, when it is solved with more or fewer
+ * others, or where memory is short; the same call under the same conditions repeats bit for bit. */
 typedef struct rpa_ctx rpa_ctx;
 
 typedef enum {
@@ -63,7 +74,9 @@ typedef enum {
 typedef struct {
     int prec;                  /* rpa_precision */
     double tol;                /* COCG: stop when ||b - A x||_2 <= tol ||b||_2 (Hermitian norm) */
-    int maxit;                 /* COCG: iteration limit per system (FP64) or per inner solve (mixed) */
+    int maxit;                 /* COCG: iteration limit per system (FP64) or per inner solve (mixed); Lanczos
+                                  kernels: steps per solve of a real right-hand side, of which a mixed
+                                  inner solve after the first has two (its real and imaginary parts) */
     int max_refine;            /* mixed: limit on FP64 residual evaluations per system */
     double inner_tol;          /* mixed: relative residual reduction asked of each FP32 inner solve */
     double eps_c;              /* subspace iteration: stop when |dE_c,m| <= eps_c * n_atoms / n_omega (Ha/atom) */
@@ -92,9 +105,13 @@ typedef struct {
                                   kernel per iteration, one block per system with whole xy planes in
                                   a shared-memory ring (grids whose nx*ny plane fits, about 1800
                                   points); where a plane does not fit, its cluster form (below); where
-                                  neither fits, as 1; before either of them, grids that fit on chip
-                                  run the Lanczos kernel (a thread-block cluster keeps a system's
-                                  real Lanczos vector in shared memory; the same iterates).  5 = the fused kernel warp-specialised: producer
+                                  neither fits, as 1; before either of them the Lanczos kernels run (the
+                                  same iterates from real vectors: a thread-block cluster keeps a
+                                  system's vector in shared memory, or streams its planes where it
+                                  does not fit), but for rpa_ec_gradient's subspace, for FP64 systems
+                                  without P_c at an omega of zero (below 1e-15 of the spectrum's
+                                  width), and where their workspace does not fit (see rpa_ctx).
+                                  5 = the fused kernel warp-specialised: producer
                                   threads form the next plane while consumer threads apply the
                                   stencil (planes of up to ~416 blocks of 2 x 2 points; else as 4).
                                   6 = the fused kernel's cluster form: the 2..8 blocks of a thread-
@@ -260,7 +277,9 @@ rpa_status rpa_ec(rpa_ctx *ctx, int n_r, const double *V0_dev, double *lambdas_h
  * where x_{n,i} is the projected Sternheimer solution for dV = nu^1/2 y_i.  The Sternheimer
  * operator is complex symmetric, so the adjoint solve is the forward solve; the solutions are
  * recomputed (one extra Sternheimer pass per frequency), never stored.  This derivative is not
- * in the paper; it differentiates the method's E_c (Eq. 10).
+ * in the paper; it differentiates the method's E_c (Eq. 10).  The subspace iteration runs on the complex
+ * COCG kernels (rpa_ec: on the Lanczos kernels, so that energies of the two calls agree to the
+ * tolerance), the responses on those that rpa_ec uses; what is asked for changes no value.
  * grad_dev: N_d doubles (written).  V_out_dev: N_d x n_r, the final subspace (may be NULL).
  * The other arguments and outputs are those of rpa_ec. */
 rpa_status rpa_ec_gradient(rpa_ctx *ctx, int n_r, const double *V0_dev, double *grad_dev, double *V_out_dev,

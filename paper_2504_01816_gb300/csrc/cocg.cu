@@ -2962,10 +2962,11 @@ int run_queue(Ctx &c, SolveSpec &sp, cudaStream_t st, std::vector<int> *iters_ou
     // rpa_options.stencil_shape: 0 = automatic (the fused kernel where a plane fits its ring, its
     // cluster form where a band of the plane does, else split variant 1), 1..3 = the split kernels'
     // variants, 4 = the fused kernel (as 0), 5 = its warp-specialised form, 6 = its cluster form
-    // with two blocks per SM where the bands fit (else as 0).  The plain FP64 form always runs the
-    // split kernels.  Periodic grids: the fused kernel needs even nx (point pairs wrap onto point
-    // pairs); the warp-specialised and cluster forms and the two-column split variant are Dirichlet
-    // only (the fused kernel or the first split variant stands in for them).
+    // with two blocks per SM where the bands fit (else as 0).  With 0 and 4 the Lanczos kernels come before
+    // all of them (below).  The plain FP64 form otherwise runs the split kernels.  Periodic grids: the fused
+    // kernel needs even nx (point pairs wrap onto point pairs); the warp-specialised and cluster forms and
+    // the two-column split variant are Dirichlet only (the fused kernel or the first split variant stands in
+    // for them).
     const int want = std::max(0, std::min(6, c.opt.stencil_shape));
     const bool per = c.opt.periodic != 0;
     const bool even_nx = (c.nx % 2) == 0;

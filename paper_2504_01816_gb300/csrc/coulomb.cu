@@ -200,7 +200,11 @@ __global__ void __launch_bounds__(256) k_axis_par(const double *__restrict__ in,
 }
 
 // The eigenvectors by parity for k_axis_par (empty: one has no parity, as within the degenerate pairs of a
-// periodic axis).
+// periodic axis).  The part of the other parity that is dropped is the eigensolver's error: rounding over the gap to
+// the next eigenvalue, 1e-13 at n = 40 and 6e-12 at n = 150.  It mixes neighbours, on which nu^p differs by as little as
+// their gap, so the operator is not the worse for it (against a long double eigensolver, p = 1/2: 3.46e-14
+// with all of Q, 3.42e-14 by parity at n = 40; 7.0e-13 and 5.6e-13 at n = 150), and the vectors stay orthonormal
+// (5e-14).
 std::vector<double> by_parity(const std::vector<double> &Q, int n) {
     const int h = (n + 1) / 2;
     std::vector<double> F((size_t)2 * h * h + h, 0.0);

@@ -159,10 +159,11 @@ struct Ctx {
     LanczosPlan lz_plan{};        // the last queue's plan, for lz_key = {slots, form, batch_load}
     int lz_key[3] = {-1, -1, -1};
     bool lz_ok = false;
-    // rpa_ec_gradient with the final subspace as an output runs the COCG kernels up to it: a subspace is R L^-T
-    // with the conditioning of R, and after the exact integer pieces of the tensor-core contractions
-    // (whose last digits turn on 1e-12 of their operands) the Lanczos kernel's rounding moves it by
-    // 2e-9 relative, more than a change of kernels may; the energies and the gradient move by 1e-10.
+    // Set while rpa_ec_gradient iterates its subspace: the COCG kernels.  A subspace is R L^-T with the conditioning of R,
+    // and after the exact integer pieces of the tensor-core contractions (whose last digits turn on
+    // 1e-12 of their operands) the Lanczos kernel's rounding moves it by 2e-9 relative, more than a change
+    // of kernels may; the energies and the gradient move by 1e-10.  It is one rule for every call, so that
+    // they do not depend on whether the subspace is an output.
     bool keep_cocg = false;
     SysState *h_state = nullptr;  // pinned host mirror of the slot states
     size_t h_state_cap = 0;

@@ -27,6 +27,9 @@
 // overwritten.  Every block of a cluster computes the same scalars from the same sums in the same order,
 // so all take the same decisions.  The factors, the stopping test and the slot's state belong to an extra
 // warp that works while the others compute the next stencil; a solve therefore ends one stencil late.
+// In the mixed form the dot products, a_k, g_k and the right-hand side's norms are FP32 throughout (the COCG
+// kernels add the threads' sums in FP64): what that costs in a solve its FP64 refinement makes good.  The
+// factors are FP64.
 //
 // What bounds it: shared-memory loads.  A unit of W x 2 points and ZC planes takes 2 (ZC + 12) 16-byte
 // loads for the z neighbours of all its planes (held against the ZC accumulators in turn), and per
@@ -34,7 +37,7 @@
 // a plane-by-plane march on complex values; the FP64 form is bound by the FP64 pipe (46 operations a
 // point).  Measured (GB300, tol 1e-11, whole chi0 application, against the fused and split COCG kernels):
 // 40^3, 1024 systems 212 -> 98 ms; 24^3, 4 systems 9.9 -> 1.9 ms; 37 x 43 x 29, 77 systems 25 -> 6.8 ms;
-// FP64 15^3, 32 systems 15.9 -> 3.2 ms, 32^3, 128 systems 197 -> 79 ms.  At 40^3 (four blocks a system) an
+// FP64 15^3, 32 systems 15.9 -> 2.6 ms, 32^3, 128 systems 197 -> 78 ms.  At 40^3 (four blocks a system) an
 // iteration takes 20 thousand cycles: x and y neighbours 9.4 (5.7 of shared-memory loads and 2.5 of
 // copies), z neighbours 2.8, sums 2.3, update 2.2, halo 0.3, and per iteration of a solve 1.4 of waiting for
 // the solution before it and 2.0 for the start.  With the solution formed at the end of each solve, by all
@@ -2026,6 +2029,8 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
     // streaming kernel is faster then.  An iteration on chip takes 1.5 times the cycles above.  Measured, chi0 in
     // ms, on chip and streaming: 44^3 32 systems 7.7, 15.4, 128 systems 23.7, 28.1, 256 systems 45.0, 40.7; 48^3
     // 11.0, 19.0; 38.1, 30.4; 73.3, 46.4; with four blocks, 40^3, 4096 systems 357, 429; with two, 32^3 175, 212.
+    // Periodic (one row a thread, 16 blocks on chip): 44^3 16.4, 23.9; 59.3, 51.8; 114.9, 86.5; 48^3 16.1, 31.8; 57.9,
+    // 58.2; 112.7, 96.8: the rule takes the dearer at 44^3 with 128 and at 48^3 with 256 systems (14 and 16%).
     LanczosPlan sp;
     double sc = 0.0;
     if (stream_plan(c, nsys, sms, optin, sp, sc) && (!found || sc < 0.93 * 1.5 * best_cost)) {

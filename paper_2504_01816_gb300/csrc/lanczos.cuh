@@ -25,8 +25,8 @@ template <typename T> struct LanczosArgs {
     double d0;                     // 3 a_0
 };
 
-// Plan for nsys systems of this context; false where the grid does not fit on chip (or its slabs
-// would be mostly halo) and the COCG kernels run instead.
+// Plan for nsys systems of this context; false where the grid neither fits on chip nor streams (fewer than 6 points
+// along x or y or 8 along z, planes too wide for the streaming kernel, or FP64) and the COCG kernels run instead.
 bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &p);
 // Once a queue, before its launches (p.ws set).
 void lanczos_prepare(const Ctx &c, const LanczosPlan &p, cudaStream_t s);
