@@ -672,11 +672,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
         const int x0 = (xyt % tl.ntx) * tl.tx, y0 = (xyt / tl.ntx) * tl.ty;
         const int zb = zc * tl.zlen, ze = min(nz, zb + tl.zlen);   // planes computed by this item
         const int gx = x0 + lx, gy = y0 + ly;
-        const bool own = in_tile && gx < nx && gy < ny;
-        // the last tile along an axis may reach past it: zero there, on a periodic grid the images of the first
-        // columns, which its last columns' neighbours are
-        const bool have = own || (per && in_tile);
-        const int col = own ? gy * nx + gx : have ? wrap_index(gy, ny) * nx + wrap_index(gx, nx) : 0;
+        // the last tile along an axis may reach past it (by less than the axis): zero there, on a periodic grid the
+        // images of the first columns, which its last columns' neighbours are
+        const bool have = in_tile && (per || (gx < nx && gy < ny));
+        const int col = (per && gy >= ny ? gy - ny : gy) * nx + (per && gx >= nx ? gx - nx : gx);
         auto pnew = [&](const C a, const C b) -> C {
             C o;
             o.x = a.x + br * b.x - bi * b.y;
@@ -740,7 +739,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
             f1r = rs[col + zplane(zb + R + 1) * plane];
             f1p = po[col + zplane(zb + R + 1) * plane];
         }
-        T vnext = own ? vloc[col + zb * plane] : (T)0;  // potential of the next plane
+        T vnext = have ? vloc[col + zb * plane] : (T)0;  // potential of the next plane
         T acc0 = 0, acc1 = 0;              // per-thread sums in the working precision (FP64 is slow)
         // The z loop is unrolled by the window length: slot (u + m) % 13 of qv holds plane z-6+m,
         // so the window turns without moving registers.
@@ -774,9 +773,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
                     f2p = po[col + zplane(z + R + 2) * plane];
                 }
                 const T vz = vnext;                          // potential of plane z (loaded one plane ago)
-                if (own && z + 1 < ze) vnext = vloc[col + (z + 1) * plane];
+                if (have && z + 1 < ze) vnext = vloc[col + (z + 1) * plane];
                 __syncthreads();
-                if (own) {
+                if (have && gx < nx && gy < ny) {            // a flag kept for it costs 5% (periodic, FP32)
                     const int idx = col + z * plane;
                     const C c = qv[(u + R) % (2 * R + 1)];
                     const T dre = (T)3 * cf.a[0] + vz + sre;
