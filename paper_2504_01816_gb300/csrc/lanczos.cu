@@ -260,6 +260,7 @@ template <typename T> struct Shared {
     unsigned opened;                     // jobs whose coefficients are there
     int item[2], flag;
     unsigned gone;                       // a wait ran out (wait_lost; 0: none did)
+    int tell;                            // the blocks told of it (0: this one)
     int taken;                           // on chip: the system taken last (first block)
     int nto, to[4 * 12];                 // the copies that fill the neighbours' halos
     unsigned expect;                     // bytes that arrive in this block's halo
@@ -352,8 +353,9 @@ __device__ __forceinline__ void put(T *own, int gx, int nvx, int nx, const Pk<T>
 // (start_part), and leave the launch before the next system.  The mark is the number of reductions (ng)
 // behind that barrier: a decision counts the marks up to its own number only, so that one made meanwhile by a
 // thread that is ahead does not divide those that still have to decide.
-template <typename T> __device__ __noinline__ void wait_lost(unsigned mark, int ncl) {
+template <typename T> __device__ __noinline__ void wait_lost(unsigned mark) {
     Shared<T> &S = sh<T>();
+    const int ncl = S.tell;
     atomicExch(S.A.err, 2);
     if (ncl == 0) atomicCAS(&S.gone, 0u, mark);          // this block; the first mark stands
     for (int t = 0; t < ncl; ++t) {
@@ -417,9 +419,9 @@ __device__ __forceinline__ void keep_wait() { asm volatile("cp.async.bulk.wait_g
 // sends its sums to all (st.async, which counts on the receiver's barrier) and waits for all.  A block
 // sends only after all its threads are done with the stencil, so the wait also says that no block reads
 // its halo any more.  The sums alternate between two buffers and barriers: a block may be one
-// reduction ahead of another, never two.  tell: the blocks told of a lost wait (wait_lost).
+// reduction ahead of another, never two.
 template <typename T>
-__device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int nmain, int tell) {
+__device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, int rank, int nmain) {
     Shared<T> &S = sh<T>();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = nmain >> 5;
     T v[3] = {a, b, c};
@@ -448,7 +450,7 @@ __device__ __forceinline__ void gather3(T a, T b, T c, unsigned &ng, int ncl, in
                       v[0], v[1], v[2]);
         __syncwarp();
     }
-    if (!mbar_wait(pb, (ng >> 1) & 1)) wait_lost<T>(ng + 1, tell);
+    if (!mbar_wait(pb, (ng >> 1) & 1)) wait_lost<T>(ng + 1);
     ++ng;
 }
 template <typename T> __device__ __forceinline__ void sum_parts(unsigned ng, int ncl, T &a, T &b, T &c) {   // after gather3
@@ -824,7 +826,7 @@ template <typename T, int ZC> __device__ __forceinline__ void finish_job(int nma
 // The scalar lane then: the flush warps are done with it too (njobs posted so far).  False where the wait ran out.
 template <typename T> __device__ __forceinline__ bool jobs_done(unsigned njobs, unsigned ng) {
     const bool ok = njobs == 0 || mbar_wait((unsigned)__cvta_generic_to_shared(&sh<T>().job_done), (njobs - 1) & 1);
-    if (!ok) wait_lost<T>(ng + 1, 0);
+    if (!ok) wait_lost<T>(ng + 1);
     return ok;
 }
 // ... and the next (not posted where the wait ran out: the flush warps still read the last).
@@ -895,6 +897,7 @@ template <typename T, int ZC> __device__ __noinline__ void block_setup(const Lan
         mbar_init(&S.job_done);
         S.next = 1 << 30;                                // no job
         S.gone = 0;
+        S.tell = 0;
         S.taken = 1 << 30;
         S.opened = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -982,7 +985,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
     if (scalar) fetch(0);
     for (;; ++ns) {
         const bool here = mbar_wait((unsigned)__cvta_generic_to_shared(&S.ibar[ns & 1]), (ns >> 1) & 1);
-        if (!here) wait_lost<T>(ng + 1, 0);
+        if (!here) wait_lost<T>(ng + 1);
         if (main_any(nmain, !here || left<T>(ng))) {    // the item is not to be read, or a solve has ended so
             if (scalar) leave<T>(G.rank, n_items, njobs, ng);
             cluster_barrier();
@@ -995,7 +998,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
         {
             T rr, ii, ri;
             start_sums<T, ZC>(s, rr, ii, ri);
-            gather3(rr, ii, ri, ng, ncl, G.rank, nmain, 0);
+            gather3(rr, ii, ri, ng, ncl, G.rank, nmain);
             if (scalar && !left<T>(ng)) {
                 fetch(ns + 1);                           // every block has read the number before this one
                 T a, b, c;
@@ -1112,7 +1115,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                         }
                     }
                 }
-                if (!mbar_wait((unsigned)__cvta_generic_to_shared(&S.bar), phase)) wait_lost<T>(ng + 1, 0);
+                const bool halo = mbar_wait((unsigned)__cvta_generic_to_shared(&S.bar), phase);
+                if (!halo) wait_lost<T>(ng + 1);
                 phase ^= 1u;
                 if (G.unit) {
 #pragma unroll
@@ -1147,7 +1151,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                     suv = t1.sum();
                     suu = t2.sum();
                 }
-                gather3(svv, suv, suu, ng, ncl, G.rank, nmain, 0);
+                gather3(svv, suv, suu, ng, ncl, G.rank, nmain);
                 if (S.flag) {                            // the last step ended the solve (k = kb: a lost wait)
                     n = k - kb;
                     break;
@@ -1192,7 +1196,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                                         }
                                 }
                         }
-                        gather3((T)0, t1.sum(), t2.sum(), ng, ncl, G.rank, nmain, 0);
+                        gather3((T)0, t1.sum(), t2.sum(), ng, ncl, G.rank, nmain);
                         if (scalar) {
                             T a, b, c;
                             sum_parts(ng, ncl, a, b, c);
@@ -1253,7 +1257,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_lanczos(const __grid_constant__ Lan
                         acc[z][1] = pk_load_l2(hl + G.c1 + z * A.plane);
                     }
                 }
-                if (scalar && !left<T>(ng)) {            // (a lost halo's barrier is not armed again)
+                if (scalar && halo) {                    // (a lost halo's barrier is not armed again)
                     const Work<T, ZC> K(A);
                     send_halos(slab);
                     keep(slab, K.H + buf * K.buf, K.hvec, k - kb, G.nzl, A.plane);
@@ -1576,6 +1580,7 @@ __global__ void __launch_bounds__(MAXT, 1)
         for (int q = 0; q < 2; ++q) mbar_init(&S.pbar[q]);
         for (int q = 0; q < kStages; ++q) mbar_init(&S.full[q]);
         S.gone = 0;
+        S.tell = ncl;
         S.A.err = A.L.err;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1609,7 +1614,7 @@ __global__ void __launch_bounds__(MAXT, 1)
         {
             float rr, ii, ri;
             stream_start<R>(&A, s, 0.f, 0.f, false, rr, ii, ri);
-            gather3(rr, ii, ri, ng, ncl, G.rank, (int)blockDim.x, ncl);
+            gather3(rr, ii, ri, ng, ncl, G.rank, (int)blockDim.x);
             if (scalar) {
                 float a, b, c;
                 sum_parts(ng, ncl, a, b, c);
@@ -1790,7 +1795,7 @@ __global__ void __launch_bounds__(MAXT, 1)
 #pragma unroll
                     for (int j = 0; j < kRadius; ++j) put_u(acc[j]);
                 before_bulk();                           // u and v_k, for the next sweep's copies
-                gather3(svv.x + svv.y, suv.x + suv.y, suu.x + suu.y, ng, ncl, G.rank, (int)blockDim.x, ncl);
+                gather3(svv.x + svv.y, suv.x + suv.y, suu.x + suu.y, ng, ncl, G.rank, (int)blockDim.x);
                 {
                     float a, b, c;
                     sum_parts(ng, ncl, a, b, c);
@@ -1805,15 +1810,16 @@ __global__ void __launch_bounds__(MAXT, 1)
                     S.F.ck = (double)cc;
                     S.F.ig = (double)ig;
                     factor<float>(0, k - 1 - kb, k, A.L.maxit);
-                    if (!G4.ok) wait_lost<float>(ng, ncl);
+                    if (!G4.ok) wait_lost<float>(ng);
                     if (A.L.prof && G.rank == 0) atomicAdd(A.L.prof + 1, (unsigned long long)A.L.nd);
                 }
                 cc = ig > 0.f ? 1.f / ig : 0.f;
                 dg -= ap;
                 cluster_barrier();                       // u and v_k of every band are written; the decision is taken
                 n = k - kb;
-                // (a vote: as a plain condition it costs the plane loop 8 registers and 2.5% of the call)
-                if (__any_sync(0xffffffffu, S.flag != 0 || left<float>(ng))) break;
+                // (a vote: as a plain condition it costs the plane loop 8 registers and 2.5% of the call, and wait_lost with
+                // the cluster's size as an argument 2% at 51 x 44 x 51)
+                if (S.flag || __any_sync(0xffffffffu, left<float>(ng))) break;
                 if (n == A.L.hist) {                     // the history is full: into x and p
                     G4 = stream_flush<R>(&A, s, n, true, have_p, pt ? -S.start[1] : S.start[0], pt ? S.start[0] : S.start[1], G4);
                     have_p = true;
