@@ -45,7 +45,7 @@ extern "C" {
 
 /* A context keeps the device memory of its largest calls until it is destroyed: up to 8 GB for the
  * systems in flight (the contexts of a batch together) and up to 4 GB (grids solved on chip) or 8 GB
- * (streamed) of Lanczos vectors (batches: about 16 GB together).  The Lanczos vectors are optional: a call that finds no
+ * (streamed) of Lanczos vectors (batches: about 16 or 32 GB together).  The Lanczos vectors are optional: a call that finds no
  * room for them (512 MB stay free) runs the COCG kernels, and a device allocation of the library that
  * fails takes back those that no running call uses, on all contexts of the device, before it reports
  * RPA_ERR_OOM.

@@ -1882,10 +1882,11 @@ void cluster_config(cudaLaunchConfig_t &lc, cudaLaunchAttribute &at, int ncl, in
 
 }  // namespace
 
-// Bytes of a history buffer: `most` for a context by itself, the share (by systems) of twice that for a batch's.
+// Bytes of a history buffer: `most` for a context by itself, the share (by systems) of four times that for a batch's
+// (of twice that, a history of 113 vectors instead of 128 cost a batch of 29 x 34 x 26 .. 33 x 25 x 34, 177 solves, 1%).
 static size_t history_budget(const Ctx &c, int nsys, size_t most) {
     if (c.batch_load <= nsys) return most;
-    return std::min(most, (size_t)(2.0 * (double)most * nsys / c.batch_load));
+    return std::min(most, (size_t)(4.0 * (double)most * nsys / c.batch_load));
 }
 
 // Plan of the streaming kernel: threads of one or two rows and 1 to 8 bands, of which a block's threads take every
@@ -1950,7 +1951,7 @@ static bool stream_plan(const Ctx &c, int nsys, int sms, int optin, LanczosPlan 
     if (best == 1e300) return false;
     cycles = best;
     const size_t nv = (size_t)c.nz * c.ny * px;
-    // history: as many vectors as 8 GB hold, 16 .. kHistMax (a batch: its share of 16 GB, by systems)
+    // history: as many vectors as 8 GB hold, 16 .. kHistMax (a batch: its share of 32 GB, by systems)
     const size_t most = history_budget(c, nsys, (size_t)8 << 30);
     p.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, most / (nv * 4 * p.clusters)));
     p.ws_stride = nv * (4 + p.hist);
@@ -2046,7 +2047,7 @@ bool lanczos_plan(const Ctx &c, int nsys, LanczosPlan &best) {
     if (!found) return false;
     best.stream = 0;
     const size_t vec = (size_t)2 * best.zc * (best.threads - kExtra) * W, hvec = (size_t)best.nch * best.zc * best.plane;
-    // history: as many vectors as 2 GB hold in each of its two buffers, 16 .. kHistMax (a batch: its share of 4 GB)
+    // history: as many vectors as 2 GB hold in each of its two buffers, 16 .. kHistMax (a batch: its share of 8 GB)
     const size_t per_vec = hvec * tsz * best.clusters * best.ncl;
     best.hist = (int)std::max<size_t>(16, std::min<size_t>(kHistMax, history_budget(c, nsys, (size_t)2 << 30) / per_vec));
     best.ws_stride = vec + 2 * hvec + 2 * hvec * best.hist;
